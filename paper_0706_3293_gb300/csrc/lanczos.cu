@@ -10,6 +10,7 @@
 #include "ef64.cuh"
 #include "hm_row.cuh"
 #include "s1blk.cuh"
+#include "tridiag.cuh"
 
 namespace hm {
 
@@ -470,128 +471,54 @@ __global__ void k_lz_beta(LzScalars *S, const double *__restrict__ part, int nbl
     }
 }
 
-// ---- tridiagonal T (diagonal al[0..m), off-diagonal be[0..m-1)) ------------------------
+// ---- tridiagonal T: eigenvalues and eigenvectors by tridiag.cuh, one CTA each ----------
 
-__device__ int sturm_count(int m, const double *al, const double *be, double x, double pivmin) {
-    int c = 0;
-    double q = al[0] - x;
-    if (fabs(q) < pivmin) q = -pivmin;
-    if (q < 0) ++c;
-    for (int i = 1; i < m; ++i) {
-        q = (al[i] - x) - be[i - 1] * be[i - 1] / q;
-        if (fabs(q) < pivmin) q = -pivmin;
-        if (q < 0) ++c;
-    }
-    return c;
+// CTA e: the e-th lowest Ritz value
+__global__ void __launch_bounds__(TRI_NT) k_ritz(const LzScalars *S, const double *alpha, const double *beta,
+                                              double *ritz) {
+    const int e = blockIdx.x, m = S->j;
+    const double v = m >= 1 && e < m ? tri_eig(m, alpha, beta, e + 1) : __longlong_as_double(0x7ff8000000000000ll);
+    if (threadIdx.x == 0) ritz[e] = v;
 }
 
-// e-th lowest eigenvalue (1-based) by bisection of the Sturm count on the Gershgorin
-// interval, until the midpoint no longer moves
-__device__ double tri_eig(int m, const double *al, const double *be, int e) {
-    double lo = 1e308, hi = -1e308, bmax = 0.0;
-    for (int i = 0; i < m; ++i) {
-        double r = (i > 0 ? fabs(be[i - 1]) : 0.0) + (i < m - 1 ? fabs(be[i]) : 0.0);
-        lo = fmin(lo, al[i] - r);
-        hi = fmax(hi, al[i] + r);
-        if (i < m - 1) bmax = fmax(bmax, fabs(be[i]));
-    }
-    const double pivmin = 2.2250738585072014e-308 * fmax(1.0, bmax * bmax);
-    const double pad = 2.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi)) + pivmin;
-    double a = lo - pad, c = hi + pad;
-    for (int it = 0; it < 400; ++it) {
-        double mid = 0.5 * (a + c);
-        if (mid <= a || mid >= c) break;
-        if (sturm_count(m, al, be, mid, pivmin) >= e) c = mid; else a = mid;
-    }
-    return 0.5 * (a + c);
-}
-
-// eigenvector of T for eigenvalue th by inverse iteration: three solves of
-// (T - th I) z = b with Gaussian elimination and partial pivoting (one extra
-// super-diagonal of fill-in); z normalised, returned in z[0..m)
-__device__ void tri_vec(int m, const double *al, const double *be, double th, double *z,
-                        double *d, double *du, double *du2, double *dl) {
-    if (m == 1) { z[0] = 1.0; return; }
-    double tnorm = 0.0;
-    for (int i = 0; i < m; ++i) tnorm = fmax(tnorm, fabs(al[i]) + (i > 0 ? fabs(be[i - 1]) : 0.0) + (i < m - 1 ? fabs(be[i]) : 0.0));
-    const double tiny = fmax(tnorm, 1e-300) * 2.220446049250313e-16;
-    for (int i = 0; i < m; ++i) z[i] = 1.0 / sqrt((double)m) * (1.0 + 1e-3 * (double)(i % 7));
-    for (int it = 0; it < 3; ++it) {
-        for (int i = 0; i < m; ++i) d[i] = al[i] - th;
-        for (int i = 0; i < m - 1; ++i) { du[i] = be[i]; dl[i] = be[i]; }
-        for (int i = 0; i < m; ++i) du2[i] = 0.0;
-        double *b = z;
-        for (int i = 0; i < m - 1; ++i) {
-            if (fabs(d[i]) >= fabs(dl[i])) {
-                if (d[i] == 0.0) d[i] = tiny;
-                const double f = dl[i] / d[i];
-                d[i + 1] -= f * du[i];
-                b[i + 1] -= f * b[i];
-            } else {
-                const double f = d[i] / dl[i];
-                d[i] = dl[i];
-                const double t = d[i + 1];
-                d[i + 1] = du[i] - f * t;
-                du[i] = t;
-                if (i < m - 2) {
-                    du2[i] = du[i + 1];
-                    du[i + 1] = -f * du[i + 1];
-                }
-                const double tb = b[i];
-                b[i] = b[i + 1];
-                b[i + 1] = tb - f * b[i + 1];
-            }
-        }
-        if (d[m - 1] == 0.0) d[m - 1] = tiny;
-        b[m - 1] = b[m - 1] / d[m - 1];
-        b[m - 2] = (b[m - 2] - du[m - 2] * b[m - 1]) / d[m - 2];
-        for (int i = m - 3; i >= 0; --i) b[i] = (b[i] - du[i] * b[i + 1] - du2[i] * b[i + 2]) / d[i];
-        double nn = 0.0;
-        for (int i = 0; i < m; ++i) nn += b[i] * b[i];
-        nn = 1.0 / sqrt(nn);
-        for (int i = 0; i < m; ++i) b[i] *= nn;
-    }
-}
-
-__global__ void k_ritz(const LzScalars *S, const double *alpha, const double *beta, int n_ritz, double *ritz) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    const int m = S->j;
-    if (e >= n_ritz) return;
-    ritz[e] = (m >= 1 && e < m) ? tri_eig(m, alpha, beta, e + 1) : __longlong_as_double(0x7ff8000000000000ll);
-}
-
-// Convergence of the lowest Ritz pair of every leading T_k (k = 1..m): thread k computes
+// Convergence of the lowest Ritz pair of every leading T_k (k = 1..m): CTA k - 1 computes
 // theta_1(T_k) and the last component s_k of its eigenvector; the residual norm of the
 // Ritz pair is beta_k |s_k|.  res[k-1] = beta_k |s_k| / max(1, |theta|).
-__global__ void k_conv_scan(const LzScalars *S, const double *alpha, const double *beta,
-                            double *scratch, int max_steps, double *res) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x + 1;
-    const int m = S->j;
-    if (k > m) return;
-    double *z = scratch + (size_t)(k - 1) * (5 * (size_t)max_steps + 4);
-    double *d = z + max_steps, *du = d + max_steps, *du2 = du + max_steps, *dl = du2 + max_steps;
+__global__ void __launch_bounds__(TRI_NT) k_conv_scan(const LzScalars *S, const double *alpha, const double *beta,
+                                                   double *scratch, int max_steps, double *res) {
+    const int k = blockIdx.x + 1;
+    if (k > S->j) return;
+    double *f = scratch + (size_t)(k - 1) * (5 * (size_t)max_steps + 4);
     const double th = tri_eig(k, alpha, beta, 1);
-    tri_vec(k, alpha, beta, th, z, d, du, du2, dl);
-    res[k - 1] = beta[k - 1] * fabs(z[k - 1]) / fmax(1.0, fabs(th));
+    if (threadIdx.x >= 32) return;
+    const double sk = tri_vec(k, alpha, beta, th, nullptr, f, f + max_steps);
+    if (threadIdx.x == 0) res[k - 1] = beta[k - 1] * sk / fmax(1.0, fabs(th));
 }
 
 // picks the shortest converged Krylov length (res <= tol), or m; computes the lowest
-// eigenvector of T_mconv into coef, and e0 / e1 into ritz[0], ritz[1]
-__global__ void k_pick_and_vec(LzScalars *S, const double *alpha, const double *beta,
-                               double *scratch, int max_steps, const double *res, double tol,
-                               double *coef, double *ritz) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    const int m = S->j;
+// eigenvector of T_mconv into coef (CTA 0), and e0 / e1 into ritz[0], ritz[1] (CTA 0 / 1)
+__global__ void __launch_bounds__(TRI_NT) k_pick_and_vec(LzScalars *S, const double *alpha, const double *beta,
+                                                      double *scratch, int max_steps, const double *res, double tol,
+                                                      double *coef, double *ritz) {
+    const int m = S->j, lane = threadIdx.x & 31;
     int mc = m;
-    for (int k = 1; k <= m; ++k)
-        if (res[k - 1] <= tol) { mc = k; break; }
-    S->mconv = mc;
-    double *d = scratch, *du = d + max_steps, *du2 = du + max_steps, *dl = du2 + max_steps;
+    for (int k0 = 0; k0 < m; k0 += 32) {
+        const unsigned ok = __ballot_sync(0xffffffffu, k0 + lane < m && res[k0 + lane] <= tol);
+        if (ok) { mc = k0 + __ffs(ok); break; }
+    }
+    if (blockIdx.x == 1) {
+        const double e1 = mc >= 2 ? tri_eig(mc, alpha, beta, 2) : __longlong_as_double(0x7ff0000000000000ll);
+        if (threadIdx.x == 0) ritz[1] = e1;
+        return;
+    }
     const double th = tri_eig(mc, alpha, beta, 1);
-    ritz[0] = th;
-    ritz[1] = mc >= 2 ? tri_eig(mc, alpha, beta, 2) : __longlong_as_double(0x7ff0000000000000ll);
-    tri_vec(mc, alpha, beta, th, coef, d, du, du2, dl);
-    for (int k = mc; k < max_steps; ++k) coef[k] = 0.0;
+    if (threadIdx.x >= 32) return;
+    tri_vec(mc, alpha, beta, th, coef, scratch, scratch + max_steps);
+    for (int k = mc + lane; k < max_steps; k += 32) coef[k] = 0.0;
+    if (lane == 0) {
+        S->mconv = mc;
+        ritz[0] = th;
+    }
 }
 
 __global__ void k_scale(double *__restrict__ v, uint64_t n, const LzScalars *S) {
@@ -837,9 +764,10 @@ static int run_steps_graph(hm_lanczos *R, int steps, cudaStream_t st) {
 
 // lowest Ritz value, steps done and status of one run (device, out[0..2]); NaN without steps
 __global__ void k_branch_out(const LzScalars *S, const double *alpha, const double *beta, double *out) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int m = S->j;
-    out[0] = m >= 1 ? tri_eig(m, alpha, beta, 1) : __longlong_as_double(0x7ff8000000000000ll);
+    const double e0 = m >= 1 ? tri_eig(m, alpha, beta, 1) : __longlong_as_double(0x7ff8000000000000ll);
+    if (threadIdx.x != 0) return;
+    out[0] = e0;
     out[1] = (double)m;
     out[2] = (double)S->status;
 }
@@ -884,7 +812,7 @@ int lz_branches(const std::vector<const hm_basis *> &bases, int n_bonds, const i
                 rc = enqueue_start(runs[i], nullptr, seeds[i], br[i]);
                 for (int k = 0; k < steps && rc == HM_OK; ++k) rc = enqueue_step(runs[i], br[i]);
                 if (rc != HM_OK) break;
-                k_branch_out<<<1, 32, 0, br[i]>>>(runs[i]->sc, runs[i]->alpha, runs[i]->beta, out + 3 * i);
+                k_branch_out<<<1, TRI_NT, 0, br[i]>>>(runs[i]->sc, runs[i]->alpha, runs[i]->beta, out + 3 * i);
                 if ((e = cudaGetLastError()) != cudaSuccess) { rc = cuda_fail(e, "k_branch_out"); break; }
                 if ((e = cudaEventRecord(done[i], br[i])) != cudaSuccess || (e = cudaStreamWaitEvent(cap, done[i], 0)) != cudaSuccess)
                     rc = cuda_fail(e, "join");
@@ -1000,7 +928,7 @@ int lanczos_run(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t 
     int rc = run_steps_graph(R, steps, st);
     double *d_ritz = (double *)(R->work + R->L.ritz);
     if (rc == HM_OK && n_ritz > 0) {
-        k_ritz<<<1, 64, 0, st>>>(R->sc, R->alpha, R->beta, n_ritz, d_ritz);
+        k_ritz<<<n_ritz, TRI_NT, 0, st>>>(R->sc, R->alpha, R->beta, d_ritz);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "k_ritz");
     }
@@ -1034,8 +962,8 @@ int e0_grad(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v, 
     if (rc == HM_OK) {
         // residual of the lowest Ritz pair of every leading T_k, then the shortest
         // converged length and the eigenvector of T there (no ghost copies yet)
-        k_conv_scan<<<(steps + 63) / 64, 64, 0, st>>>(R->sc, R->alpha, R->beta, tri, steps, res);
-        k_pick_and_vec<<<1, 1, 0, st>>>(R->sc, R->alpha, R->beta, tri, steps, res, 1e-10, R->coef, d_ritz);
+        k_conv_scan<<<steps, TRI_NT, 0, st>>>(R->sc, R->alpha, R->beta, tri, steps, res);
+        k_pick_and_vec<<<2, TRI_NT, 0, st>>>(R->sc, R->alpha, R->beta, tri, steps, res, 1e-10, R->coef, d_ritz);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "e0_grad: eigenvector");
     }

@@ -1,0 +1,36 @@
+"""GPU tests of the tridiagonal eigensolvers (csrc/tridiag.cuh, the Ritz values of lanczos_run, and
+the finite-temperature eigen-decomposition) at the edges of their 32-row chunks."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_0706_3293_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def hm():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_0706_3293_gb300 import api
+    return api
+
+
+@pytest.mark.parametrize("m", [1, 2, 7, 8, 9, 31, 32, 33, 63, 64, 65, 130])
+def test_ritz_values_vs_lapack(hm, m):
+    """Every Ritz value of T_m (up to 64 of them) against LAPACK on the returned alpha, beta, ghosts
+    included.  Bound: the minors' rounding perturbs the entries of T by at most 7 eps of its
+    Gershgorin bound, the bracket adds one eps, LAPACK's own error is at most m eps."""
+    inst = W.small_ring(14, -1.0, -0.4)
+    b = hm.Basis(inst.n_sites, inst.two_s, inst.two_m)
+    r = hm.lanczos_run(b, hm.bonds_of(inst), m, seed=5, n_ritz=min(m + 2, 64))
+    al, be = r.alpha, r.beta
+    assert r.steps_done == m
+    T = np.diag(al) + np.diag(be[: m - 1], 1) + np.diag(be[: m - 1], -1)
+    ref = np.linalg.eigvalsh(T)
+    n = min(m, 64)
+    bound = np.abs(T).sum(1).max()
+    assert np.abs(r.ritz[:n] - ref[:n]).max() <= (8 + m) * np.finfo(float).eps * bound
+    assert np.isnan(r.ritz[n:]).all()                    # past the dimension of T
