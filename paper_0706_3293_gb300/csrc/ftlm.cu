@@ -559,6 +559,11 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
 // Implicit symmetric QR with Wilkinson shifts (Golub and Van Loan, Sec. 8.3): each sweep
 // chases a bulge down the unreduced block with Givens rotations; the rotations are also
 // applied to z, the first row of the accumulated eigenvector matrix.
+// One thread per matrix: a sweep is one chain of dependent binary64 operations, so its
+// number is what counts.  A rotation takes its cosine and sine from one rsqrt (six binary64
+// instructions where hypot and two divisions took forty), and the values the next rotation
+// needs stay in registers.  T is scaled to norm 1, so squares
+// neither overflow nor lose anything that matters when they underflow.
 __device__ void tri_ql_first(int m, double *dg, double *e, double *z) {
     for (int i = 0; i < m; ++i) z[i] = i == 0 ? 1.0 : 0.0;
     int hi = m - 1, guard = 0;
@@ -573,43 +578,62 @@ __device__ void tri_ql_first(int m, double *dg, double *e, double *z) {
         const double eh = e[hi - 1];
         const double den = dd + copysign(sqrt(dd * dd + eh * eh), dd == 0.0 ? 1.0 : dd);
         const double mu = dg[hi] - eh * eh / den;
-        double x = dg[lo] - mu, y = e[lo];
+        double a = dg[lo], b = e[lo], zk = z[lo], x = a - mu, y = b;
         for (int kk = lo; kk < hi; ++kk) {
-            const double r = hypot(x, y);
-            const double c = r == 0.0 ? 1.0 : x / r, s = r == 0.0 ? 0.0 : y / r;
-            if (kk > lo) e[kk - 1] = r;
-            const double a = dg[kk], b = e[kk], cc = dg[kk + 1];
-            dg[kk] = c * c * a + 2.0 * c * s * b + s * s * cc;
-            dg[kk + 1] = s * s * a - 2.0 * c * s * b + c * c * cc;
-            e[kk] = c * s * (cc - a) + (c * c - s * s) * b;
-            const double zk = z[kk], zk1 = z[kk + 1];
+            const double cc = dg[kk + 1], zk1 = z[kk + 1], en = kk + 1 < hi ? e[kk + 1] : 0.0;
+            const double r2 = fma(x, x, y * y);
+            const double ri = rsqrt(r2);
+            const double c = r2 > 0.0 ? x * ri : 1.0, s = r2 > 0.0 ? y * ri : 0.0;
+            if (kk > lo) e[kk - 1] = r2 > 0.0 ? r2 * ri : 0.0;
+            const double c2 = c * c, s2 = s * s, cs = c * s, csb = 2.0 * cs * b;
+            dg[kk] = c2 * a + csb + s2 * cc;
+            x = cs * (cc - a) + (c2 - s2) * b;
+            a = s2 * a - csb + c2 * cc;
             z[kk] = c * zk + s * zk1;
-            z[kk + 1] = -s * zk + c * zk1;
-            if (kk + 1 < hi) {
-                x = e[kk];
-                y = s * e[kk + 1];
-                e[kk + 1] = c * e[kk + 1];
-            }
+            zk = c * zk1 - s * zk;
+            y = s * en;
+            b = c * en;
         }
+        dg[hi] = a;
+        e[hi - 1] = x;
+        z[hi] = zk;
     }
 }
 
-__global__ void k_ft_eig(FtParams F, double *scratch) {
+// theta and tau of every (sector, vector): FT_EIG matrices to a CTA.  Few to a CTA spreads
+// the chains over the SMs (a warp's binary64 instruction occupies its quarter of an SM for 64
+// cycles however many lanes take part) and keeps lanes with unequal deflation patterns apart:
+// 25.7 ms with 128 to a CTA and the hypot form against 12.7 ms at N = 20, 672 matrices of 80
+// rows.
+constexpr int FT_EIG = 4;
+__host__ __device__ __forceinline__ size_t ft_eig_smem(int steps) {
+    const size_t b = (size_t)FT_EIG * 3 * steps * 8;
+    return b <= 40 * 1024 ? b : 0;                     // more rows: the scratch in device memory
+}
+
+__global__ void __launch_bounds__(FT_EIG) k_ft_eig(FtParams F, double *scratch) {
+    extern __shared__ __align__(16) double ft_eig_sh[];
     const FtDev &d = F.d;
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * FT_EIG + threadIdx.x;
     if (t >= F.nsec * FT_W) return;
     const int v = t % FT_W;
     if ((F.exact_mask >> (t / FT_W)) & 1ull) return;   // filled by k_ft_exact
     const int m = (v < F.R) ? d.nsteps[t] : 0;
     d.mlen[t] = m;
     if (m == 0) return;
-    double *dg = scratch + (size_t)t * 3 * F.steps, *e = dg + F.steps, *z = e + F.steps;
-    for (int i = 0; i < m; ++i) dg[i] = d.alpha[(size_t)t * F.steps + i];
-    for (int i = 0; i + 1 < m; ++i) e[i] = d.beta[(size_t)t * F.steps + i];
+    double *dg = ft_eig_smem(F.steps) ? ft_eig_sh + (size_t)threadIdx.x * 3 * F.steps
+                                      : scratch + (size_t)t * 3 * F.steps;
+    double *e = dg + F.steps, *z = e + F.steps;
+    const double *al = d.alpha + (size_t)t * F.steps, *be = d.beta + (size_t)t * F.steps;
+    double nrm = 0.0;
+    for (int i = 0; i < m; ++i) nrm = fmax(nrm, fmax(fabs(al[i]), i + 1 < m ? fabs(be[i]) : 0.0));
+    const int ex = nrm > 0.0 && nrm < 1e308 ? min(max(ilogb(nrm), -1000), 1000) : 0;
+    for (int i = 0; i < m; ++i) dg[i] = ldexp(al[i], -ex);
+    for (int i = 0; i + 1 < m; ++i) e[i] = ldexp(be[i], -ex);
     if (m > 1) e[m - 1] = 0.0;
     tri_ql_first(m, dg, e, z);
     for (int i = 0; i < m; ++i) {
-        d.theta[(size_t)t * F.steps + i] = dg[i];
+        d.theta[(size_t)t * F.steps + i] = ldexp(dg[i], ex);
         d.tau[(size_t)t * F.steps + i] = z[i] * z[i];
     }
 }
@@ -717,52 +741,82 @@ __global__ void __launch_bounds__(256) k_ft_exact(FtParams F, BondParams bp, con
     for (int r = threadIdx.x; r < FT_W; r += blockDim.x) d.mlen[(size_t)ex.A * FT_W + r] = r < F.R ? n : 0;
 }
 
-// one block: e_ref = min theta, then Z and E sums for each temperature (fixed order)
-__global__ void k_ft_thermo(FtParams F, const double *temps, int n_t) {
+// Thermal sums.  Every (temperature, Ritz value) pair costs an exponential, about 25 binary64
+// operations on a pipe that takes 1.7 a cycle and SM: on one SM the 1.3 M pairs of 24
+// temperatures at N = 20 took 8.9 ms, over all of them 0.09 ms.
+// mins[s] = lowest Ritz value of sector s
+__global__ void __launch_bounds__(256) k_ft_min(FtParams F, double *__restrict__ mins) {
     const FtDev &d = F.d;
-    __shared__ double red[32];
-    __shared__ double s_ref;
-    const int nst = F.nsec * FT_W;
+    __shared__ double red[8];
+    const int s = blockIdx.x;
     double mn = 1e308;
-    for (int t = threadIdx.x; t < nst; t += blockDim.x)
-        for (int i = 0; i < d.mlen[t]; ++i) mn = fmin(mn, d.theta[(size_t)t * F.steps + i]);
+    for (int p = threadIdx.x; p < F.R * F.steps; p += 256) {
+        const int t = s * FT_W + p / F.steps, i = p % F.steps;
+        if (i < d.mlen[t]) mn = fmin(mn, d.theta[(size_t)t * F.steps + i]);
+    }
     for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_down_sync(0xffffffffu, mn, o));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mn;
     __syncthreads();
     if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) mn = fmin(mn, red[w]);
+        mins[s] = mn;
+    }
+}
+
+// CTA (s, it): the sums of sector s at temperature temps[it], zs / es [it nsec + s]
+__global__ void __launch_bounds__(256) k_ft_thermo(FtParams F, const double *__restrict__ temps,
+                                                    const double *__restrict__ mins, double *__restrict__ zs,
+                                                    double *__restrict__ es) {
+    const FtDev &d = F.d;
+    __shared__ double red[8];
+    const int s = blockIdx.x, it = blockIdx.y;
+    double e_ref = 1e308;
+    for (int k = 0; k < F.nsec; ++k) e_ref = fmin(e_ref, mins[k]);
+    const double T = temps[it], wgt = (double)d.secdim[s] / (double)F.R;
+    double z = 0.0, ez = 0.0;
+    for (int p = threadIdx.x; p < F.R * F.steps; p += 256) {
+        const int t = s * FT_W + p / F.steps, i = p % F.steps;
+        if (i < d.mlen[t]) {
+            const double th = d.theta[(size_t)t * F.steps + i];
+            const double b = d.tau[(size_t)t * F.steps + i] * exp(-(th - e_ref) / T) * wgt;
+            z += b;
+            ez += b * th;
+        }
+    }
+    z = block_sum<256>(z, red);
+    __syncthreads();
+    ez = block_sum<256>(ez, red);
+    if (threadIdx.x == 0) {
+        zs[(size_t)it * F.nsec + s] = z;
+        es[(size_t)it * F.nsec + s] = ez;
+    }
+}
+
+// e_ref, Z and E from the sectors' sums, in sector order
+__global__ void __launch_bounds__(256) k_ft_thermo_fin(FtParams F, const double *__restrict__ mins,
+                                                        const double *__restrict__ zs, const double *__restrict__ es,
+                                                        int n_t) {
+    const FtDev &d = F.d;
+    const int it = blockIdx.x * 256 + threadIdx.x;
+    if (it == 0) {
         double m = 1e308;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmin(m, red[w]);
-        s_ref = m;
+        for (int k = 0; k < F.nsec; ++k) m = fmin(m, mins[k]);
         *d.eref = m;
     }
-    __syncthreads();
-    const double e_ref = s_ref;
-    for (int it = 0; it < n_t; ++it) {
-        const double T = temps[it];
-        double z = 0.0, ez = 0.0;
-        for (int t = threadIdx.x; t < nst; t += blockDim.x) {
-            const int s = t / FT_W;
-            const double wgt = (double)d.secdim[s] / (double)F.R;
-            for (int i = 0; i < d.mlen[t]; ++i) {
-                const double th = d.theta[(size_t)t * F.steps + i];
-                const double b = d.tau[(size_t)t * F.steps + i] * exp(-(th - e_ref) / T) * wgt;
-                z += b;
-                ez += b * th;
-            }
-        }
-        __syncthreads();
-        double zs = block_sum<1024>(z, red);
-        __syncthreads();
-        double es = block_sum<1024>(ez, red);
-        if (threadIdx.x == 0) { d.zsum[it] = zs; d.esum[it] = es / zs; }
-        __syncthreads();
+    if (it >= n_t) return;
+    double z = 0.0, e = 0.0;
+    for (int s = 0; s < F.nsec; ++s) {
+        z += zs[(size_t)it * F.nsec + s];
+        e += es[(size_t)it * F.nsec + s];
     }
+    d.zsum[it] = z;
+    d.esum[it] = e / z;
 }
 
 // ---- host --------------------------------------------------------------------------------
 struct FtLayout {
-    size_t q0, q1, st, ab, part, wr, slo, parta, partc, ckit, ckcs, sec, bar, items, rowoff, secdim, theta, tau, mlen, therm, temps, eigs,
-        xcd, xmat, total;
+    size_t q0, q1, st, ab, part, wr, slo, parta, partc, ckit, ckcs, sec, bar, items, rowoff, secdim, theta, tau, mlen, therm, tsum, temps,
+        eigs, xcd, xmat, total;
 };
 
 static int ft_choose_K(int N) {
@@ -806,6 +860,7 @@ static FtLayout ft_layout(int N, int nsec, int R, int steps, int nitems, int nct
     L.tau = o; o += a(nst * (size_t)steps * 8);
     L.mlen = o; o += a(nst * 4);
     L.therm = o; o += a((size_t)(2 * n_t + 1) * 8);
+    L.tsum = o; o += a((size_t)nsec * (2 * (size_t)n_t + 1) * 8);
     L.temps = o; o += a((size_t)(n_t > 0 ? n_t : 1) * 8);
     L.eigs = o; o += a(nst * 3 * (size_t)steps * 8);
     L.xcd = o; o += a((xcd_words > 0 ? xcd_words : 1) * 4);
@@ -1142,7 +1197,7 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
         if (rc == HM_OK) rc = ft_launch_persistent(&S, use_vt, cap);
         if (rc == HM_OK) {
             const int nst = nsec * FT_W;
-            k_ft_eig<<<(nst + 127) / 128, 128, 0, cap>>>(S.F, (double *)(w + S.L.eigs));
+            k_ft_eig<<<nst / FT_EIG, FT_EIG, ft_eig_smem(S.F.steps), cap>>>(S.F, (double *)(w + S.L.eigs));
             if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ft_eig");
             if (rc == HM_OK && S.F.nexact > 0) {
                 k_ft_exact<<<S.F.nexact, 256, 0, cap>>>(S.F, S.bp, (const uint32_t *)(w + S.L.xcd),
@@ -1160,7 +1215,10 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
     cudaStreamDestroy(cap);
     HM_TRY(rc);
     if (n_t > 0) {
-        k_ft_thermo<<<1, 1024, 0, st>>>(S.F, d_temps, n_t);
+        double *mins = (double *)(w + S.L.tsum), *zs = mins + nsec, *es = zs + (size_t)nsec * n_t;
+        k_ft_min<<<nsec, 256, 0, st>>>(S.F, mins);
+        k_ft_thermo<<<dim3(nsec, n_t), 256, 0, st>>>(S.F, d_temps, mins, zs, es);
+        k_ft_thermo_fin<<<(n_t + 255) / 256, 256, 0, st>>>(S.F, mins, zs, es, n_t);
         HM_CUDA(cudaGetLastError());
     }
     GridBar bar;

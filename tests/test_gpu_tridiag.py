@@ -34,3 +34,18 @@ def test_ritz_values_vs_lapack(hm, m):
     bound = np.abs(T).sum(1).max()
     assert np.abs(r.ritz[:n] - ref[:n]).max() <= (8 + m) * np.finfo(float).eps * bound
     assert np.isnan(r.ritz[n:]).all()                    # past the dimension of T
+
+
+def test_ftlm_long_krylov_spaces(hm):
+    """Past 426 steps the eigen-decomposition works in device memory instead of shared memory.  The
+    quadrature over 32 vectors has converged long before, so Z and E agree with a shorter run up to the
+    FP32 vectors' rounding, 430 steps of 2^-24."""
+    inst = W.small_ring(12, -1.0, -0.3)
+    T = [0.3, 1.0, 5.0]
+    a = hm.ftlm_run(12, hm.bonds_of(inst), 32, 100, 9, T)
+    c = hm.ftlm_run(12, hm.bonds_of(inst), 32, 430, 9, T)
+    tol = 430 * 2.0**-24
+    assert np.allclose(c.Z * np.exp(-(c.e_ref - a.e_ref) / np.array(T)), a.Z, rtol=tol)
+    assert np.allclose(c.E, a.E, rtol=tol)
+    k = int(np.argmax(a.mlen[:, 0]))
+    assert abs(c.tau[k, 0, : c.mlen[k, 0]].sum() - 1.0) <= 430 * 16 * np.finfo(float).eps
