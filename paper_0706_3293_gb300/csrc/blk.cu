@@ -365,13 +365,19 @@ static int launch_blk_matvec(hm_basis *b, const BlkParams &P, const T *x, T *y, 
     return HM_OK;
 }
 
-// split position: 15 low sites (blocks <= 6435 rows: three 512-thread CTAs per SM), or
-// the largest K <= 15 that leaves two high sites
-// split position of the block path: the low part holds K = min(15, N - 2) sites
-// (HM_BLK_K = 8..15 overrides, for tuning); the thread-per-row slots need K <= 15.  The
-// Lanczos workspace sizes its per-block partials (2^(N-K) blocks) with the same function.
+// Split position of the block path: the low part holds K = min(15, N / 2 + 2) sites, at least 8
+// and at most N - 2 (HM_BLK_K = 8..15 overrides, for tuning).  The thread-per-row slots need
+// K <= 15, where the largest block (6435 rows) still leaves three 512-thread CTAs per SM.
+// Below N = 26 a block is a CTA's unit of work, and K = 15 leaves too few of them (2^(N-15):
+// 4 at N = 16 with N - 2, 32 at N = 20) for 152 SMs; too small a K spends the time on the set-up
+// of blocks of few rows.  Measured on GB300 (J1-J2 ring, M = 0, FP64 Lanczos product and
+// alpha, us; K = 15 or N - 2 / K of the rule / one less / one more):
+//   N = 16: 27.8 / 19.4 / 19.2 / 19.5      N = 18: 38.6 / 20.0 / 21.2 / 21.6
+//   N = 20: 40.3 / 25.3 / 29.7 / 25.7      N = 22: 42.5 / 42.0 / 46.8 / 38.0
+//   N = 24: 84.4 / 79.6 / 88.5 / 84.4      N = 26: K = 15, 231.9 (14: 244.4)
+// The Lanczos workspace sizes its per-block partials (2^(N-K) blocks) with the same function.
 int blk_K(const hm_basis *b) {
-    int K = 15;
+    int K = std::max(8, std::min(15, b->view.N / 2 + 2));
     if (const char *e = getenv("HM_BLK_K")) K = std::max(8, std::min(15, atoi(e)));
     return std::min(K, b->view.N - 2);
 }

@@ -78,7 +78,7 @@ static LzLayout lz_layout(const hm_basis *b, int dtype, int max_steps, bool grad
         L.xs[1] = o; o += al256(dim * 8);
         L.qqp = o; o += al256(npart * sizeof(double));
     }
-    // per-block partials of the s = 1/2 block path (split K = min(15, N - 2): H <= 17)
+    // per-block partials of the s = 1/2 block path (split blk_K: H <= 17)
     if (!mom && b->view.S2 == 1 && b->view.N >= 10 && b->view.N <= 32 && !b->view.idx64) {
         const int H = b->view.N - blk_K(b);
         L.hpart_H = H;
