@@ -108,7 +108,7 @@ static int blk_tables(hm_basis *b, int K, const void **dev, int *bytes, int *oU,
 }
 
 // integer coefficient of a per-bond plan: round(h 2^pb_s)
-long long pb_coef(const BlkParams &P, double h) { return std::llround(std::ldexp(h, P.pb_s)); }
+static long long pb_coef(const BlkParams &P, double h) { return std::llround(std::ldexp(h, P.pb_s)); }
 
 // Compile-time slots of the thread-per-row kernels (BlkParams::ln ..).  Sets rows_ok = 0
 // when a class has more bonds of one kind than the slots hold.
@@ -184,11 +184,10 @@ int blk_plan(hm_basis *b, const BondParams &bp_all, int K, BlkParams *P, bool bo
             g0 += bp.jm[t] / 4.0;                                 // -J_b / 4
             mx = std::max(mx, std::fabs(bp.jm[t] / 2.0));
         }
-        P->pb_g0 = g0;
-        mx = std::max(mx, std::fabs(g0));
+        P->pb_g0 = g0;                                            // |g0| <= 64 mx / 2
         int ex = 0;
         std::frexp(mx, &ex);                                      // mx < 2^ex
-        P->pb_s = mx > 0.0 ? 61 - ex : 0;                         // |C| <= 2^61
+        P->pb_s = mx > 0.0 ? 56 - ex : 0;                         // |C_b| < 2^56, |C0| < 2^62
         P->pb_c0 = std::llround(std::ldexp(g0, P->pb_s));
     }
     P->nc = (int)cls.size() > 0 ? (int)cls.size() : 1;
@@ -253,6 +252,13 @@ int blk_plan(hm_basis *b, const BondParams &bp_all, int K, BlkParams *P, bool bo
 // the slots, groups and tables of a plan whose classes are set: bonds bp with classes bc
 static int blk_plan_bonds(hm_basis *b, const BondParams &bp, const std::vector<int> &bc, int K, BlkParams *P) {
     const SectorView &sv = b->view;
+    if (P->perbond)
+        for (int t = 0; t < bp.nb; ++t) {                        // J_b / 2
+            const long long C = pb_coef(*P, -bp.jm[t] / 2.0);
+            P->pb_cl[t] = (int)(C & ((1ll << 27) - 1));
+            P->pb_ch[t] = (int)(C >> 27);
+            P->pb_cf[t] = (float)(-bp.jm[t] / 2.0);
+        }
     // low groups keyed by (class, type, d); high and cross bonds by class
     std::map<std::tuple<int, int, int>, uint32_t> groups;
     std::vector<std::tuple<int, int, int>> hi[HM_BLK_MAXC], cr[HM_BLK_MAXC];   // (p, q, bond)
@@ -287,7 +293,6 @@ static int blk_plan_bonds(hm_basis *b, const BondParams &bp, const std::vector<i
         for (auto &e : hi[c]) {
             P->hb_p[nh] = (uint8_t)std::get<0>(e);
             P->hb_q[nh] = (uint8_t)std::get<1>(e);
-            if (P->perbond) P->pb_hc[nh] = pb_coef(*P, -bp.jm[std::get<2>(e)] / 2.0);   // J_b / 2
             P->pb_hbb[nh] = (uint8_t)std::get<2>(e);
             ++nh;
         }
@@ -424,15 +429,15 @@ int blk_lz_plan(hm_basis *b, const BondParams &bp, int dtype, BlkParams *P, int 
 }
 
 // kernel specialised to the plan (jit.cu), with its launch attributes; 1 = not available
-int jit_lz_kernel(const BlkParams &P, int dtype, const BondParams &bp, const void **kern, int split = 0);
-int jit_mv_kernel(const BlkParams &P, int dtype, const BondParams &bp, const void **kern);
+int jit_lz_kernel(const BlkParams &P, int dtype, const void **kern, int split = 0);
+int jit_mv_kernel(const BlkParams &P, int dtype, const void **kern);
 // pad elements after the staged rows of a specialised kernel (jit.cu)
 int jit_pad(const void *kern);
 
-int blk_lz_jit(const BlkParams &P, int dtype, const BondParams &bp, const void **kern, int *blocks, int split) {
+int blk_lz_jit(const BlkParams &P, int dtype, const void **kern, int *blocks, int split) {
     *kern = nullptr;
     const void *k = nullptr;
-    if (jit_lz_kernel(P, dtype, bp, &k, split) != 0) return 1;
+    if (jit_lz_kernel(P, dtype, &k, split) != 0) return 1;
     const size_t sm = blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, jit_pad(k));
     if (raise_smem_limit(k, (int)sm) != cudaSuccess) {
         cudaGetLastError();
@@ -611,7 +616,7 @@ int blk_lz_split(hm_basis *b, const BondParams &bp, const BlkParams &P, int dtyp
     PB->split = 2;
     PB->rot = std::min(PB->H, 9);
     if (blk_target_table(b, PA, 8) < 0 || blk_target_table(b, PB, 8) < 0) return 1;
-    if (blk_lz_jit(*PA, dtype, bp, kA, blkA, 1) != 0 || blk_lz_jit(*PB, dtype, bp, kB, blkB, 2) != 0) return 1;
+    if (blk_lz_jit(*PA, dtype, kA, blkA, 1) != 0 || blk_lz_jit(*PB, dtype, kB, blkB, 2) != 0) return 1;
     return 0;
 }
 
@@ -648,13 +653,13 @@ int blk_lz32_launch(const BlkParams &P, const float *qc, float *qp, LzScalars *S
 }
 
 // per-bond plan: the specialised y = H x kernel (jit.cu); 1 when it is not available
-static int launch_blk_matvec_pb(hm_basis *b, const BlkParams &P0, const BondParams &bp, const void *x, void *y,
+static int launch_blk_matvec_pb(hm_basis *b, const BlkParams &P0, const void *x, void *y,
                                 int dtype, cudaStream_t st) {
     BlkParams P = P0;
     const int trc = blk_target_table(b, &P, dtype == HM_F64 ? 8 : 4);
     if (trc < 0) return trc;
     const void *k = nullptr;
-    if (jit_mv_kernel(P, dtype, bp, &k) != 0) return 1;
+    if (jit_mv_kernel(P, dtype, &k) != 0) return 1;
     const size_t sm = blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
     HM_CUDA(raise_smem_limit(k, (int)sm));
     int *Ed = nullptr;
@@ -763,7 +768,7 @@ const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int 
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return nullptr;
     if (!P.perbond) return "k_blk_matvec";
     const void *k = nullptr;
-    return jit_mv_kernel(P, dtype, bp, &k) == 0 ? "k_blk_matvec_jit" : nullptr;
+    return jit_mv_kernel(P, dtype, &k) == 0 ? "k_blk_matvec_jit" : nullptr;
 }
 
 // returns 1 when the block path does not apply (caller falls back to the row kernel)
@@ -774,7 +779,7 @@ int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dt
     int rc = blk_plan(b, bp, blk_K(b), &P);
     if (rc != 0) return rc;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return 1;
-    if (P.perbond) return launch_blk_matvec_pb(b, P, bp, x, y, dtype, st);
+    if (P.perbond) return launch_blk_matvec_pb(b, P, x, y, dtype, st);
     if (dtype == HM_F64) {
         switch (P.nc) {
             case 1: return launch_blk_matvec<double, 1>(b, P, (const double *)x, (double *)y, st);

@@ -71,15 +71,18 @@ struct BlkParams {
     // per-bond couplings (more than HM_BLK_MAXC distinct J): every bond sits in the slots of
     // class 0 and a row is y_i = g0 x_i + sum over its allowed exchanges of
     // h_b (x_i - x_target), h_b = J_b / 2, g0 = -sum_b J_b / 4 (Eq. E-2-1).  In FP64 the
-    // coefficients are integers scaled by 2^pb_s (|C| < 2^62): C_b = round(h_b 2^pb_s),
-    // pb_c0 = round(g0 2^pb_s), and a row is one exact int128 sum, rounded once
+    // coefficients are integers scaled by 2^pb_s: C_b = round(h_b 2^pb_s), |C_b| < 2^56, so that
+    // couplings down to 1/16 of the largest keep all 53 bits, pb_c0 = round(g0 2^pb_s), and a
+    // row is one exact 128-bit sum, rounded once (PbSum, blk_sweep.cuh).  C_b is kept as the pair
+    // {C & (2^27 - 1), C >> 27}
     int perbond;
     int pb_s;
     long long pb_c0;
     double pb_g0;
     uint8_t pb_lb[3][HM_BLK_SL], pb_xb[2][HM_BLK_SX];   // bond index of each low / cross slot
     uint8_t pb_hbb[HM_BLK_MAXB];                      // bond index of each high bond
-    long long pb_hc[HM_BLK_MAXB];                     // C_b of each high bond (hb_p / hb_q order)
+    int pb_cl[HM_BLK_MAXB], pb_ch[HM_BLK_MAXB];       // C_b of each bond (bond order)
+    float pb_cf[HM_BLK_MAXB];                         // h_b of each bond
     // bond-correlation plan (one chunk of bonds, per-bond slots): the block setup keeps the
     // high targets uncompacted, hbi[j] for high bond j or ~0 when its spins are parallel
     int bcmode;

@@ -62,8 +62,9 @@ struct BlkMetaXF {
 };
 struct BlkMetaX : BlkMetaXF {
     // per-bond plan (a spin-flip plan with classes allocates only the BlkMetaXF part):
-    // coefficient of each entry of hbi and of hbf, integer (C_b, FP64 rows) and float (FP32 rows)
-    long long hbc[BLK_HBI], hbfc[HM_BLK_MAXB];
+    // coefficient of each entry of hbi and of hbf, integer pair (C_b, FP64 rows) and float (FP32
+    // rows)
+    int2 hbc[BLK_HBI], hbfc[HM_BLK_MAXB];
     float hbcf[BLK_HBI], hbfcf[HM_BLK_MAXB];
 };
 
@@ -130,12 +131,32 @@ __device__ __forceinline__ Sv blk_flip_sum(const BlkMeta &B, int c, const unsign
 }
 
 // ---- per-bond rows: y_i = g0 x_i + sum over allowed exchanges of h_b (x_i - x_t) ----------
-// fixed-point rows: exact int128 sum of C_b (x_i - x_t) (|C_b| <= 2^61, |x_i - x_t| < 2^54,
-// at most 64 terms and C0 x_i: below 2^123); FP32 rows: float multiply-adds
-template <class Sv> struct PbAcc { using T = __int128; };
+// Fixed-point rows: the exact sum of C_b (x_i - x_t), |C_b| < 2^56, |x_i - x_t| <= 2^54, at most
+// 64 terms.  With C = c1 2^27 + c0 and d = d1 2^27 + d0 (c0, d0 >= 0) it is kept as the 64-bit
+// sums of c0 d0, c1 d1 and (c0 + c1)(d0 + d1) (Karatsuba): three 32 x 32-bit multiply-adds a
+// term and no carries between them.  These rows are bound by the multiply pipe (half rate), and
+// a 64 x 64-bit product a term takes four.  |sum c0 d1 + c1 d0| <= 64 (2^54 + 2^56) fits, so the
+// cross sum may wrap on the way, and sum |c1 d1| <= 64 2^56.  Products at 48 couplings, against
+// 128-bit sums with the couplings as literals: N = 24 219 -> 190 us (half of it the split K),
+// N = 26 719 -> 695 us.  FP32 rows: float multiply-adds.
+struct PbSum {
+    long long s0, s2;
+    unsigned long long s1;
+    __device__ __forceinline__ PbSum(int) : s0(0), s2(0), s1(0) {}
+    __device__ __forceinline__ __int128 value() const {
+        return (__int128)s0 + ((__int128)(long long)(s1 - (unsigned long long)s0 - (unsigned long long)s2) << 27) + ((__int128)s2 << 54);
+    }
+};
+template <class Sv> struct PbAcc { using T = PbSum; };
 template <> struct PbAcc<float> { using T = float; };
-__device__ __forceinline__ __int128 pb_mac(long long C, float, int64_t d, __int128 a) { return a + (__int128)C * d; }
-__device__ __forceinline__ float pb_mac(long long, float Cf, float d, float a) { return fmaf(Cf, d, a); }
+__device__ __forceinline__ PbSum pb_mac(int c0, int c1, float, int64_t d, PbSum a) {
+    const int d0 = (int)d & 0x7FFFFFF, d1 = (int)(d >> 27);
+    a.s0 += (long long)c0 * d0;
+    a.s1 += (unsigned long long)((long long)(c0 + c1) * (d0 + d1));
+    a.s2 += (long long)c1 * d1;
+    return a;
+}
+__device__ __forceinline__ float pb_mac(int, int, float Cf, float d, float a) { return fmaf(Cf, d, a); }
 
 __device__ __forceinline__ double i128_to_double(__int128 v) {
     const long long hi = (long long)(v >> 64);
@@ -152,20 +173,24 @@ __device__ __forceinline__ typename PbAcc<Sv>::T blk_high_pb(const BlkParams &P,
     const BlkMetaX &X = *B.x;
     const int e1 = B.he[0];
     const uint4 *h4 = reinterpret_cast<const uint4 *>(B.hbi);
+    auto mac = [&](int e, Sv v) {
+        if constexpr (sizeof(Sv) == 8) a = pb_mac(X.hbc[e].x, X.hbc[e].y, 0.0f, xo - v, a);
+        else a = pb_mac(0, 0, X.hbcf[e], xo - v, a);
+    };
     int e = B.hs[0];
     for (; e + 4 <= e1; e += 4) {
         const uint4 t = h4[e >> 2];
         const Sv v0 = gx(Xg + (size_t)(t.x + r) * sizeof(Sv)), v1 = gx(Xg + (size_t)(t.y + r) * sizeof(Sv));
         const Sv v2 = gx(Xg + (size_t)(t.z + r) * sizeof(Sv)), v3 = gx(Xg + (size_t)(t.w + r) * sizeof(Sv));
-        a = pb_mac(X.hbc[e], X.hbcf[e], xo - v0, a);
-        a = pb_mac(X.hbc[e + 1], X.hbcf[e + 1], xo - v1, a);
-        a = pb_mac(X.hbc[e + 2], X.hbcf[e + 2], xo - v2, a);
-        a = pb_mac(X.hbc[e + 3], X.hbcf[e + 3], xo - v3, a);
+        mac(e, v0);
+        mac(e + 1, v1);
+        mac(e + 2, v2);
+        mac(e + 3, v3);
     }
-    for (; e < e1; ++e) a = pb_mac(X.hbc[e], X.hbcf[e], xo - gx(Xg + (size_t)(B.hbi[e] + r) * sizeof(Sv)), a);
+    for (; e < e1; ++e) mac(e, gx(Xg + (size_t)(B.hbi[e] + r) * sizeof(Sv)));
     for (int f = X.fs[0]; f < X.fe[0]; ++f) {
         const Sv v = gx(Xg + (size_t)(X.hbf[f] - r) * sizeof(Sv));
-        a = pb_mac(X.hbfc[f], X.hbfcf[f], xo - (P.par < 0 ? -v : v), a);
+        a = pb_mac(X.hbfc[f].x, X.hbfc[f].y, X.hbfcf[f], xo - (P.par < 0 ? -v : v), a);
     }
     return a;
 }
@@ -441,17 +466,21 @@ __device__ __forceinline__ void blk_sweep(const BlkParams &P, const unsigned cha
                 const int b0 = popc_below(hm, P.hb_start[c]), b1 = popc_below(hm, P.hb_start[c + 1]);
                 const int f0 = popc_below(fm, P.hb_start[c]), f1 = popc_below(fm, P.hb_start[c + 1]);
                 if (tid >= P.hb_start[c] && tid < P.hb_start[c + 1]) {
-                    const float cf = P.perbond ? (float)ldexp((double)P.pb_hc[tid], -P.pb_s) : 0.0f;
+                    const int pb = P.pb_hbb[tid];
+                    const float cf = P.pb_cf[pb];
                     if (hval) {
                         B.hbi[start + popc_below(hm, tid) - b0] = hidx;
                         if (P.perbond) {
-                            BX->hbc[start + popc_below(hm, tid) - b0] = P.pb_hc[tid];
+                            BX->hbc[start + popc_below(hm, tid) - b0] = make_int2(P.pb_cl[pb], P.pb_ch[pb]);
                             BX->hbcf[start + popc_below(hm, tid) - b0] = cf;
                         }
                     }
                     if (hflip) {
                         BX->hbf[popc_below(fm, tid)] = hidx;
-                        if (P.perbond) { BX->hbfc[popc_below(fm, tid)] = P.pb_hc[tid]; BX->hbfcf[popc_below(fm, tid)] = cf; }
+                        if (P.perbond) {
+                            BX->hbfc[popc_below(fm, tid)] = make_int2(P.pb_cl[pb], P.pb_ch[pb]);
+                            BX->hbfcf[popc_below(fm, tid)] = cf;
+                        }
                     }
                 }
                 if (tid == c) {
@@ -561,8 +590,8 @@ __device__ __forceinline__ void matvec_body(const BlkParams &P, const T *__restr
         if constexpr (Row::kPerBond) {
             const double sy = ef::pow2d(u - P.pb_s);
             blk_sweep<int64_t, NC, false, Row>(P, (const unsigned char *)x, GF64{E}, nullptr, [](uint32_t) { return 0; },
-                                          [&](uint32_t off, uint32_t r, int64_t xo, __int128 sv, int) {
-                                              const __int128 t = (__int128)P.pb_c0 * xo + sv;
+                                          [&](uint32_t off, uint32_t r, int64_t xo, const PbSum &sv, int) {
+                                              const __int128 t = (__int128)P.pb_c0 * xo + sv.value();
                                               yb[off + r] = ef::d2u(i128_to_double(t) * sy);
                                           },
                                           [](int) {}, [](uint32_t, int) {});
@@ -697,8 +726,8 @@ __device__ __forceinline__ void lz64_body(const BlkParams &P, const long long *_
         }
     };
     const double sy = ef::pow2d(u - P.pb_s);
-    auto rowb = [&](uint32_t off, uint32_t r, int64_t xo, __int128 sv, int) {
-        const __int128 t = (__int128)P.pb_c0 * xo + sv;
+    auto rowb = [&](uint32_t off, uint32_t r, int64_t xo, const PbSum &sv, int) {
+        const __int128 t = (__int128)P.pb_c0 * xo + sv.value();
         const unsigned long long yb = ef::d2u(i128_to_double(t) * sy);
         __stcs(Y + off + r, yb);
         d1f = ef::df_add(d1f, ef::df_mul(ef::df_from_fix(xo, E, 0, E - 1023), ef::df_from_bits(yb, E - 1023)));

@@ -35,7 +35,6 @@
 #endif
 
 namespace hm {
-long long pb_coef(const BlkParams &P, double h);   // blk.cu: round(h 2^pb_s)
 
 namespace {
 
@@ -284,19 +283,20 @@ std::string gen_row_table(const BlkParams &P) {
 }
 
 // The row policy of a per-bond plan (BlkParams::perbond): the slots of class 0 written out
-// as in gen_row_slots, each with its own coefficient h_b = J_b / 2 as a literal, summed
-// as h_b (x_i - x_t) (blk_sweep.cuh, per-bond rows).  A slot whose spins are parallel reads
+// as in gen_row_slots, each with its own coefficient h_b = J_b / 2, summed as h_b (x_i - x_t)
+// (blk_sweep.cuh, per-bond rows).  The coefficients come from the kernel parameters, not as
+// literals: a kernel then serves every coupling of a bond layout, where literals cost a new
+// compilation (150 ms) for each step of a fit.  A slot whose spins are parallel reads
 // a fixed address (a broadcast) and adds a zero difference.
-std::string gen_row_pb_table(const BlkParams &P, const BondParams &bp);
+std::string gen_row_pb_table(const BlkParams &P);
 
-std::string gen_row_pb(const BlkParams &P, const BondParams &bp) {
-    if (P.tt) return gen_row_pb_table(P, bp);
-    auto hb = [&](int t) { return -bp.jm[t] / 2.0; };
-    // coefficient arguments of hm::pb_mac: C_b (integer, FP64 rows) and h_b (float, FP32 rows)
+std::string gen_row_pb(const BlkParams &P) {
+    if (P.tt) return gen_row_pb_table(P);
+    // coefficient arguments of hm::pb_mac: C_b (integer, FP64 rows) and h_b (float, FP32 rows),
+    // read from the kernel parameters
     auto cf = [&](int t) {
-        char buf[96];
-        snprintf(buf, sizeof buf, "%lldLL, %.9gf", pb_coef(P, hb(t)), hb(t));
-        return std::string(buf);
+        const std::string i = std::to_string(t);
+        return "P.pb_cl[" + i + "], P.pb_ch[" + i + "], P.pb_cf[" + i + "]";
     };
     std::string s;
     s += "struct RowJit {\n"
@@ -318,7 +318,7 @@ std::string gen_row_pb(const BlkParams &P, const BondParams &bp) {
          "    const uint32_t R0own = hm::r0s_at(l4 & 0x3FCu), R1own = hm::us_at(lh4k);\n"
          "    const uint32_t zo = (uint32_t)((P.max_block + hm::BLK_XPAD - 1) * sizeof(Sv));   // fixed address\n"
          "    (void)R0own; (void)R1own; (void)lh4; (void)gx; (void)zo;\n"
-         "    typename hm::PbAcc<Sv>::T a = 0;\n";
+         "    typename hm::PbAcc<Sv>::T a(0);\n";
     std::set<int> ds;
     for (int t = 0; t < 3; ++t)
         for (int k = 0; k < P.ln[0][t]; ++k) ds.insert(P.ld[0][t][k]);
@@ -358,12 +358,10 @@ std::string gen_row_pb(const BlkParams &P, const BondParams &bp) {
 // low slot gathers the row its entry names -- the exchange target, or the row itself when the
 // exchange is not allowed, so that h_b (x_i - x_t) is zero without a test -- and cross slots
 // take the rank of l ^ 2^p from the table.
-std::string gen_row_pb_table(const BlkParams &P, const BondParams &bp) {
-    auto hb = [&](int t) { return -bp.jm[t] / 2.0; };
+std::string gen_row_pb_table(const BlkParams &P) {
     auto cf = [&](int t) {
-        char buf[96];
-        snprintf(buf, sizeof buf, "%lldLL, %.9gf", pb_coef(P, hb(t)), hb(t));
-        return std::string(buf);
+        const std::string i = std::to_string(t);
+        return "P.pb_cl[" + i + "], P.pb_ch[" + i + "], P.pb_cf[" + i + "]";
     };
     std::string s;
     s += "struct RowJit {\n"
@@ -381,7 +379,7 @@ std::string gen_row_pb_table(const BlkParams &P, const BondParams &bp) {
          "        const G &gx, Sv xo) {\n"
          "    (void)l; (void)Xg;\n"
          "    const uint4 *tt = P.tt + (B.lwo + r);\n"
-         "    typename hm::PbAcc<Sv>::T a = 0;\n";
+         "    typename hm::PbAcc<Sv>::T a(0);\n";
     const int nch = (P.tt_n + 7) / 8;
     for (int j = 0; j < nch; ++j) put(s, "    const uint4 q%d = hm::ldg_v4(tt + %uu);\n", j, (unsigned)j * P.tt_stride);
     static const char *comp[4] = {"x", "y", "z", "w"};
@@ -738,12 +736,12 @@ int compile(const std::string &src, const char *name, int device, const void **o
 // handle (usable with cudaLaunchKernel / cudaFuncSetAttribute), or 1 when the generic
 // kernel has to serve.
 // source of the row policy for plan P: per-bond, per-byte delta tables, or slots
-static bool jit_row_source(const BlkParams &P, const BondParams &bp, std::string *src, bool *delta) {
+static bool jit_row_source(const BlkParams &P, std::string *src, bool *delta) {
     bool gen_ok = true;
     const char *rowk = getenv("HM_JIT_ROW");
     *delta = !P.perbond && rowk && strcmp(rowk, "delta") == 0 && !P.par;   // no spin-flip or per-bond form
     *src = std::string("#include \"blk_sweep.cuh\"\n") +
-           (P.perbond ? gen_row_pb(P, bp) : *delta ? gen_row(P, gen_ok) : P.tt ? gen_row_table(P) : gen_row_slots(P));
+           (P.perbond ? gen_row_pb(P) : *delta ? gen_row(P, gen_ok) : P.tt ? gen_row_table(P) : gen_row_slots(P));
     return gen_ok;
 }
 
@@ -768,14 +766,14 @@ static int jit_get(const std::string &src, const char *name, int dev, int pad, c
 
 // y = H x kernel (matvec API) for a per-bond plan: k_blk_matvec_jit, one vector, dtype
 // HM_F64 (binary64 x, E = its largest exponent field in Eptr) or HM_F32
-int jit_mv_kernel(const BlkParams &P, int dtype, const BondParams &bp, const void **kern) {
+int jit_mv_kernel(const BlkParams &P, int dtype, const void **kern) {
     const char *env = getenv("HM_JIT");
     if ((env && env[0] == '0') || !P.rows_ok || !P.perbond) return 1;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 1; }
     std::string src;
     bool delta = false;
-    if (!jit_row_source(P, bp, &src, &delta)) return 1;
+    if (!jit_row_source(P, &src, &delta)) return 1;
     const char *T = dtype == HM_F64 ? "double" : "float";
     put(src,
         "extern \"C\" __global__ void __launch_bounds__(512, 3) k_blk_matvec_jit(hm::BlkParams P,\n"
@@ -803,7 +801,7 @@ int jit_bc_kernel(const BlkParams &P, int dtype, int nbk, const void **kern) {
 
 // split = 1 / 2: the passes of the split FP64 product (k_blk_lz64a_jit / k_blk_lz64b_jit,
 // plans of the near and of the far bonds; blk_sweep.cuh, lz64_body)
-int jit_lz_kernel(const BlkParams &P, int dtype, const BondParams &bp, const void **kern, int split) {
+int jit_lz_kernel(const BlkParams &P, int dtype, const void **kern, int split) {
     const char *env = getenv("HM_JIT");
     if (env && env[0] == '0') return 1;
     if (!P.rows_ok) return 1;
@@ -812,14 +810,15 @@ int jit_lz_kernel(const BlkParams &P, int dtype, const BondParams &bp, const voi
     if (cudaGetDevice(&dev) != cudaSuccess) { cudaGetLastError(); return 1; }
     std::string src;
     bool delta = false;
-    if (!jit_row_source(P, bp, &src, &delta)) return 1;
+    if (!jit_row_source(P, &src, &delta)) return 1;
     const bool f64 = dtype == HM_F64;
     const int nc = P.nc == 1 ? 1 : (P.nc == 2 ? 2 : 4);
     const char *name = !f64 ? "k_blk_lz32_jit" : split == 1 ? "k_blk_lz64a_jit" : split == 2 ? "k_blk_lz64b_jit"
                                                                                          : "k_blk_lz64_jit";
     // resident CTAs per SM the register budget is cut for (3: 40 registers a thread, 2: 64);
-    // HM_JIT_CTAS overrides the default
-    int ctas = 3;
+    // HM_JIT_CTAS overrides the default.  FP64 per-bond rows are bound by the multiply pipe, not
+    // by latency, and spill at 40 registers (N = 26: 620 us with 3, 600 with 2)
+    int ctas = f64 && P.perbond ? 2 : 3;
     if (const char *e = getenv("HM_JIT_CTAS")) ctas = atoi(e) == 2 ? 2 : 3;
     if (f64)
         put(src,
