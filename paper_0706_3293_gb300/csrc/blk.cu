@@ -380,9 +380,12 @@ static int launch_blk_matvec(hm_basis *b, const BlkParams &P, const T *x, T *y, 
 //   N = 16: 27.8 / 19.4 / 19.2 / 19.5      N = 18: 38.6 / 20.0 / 21.2 / 21.6
 //   N = 20: 40.3 / 25.3 / 29.7 / 25.7      N = 22: 42.5 / 42.0 / 46.8 / 38.0
 //   N = 24: 84.4 / 79.6 / 88.5 / 84.4      N = 26: K = 15, 231.9 (14: 244.4)
+// fp32_run: FP32 Lanczos runs keep K = 15.  The split decides the order in which a float row adds
+// its exchanges, and a run carries a changed rounding into every alpha and beta (FP64 rows are
+// exact integer sums, whatever the order).
 // The Lanczos workspace sizes its per-block partials (2^(N-K) blocks) with the same function.
-int blk_K(const hm_basis *b) {
-    int K = std::max(8, std::min(15, b->view.N / 2 + 2));
+int blk_K(const hm_basis *b, bool fp32_run) {
+    int K = fp32_run ? 15 : std::max(8, std::min(15, b->view.N / 2 + 2));
     if (const char *e = getenv("HM_BLK_K")) K = std::max(8, std::min(15, atoi(e)));
     return std::min(K, b->view.N - 2);
 }
@@ -408,7 +411,7 @@ static int set_smem(K_t kern, size_t sm) {
 
 // Lanczos hooks: plan (0 = block path usable), attribute setup, launch
 int blk_lz_plan(hm_basis *b, const BondParams &bp, int dtype, BlkParams *P, int *blocks) {
-    int rc = blk_plan(b, bp, blk_K(b), P);
+    int rc = blk_plan(b, bp, blk_K(b, dtype == HM_F32), P);
     if (rc != 0) return rc;
     const size_t sm = blk_row_smem_bytes(*P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
     if (!P->rows_ok || sm > 200 * 1024) return 1;
@@ -725,7 +728,7 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
             bc.jm[i] = bp.jm[c0 + i]; bc.jmf[i] = bp.jmf[c0 + i];
         }
         BlkParams &P = plans[c];
-        if (blk_plan(b, bc, blk_K(b), &P, true) != 0 || !P.rows_ok) return 1;
+        if (blk_plan(b, bc, blk_K(b, false), &P, true) != 0 || !P.rows_ok) return 1;
         const size_t sm = blk_row_smem_bytes(P, es, BLK_XPAD);
         if (sm > 200 * 1024 || jit_bc_kernel(P, dtype, nbk, &kerns[c]) != 0) return 1;
         if (raise_smem_limit(kerns[c], (int)sm) != cudaSuccess) {
@@ -764,7 +767,7 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
 const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int nvec) {
     if (nvec != 1) return nullptr;
     BlkParams P;
-    if (blk_plan(b, bp, blk_K(b), &P) != 0) return nullptr;
+    if (blk_plan(b, bp, blk_K(b, false), &P) != 0) return nullptr;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return nullptr;
     if (!P.perbond) return "k_blk_matvec";
     const void *k = nullptr;
@@ -776,7 +779,7 @@ int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dt
                cudaStream_t st) {
     if (nvec != 1) return 1;
     BlkParams P;
-    int rc = blk_plan(b, bp, blk_K(b), &P);
+    int rc = blk_plan(b, bp, blk_K(b, false), &P);
     if (rc != 0) return rc;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return 1;
     if (P.perbond) return launch_blk_matvec_pb(b, P, x, y, dtype, st);

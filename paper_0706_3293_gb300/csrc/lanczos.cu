@@ -19,7 +19,7 @@ int blk_lz_jit(const BlkParams &P, int dtype, const void **kern, int *blocks, in
 int blk_lz_split(hm_basis *b, const BondParams &bp, const BlkParams &P, int dtype, BlkParams *PA, BlkParams *PB,
                  const void **kA, const void **kB, int *blkA, int *blkB);
 int blk_target_table(hm_basis *b, BlkParams *P, int esize);
-int blk_K(const hm_basis *b);   // blk.cu: split position of the block path
+int blk_K(const hm_basis *b, bool fp32_run);   // blk.cu: split position of the block path
 int blk_lz64_launch(const BlkParams &P, const long long *Xc, unsigned long long *Y, LzScalars *S, int pc,
                     double *part, int blocks, cudaStream_t st, const void *jit);
 int blk_lz32_launch(const BlkParams &P, const float *qc, float *qp, LzScalars *S, double *part, int blocks,
@@ -80,7 +80,7 @@ static LzLayout lz_layout(const hm_basis *b, int dtype, int max_steps, bool grad
     }
     // per-block partials of the s = 1/2 block path (split blk_K: H <= 17)
     if (!mom && b->view.S2 == 1 && b->view.N >= 10 && b->view.N <= 32 && !b->view.idx64) {
-        const int H = b->view.N - blk_K(b);
+        const int H = b->view.N - blk_K(b, dtype == HM_F32);
         L.hpart_H = H;
         L.hpart = o; o += al256(((size_t)2 << H) * sizeof(double));
     }
