@@ -1,13 +1,14 @@
 // basis.cu -- sector tables (Sec. 3, Eq. E-3-c), the codec test hooks (Sec. 3.1, 3.2),
 // bond preparation, seeded start vectors and error reporting.
 #include <stdlib.h>
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
 #include <new>
 
-#include "hm_internal.cuh"
+#include "hm_row.cuh"
 
 namespace hm {
 
@@ -140,6 +141,97 @@ int make_bonds(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *
     return HM_OK;
 }
 
+// the device tables of a basis: CD, then per entry (p, S, a) the rank changes {E+, F+, E-, F-}
+// and {G+, G-} of the exchanges that the row sweep reads (hm_row.cuh), zero where there is none
+static std::vector<uint64_t> row_tables(const hm_basis *b) {
+    const SectorView &v = b->view;
+    const size_t n = (size_t)v.cd_len;
+    std::vector<uint64_t> t(7 * n, 0);
+    std::copy(b->cd.begin(), b->cd.end(), t.begin());
+    auto at = [&](int p, int S, int a) { return b->cd[(size_t)p * v.cd_rowlen + (size_t)S * v.cd_w + a]; };
+    for (int p = 1; p < v.N; ++p)                    // position 0 has no rank term
+        for (int S = 0; S <= v.A; ++S)
+            for (int a = 0; a <= std::min(S, v.S2); ++a) {
+                const uint64_t c = at(p, S, a);
+                uint64_t *e = t.data() + n + 4 * ((size_t)p * v.cd_rowlen + (size_t)S * v.cd_w + a);
+                uint64_t *g = t.data() + 5 * n + 2 * ((size_t)p * v.cd_rowlen + (size_t)S * v.cd_w + a);
+                if (S < v.A) {
+                    if (a < v.S2) e[0] = at(p, S + 1, a + 1) - c;
+                    g[0] = at(p, S + 1, a) - c;
+                }
+                if (a >= 1) e[1] = at(p, S, a - 1) - c;
+                if (S >= 1) {
+                    if (a >= 1) e[2] = at(p, S - 1, a - 1) - c;
+                    g[1] = at(p, S - 1, a) - c;
+                }
+                if (a < v.S2) e[3] = at(p, S, a + 1) - c;
+            }
+    return t;
+}
+
+int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, size_t *smem) {
+    if (row_run_len() > 1 || bp.nb > ROW_MB) return 1;
+    const int N = sv.N, S2 = sv.S2, n1 = S2 + 1;
+    P->nb = bp.nb;
+    P->nc = P->nslots = 0;
+    memcpy(P->hs_pdn, bp.hs_pdn, sizeof P->hs_pdn);
+    memcpy(P->hs_pup, bp.hs_pup, sizeof P->hs_pup);
+    // classes of equal coupling (bonds of one class mostly follow each other), bonds by lower end
+    uint16_t bc[ROW_MB];
+    int last[HM_MAX_SITES], slot_of[HM_MAX_SITES], freed[HM_MAX_SITES], nf = 0;    // last[q]: lowest partner below q
+    for (int r = 0; r < N; ++r) last[r] = N;
+    double mx = 0.0;
+    int count[HM_MAX_SITES + 1] = {};
+    for (int t = 0; t < bp.nb; ++t) {
+        int c = t > 0 && bp.jm[t] == bp.jm[t - 1] ? bc[t - 1] : 0;
+        while (c < P->nc && P->jm[c] != bp.jm[t]) ++c;
+        if (c == P->nc) P->jm[P->nc++] = bp.jm[t];
+        bc[t] = (uint16_t)c;
+        mx = std::max(mx, std::fabs(bp.jm[t] / 4.0));
+        last[bp.q[t]] = std::min(last[bp.q[t]], (int)bp.p[t]);
+        ++count[bp.p[t]];
+    }
+    // slots: a site holds one from its own position down to its lowest partner's
+    for (int r = N - 1; r >= 0; --r) {
+        P->slot[r] = ROW_SLOT_NONE;
+        if (last[r] < r) {
+            if (nf == 0) freed[nf++] = P->nslots++;
+            slot_of[r] = freed[--nf];
+            P->slot[r] = (uint8_t)slot_of[r];
+        }
+        for (int q = r + 1; q < N; ++q)
+            if (last[q] == r) freed[nf++] = slot_of[q];
+    }
+    int at[HM_MAX_SITES + 1];
+    P->bs[0] = 0;
+    for (int r = 0; r < N; ++r) {
+        at[r] = P->bs[r];
+        P->bs[r + 1] = (uint16_t)(P->bs[r] + count[r]);
+    }
+    for (int t = 0; t < bp.nb; ++t) {
+        const int n = at[bp.p[t]]++;
+        P->q[n] = bp.q[t];
+        P->qs[n] = (uint8_t)slot_of[bp.q[t]];
+        P->cls[n] = bc[t];
+    }
+    // diagonal sum_b dC_b k_b with |k_b| <= S2^2, below 2^62; taken when that leaves the largest
+    // coupling 52 bits or more (a binary64 sum of the terms rounds no finer)
+    int ex = 0, kb = 0;
+    std::frexp(mx, &ex);                             // mx < 2^ex
+    while ((1 << kb) < S2 * S2 * std::max(1, bp.nb)) ++kb;
+    const int s = 62 - kb - ex;
+    P->dint = 62 - kb >= 52 && s > -1000 && s < 1000;
+    if (P->dint) {
+        P->dscale = std::ldexp(1.0, -s);
+        for (int c = 0; c < P->nc; ++c) P->dC[c] = std::llround(std::ldexp(P->jm[c] / 4.0, s));
+    }
+    P->tab = (size_t)P->nc * 2 * n1 * n1 * es <= 16 * 1024;
+    const size_t tabs = sv.idx64 ? row_tab_bytes<uint64_t>(sv) : row_tab_bytes<uint32_t>(sv);
+    *smem = row_coef_bytes(*P, S2, es) + tabs + (size_t)P->nslots * ROW_NT * (sv.idx64 ? 16 : 8);
+    // at least two CTAs on an SM; more shared memory than that leaves the table form ahead
+    return *smem <= 110 * 1024 ? 0 : 1;
+}
+
 // ---------------------------------------------------------------------------------------
 // codec test hooks
 // ---------------------------------------------------------------------------------------
@@ -223,12 +315,13 @@ int basis_build(int n_sites, int two_s, int two_m, hm_basis **out) {
     int rc = build_tables(n_sites, two_s, two_m, b);
     if (rc < 0) { delete b; return rc; }
     SectorView &v = b->view;
-    size_t bytes = v.idx64 ? (size_t)v.cd_len * 8 : (size_t)v.cd_len * 4;
+    const std::vector<uint64_t> tab = row_tables(b);
+    size_t bytes = v.idx64 ? tab.size() * 8 : tab.size() * 4;
     std::vector<uint32_t> c32;
-    const void *src = b->cd.data();
+    const void *src = tab.data();
     if (!v.idx64) {
-        c32.resize(v.cd_len);
-        for (int k = 0; k < v.cd_len; ++k) c32[k] = (uint32_t)b->cd[k];
+        c32.resize(tab.size());
+        for (size_t k = 0; k < tab.size(); ++k) c32[k] = (uint32_t)tab[k];
         src = c32.data();
     }
     cudaError_t e = cudaGetDevice(&b->device);

@@ -1,10 +1,224 @@
-// hm_row.cuh -- the per-row kernel body of Eq. (E-4-b): apply every bond term of
+// hm_row.cuh -- the per-row kernel bodies of Eq. (E-4-b): apply every bond term of
 // Eq. (E-2-1) to the row's own basis state, encode each target, gather x there.
+//
+// Two forms.  The sweep form (RowPlan, row_sweep) decodes the row and forms every exchange
+// target in one pass over the positions; it serves every sector whose tables fit in shared
+// memory (row_plan).  The table form below it (row_apply) is the general one: it also serves the
+// larger tables and the successor-rule row runs (HM_ROW_RUN).
 #pragma once
 
 #include "hm_internal.cuh"
 
 namespace hm {
+
+// ---- the sweep form ------------------------------------------------------------------------
+// An exchange of p < q by dp (digit at p by dp, at q by -dp) changes the rank terms of
+// positions p..q (Sec. 3.2).  With the running digit sums S_r of the row and CD of hm_internal.cuh
+//   E_dp = CD[p][S_p + dp][a_p + dp] - CD[p][S_p][a_p]
+//   F_dp = CD[q][S_q][a_q - dp] - CD[q][S_q][a_q]
+//   G_dp[r] = CD[r][S_r + dp][a_r] - CD[r][S_r][a_r]        (p < r < q)
+// the index change is E_dp + sum_{p < r < q} G_dp[r] + F_dp.  The differences are tables beside CD
+// (basis_build), so a position costs one lookup.  The sweep goes down from position N - 1: it
+// finds the digit (Sec. 3.1), adds G to the suffix sums Q_dp, keeps R_dp = F_dp - Q_dp[q] of a
+// site that is the upper end of a bond in one of a few per-thread slots, and, for the bonds whose
+// lower end the position is, has the target as i + (E_dp + Q_dp[p + 1]) + R_dp.
+// What bounds it in FP64 is the binary64 pipe (64 cycles a warp instruction and SM quarter), so
+// the exchange coefficients -J_b f are tables too (one multiply-add an exchange) and the
+// diagonal is an exact integer sum, converted once a row.  The gathers of one bond are in flight
+// while those of the bond before are added.  Measured (s = 3/2 ring, N = 12, 1.7 M rows, FP64):
+// k_matvec, the table form, 362 us; this form 172 us.
+template <class I> struct alignas(4 * sizeof(I)) RowEF { I ep, fp, em, fm; };
+template <class I> struct alignas(2 * sizeof(I)) RowG { I gp, gm; };
+
+constexpr int ROW_NT = 256;          // threads per CTA of the row kernels
+constexpr int ROW_SLOT_NONE = 255;
+
+// Lists of more than ROW_MB bonds take the table form: a kernel's parameters are copied at every
+// launch (3.9 KB here)
+constexpr int ROW_MB = 128;
+struct RowPlan {
+    int nb, nslots, nc;
+    int tab;                         // exchange coefficients from a table per class (else J f formed per exchange)
+    int dint;                        // diagonal as the integer sum of dC k (else J k / 4 added in the Acc type)
+    double dscale;                   // 2^-s of dC
+    uint8_t slot[HM_MAX_SITES];      // slot of the site's R, or ROW_SLOT_NONE
+    uint16_t bs[HM_MAX_SITES + 1];   // bonds with lower end r: [bs[r], bs[r + 1])
+    uint8_t q[ROW_MB], qs[ROW_MB];          // upper end and its slot
+    uint16_t cls[ROW_MB];              // class: index of the bond's distinct coupling
+    double jm[ROW_MB];                // by class: -J
+    long long dC[ROW_MB];             // by class: round(-J / 4 2^s)
+    double hs_pdn[64], hs_pup[64];   // as in BondParams
+};
+
+// the plan of a bond list; 0, or 1 when the sector's tables, the bonds (more than ROW_MB) or the run
+// length (HM_ROW_RUN) ask for the table form.  *smem: dynamic shared memory of a CTA for
+// accumulation type size es
+int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, size_t *smem);
+
+// resident CTAs per SM that the registers of kernel K allow
+template <auto K>
+inline int row_most() {
+    static const int most = [] {
+        int per = 1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, K, ROW_NT, 0) != cudaSuccess) cudaGetLastError();
+        return per < 1 ? 1 : per;
+    }();
+    return most;
+}
+// CTAs of a row kernel: one resident wave at most (every CTA stages the tables), and no more
+// than grid_blocks, for which the workspaces' partial sums are sized
+inline int row_grid(uint64_t rows, int most, size_t smem) {
+    const int fit = (int)((228 * 1024) / (smem + 1024));
+    const int wave = sm_count() * (fit < 1 ? 1 : fit < most ? fit : most), need = grid_blocks(rows, ROW_NT);
+    return need < wave ? need : wave;
+}
+
+__host__ __device__ __forceinline__ size_t row_coef_bytes(const RowPlan &P, int S2, int es) {
+    const int n1 = S2 + 1;
+    return ((size_t)(P.tab ? P.nc * 2 * n1 * n1 : 2 * n1 * n1) * es + 15) & ~(size_t)15;
+}
+
+// shared layout: exchange coefficients | E, F | G | CD | slots
+template <class I, class Acc>
+struct RowTabs {
+    const Acc *coef;
+    const RowEF<I> *ef;
+    const RowG<I> *g;
+    const I *cd;
+    RowG<I> *slots;                  // this thread's, stride ROW_NT
+};
+template <class I>
+__host__ __device__ __forceinline__ size_t row_tab_bytes(const SectorView &sv) {
+    return ((size_t)sv.cd_len * 7 * sizeof(I) + 15) & ~(size_t)15;
+}
+
+template <class I, class Acc>
+__device__ __forceinline__ RowTabs<I, Acc> row_stage(const SectorView &sv, const RowPlan &P, unsigned char *smem) {
+    const int n1 = sv.S2 + 1, n2 = n1 * n1;
+    Acc *coef = reinterpret_cast<Acc *>(smem);
+    for (int k = threadIdx.x; k < (P.tab ? P.nc : 1) * 2 * n2; k += ROW_NT) {
+        const int c = k / (2 * n2), m = k % (2 * n2), e = m % n2, h = (e / n1) * 8 + e % n1;
+        const double f = m < n2 ? P.hs_pdn[h] : P.hs_pup[h];
+        if constexpr (sizeof(Acc) == 8) coef[k] = P.tab ? P.jm[c] * f : f;
+        else coef[k] = P.tab ? (float)P.jm[c] * (float)f : (float)f;
+    }
+    I *cd = reinterpret_cast<I *>(smem + row_coef_bytes(P, sv.S2, sizeof(Acc)));
+    // device tables: CD, then E/F, then G (basis_build); in shared memory the wide ones first
+    const I *src = (const I *)sv.cd;
+    for (int k = threadIdx.x; k < 6 * sv.cd_len; k += ROW_NT) cd[k] = src[sv.cd_len + k];
+    for (int k = threadIdx.x; k < sv.cd_len; k += ROW_NT) cd[6 * (size_t)sv.cd_len + k] = src[k];
+    RowTabs<I, Acc> t;
+    t.coef = coef;
+    t.ef = reinterpret_cast<const RowEF<I> *>(cd);
+    t.g = reinterpret_cast<const RowG<I> *>(cd + 4 * (size_t)sv.cd_len);
+    t.cd = cd + 6 * (size_t)sv.cd_len;
+    t.slots = reinterpret_cast<RowG<I> *>(smem + row_coef_bytes(P, sv.S2, sizeof(Acc)) + row_tab_bytes<I>(sv)) + threadIdx.x;
+    __syncthreads();
+    return t;
+}
+
+// every bond of the state of index i: f(t, a_p, a_q, target of s-_p s+_q (dp = +1), target of
+// s+_p s-_q (dp = -1)); a target is meaningful only when the exchange is allowed
+template <class I, class Acc, class F>
+__device__ __forceinline__ void row_sweep(const SectorView &sv, const RowPlan &P, const RowTabs<I, Acc> &T, I i, F &&f) {
+    const int bits = sv.bits, S2 = sv.S2, mask = (1 << bits) - 1;
+    uint64_t w = 0;
+    int S = sv.A;
+    I res = i, qp = 0, qm = 0;
+    for (int r = sv.N - 1; r >= 0; --r) {
+        const int ix = r * sv.cd_rowlen + S * sv.cd_w;
+        int a = S;
+        if (r > 0) {                               // the digit whose cumulative range holds res
+            a = 0;
+            for (int k = 1; k <= S2; ++k) a += T.cd[ix + k] <= res;
+            res -= T.cd[ix + a];
+        }
+        w |= (uint64_t)a << (r * bits);
+        const RowEF<I> e = T.ef[ix + a];
+        const RowG<I> g = T.g[ix + a];
+        const I lp = i + e.ep + qp, lm = i + e.em + qm;
+        qp += g.gp;
+        qm += g.gm;
+        const int sl = P.slot[r];
+        if (sl != ROW_SLOT_NONE) T.slots[sl * ROW_NT] = RowG<I>{(I)(e.fp - qp), (I)(e.fm - qm)};
+        for (int t = P.bs[r]; t < P.bs[r + 1]; ++t) {
+            const int aq = (int)(w >> (P.q[t] * bits)) & mask;
+            const RowG<I> R = T.slots[P.qs[t] * ROW_NT];
+            f(t, a, aq, (I)(lp + R.gp), (I)(lm + R.gm));
+        }
+        S -= a;
+    }
+}
+
+// (H x)_i for NV columns: *dg the diagonal element, acc the exchange sums.  HALF: s = 1/2, where
+// at most one direction of a bond is allowed
+template <class I, class T, class Acc, int NV, bool HALF>
+__device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P, const RowTabs<I, Acc> &Tb, I i,
+                                         const T *__restrict__ x, int ld, int c0, Acc *acc, Acc *dg_out) {
+    const int S2 = sv.S2, n1 = S2 + 1, n2 = n1 * n1;
+    Acc dg = Acc(0), cp[2] = {Acc(0), Acc(0)};     // the bond before: coefficients and gathered values
+    T vp[HALF ? 1 : 2][NV];
+    long long di = 0;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        acc[k] = Acc(0);
+        vp[0][k] = T(0);
+        if constexpr (!HALF) vp[1][k] = T(0);
+    }
+    row_sweep(sv, P, Tb, i, [&](int t, int ap, int aq, I jp, I jm) {
+        const int c = P.cls[t], k4 = (S2 - 2 * ap) * (S2 - 2 * aq);
+        if (P.dint) di += P.dC[c] * k4;
+        else if constexpr (sizeof(Acc) == 8) dg = fma(0.25 * P.jm[c], (double)k4, dg);
+        else dg = fmaf(0.25f * (float)P.jm[c], (float)k4, dg);
+        const Acc *co = Tb.coef + (P.tab ? c * 2 * n2 : 0) + ap * n1 + aq;
+        auto cf = [&](int d) -> Acc {
+            const Acc v = co[d * n2];
+            if (P.tab) return v;
+            if constexpr (sizeof(Acc) == 8) return P.jm[c] * v;
+            else return (float)P.jm[c] * v;
+        };
+        auto pend = [&](int d, bool ok, I j, Acc &cn, T *vn) {
+            cn = ok ? cf(d) : Acc(0);
+            const T *xr = x + (size_t)j * ld + c0;
+#pragma unroll
+            for (int k = 0; k < NV; ++k) vn[k] = ok ? __ldg(xr + k) : T(0);
+        };
+        const bool dn = ap >= 1 && aq < S2, up = ap < S2 && aq >= 1;
+        if constexpr (HALF) {
+            Acc c1;
+            T v1[NV];
+            pend(dn ? 0 : 1, dn || up, dn ? jm : jp, c1, v1);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
+                vp[0][k] = v1[k];
+            }
+            cp[0] = c1;
+        } else {
+            Acc c1, c2;
+            T v1[NV], v2[NV];
+            pend(0, dn, jm, c1, v1);
+            pend(1, up, jp, c2, v2);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
+                acc[k] = fma(cp[1], (Acc)vp[1][k], acc[k]);
+                vp[0][k] = v1[k];
+                vp[1][k] = v2[k];
+            }
+            cp[0] = c1;
+            cp[1] = c2;
+        }
+    });
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
+        if constexpr (!HALF) acc[k] = fma(cp[1], (Acc)vp[1][k], acc[k]);
+    }
+    *dg_out = P.dint ? (Acc)((double)di * P.dscale) : dg;
+}
+
+// ---- the table form ------------------------------------------------------------------------
 
 // Tables one CTA needs in shared memory: the exchange factors, then the rank table CD.
 // Layout: double hs[128] | float hsf[128] | CD.  hs[0..64) = pdn, hs[64..128) = pup.
@@ -33,7 +247,6 @@ __device__ __forceinline__ I *stage_tables(const SectorView &sv, const BondParam
 // running digit sum causes at positions r..N-1, and the running digit sums S[r].  Laid
 // out [slot][thread]: the threads of a warp visit the same bond together, so they read
 // the same slot of consecutive threads (no bank conflict).
-constexpr int ROW_NT = 256;          // threads per CTA of the row kernels
 template <class I>
 __host__ __device__ __forceinline__ size_t row_px_bytes(const SectorView &sv) {
     const size_t a = (size_t)2 * (sv.N + 1) * ROW_NT * sizeof(I);

@@ -116,6 +116,9 @@ struct hm_lanczos {
     hm::BlkParams blk2;
     const void *jit2;
     int run;                // rows per thread run of the general product (row_runs)
+    hm::RowPlan rowp;       // its sweep form (row_blocks > 0 CTAs; 0: the table form)
+    size_t row_smem;
+    int row_blocks;
     int use_s1;             // s = 1 block path (s1blk.cu)
     int use_mom;            // momentum basis: product k_mom_matvec, then the epilogue kernel
     hm::S1Plan s1;
@@ -204,6 +207,31 @@ k_lz_matvec(SectorView sv, BondParams bp, const T *__restrict__ qc, T *__restric
         }
     });
     dot = block_sum<NT>(dot + (double)dotf.hi + (double)dotf.lo, red);
+    if (threadIdx.x == 0) part[blockIdx.x] = dot;
+}
+
+// the same by the sweep form of the row product (hm_row.cuh), FP64 vectors.  FP32 runs keep the
+// table form, which adds a row's bonds in list order: another order rounds a float row
+// differently, and a run carries that into every alpha and beta
+template <class I, bool HALF>
+__global__ void __launch_bounds__(ROW_NT)
+k_lz_row(SectorView sv, RowPlan P, const double *__restrict__ qc, double *__restrict__ qp,
+         const LzScalars *__restrict__ S, double *__restrict__ part) {
+    if (S->done) return;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double red[ROW_NT / 32];
+    const RowTabs<I, double> Tb = row_stage<I, double>(sv, P, smem_raw);
+    const double sc = S->sigma_cur, bp_ = S->beta_prev * S->sigma_prev;
+    double dot = 0.0;
+    for (uint64_t r = blockIdx.x * (uint64_t)ROW_NT + threadIdx.x; r < sv.dim; r += (uint64_t)gridDim.x * ROW_NT) {
+        double acc[1], dg;
+        row_hops<I, double, double, 1, HALF>(sv, P, Tb, (I)r, qc, 1, 0, acc, &dg);
+        const double hv = dg * qc[r] + acc[0];
+        const double u = sc * hv - bp_ * qp[r];
+        qp[r] = u;
+        dot += (sc * qc[r]) * u;
+    }
+    dot = block_sum<ROW_NT>(dot, red);
     if (threadIdx.x == 0) part[blockIdx.x] = dot;
 }
 
@@ -574,9 +602,15 @@ static int enqueue_phase_t(hm_lanczos *R, int parity, int phase, cudaStream_t st
             HM_TRY(s1_lz32(R->s1, (const float *)qc, (float *)qp, R->sc, s1part, st));
             k_lz_alpha<<<1, NT, 0, st>>>(R->sc, s1part, R->s1.nblocks, R->alpha, pprev);
         } else {
-            const size_t sm = row_smem_bytes<I>(sv);
-            k_lz_matvec<I, T, Acc><<<nblk, NT, sm, st>>>(sv, R->bp, qc, qp, R->sc, R->part, R->run);
-            k_lz_alpha<<<1, NT, 0, st>>>(R->sc, R->part, nblk, R->alpha, pprev);
+            const int np = R->row_blocks > 0 ? R->row_blocks : nblk;
+            if (R->row_blocks > 0) {
+                auto kern = sv.S2 == 1 ? k_lz_row<I, true> : k_lz_row<I, false>;
+                kern<<<np, ROW_NT, R->row_smem, st>>>(sv, R->rowp, (const double *)qc, (double *)qp, R->sc, R->part);
+            } else {
+                const size_t sm = row_smem_bytes<I>(sv);
+                k_lz_matvec<I, T, Acc><<<np, NT, sm, st>>>(sv, R->bp, qc, qp, R->sc, R->part, R->run);
+            }
+            k_lz_alpha<<<1, NT, 0, st>>>(R->sc, R->part, np, R->alpha, pprev);
         }
     } else if (b64) {
         if (R->psi)
@@ -598,17 +632,26 @@ static int enqueue_phase_t(hm_lanczos *R, int parity, int phase, cudaStream_t st
     return HM_OK;
 }
 
-// raises the dynamic shared-memory limit of the product kernel (outside any capture)
+// plans the general row product and raises its dynamic shared-memory limit (outside any capture)
 template <class I, class T, class Acc>
-static int prepare_t(const hm_basis *b) {
-    HM_CUDA(raise_smem_limit(k_lz_matvec<I, T, Acc>, (int)row_smem_bytes<I>(b->view)));
+static int prepare_t(const hm_basis *b, hm_lanczos *R) {
+    const SectorView &sv = b->view;
+    R->row_blocks = 0;
+    if (sizeof(T) == 8 && row_plan(sv, R->bp, 8, &R->rowp, &R->row_smem) == 0) {
+        auto kern = sv.S2 == 1 ? k_lz_row<I, true> : k_lz_row<I, false>;
+        HM_CUDA(raise_smem_limit(kern, R->row_smem));
+        R->row_blocks = row_grid(sv.dim, sv.S2 == 1 ? row_most<k_lz_row<I, true>>() : row_most<k_lz_row<I, false>>(), R->row_smem);
+        return HM_OK;
+    }
+    HM_CUDA(raise_smem_limit(k_lz_matvec<I, T, Acc>, (int)row_smem_bytes<I>(sv)));
     return HM_OK;
 }
 
-static int prepare(const hm_basis *b, int dtype) {
+static int prepare(const hm_basis *b, int dtype, hm_lanczos *R) {
     const bool i64 = b->view.idx64 != 0;
-    if (dtype == HM_F64) return i64 ? prepare_t<uint64_t, double, double>(b) : prepare_t<uint32_t, double, double>(b);
-    return i64 ? prepare_t<uint64_t, float, float>(b) : prepare_t<uint32_t, float, float>(b);
+    if (dtype == HM_F64)
+        return i64 ? prepare_t<uint64_t, double, double>(b, R) : prepare_t<uint32_t, double, double>(b, R);
+    return i64 ? prepare_t<uint64_t, float, float>(b, R) : prepare_t<uint32_t, float, float>(b, R);
 }
 
 static int enqueue_phase(hm_lanczos *R, int phase, cudaStream_t st) {
@@ -674,7 +717,7 @@ static int lz_create(const hm_basis *b, int n_bonds, const int32_t *u, const int
         delete R;
         return fail(HM_EWORKSPACE, "workspace must be >= %zu bytes, 256-byte aligned", need);
     }
-    rc = prepare(b, dtype);
+    rc = prepare(b, dtype, R);
     if (rc < 0) { delete R; return rc; }
     R->use_blk = 0;
     R->use_mom = b->mom_k >= 0;

@@ -30,10 +30,37 @@ k_matvec(SectorView sv, BondParams bp, const T *__restrict__ x, T *__restrict__ 
     });
 }
 
+template <class I, class T, class Acc, int NV, bool HALF>
+__global__ void __launch_bounds__(ROW_NT)
+k_row_matvec(SectorView sv, RowPlan P, const T *__restrict__ x, T *__restrict__ y, int ld, int c0) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const RowTabs<I, Acc> Tb = row_stage<I, Acc>(sv, P, smem_raw);
+    for (uint64_t r = blockIdx.x * (uint64_t)ROW_NT + threadIdx.x; r < sv.dim; r += (uint64_t)gridDim.x * ROW_NT) {
+        Acc acc[NV], dg;
+        row_hops<I, T, Acc, NV, HALF>(sv, P, Tb, (I)r, x, ld, c0, acc, &dg);
+        const T *xi = x + r * ld + c0;
+        T *yi = y + r * ld + c0;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) yi[k] = (T)(dg * (Acc)xi[k] + acc[k]);
+    }
+}
+
 template <class I, class T, class Acc, int NV>
 static int launch_matvec(const SectorView &sv, const BondParams &bp, const T *x, T *y, int ld,
                          int c0, cudaStream_t st) {
-    size_t sm = row_smem_bytes<I>(sv);
+    RowPlan P;
+    size_t sm = 0;
+    if (row_plan(sv, bp, sizeof(Acc), &P, &sm) == 0) {
+        auto run = [&](auto kern, int most) -> int {
+            if (sm > 48 * 1024) HM_CUDA(raise_smem_limit(kern, sm));
+            kern<<<row_grid(sv.dim, most, sm), ROW_NT, sm, st>>>(sv, P, x, y, ld, c0);
+            HM_CUDA(cudaGetLastError());
+            return HM_OK;
+        };
+        return sv.S2 == 1 ? run(k_row_matvec<I, T, Acc, NV, true>, row_most<k_row_matvec<I, T, Acc, NV, true>>())
+                          : run(k_row_matvec<I, T, Acc, NV, false>, row_most<k_row_matvec<I, T, Acc, NV, false>>());
+    }
+    sm = row_smem_bytes<I>(sv);
     HM_CUDA(raise_smem_limit(k_matvec<I, T, Acc, NV>, (int)sm));
     k_matvec<I, T, Acc, NV><<<grid_blocks(sv.dim, 256), 256, sm, st>>>(sv, bp, x, y, ld, c0, row_run_len());
     HM_CUDA(cudaGetLastError());
