@@ -170,9 +170,8 @@ static std::vector<uint64_t> row_tables(const hm_basis *b) {
 }
 
 int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, size_t *smem) {
-    if (row_run_len() > 1 || bp.nb > ROW_MB) return 1;
+    if (row_run_len() > 1 || bp.nb > ROW_MB || bp.nb == 0) return 1;
     const int N = sv.N, S2 = sv.S2, n1 = S2 + 1;
-    P->nb = bp.nb;
     P->nc = P->nslots = 0;
     memcpy(P->hs_pdn, bp.hs_pdn, sizeof P->hs_pdn);
     memcpy(P->hs_pup, bp.hs_pup, sizeof P->hs_pup);
@@ -181,7 +180,7 @@ int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, siz
     int last[HM_MAX_SITES], slot_of[HM_MAX_SITES], freed[HM_MAX_SITES], nf = 0;    // last[q]: lowest partner below q
     for (int r = 0; r < N; ++r) last[r] = N;
     double mx = 0.0;
-    int count[HM_MAX_SITES + 1] = {};
+    int count[HM_MAX_SITES] = {};
     for (int t = 0; t < bp.nb; ++t) {
         int c = t > 0 && bp.jm[t] == bp.jm[t - 1] ? bc[t - 1] : 0;
         while (c < P->nc && P->jm[c] != bp.jm[t]) ++c;
@@ -193,39 +192,31 @@ int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, siz
     }
     // slots: a site holds one from its own position down to its lowest partner's
     for (int r = N - 1; r >= 0; --r) {
-        P->slot[r] = ROW_SLOT_NONE;
+        slot_of[r] = ROW_SLOT_NONE;
         if (last[r] < r) {
             if (nf == 0) freed[nf++] = P->nslots++;
             slot_of[r] = freed[--nf];
-            P->slot[r] = (uint8_t)slot_of[r];
         }
         for (int q = r + 1; q < N; ++q)
             if (last[q] == r) freed[nf++] = slot_of[q];
     }
-    int at[HM_MAX_SITES + 1];
-    P->bs[0] = 0;
+    int at[HM_MAX_SITES], n = 0;
     for (int r = 0; r < N; ++r) {
-        at[r] = P->bs[r];
-        P->bs[r + 1] = (uint16_t)(P->bs[r] + count[r]);
+        at[r] = n;
+        P->pos[r] = (uint32_t)n | ((uint32_t)count[r] << 10) | ((uint32_t)slot_of[r] << 20);
+        n += count[r];
     }
-    for (int t = 0; t < bp.nb; ++t) {
-        const int n = at[bp.p[t]]++;
-        P->q[n] = bp.q[t];
-        P->qs[n] = (uint8_t)slot_of[bp.q[t]];
-        P->cls[n] = bc[t];
-    }
+    for (int t = 0; t < bp.nb; ++t)
+        P->bond[at[bp.p[t]]++] = (uint32_t)(bp.q[t] * sv.bits) | ((uint32_t)slot_of[bp.q[t]] << 8) | ((uint32_t)bc[t] << 16);
     // diagonal sum_b dC_b k_b with |k_b| <= S2^2, below 2^62; taken when that leaves the largest
     // coupling 52 bits or more (a binary64 sum of the terms rounds no finer)
     int ex = 0, kb = 0;
     std::frexp(mx, &ex);                             // mx < 2^ex
     while ((1 << kb) < S2 * S2 * std::max(1, bp.nb)) ++kb;
     const int s = 62 - kb - ex;
-    P->dint = 62 - kb >= 52 && s > -1000 && s < 1000;
-    if (P->dint) {
-        P->dscale = std::ldexp(1.0, -s);
-        for (int c = 0; c < P->nc; ++c) P->dC[c] = std::llround(std::ldexp(P->jm[c] / 4.0, s));
-    }
-    P->tab = (size_t)P->nc * 2 * n1 * n1 * es <= 16 * 1024;
+    if (62 - kb < 52 || s <= -1000 || s >= 1000) return 1;
+    P->dscale = std::ldexp(1.0, -s);
+    for (int c = 0; c < P->nc; ++c) P->dC[c] = std::llround(std::ldexp(P->jm[c] / 4.0, s));
     const size_t tabs = sv.idx64 ? row_tab_bytes<uint64_t>(sv) : row_tab_bytes<uint32_t>(sv);
     *smem = row_coef_bytes(*P, S2, es) + tabs + (size_t)P->nslots * ROW_NT * (sv.idx64 ? 16 : 8);
     // at least two CTAs on an SM; more shared memory than that leaves the table form ahead

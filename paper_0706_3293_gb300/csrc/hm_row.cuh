@@ -26,7 +26,7 @@ namespace hm {
 // the exchange coefficients -J_b f are tables too (one multiply-add an exchange) and the
 // diagonal is an exact integer sum, converted once a row.  The gathers of one bond are in flight
 // while those of the bond before are added.  Measured (s = 3/2 ring, N = 12, 1.7 M rows, FP64):
-// k_matvec, the table form, 362 us; this form 172 us.
+// k_matvec, the table form, 362 us; this form 110 us.
 template <class I> struct alignas(4 * sizeof(I)) RowEF { I ep, fp, em, fm; };
 template <class I> struct alignas(2 * sizeof(I)) RowG { I gp, gm; };
 
@@ -37,22 +37,20 @@ constexpr int ROW_SLOT_NONE = 255;
 // launch (3.9 KB here)
 constexpr int ROW_MB = 128;
 struct RowPlan {
-    int nb, nslots, nc;
-    int tab;                         // exchange coefficients from a table per class (else J f formed per exchange)
-    int dint;                        // diagonal as the integer sum of dC k (else J k / 4 added in the Acc type)
+    int nslots, nc;
     double dscale;                   // 2^-s of dC
-    uint8_t slot[HM_MAX_SITES];      // slot of the site's R, or ROW_SLOT_NONE
-    uint16_t bs[HM_MAX_SITES + 1];   // bonds with lower end r: [bs[r], bs[r + 1])
-    uint8_t q[ROW_MB], qs[ROW_MB];          // upper end and its slot
-    uint16_t cls[ROW_MB];              // class: index of the bond's distinct coupling
-    double jm[ROW_MB];                // by class: -J
-    long long dC[ROW_MB];             // by class: round(-J / 4 2^s)
+    // per position: first bond whose lower end it is | their number << 10 | slot of its R << 20
+    // (ROW_SLOT_NONE: not the upper end of a bond)
+    uint32_t pos[HM_MAX_SITES];
+    uint32_t bond[ROW_MB];           // bit offset of the upper end's digit | its slot << 8 | class << 16
+    double jm[ROW_MB];               // by class (distinct coupling): -J
+    long long dC[ROW_MB];            // by class: round(-J / 4 2^s)
     double hs_pdn[64], hs_pup[64];   // as in BondParams
 };
 
-// the plan of a bond list; 0, or 1 when the sector's tables, the bonds (more than ROW_MB) or the run
-// length (HM_ROW_RUN) ask for the table form.  *smem: dynamic shared memory of a CTA for
-// accumulation type size es
+// the plan of a bond list; 0, or 1 when the table form has to serve: more than ROW_MB bonds, tables
+// above the shared memory, couplings the integer diagonal does not hold to 52 bits, or row
+// runs (HM_ROW_RUN).  *smem: dynamic shared memory of a CTA for accumulation type size es
 int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, size_t *smem);
 
 // resident CTAs per SM that the registers of kernel K allow
@@ -75,7 +73,7 @@ inline int row_grid(uint64_t rows, int most, size_t smem) {
 
 __host__ __device__ __forceinline__ size_t row_coef_bytes(const RowPlan &P, int S2, int es) {
     const int n1 = S2 + 1;
-    return ((size_t)(P.tab ? P.nc * 2 * n1 * n1 : 2 * n1 * n1) * es + 15) & ~(size_t)15;
+    return ((size_t)P.nc * 2 * n1 * n1 * es + 15) & ~(size_t)15;
 }
 
 // shared layout: exchange coefficients | E, F | G | CD | slots
@@ -96,11 +94,10 @@ template <class I, class Acc>
 __device__ __forceinline__ RowTabs<I, Acc> row_stage(const SectorView &sv, const RowPlan &P, unsigned char *smem) {
     const int n1 = sv.S2 + 1, n2 = n1 * n1;
     Acc *coef = reinterpret_cast<Acc *>(smem);
-    for (int k = threadIdx.x; k < (P.tab ? P.nc : 1) * 2 * n2; k += ROW_NT) {
+    for (int k = threadIdx.x; k < P.nc * 2 * n2; k += ROW_NT) {
         const int c = k / (2 * n2), m = k % (2 * n2), e = m % n2, h = (e / n1) * 8 + e % n1;
         const double f = m < n2 ? P.hs_pdn[h] : P.hs_pup[h];
-        if constexpr (sizeof(Acc) == 8) coef[k] = P.tab ? P.jm[c] * f : f;
-        else coef[k] = P.tab ? (float)P.jm[c] * (float)f : (float)f;
+        coef[k] = (Acc)P.jm[c] * (Acc)f;
     }
     I *cd = reinterpret_cast<I *>(smem + row_coef_bytes(P, sv.S2, sizeof(Acc)));
     // device tables: CD, then E/F, then G (basis_build); in shared memory the wide ones first
@@ -117,21 +114,24 @@ __device__ __forceinline__ RowTabs<I, Acc> row_stage(const SectorView &sv, const
     return t;
 }
 
-// every bond of the state of index i: f(t, a_p, a_q, target of s-_p s+_q (dp = +1), target of
+// every bond of the state of index i: f(class, a_p, a_q, target of s-_p s+_q (dp = +1), target of
 // s+_p s-_q (dp = -1)); a target is meaningful only when the exchange is allowed
 template <class I, class Acc, class F>
 __device__ __forceinline__ void row_sweep(const SectorView &sv, const RowPlan &P, const RowTabs<I, Acc> &T, I i, F &&f) {
-    const int bits = sv.bits, S2 = sv.S2, mask = (1 << bits) - 1;
+    const int bits = sv.bits, S2 = sv.S2;
+    const uint32_t mask = (1u << bits) - 1u;
+    const int o2 = S2 + 1 < 2 ? S2 + 1 : 2, o3 = S2 + 1 < 3 ? S2 + 1 : 3;   // entry S2 + 1 is above every index
     uint64_t w = 0;
-    int S = sv.A;
+    int S = sv.A, row = (sv.N - 1) * sv.cd_rowlen;
     I res = i, qp = 0, qm = 0;
-    for (int r = sv.N - 1; r >= 0; --r) {
-        const int ix = r * sv.cd_rowlen + S * sv.cd_w;
+    for (int r = sv.N - 1; r >= 0; --r, row -= sv.cd_rowlen) {
+        const int ix = row + S * sv.cd_w;
         int a = S;
         if (r > 0) {                               // the digit whose cumulative range holds res
-            a = 0;
-            for (int k = 1; k <= S2; ++k) a += T.cd[ix + k] <= res;
-            res -= T.cd[ix + a];
+            const I *c = T.cd + ix;
+            a = (c[1] <= res) + (c[o2] <= res) + (c[o3] <= res);
+            for (int k = 4; k <= S2; ++k) a += c[k] <= res;
+            res -= c[a];
         }
         w |= (uint64_t)a << (r * bits);
         const RowEF<I> e = T.ef[ix + a];
@@ -139,66 +139,66 @@ __device__ __forceinline__ void row_sweep(const SectorView &sv, const RowPlan &P
         const I lp = i + e.ep + qp, lm = i + e.em + qm;
         qp += g.gp;
         qm += g.gm;
-        const int sl = P.slot[r];
+        const uint32_t pr = P.pos[r];
+        const int sl = (int)(pr >> 20);
         if (sl != ROW_SLOT_NONE) T.slots[sl * ROW_NT] = RowG<I>{(I)(e.fp - qp), (I)(e.fm - qm)};
-        for (int t = P.bs[r]; t < P.bs[r + 1]; ++t) {
-            const int aq = (int)(w >> (P.q[t] * bits)) & mask;
-            const RowG<I> R = T.slots[P.qs[t] * ROW_NT];
-            f(t, a, aq, (I)(lp + R.gp), (I)(lm + R.gm));
+        const int t1 = (int)(pr & 1023u) + (int)((pr >> 10) & 1023u);
+        for (int t = (int)(pr & 1023u); t < t1; ++t) {
+            const uint32_t br = P.bond[t];
+            const int aq = (int)((uint32_t)(w >> (br & 255u)) & mask);
+            const RowG<I> R = T.slots[((br >> 8) & 255u) * ROW_NT];
+            f((int)(br >> 16), a, aq, (I)(lp + R.gp), (I)(lm + R.gm));
         }
         S -= a;
     }
 }
 
-// (H x)_i for NV columns: *dg the diagonal element, acc the exchange sums.  HALF: s = 1/2, where
-// at most one direction of a bond is allowed
-template <class I, class T, class Acc, int NV, bool HALF>
+// (H x)_i for NV columns: *dg the diagonal element, acc the exchange sums.  MODE: ROW_ONE one class
+// of couplings (a ring, a uniform lattice); ROW_HALF s = 1/2, where a bond allows one direction at
+// most, so one gather and one multiply-add serve it; ROW_ANY the rest
+enum { ROW_ANY = 0, ROW_ONE = 1, ROW_HALF = 2 };
+template <class I, class T, class Acc, int NV, int MODE>
 __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P, const RowTabs<I, Acc> &Tb, I i,
-                                         const T *__restrict__ x, int ld, int c0, Acc *acc, Acc *dg_out) {
+                                         const T *__restrict__ x, int ld, int c0, Acc *acc, Acc *dg) {
     const int S2 = sv.S2, n1 = S2 + 1, n2 = n1 * n1;
-    Acc dg = Acc(0), cp[2] = {Acc(0), Acc(0)};     // the bond before: coefficients and gathered values
-    T vp[HALF ? 1 : 2][NV];
+    Acc cp[2] = {Acc(0), Acc(0)};                  // the bond before: coefficients and gathered values
+    T vp[2][NV];
     long long di = 0;
+    int k1 = 0;
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
         acc[k] = Acc(0);
-        vp[0][k] = T(0);
-        if constexpr (!HALF) vp[1][k] = T(0);
+        vp[0][k] = vp[1][k] = T(0);
     }
-    row_sweep(sv, P, Tb, i, [&](int t, int ap, int aq, I jp, I jm) {
-        const int c = P.cls[t], k4 = (S2 - 2 * ap) * (S2 - 2 * aq);
-        if (P.dint) di += P.dC[c] * k4;
-        else if constexpr (sizeof(Acc) == 8) dg = fma(0.25 * P.jm[c], (double)k4, dg);
-        else dg = fmaf(0.25f * (float)P.jm[c], (float)k4, dg);
-        const Acc *co = Tb.coef + (P.tab ? c * 2 * n2 : 0) + ap * n1 + aq;
-        auto cf = [&](int d) -> Acc {
-            const Acc v = co[d * n2];
-            if (P.tab) return v;
-            if constexpr (sizeof(Acc) == 8) return P.jm[c] * v;
-            else return (float)P.jm[c] * v;
-        };
-        auto pend = [&](int d, bool ok, I j, Acc &cn, T *vn) {
-            cn = ok ? cf(d) : Acc(0);
-            const T *xr = x + (size_t)j * ld + c0;
-#pragma unroll
-            for (int k = 0; k < NV; ++k) vn[k] = ok ? __ldg(xr + k) : T(0);
-        };
+    row_sweep(sv, P, Tb, i, [&](int c, int ap, int aq, I jp, I jm) {
+        const int kk = (S2 - 2 * ap) * (S2 - 2 * aq);
+        if constexpr (MODE == ROW_ONE) k1 += kk;
+        else di += P.dC[c] * kk;
+        const Acc *co = Tb.coef + ap * n1 + aq;
+        if constexpr (MODE != ROW_ONE) co += c * 2 * n2;
         const bool dn = ap >= 1 && aq < S2, up = ap < S2 && aq >= 1;
-        if constexpr (HALF) {
-            Acc c1;
-            T v1[NV];
-            pend(dn ? 0 : 1, dn || up, dn ? jm : jp, c1, v1);
+        if constexpr (MODE == ROW_HALF) {
+            const Acc cn = co[dn ? 0 : n2];        // zero in the table when neither is allowed
+            const T *xr = x + (size_t)(dn ? jm : jp) * ld + c0;
+            T vn[NV];
+#pragma unroll
+            for (int k = 0; k < NV; ++k) vn[k] = dn || up ? __ldg(xr + k) : T(0);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
                 acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
-                vp[0][k] = v1[k];
+                vp[0][k] = vn[k];
             }
-            cp[0] = c1;
+            cp[0] = cn;
         } else {
-            Acc c1, c2;
+            // a coefficient whose exchange is not allowed is zero in the table
+            const Acc c1 = co[0], c2 = co[n2];
+            const T *x1 = x + (size_t)jm * ld + c0, *x2 = x + (size_t)jp * ld + c0;
             T v1[NV], v2[NV];
-            pend(0, dn, jm, c1, v1);
-            pend(1, up, jp, c2, v2);
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                v1[k] = dn ? __ldg(x1 + k) : T(0);
+                v2[k] = up ? __ldg(x2 + k) : T(0);
+            }
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
                 acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
@@ -213,9 +213,9 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
         acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
-        if constexpr (!HALF) acc[k] = fma(cp[1], (Acc)vp[1][k], acc[k]);
+        if constexpr (MODE != ROW_HALF) acc[k] = fma(cp[1], (Acc)vp[1][k], acc[k]);
     }
-    *dg_out = P.dint ? (Acc)((double)di * P.dscale) : dg;
+    *dg = MODE == ROW_ONE ? (Acc)(0.25 * P.jm[0] * (double)k1) : (Acc)((double)di * P.dscale);
 }
 
 // ---- the table form ------------------------------------------------------------------------

@@ -213,7 +213,7 @@ k_lz_matvec(SectorView sv, BondParams bp, const T *__restrict__ qc, T *__restric
 // the same by the sweep form of the row product (hm_row.cuh), FP64 vectors.  FP32 runs keep the
 // table form, which adds a row's bonds in list order: another order rounds a float row
 // differently, and a run carries that into every alpha and beta
-template <class I, bool HALF>
+template <class I, int MODE>
 __global__ void __launch_bounds__(ROW_NT)
 k_lz_row(SectorView sv, RowPlan P, const double *__restrict__ qc, double *__restrict__ qp,
          const LzScalars *__restrict__ S, double *__restrict__ part) {
@@ -225,7 +225,7 @@ k_lz_row(SectorView sv, RowPlan P, const double *__restrict__ qc, double *__rest
     double dot = 0.0;
     for (uint64_t r = blockIdx.x * (uint64_t)ROW_NT + threadIdx.x; r < sv.dim; r += (uint64_t)gridDim.x * ROW_NT) {
         double acc[1], dg;
-        row_hops<I, double, double, 1, HALF>(sv, P, Tb, (I)r, qc, 1, 0, acc, &dg);
+        row_hops<I, double, double, 1, MODE>(sv, P, Tb, (I)r, qc, 1, 0, acc, &dg);
         const double hv = dg * qc[r] + acc[0];
         const double u = sc * hv - bp_ * qp[r];
         qp[r] = u;
@@ -565,6 +565,11 @@ __global__ void k_store_nrm2(LzScalars *S, const double *__restrict__ part, int 
 // ---------------------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------------------
+template <class I>
+static auto lz_row_kernel(const hm_lanczos *R) {
+    return R->basis->view.S2 == 1 ? k_lz_row<I, ROW_HALF> : R->rowp.nc == 1 ? k_lz_row<I, ROW_ONE> : k_lz_row<I, ROW_ANY>;
+}
+
 template <class I, class T, class Acc>
 static int enqueue_phase_t(hm_lanczos *R, int parity, int phase, cudaStream_t st) {
     const SectorView &sv = R->basis->view;
@@ -604,7 +609,7 @@ static int enqueue_phase_t(hm_lanczos *R, int parity, int phase, cudaStream_t st
         } else {
             const int np = R->row_blocks > 0 ? R->row_blocks : nblk;
             if (R->row_blocks > 0) {
-                auto kern = sv.S2 == 1 ? k_lz_row<I, true> : k_lz_row<I, false>;
+                auto kern = lz_row_kernel<I>(R);
                 kern<<<np, ROW_NT, R->row_smem, st>>>(sv, R->rowp, (const double *)qc, (double *)qp, R->sc, R->part);
             } else {
                 const size_t sm = row_smem_bytes<I>(sv);
@@ -638,9 +643,10 @@ static int prepare_t(const hm_basis *b, hm_lanczos *R) {
     const SectorView &sv = b->view;
     R->row_blocks = 0;
     if (sizeof(T) == 8 && row_plan(sv, R->bp, 8, &R->rowp, &R->row_smem) == 0) {
-        auto kern = sv.S2 == 1 ? k_lz_row<I, true> : k_lz_row<I, false>;
-        HM_CUDA(raise_smem_limit(kern, R->row_smem));
-        R->row_blocks = row_grid(sv.dim, sv.S2 == 1 ? row_most<k_lz_row<I, true>>() : row_most<k_lz_row<I, false>>(), R->row_smem);
+        HM_CUDA(raise_smem_limit(lz_row_kernel<I>(R), R->row_smem));
+        const int most = std::min(row_most<k_lz_row<I, ROW_HALF>>(),
+                                  std::min(row_most<k_lz_row<I, ROW_ONE>>(), row_most<k_lz_row<I, ROW_ANY>>()));
+        R->row_blocks = row_grid(sv.dim, most, R->row_smem);
         return HM_OK;
     }
     HM_CUDA(raise_smem_limit(k_lz_matvec<I, T, Acc>, (int)row_smem_bytes<I>(sv)));
@@ -717,7 +723,7 @@ static int lz_create(const hm_basis *b, int n_bonds, const int32_t *u, const int
         delete R;
         return fail(HM_EWORKSPACE, "workspace must be >= %zu bytes, 256-byte aligned", need);
     }
-    rc = prepare(b, dtype, R);
+    rc = prepare(b, dtype, R);   // reads R->basis
     if (rc < 0) { delete R; return rc; }
     R->use_blk = 0;
     R->use_mom = b->mom_k >= 0;

@@ -30,14 +30,14 @@ k_matvec(SectorView sv, BondParams bp, const T *__restrict__ x, T *__restrict__ 
     });
 }
 
-template <class I, class T, class Acc, int NV, bool HALF>
+template <class I, class T, class Acc, int NV, int MODE>
 __global__ void __launch_bounds__(ROW_NT)
 k_row_matvec(SectorView sv, RowPlan P, const T *__restrict__ x, T *__restrict__ y, int ld, int c0) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const RowTabs<I, Acc> Tb = row_stage<I, Acc>(sv, P, smem_raw);
     for (uint64_t r = blockIdx.x * (uint64_t)ROW_NT + threadIdx.x; r < sv.dim; r += (uint64_t)gridDim.x * ROW_NT) {
         Acc acc[NV], dg;
-        row_hops<I, T, Acc, NV, HALF>(sv, P, Tb, (I)r, x, ld, c0, acc, &dg);
+        row_hops<I, T, Acc, NV, MODE>(sv, P, Tb, (I)r, x, ld, c0, acc, &dg);
         const T *xi = x + r * ld + c0;
         T *yi = y + r * ld + c0;
 #pragma unroll
@@ -57,8 +57,9 @@ static int launch_matvec(const SectorView &sv, const BondParams &bp, const T *x,
             HM_CUDA(cudaGetLastError());
             return HM_OK;
         };
-        return sv.S2 == 1 ? run(k_row_matvec<I, T, Acc, NV, true>, row_most<k_row_matvec<I, T, Acc, NV, true>>())
-                          : run(k_row_matvec<I, T, Acc, NV, false>, row_most<k_row_matvec<I, T, Acc, NV, false>>());
+        if (sv.S2 == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_HALF>, row_most<k_row_matvec<I, T, Acc, NV, ROW_HALF>>());
+        if (P.nc == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_ONE>, row_most<k_row_matvec<I, T, Acc, NV, ROW_ONE>>());
+        return run(k_row_matvec<I, T, Acc, NV, ROW_ANY>, row_most<k_row_matvec<I, T, Acc, NV, ROW_ANY>>());
     }
     sm = row_smem_bytes<I>(sv);
     HM_CUDA(raise_smem_limit(k_matvec<I, T, Acc, NV>, (int)sm));
