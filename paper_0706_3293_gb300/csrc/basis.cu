@@ -217,6 +217,8 @@ int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, siz
     if (62 - kb < 52 || s <= -1000 || s >= 1000) return 1;
     P->dscale = std::ldexp(1.0, -s);
     for (int c = 0; c < P->nc; ++c) P->dC[c] = std::llround(std::ldexp(P->jm[c] / 4.0, s));
+    P->dsum = 0;
+    for (int t = 0; t < bp.nb; ++t) P->dsum += P->dC[bc[t]];
     const size_t tabs = sv.idx64 ? row_tab_bytes<uint64_t>(sv) : row_tab_bytes<uint32_t>(sv);
     *smem = row_coef_bytes(*P, S2, es) + tabs + (size_t)P->nslots * ROW_NT * (sv.idx64 ? 16 : 8);
     // at least two CTAs on an SM; more shared memory than that leaves the table form ahead

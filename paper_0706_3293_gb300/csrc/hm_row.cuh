@@ -45,6 +45,7 @@ struct RowPlan {
     uint32_t bond[ROW_MB];           // bit offset of the upper end's digit | its slot << 8 | class << 16
     double jm[ROW_MB];               // by class (distinct coupling): -J
     long long dC[ROW_MB];            // by class: round(-J / 4 2^s)
+    long long dsum;                  // sum of dC over the bonds (s = 1/2: the diagonal is dsum - 2 sum over unequal spins)
     double hs_pdn[64], hs_pup[64];   // as in BondParams
 };
 
@@ -53,21 +54,16 @@ struct RowPlan {
 // runs (HM_ROW_RUN).  *smem: dynamic shared memory of a CTA for accumulation type size es
 int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, size_t *smem);
 
-// resident CTAs per SM that the registers of kernel K allow
-template <auto K>
-inline int row_most() {
-    static const int most = [] {
-        int per = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, K, ROW_NT, 0) != cudaSuccess) cudaGetLastError();
-        return per < 1 ? 1 : per;
-    }();
-    return most;
-}
 // CTAs of a row kernel: one resident wave at most (every CTA stages the tables), and no more
 // than grid_blocks, for which the workspaces' partial sums are sized
-inline int row_grid(uint64_t rows, int most, size_t smem) {
-    const int fit = (int)((228 * 1024) / (smem + 1024));
-    const int wave = sm_count() * (fit < 1 ? 1 : fit < most ? fit : most), need = grid_blocks(rows, ROW_NT);
+template <class F>
+inline int row_grid(uint64_t rows, F kern, size_t smem) {
+    int per = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, ROW_NT, smem) != cudaSuccess) {
+        cudaGetLastError();
+        per = 1;
+    }
+    const int wave = sm_count() * (per < 1 ? 1 : per), need = grid_blocks(rows, ROW_NT);
     return need < wave ? need : wave;
 }
 
@@ -171,18 +167,15 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
         vp[0][k] = vp[1][k] = T(0);
     }
     row_sweep(sv, P, Tb, i, [&](int c, int ap, int aq, I jp, I jm) {
-        const int kk = (S2 - 2 * ap) * (S2 - 2 * aq);
-        if constexpr (MODE == ROW_ONE) k1 += kk;
-        else di += P.dC[c] * kk;
-        const Acc *co = Tb.coef + ap * n1 + aq;
-        if constexpr (MODE != ROW_ONE) co += c * 2 * n2;
-        const bool dn = ap >= 1 && aq < S2, up = ap < S2 && aq >= 1;
         if constexpr (MODE == ROW_HALF) {
-            const Acc cn = co[dn ? 0 : n2];        // zero in the table when neither is allowed
-            const T *xr = x + (size_t)(dn ? jm : jp) * ld + c0;
+            // a_p = 1: the first digits (1, 0) of the table, -J / 2 as for (0, 1)
+            const bool ne = ap != aq;
+            if (ne) di += P.dC[c];
+            const Acc cn = Tb.coef[c * 8 + 2];
+            const T *xr = x + (size_t)(ap ? jm : jp) * ld + c0;
             T vn[NV];
 #pragma unroll
-            for (int k = 0; k < NV; ++k) vn[k] = dn || up ? __ldg(xr + k) : T(0);
+            for (int k = 0; k < NV; ++k) vn[k] = ne ? __ldg(xr + k) : T(0);
 #pragma unroll
             for (int k = 0; k < NV; ++k) {
                 acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
@@ -190,6 +183,12 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
             }
             cp[0] = cn;
         } else {
+            const int kk = (S2 - 2 * ap) * (S2 - 2 * aq);
+            if constexpr (MODE == ROW_ONE) k1 += kk;
+            else di += P.dC[c] * kk;
+            const Acc *co = Tb.coef + ap * n1 + aq;
+            if constexpr (MODE != ROW_ONE) co += c * 2 * n2;
+            const bool dn = ap >= 1 && aq < S2, up = ap < S2 && aq >= 1;
             // a coefficient whose exchange is not allowed is zero in the table
             const Acc c1 = co[0], c2 = co[n2];
             const T *x1 = x + (size_t)jm * ld + c0, *x2 = x + (size_t)jp * ld + c0;
@@ -215,6 +214,7 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
         acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
         if constexpr (MODE != ROW_HALF) acc[k] = fma(cp[1], (Acc)vp[1][k], acc[k]);
     }
+    if constexpr (MODE == ROW_HALF) di = P.dsum - 2 * di;
     *dg = MODE == ROW_ONE ? (Acc)(0.25 * P.jm[0] * (double)k1) : (Acc)((double)di * P.dscale);
 }
 

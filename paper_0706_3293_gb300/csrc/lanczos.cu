@@ -644,9 +644,7 @@ static int prepare_t(const hm_basis *b, hm_lanczos *R) {
     R->row_blocks = 0;
     if (sizeof(T) == 8 && row_plan(sv, R->bp, 8, &R->rowp, &R->row_smem) == 0) {
         HM_CUDA(raise_smem_limit(lz_row_kernel<I>(R), R->row_smem));
-        const int most = std::min(row_most<k_lz_row<I, ROW_HALF>>(),
-                                  std::min(row_most<k_lz_row<I, ROW_ONE>>(), row_most<k_lz_row<I, ROW_ANY>>()));
-        R->row_blocks = row_grid(sv.dim, most, R->row_smem);
+        R->row_blocks = row_grid(sv.dim, lz_row_kernel<I>(R), R->row_smem);
         return HM_OK;
     }
     HM_CUDA(raise_smem_limit(k_lz_matvec<I, T, Acc>, (int)row_smem_bytes<I>(sv)));

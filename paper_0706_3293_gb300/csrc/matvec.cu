@@ -51,15 +51,15 @@ static int launch_matvec(const SectorView &sv, const BondParams &bp, const T *x,
     RowPlan P;
     size_t sm = 0;
     if (row_plan(sv, bp, sizeof(Acc), &P, &sm) == 0) {
-        auto run = [&](auto kern, int most) -> int {
+        auto run = [&](auto kern) -> int {
             if (sm > 48 * 1024) HM_CUDA(raise_smem_limit(kern, sm));
-            kern<<<row_grid(sv.dim, most, sm), ROW_NT, sm, st>>>(sv, P, x, y, ld, c0);
+            kern<<<row_grid(sv.dim, kern, sm), ROW_NT, sm, st>>>(sv, P, x, y, ld, c0);
             HM_CUDA(cudaGetLastError());
             return HM_OK;
         };
-        if (sv.S2 == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_HALF>, row_most<k_row_matvec<I, T, Acc, NV, ROW_HALF>>());
-        if (P.nc == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_ONE>, row_most<k_row_matvec<I, T, Acc, NV, ROW_ONE>>());
-        return run(k_row_matvec<I, T, Acc, NV, ROW_ANY>, row_most<k_row_matvec<I, T, Acc, NV, ROW_ANY>>());
+        if (sv.S2 == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_HALF>);
+        if (P.nc == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_ONE>);
+        return run(k_row_matvec<I, T, Acc, NV, ROW_ANY>);
     }
     sm = row_smem_bytes<I>(sv);
     HM_CUDA(raise_smem_limit(k_matvec<I, T, Acc, NV>, (int)sm));

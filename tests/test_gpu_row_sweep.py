@@ -70,3 +70,25 @@ def test_sweep_form_lanczos(hm, n, two_s, two_m, monkeypatch):
     scale = np.abs(res["2"].alpha).max()
     assert np.abs(res["1"].alpha - res["2"].alpha).max() <= 1e3 * len(bl) * 2.0**-46 * scale
     assert np.abs(res["1"].beta - res["2"].beta).max() <= 1e3 * len(bl) * 2.0**-46 * scale
+
+
+@pytest.mark.parametrize("k", ["0", "half"])
+@pytest.mark.parametrize("n,two_s,two_m", [(6, 1, 0), (12, 1, 0), (13, 1, 1), (16, 1, 4), (8, 2, 0), (6, 3, 0), (6, 4, 2)])
+def test_sweep_form_momentum(hm, n, two_s, two_m, k, monkeypatch):
+    """Momentum blocks, orbits of short period among the targets: the sweep form against the table
+    form, within the rounding of a row of T terms (x of size 1, row sums of |H| below sum |J| s (2s + 1),
+    orbit factors below sqrt(N))."""
+    if k == "half" and n % 2:
+        pytest.skip("momentum pi needs an even ring")
+    b = hm.Basis(n, two_s, two_m, momentum=0 if k == "0" else n // 2)
+    u, v, J = W.ring_bonds(n, -1.0, -0.375)
+    bl = hm.BondList.make(u, v, J)
+    bound = np.abs(J).sum() * (two_s / 2.0) * (two_s + 1) * np.sqrt(n)
+    rng = np.random.default_rng(n)
+    for dtype, eps in ((torch.float64, 2.0**-53), (torch.float32, 2.0**-24)):
+        x = torch.from_numpy(rng.uniform(-1, 1, b.dim)).to(dtype).cuda()
+        out = {}
+        for run in ("1", "2"):
+            monkeypatch.setenv("HM_ROW_RUN", run)
+            out[run] = hm.matvec(b, bl, x).double().cpu().numpy()
+        assert np.abs(out["1"] - out["2"]).max() <= 2 * (3 * len(bl) + 4) * eps * bound
