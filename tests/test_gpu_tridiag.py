@@ -49,3 +49,25 @@ def test_ftlm_long_krylov_spaces(hm):
     assert np.allclose(c.E, a.E, rtol=tol)
     k = int(np.argmax(a.mlen[:, 0]))
     assert abs(c.tau[k, 0, : c.mlen[k, 0]].sum() - 1.0) <= 430 * 16 * np.finfo(float).eps
+
+
+@pytest.mark.parametrize("n,two_m,steps", [(11, 1, 7), (11, 1, 8), (12, 4, 33), (13, 1, 192), (13, 1, 200)])
+def test_arnoldi_gram_schmidt_tiles(hm, n, two_m, steps):
+    """Gram-Schmidt over row tiles (up to 192 vectors, then the untiled kernels) at row counts that are no
+    multiple of a tile: H is tridiagonal to the double-float dots' rounding (dim terms of 2^-46 of the
+    vectors' products, |v| = |w| / beta = 1, scaled by |H|), as a Hermitian H's Arnoldi matrix is, and
+    its lowest eigenvalue is the sector's once the space holds it."""
+    inst = W.small_ring(n, -1.0, -0.4, two_m=two_m)
+    b = hm.Basis(inst.n_sites, inst.two_s, inst.two_m)
+    r = hm.arnoldi_run(b, hm.bonds_of(inst), steps, seed=11, n_ritz=1)
+    assert r.steps == steps
+    H = r.H[:steps, :steps]
+    scale = np.abs(r.H).max()
+    off = H - np.triu(np.tril(H, 1), -1)
+    assert np.abs(off).max() <= b.dim * 2.0**-46 * scale
+    assert np.abs(np.diag(H, 1) - np.diag(H, -1)).max() <= b.dim * 2.0**-46 * scale
+    if steps >= 192:
+        eye = torch.eye(b.dim, dtype=torch.float64, device="cuda")
+        dense = torch.stack([hm.matvec(b, hm.bonds_of(inst), eye[k].contiguous()) for k in range(b.dim)])
+        e0 = np.linalg.eigvalsh(dense.cpu().numpy())[0]
+        assert abs(r.ritz[0] - e0) <= 1e-11 * abs(e0)
