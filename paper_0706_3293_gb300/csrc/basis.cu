@@ -319,7 +319,7 @@ int basis_build(int n_sites, int two_s, int two_m, hm_basis **out) {
     }
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_cd, bytes > 0 ? bytes : 8);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_scratch, 256);
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_scratch, (size_t)HM_ESLOTS * HM_EPART * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_cd, src, bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         if (b->d_cd) cudaFree(b->d_cd);

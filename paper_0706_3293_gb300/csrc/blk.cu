@@ -5,6 +5,7 @@
 #include <cstring>
 #include <cmath>
 #include <map>
+#include <memory>
 #include <tuple>
 #include <type_traits>
 
@@ -60,6 +61,7 @@ int blk_host_tables(const hm_basis *b, int K, std::vector<uint16_t> &U, std::vec
 
 static int blk_tables(hm_basis *b, int K, const void **dev, int *bytes, int *oU, int *oR0, int *oC,
                       const uint16_t **lw, int *lwoff) {
+    std::lock_guard<std::mutex> lk(b->tab_mu);
     auto it = b->blk_tabs.find(K);
     if (it == b->blk_tabs.end()) {
         std::vector<uint16_t> U;
@@ -323,10 +325,11 @@ static int blk_plan_bonds(hm_basis *b, const BondParams &bp, const std::vector<i
 // kernels with the generic row policy (blk_sweep.cuh); jit.cu builds the same bodies
 // with the plan's bonds written out
 // ---------------------------------------------------------------------------------------
-template <class T, int NC>
+template <class T, int NC, bool TAB>
 __global__ void __launch_bounds__(BLK_NT, 3)
-k_blk_matvec(BlkParams P, const T *__restrict__ x, T *__restrict__ y, const int *__restrict__ Eptr) {
-    matvec_body<T, NC, RowGeneric<NC>>(P, x, y, Eptr);
+k_blk_matvec(BlkParams P, const T *__restrict__ x, T *__restrict__ y, const int *__restrict__ Eptr, int nE) {
+    if constexpr (TAB) matvec_body<T, NC, RowTable<NC>>(P, x, y, Eptr, nE);
+    else matvec_body<T, NC, RowGeneric<NC>>(P, x, y, Eptr, nE);
 }
 
 template <int NC, bool IR>
@@ -342,32 +345,47 @@ k_blk_lz32(BlkParams P, const float *__restrict__ qc, float *__restrict__ qp, Lz
     lz32_body<NC, RowGeneric<NC>>(P, qc, qp, S, part);
 }
 
-// largest exponent field of a double vector (for the fixed-point unit)
-__global__ void k_max_exp(const unsigned long long *__restrict__ x, uint64_t n, int *out) {
-    int m = 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
-        m = max(m, (int)((x[i] >> 52) & 0x7FF));
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+// largest exponent field of a double vector (for the fixed-point unit), one partial maximum a CTA.
+// Two elements a load (x is 8-byte aligned only: an odd first element goes alone)
+__global__ void __launch_bounds__(256) k_max_exp(const unsigned long long *__restrict__ x, uint64_t n,
+                                                  int *__restrict__ part) {
+    __shared__ int red[8];
+    uint32_t m = 0;
+    const uint64_t head = ((uintptr_t)x & 15) && n ? 1 : 0, n2 = (n - head) / 2;
+    const uint4 *x2 = reinterpret_cast<const uint4 *>(x + head);
+    for (uint64_t i = blockIdx.x * (uint64_t)256 + threadIdx.x; i < n2; i += (uint64_t)gridDim.x * 256) {
+        const uint4 v = __ldg(x2 + i);
+        m = max(m, max(v.y & 0x7FF00000u, v.w & 0x7FF00000u));
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (head) m = max(m, (uint32_t)(x[0] >> 32) & 0x7FF00000u);
+        if (head + 2 * n2 < n) m = max(m, (uint32_t)(x[n - 1] >> 32) & 0x7FF00000u);
+    }
+    const int w = (int)__reduce_max_sync(0xffffffffu, m >> 20);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = red[0];
+        for (int k = 1; k < 8; ++k) t = max(t, red[k]);
+        part[blockIdx.x] = t;
+    }
 }
 
-template <class T, int NC>
-static int launch_blk_matvec(hm_basis *b, const BlkParams &P, const T *x, T *y, cudaStream_t st) {
-    const size_t sm = blk_row_smem_bytes(P, sizeof(T) == 8 ? 8 : 4, BLK_XPAD);
-    HM_CUDA(raise_smem_limit(k_blk_matvec<T, NC>, sm));
-    int *Ed = nullptr;
-    if constexpr (sizeof(T) == 8) {
-        Ed = (int *)b->d_scratch;
-        HM_CUDA(cudaMemsetAsync(Ed, 0, sizeof(int), st));
-        k_max_exp<<<grid_blocks(P.dim, 256), 256, 0, st>>>((const unsigned long long *)x, P.dim, Ed);
-        HM_CUDA(cudaGetLastError());
-    }
-    int per = 1;
-    HM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_blk_matvec<T, NC>, BLK_NT, sm));
-    const int blocks = std::min<int>(sm_count() * std::max(per, 1), 1 << P.H);
-    k_blk_matvec<T, NC><<<blocks, BLK_NT, sm, st>>>(P, x, y, Ed);
+// enqueues k_max_exp of x into the next exponent slot of the basis; its partial maxima are at *part,
+// *n of them
+static int launch_max_exp(hm_basis *b, const void *x, uint64_t n, int **part, int *np, cudaStream_t st) {
+    *part = (int *)b->d_scratch + (size_t)(b->eslot.fetch_add(1) % HM_ESLOTS) * HM_EPART;
+    const uint64_t want = (n + 2047) / 2048;                  // four loads a thread
+    *np = (int)std::min<uint64_t>(std::min(HM_EPART, sm_count() * 3), want ? want : 1);
+    k_max_exp<<<*np, 256, 0, st>>>((const unsigned long long *)x, n, *part);
     HM_CUDA(cudaGetLastError());
     return HM_OK;
+}
+
+template <class T, bool TAB>
+static const void *blk_mv_kernel(int nc) {
+    return nc == 1 ? (const void *)k_blk_matvec<T, 1, TAB> : nc == 2 ? (const void *)k_blk_matvec<T, 2, TAB>
+                                                                     : (const void *)k_blk_matvec<T, 4, TAB>;
 }
 
 // Split position of the block path: the low part holds K = min(15, N / 2 + 2) sites, at least 8
@@ -476,8 +494,9 @@ int blk_lz_jit(const BlkParams &P, int dtype, const void **kern, int *blocks, in
 // ring), built once per basis, layout and element size.  A per-bond plan (each bond its own
 // coefficient) takes no triangles, and a slot whose exchange is not allowed points at the
 // row itself, so that its difference x_i - x_t vanishes.  Returns 0 and sets P->tt, or 1 when
-// the policy does not apply (more than 48 entries, or HM_JIT_ROW selects another policy).
-int blk_target_table(hm_basis *b, BlkParams *P, int esize) {
+// the policy does not apply (more than 48 entries, or HM_JIT_ROW selects another policy) or the table
+// is not there yet and build is false (no allocation, no copy).
+int blk_target_table(hm_basis *b, BlkParams *P, int esize, bool build) {
     P->tt = nullptr;
     const char *rowk = getenv("HM_JIT_ROW");
     if (rowk && *rowk && strcmp(rowk, "table") != 0) return 1;
@@ -534,8 +553,10 @@ int blk_target_table(hm_basis *b, BlkParams *P, int esize) {
     for (auto &sl : low) key += std::to_string(sl.p) + "-" + std::to_string(sl.q) + "/" + std::to_string(sl.c) + ",";
     key += "|";
     for (int p : cps) key += std::to_string(p) + ",";
+    std::lock_guard<std::mutex> lk(b->tab_mu);
     auto it = b->blk_ttabs.find(key);
     if (it == b->blk_ttabs.end()) {
+        if (!build) return 1;
         const uint32_t rows = 1u << K;
         std::vector<uint32_t> rank(rows);                 // colex rank within the popcount class
         {
@@ -575,6 +596,8 @@ int blk_target_table(hm_basis *b, BlkParams *P, int esize) {
     P->tt_n = n;
     P->tt_ncross = (int)cps.size();
     for (size_t i = 0; i < cps.size(); ++i) P->tt_cross_p[i] = cps[i];
+    for (int e = 0; e < P->nxf; ++e)
+        P->tt_xe[P->xf_dst[e]] = (uint8_t)(2 * ntri + nsgl + (std::find(cps.begin(), cps.end(), (int)P->xf_p[e]) - cps.begin()));
     P->tt_ntri = ntri;
     P->tt_nsgl = nsgl;
     for (int t = 0; t < ntri; ++t) {
@@ -618,7 +641,7 @@ int blk_lz_split(hm_basis *b, const BondParams &bp, const BlkParams &P, int dtyp
     PA->split = 1;
     PB->split = 2;
     PB->rot = std::min(PB->H, 9);
-    if (blk_target_table(b, PA, 8) < 0 || blk_target_table(b, PB, 8) < 0) return 1;
+    if (blk_target_table(b, PA, 8, true) < 0 || blk_target_table(b, PB, 8, true) < 0) return 1;
     if (blk_lz_jit(*PA, dtype, kA, blkA, 1) != 0 || blk_lz_jit(*PB, dtype, kB, blkB, 2) != 0) return 1;
     return 0;
 }
@@ -655,53 +678,30 @@ int blk_lz32_launch(const BlkParams &P, const float *qc, float *qp, LzScalars *S
     return HM_OK;
 }
 
-// per-bond plan: the specialised y = H x kernel (jit.cu); 1 when it is not available
-static int launch_blk_matvec_pb(hm_basis *b, const BlkParams &P0, const void *x, void *y,
-                                int dtype, cudaStream_t st) {
-    BlkParams P = P0;
-    const int trc = blk_target_table(b, &P, dtype == HM_F64 ? 8 : 4);
-    if (trc < 0) return trc;
-    const void *k = nullptr;
-    if (jit_mv_kernel(P, dtype, &k) != 0) return 1;
-    const size_t sm = blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
-    HM_CUDA(raise_smem_limit(k, (int)sm));
-    int *Ed = nullptr;
-    if (dtype == HM_F64) {
-        Ed = (int *)b->d_scratch;
-        HM_CUDA(cudaMemsetAsync(Ed, 0, sizeof(int), st));
-        k_max_exp<<<grid_blocks(P.dim, 256), 256, 0, st>>>((const unsigned long long *)x, P.dim, Ed);
-        HM_CUDA(cudaGetLastError());
-    }
-    int per = 0;
-    HM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, BLK_NT, sm));
-    const int blocks = std::min<int>(sm_count() * std::max(per, 1), 1 << P.H);
-    void *args[] = {(void *)&P, (void *)&x, (void *)&y, (void *)&Ed};
-    HM_CUDA(cudaLaunchKernel(k, dim3(blocks), dim3(BLK_NT), args, sm, st));
-    return HM_OK;
-}
-
 // ---- bond correlations on the block path -------------------------------------------------
 int jit_bc_kernel(const BlkParams &P, int dtype, int nbk, const void **kern);
 
 constexpr int BC_CHUNK = 16;               // bonds per bond-correlation launch
 constexpr uint64_t BC_MIN_ROWS = 100000;   // smaller sectors: the general kernel (no compile)
 
-// out[k] = sign 2^u (T0 / 4 - C_k / 2) / div from the CTA partials of one chunk (fixed order)
-__global__ void k_bc_final(const double *__restrict__ part, int nctas, int nbk, const int *Eptr, double sign,
-                           const double *div, double *__restrict__ out) {
+// out[k] = sign 2^u (T0 / 4 - C_k / 2) / div from the CTA partials of one chunk: warp k sums the
+// partials of bond k (the last warp T0) in a fixed order.  One thread summing 304 of them one
+// after the other took 44 us.
+__global__ void __launch_bounds__(32 * (BC_CHUNK + 1))
+k_bc_final(const double *__restrict__ part, int nctas, int nbk, const int *__restrict__ Eptr, int nE, double sign,
+           const double *div, double *__restrict__ out) {
     __shared__ double t0s;
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int c = 0; c < nctas; ++c) t += part[(size_t)c * (nbk + 1) + nbk];
-        t0s = t;
-    }
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31, col = k == BC_CHUNK ? nbk : k;
+    double s = 0.0;
+    if (col <= nbk && (k == BC_CHUNK || k < nbk))
+        for (int c = lane; c < nctas; c += 32) s += part[(size_t)c * (nbk + 1) + col];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (k == BC_CHUNK && lane == 0) t0s = s;
+    const int E = Eptr ? blk_emax(Eptr, nE) : 0;
     __syncthreads();
-    const int k = threadIdx.x;
-    if (k >= nbk) return;
-    double ck = 0.0;
-    for (int c = 0; c < nctas; ++c) ck += part[(size_t)c * (nbk + 1) + k];
-    double v = 0.25 * t0s - 0.5 * ck;
-    if (Eptr) v = ldexp(v, *Eptr - 1022 - ef::FIX_BITS);
+    if (lane != 0 || k >= nbk) return;
+    double v = 0.25 * t0s - 0.5 * s;
+    if (Eptr) v = ldexp(v, E - 1022 - ef::FIX_BITS);
     out[k] = sign * (div ? v / *div : v);
 }
 
@@ -743,20 +743,15 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
         blocks[c] = std::min<int>(sm_count() * std::min(per, 4), 1 << P.H);
         if (!work || work_bytes < (size_t)blocks[c] * (nbk + 1) * sizeof(double)) return 1;
     }
-    int *Ed = nullptr;
-    if (dtype == HM_F64) {
-        Ed = (int *)b->d_scratch;
-        HM_CUDA(cudaMemsetAsync(Ed, 0, sizeof(int), st));
-        k_max_exp<<<grid_blocks(sv.dim, 256), 256, 0, st>>>((const unsigned long long *)x, sv.dim, Ed);
-        HM_CUDA(cudaGetLastError());
-    }
+    int *Ed = nullptr, nE = 0;
+    if (dtype == HM_F64) HM_TRY(launch_max_exp(b, x, sv.dim, &Ed, &nE, st));
     double *part = (double *)work;
     for (int c = 0; c < nch; ++c) {
         const int nbk = std::min(BC_CHUNK, bp.nb - c * BC_CHUNK);
         const size_t sm = blk_row_smem_bytes(plans[c], es, BLK_XPAD);
-        void *args[] = {(void *)&plans[c], (void *)&x, (void *)&g, (void *)&Ed, (void *)&part};
+        void *args[] = {(void *)&plans[c], (void *)&x, (void *)&g, (void *)&Ed, (void *)&nE, (void *)&part};
         HM_CUDA(cudaLaunchKernel(kerns[c], dim3(blocks[c]), dim3(BLK_NT), args, sm, st));
-        k_bc_final<<<1, 32, 0, st>>>(part, blocks[c], nbk, Ed, sign, div, out + c * BC_CHUNK);
+        k_bc_final<<<1, 32 * (BC_CHUNK + 1), 0, st>>>(part, blocks[c], nbk, Ed, nE, sign, div, out + c * BC_CHUNK);
         HM_CUDA(cudaGetLastError());
     }
     return HM_OK;
@@ -774,27 +769,96 @@ const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int 
     return jit_mv_kernel(P, dtype, &k) == 0 ? "k_blk_matvec_jit" : nullptr;
 }
 
+// The plan of y = H x for one bond list.  Planning takes 20 to 60 us of host time (groups, table
+// layout, the source text that names a run-time compiled kernel), more than the product itself
+// below N = 22, so a basis keeps its last BLK_MV_PLANS of them, found by the values of the bonds
+// (never by an address), the type and the environment knobs that enter.
+struct BlkMvPlan {
+    int nb, dtype, K, env;
+    unsigned char p[HM_BLK_MAXB], q[HM_BLK_MAXB];
+    double jm[HM_BLK_MAXB];
+    BlkParams P;
+    const void *kern;
+    size_t smem;
+    int blocks;
+};
+constexpr unsigned BLK_MV_PLANS = 8;
+
+// what of the environment enters a plan besides the split
+static int blk_env() {
+    const char *row = getenv("HM_JIT_ROW"), *jit = getenv("HM_JIT");
+    return (row && *row && strcmp(row, "table") != 0 ? 1 : 0) | (jit && jit[0] == '0' ? 2 : 0);
+}
+
+// 0 and the plan, or 1 when the block path does not apply
+static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, cudaStream_t st,
+                       std::shared_ptr<const BlkMvPlan> *out) {
+    if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB) return 1;
+    const int K = blk_K(b, false), env = blk_env(), nb = bp.nb;
+    {
+        std::lock_guard<std::mutex> lk(b->tab_mu);
+        for (const auto &m : b->mv_plans)
+            if (m->nb == nb && m->dtype == dtype && m->K == K && m->env == env && !memcmp(m->p, bp.p, nb) &&
+                !memcmp(m->q, bp.q, nb) && !memcmp(m->jm, bp.jm, nb * sizeof(double))) {
+                *out = m;
+                return 0;
+            }
+    }
+    auto m = std::make_shared<BlkMvPlan>();
+    BlkParams &P = m->P;
+    const int rc = blk_plan(b, bp, K, &P);
+    if (rc != 0) return rc;
+    const int es = dtype == HM_F64 ? 8 : 4;
+    m->smem = blk_row_smem_bytes(P, es, BLK_XPAD);
+    if (!P.rows_ok || m->smem > 200 * 1024) return 1;
+    // target tables: built on the first product of a layout, but for class plans neither inside a
+    // stream capture (no allocation there) nor without end on a basis that sees many bond lists; the
+    // generic rows then serve, with the same result (FP64: the same exact sums)
+    bool build = true;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    HM_CUDA(cudaStreamIsCapturing(st, &cs));
+    if (!P.perbond) {
+        std::lock_guard<std::mutex> lk(b->tab_mu);
+        build = cs == cudaStreamCaptureStatusNone && b->blk_ttabs.size() < 32;
+    }
+    const int trc = blk_target_table(b, &P, es, build);
+    if (trc < 0) return trc;
+    if (P.perbond) {
+        if (jit_mv_kernel(P, dtype, &m->kern) != 0) return 1;
+    } else if (dtype == HM_F64) {
+        m->kern = P.tt ? blk_mv_kernel<double, true>(P.nc) : blk_mv_kernel<double, false>(P.nc);
+    } else {
+        m->kern = P.tt ? blk_mv_kernel<float, true>(P.nc) : blk_mv_kernel<float, false>(P.nc);
+    }
+    HM_CUDA(raise_smem_limit(m->kern, m->smem));
+    int per = 0;
+    HM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, m->kern, BLK_NT, m->smem));
+    m->blocks = std::min<int>(sm_count() * std::max(per, 1), 1 << P.H);
+    m->nb = nb; m->dtype = dtype; m->K = K; m->env = env;
+    memcpy(m->p, bp.p, nb);
+    memcpy(m->q, bp.q, nb);
+    memcpy(m->jm, bp.jm, nb * sizeof(double));
+    if (P.perbond || P.tt || cs == cudaStreamCaptureStatusNone) {   // a capture's plan without its table is not kept
+        std::lock_guard<std::mutex> lk(b->tab_mu);
+        if (b->mv_plans.size() < BLK_MV_PLANS) b->mv_plans.push_back(m);
+        else b->mv_plans[b->mv_next++ % BLK_MV_PLANS] = m;
+    }
+    *out = m;
+    return 0;
+}
+
 // returns 1 when the block path does not apply (caller falls back to the row kernel)
 int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dtype, int nvec,
                cudaStream_t st) {
     if (nvec != 1) return 1;
-    BlkParams P;
-    int rc = blk_plan(b, bp, blk_K(b, false), &P);
+    std::shared_ptr<const BlkMvPlan> m;
+    const int rc = blk_mv_plan(b, bp, dtype, st, &m);
     if (rc != 0) return rc;
-    if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return 1;
-    if (P.perbond) return launch_blk_matvec_pb(b, P, x, y, dtype, st);
-    if (dtype == HM_F64) {
-        switch (P.nc) {
-            case 1: return launch_blk_matvec<double, 1>(b, P, (const double *)x, (double *)y, st);
-            case 2: return launch_blk_matvec<double, 2>(b, P, (const double *)x, (double *)y, st);
-            default: return launch_blk_matvec<double, 4>(b, P, (const double *)x, (double *)y, st);
-        }
-    }
-    switch (P.nc) {
-        case 1: return launch_blk_matvec<float, 1>(b, P, (const float *)x, (float *)y, st);
-        case 2: return launch_blk_matvec<float, 2>(b, P, (const float *)x, (float *)y, st);
-        default: return launch_blk_matvec<float, 4>(b, P, (const float *)x, (float *)y, st);
-    }
+    int *Ed = nullptr, nE = 0;
+    if (dtype == HM_F64) HM_TRY(launch_max_exp(b, x, m->P.dim, &Ed, &nE, st));
+    void *args[] = {(void *)&m->P, (void *)&x, (void *)&y, (void *)&Ed, (void *)&nE};
+    HM_CUDA(cudaLaunchKernel(m->kern, dim3(m->blocks), dim3(BLK_NT), args, m->smem, st));
+    return HM_OK;
 }
 
 }  // namespace hm

@@ -347,6 +347,89 @@ static __device__ __forceinline__ void sums(const BlkParams &P, const BlkMeta &B
     }
 }
 };
+
+// The rows of a class plan with per-class target tables (BlkParams::tt) at run-time counts: the
+// policy that gen_row_table (jit.cu) writes out per plan, compiled once.  An exchange among the low
+// sites is a table field and a shared-memory gather instead of the generic policy's rank-table
+// reads and spin test (about twenty instructions); y = H x needs no run-time compilation for it.
+// FP64 J1-J2 ring, M = 0, product with the exponent pass: N = 24 163 -> 150 us, N = 28 2337 -> 2118 us.
+template <int NC>
+struct RowTable {
+static constexpr int kPad = BLK_XPAD;
+static constexpr bool kRelUS = false;
+static constexpr bool kPerBond = false;
+static constexpr bool kBC = false;
+template <class Sv>
+static __device__ __forceinline__ void stage(const BlkParams &P, unsigned char *dyn) {
+    if (threadIdx.x == 0) *(Sv *)(dyn + (P.max_block + BLK_XPAD - 1) * sizeof(Sv)) = Sv(0);
+}
+template <class Sv>
+static __device__ __forceinline__ void block(const BlkParams &, uint32_t) {}
+template <class Sv, class G>
+static __device__ __forceinline__ void sums(const BlkParams &P, const BlkMeta &B, const unsigned char *Xsb,
+                                            const unsigned char *Xg, uint32_t l, uint32_t r, const G &gx, Sv xo,
+                                            Sv *acc, int *cnt) {
+    (void)xo;
+    const uint32_t g = B.lwo + r;
+    const int ntri = P.tt_ntri, nsgl = P.tt_nsgl, nw = ntri + (nsgl + 1) / 2;   // pairs of entries
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = Sv(0);
+    auto add = [&](int c, Sv v) {
+#pragma unroll
+        for (int k = 0; k < NC; ++k)
+            if (NC == 1 || c == k) acc[k] += v;
+    };
+    const uint4 *tt = P.tt + g;
+    uint4 q = nw > 0 ? ldg_v4(tt) : make_uint4(0u, 0u, 0u, 0u);
+    for (int w = 0; w < nw; w += 4) {
+        const uint32_t e4[4] = {q.x, q.y, q.z, q.w};
+        if (w + 4 < nw) q = ldg_v4(tt += P.tt_stride);             // the next chunk, one round ahead
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int i = w + k;
+            if (i >= nw) break;
+            const Sv x1 = HM_XS(e4[k] & 0xFFFFu), x2 = HM_XS(e4[k] >> 16);
+            if (i < ntri) {
+                const int ca = P.tt_tri_ca[i], cb = P.tt_tri_cb[i];
+                if (NC == 1 || ca == cb) {
+                    add(ca, x1 + x2);
+                } else {       // the second edge is of class ca when the spins of a and c are parallel
+                    const Sv xa = ((l >> P.tt_tri_a[i]) ^ (l >> P.tt_tri_c[i])) & 1u ? Sv(0) : x2;
+                    add(ca, x1 + xa);
+                    add(cb, x2 - xa);
+                }
+            } else {
+                const int s = 2 * (i - ntri);
+                add(P.tt_sgl_c[s], x1);
+                if (s + 1 < nsgl) add(P.tt_sgl_c[s + 1], x2);      // else a cross entry shares the pair
+            }
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        int m = 0;
+        Sv a = Sv(0);
+        switch (P.lgn[c]) { HM_RUN6(HM_LG) }
+        for (int t = 0; t < 2; ++t)
+            for (int s = 0; s < P.xn[c][t]; ++s) {
+                const int d = (2 * c + t) * HM_BLK_SX + s;
+                const XSlot x_ = B.xs[d];
+                if ((l ^ x_.wm) & x_.vm) {
+                    const int e = P.tt_xe[d];
+                    const uint32_t v_ = __ldg((const uint16_t *)P.tt + ((size_t)(e >> 3) * P.tt_stride + g) * 8 + (e & 7));
+                    HM_XADD(v_)
+                }
+            }
+        a += blk_high_sum<Sv>(B, c, Xg, r, gx);
+        if (P.par) {
+            const Sv f = blk_flip_sum<Sv>(B, c, Xg, r, gx);
+            a += P.par < 0 ? -f : f;
+        }
+        acc[c] += a;
+        cnt[c] = m + (B.he[c] - B.hs[c]) + (P.par ? B.x->fe[c] - B.x->fs[c] : 0);
+    }
+}
+};
 #undef HM_XS
 #undef HM_L0
 #undef HM_L1
@@ -577,14 +660,22 @@ __device__ __forceinline__ float blk_y_f32(const BlkParams &P, const float *acc,
     return y;
 }
 
+// largest exponent field of the vector from the partial maxima of k_max_exp (every warp for itself:
+// no barrier, no reset between calls)
+__device__ __forceinline__ int blk_emax(const int *__restrict__ part, int n) {
+    int m = 0;
+    for (int i = threadIdx.x & 31; i < n; i += 32) m = max(m, __ldg(part + i));
+    return __reduce_max_sync(0xffffffffu, m);
+}
+
 // ---------------------------------------------------------------------------------------
 // y = H x (matvec API)
 // ---------------------------------------------------------------------------------------
 template <class T, int NC, class Row>
 __device__ __forceinline__ void matvec_body(const BlkParams &P, const T *__restrict__ x, T *__restrict__ y,
-                                            const int *__restrict__ Eptr) {
+                                            const int *__restrict__ Eptr, int nE) {
     if constexpr (sizeof(T) == 8) {
-        const int E = Eptr ? *Eptr : 0;
+        const int E = blk_emax(Eptr, nE);
         const int u = E - 1022 - ef::FIX_BITS;
         unsigned long long *yb = (unsigned long long *)y;
         if constexpr (Row::kPerBond) {
@@ -832,13 +923,13 @@ __device__ __forceinline__ void bc_sweep(const BlkParams &P, const T *__restrict
 
 template <class T, class Row>
 __device__ __forceinline__ void bc_body(const BlkParams &P, const T *__restrict__ x, const T *__restrict__ g,
-                                        const int *__restrict__ Eptr, double *__restrict__ part) {
+                                        const int *__restrict__ Eptr, int nE, double *__restrict__ part) {
     using Sv = typename BcSv<T>::S;
     ef::df acc[Row::kNB];
 #pragma unroll
     for (int k = 0; k < Row::kNB; ++k) acc[k] = ef::df{0.0f, 0.0f};
     double t0 = 0.0;
-    if constexpr (sizeof(T) == 8) bc_sweep<T, Row, Sv>(P, x, g, GF64{Eptr ? *Eptr : 0}, acc, t0);
+    if constexpr (sizeof(T) == 8) bc_sweep<T, Row, Sv>(P, x, g, GF64{blk_emax(Eptr, nE)}, acc, t0);
     else bc_sweep<T, Row, Sv>(P, x, g, GF32{}, acc, t0);
     __shared__ double red[BLK_NT / 32];
     double *pc = part + (size_t)blockIdx.x * (Row::kNB + 1);

@@ -7,7 +7,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <map>
+#include <memory>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -79,12 +82,23 @@ struct S1Tab {                      // tables of the s = 1 block path (s1blk.cu)
 };
 }  // namespace hm
 
+namespace hm {
+struct BlkMvPlan;
+}
+constexpr int HM_ESLOTS = 16, HM_EPART = 512;
+
 struct hm_basis {
     hm::SectorView view;
     std::vector<uint64_t> D;        // host D(k, a), (N+1) x (S2*N+1)
     std::vector<uint64_t> cd;       // host CD, cd_len entries
     void *d_cd = nullptr;           // device copy (owned)
-    void *d_scratch = nullptr;      // 256 bytes of device scratch (owned), e.g. exponents
+    // device scratch (owned): HM_ESLOTS slots of HM_EPART ints for the exponent maxima of a product's
+    // vector; a call takes the next slot, so calls in flight on several streams do not share one
+    void *d_scratch = nullptr;
+    std::atomic<unsigned> eslot{0};
+    std::mutex tab_mu;              // guards blk_tabs, blk_ttabs and mv_plans (built on first use)
+    std::vector<std::shared_ptr<const hm::BlkMvPlan>> mv_plans;   // the last plans of y = H x (blk.cu)
+    unsigned mv_next = 0;
     std::map<int, hm::BlkTab> blk_tabs;   // per split position K (owned device memory)
     std::map<std::string, void *> blk_ttabs;   // per-class target tables by layout (owned device memory)
     std::map<int, hm::S1Tab> s1_tabs;     // s = 1 block path, per split K (owned device memory)

@@ -777,8 +777,8 @@ int jit_mv_kernel(const BlkParams &P, int dtype, const void **kern) {
     const char *T = dtype == HM_F64 ? "double" : "float";
     put(src,
         "extern \"C\" __global__ void __launch_bounds__(512, 3) k_blk_matvec_jit(hm::BlkParams P,\n"
-        "        const %s *__restrict__ x, %s *__restrict__ y, const int *__restrict__ Eptr) {\n"
-        "    hm::matvec_body<%s, 1, RowJit>(P, x, y, Eptr);\n}\n", T, T, T);
+        "        const %s *__restrict__ x, %s *__restrict__ y, const int *__restrict__ Eptr, int nE) {\n"
+        "    hm::matvec_body<%s, 1, RowJit>(P, x, y, Eptr, nE);\n}\n", T, T, T);
     return jit_get(src, "k_blk_matvec_jit", dev, BLK_XPAD, kern);
 }
 
@@ -793,9 +793,9 @@ int jit_bc_kernel(const BlkParams &P, int dtype, int nbk, const void **kern) {
     const char *T = dtype == HM_F64 ? "double" : "float";
     put(src,
         "extern \"C\" __global__ void __launch_bounds__(512, 2) k_blk_bc_jit(hm::BlkParams P,\n"
-        "        const %s *__restrict__ x, const %s *__restrict__ g, const int *__restrict__ Eptr,\n"
+        "        const %s *__restrict__ x, const %s *__restrict__ g, const int *__restrict__ Eptr, int nE,\n"
         "        double *__restrict__ part) {\n"
-        "    hm::bc_body<%s, RowJit>(P, x, g, Eptr, part);\n}\n", T, T, T);
+        "    hm::bc_body<%s, RowJit>(P, x, g, Eptr, nE, part);\n}\n", T, T, T);
     return jit_get(src, "k_blk_bc_jit", dev, BLK_XPAD, kern);
 }
 
