@@ -72,11 +72,12 @@ struct FtDev {
     double *alpha, *beta;           // [(s * FT_W + v) * steps + j]
     double *part;                   // [slot][v]: warp partials of the update phase (FtRange)
     double *parta;                  // [sector][warp][v]: warp partials of the product phase
-    double *partc;                  // [sector][cta][v]: the same summed over each CTA's warps
+    double *partc;                  // [sector][cta][v]: the sums over each CTA's warps, of either phase
     const uint32_t *ck_it0;         // [chunk]: the block holding the chunk's first row
     const uint32_t *ck_cs;          // [nsec + 1]: sector s owns chunks ck_cs[s] .. ck_cs[s + 1] - 1
     const FtRange *wr;              // [warp]
     const uint32_t *slo;            // [nsec + 1]: sector s owns slots slo[s] .. slo[s + 1] - 1
+    const uint2 *cta_rng;           // [nsec]: the CTAs [x, y) whose update rows include rows of sector s
     int *sec_active;                // [s]
     GridBar *bar;
     const uint32_t *items;          // (A << 16) | h, sorted by A
@@ -137,7 +138,7 @@ __device__ bool grid_sync(GridBar *gb, unsigned nctas, unsigned long long limit_
             while (*vgen == g) {
                 if (*vab) break;
                 if (globaltimer_ns() - t0 > limit_ns) { atomicExch(&gb->abort, 1); break; }
-                __nanosleep(200);
+                __nanosleep(32);
             }
         }
         __threadfence();
@@ -241,50 +242,22 @@ __device__ __forceinline__ void ft_warp_setup(const BlkParams &P, const BlkTabs 
     }
 }
 
-// Per (sector, vector) sums of the warp partials: the slots of sector s, slo[s] ..
-// slo[s + 1] - 1, in a fixed order (16 strided chunks, then the chunks in order);
-// f(s, v, sum) runs on warp 0 of the CTA that owns sector s.  All threads call it.
-template <class F>
-__device__ __forceinline__ void ft_sector_sums(const FtParams &Fp, double *red, F &&f) {
-    const FtDev &d = Fp.d;
-    constexpr int NCH = FT_NT / FT_W;
-    const int v = threadIdx.x % FT_W, c = threadIdx.x / FT_W;
-    for (int s = blockIdx.x; s < Fp.nsec; s += gridDim.x) {
-        const uint32_t s0 = d.slo[s], s1 = d.slo[s + 1];
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        uint32_t sl = s0 + c;
-        for (; sl + 3 * NCH < s1; sl += 4 * NCH) {
-            a0 += d.part[(size_t)sl * FT_W + v];
-            a1 += d.part[(size_t)(sl + NCH) * FT_W + v];
-            a2 += d.part[(size_t)(sl + 2 * NCH) * FT_W + v];
-            a3 += d.part[(size_t)(sl + 3 * NCH) * FT_W + v];
-        }
-        for (; sl < s1; sl += NCH) a0 += d.part[(size_t)sl * FT_W + v];
-        const double a = (a0 + a1) + (a2 + a3);
-        red[c * FT_W + v] = a;
-        __syncthreads();
-        if (c == 0) {
-            double t = 0.0;
-            for (int i = 0; i < NCH; ++i) t += red[i * FT_W + v];
-            f(s, v, t);
-        }
-        __syncthreads();
-    }
-}
-
-// Per (sector, vector) sums of the product-phase partials partc[s][b][v] over all CTAs b
+// Per (sector, vector) sums of the CTA partials partc[s][b][v] over the CTAs b in [lo(s), hi(s))
 // in a fixed order (16 strided chunks of four running sums, then the chunks in order);
-// f(s, v, sum) runs on warp 0 of the CTA that owns sector s.  All threads call it.
-template <class F>
-__device__ __forceinline__ void ft_sector_sums_a(const FtParams &Fp, double *red, F &&f) {
+// f(s, v, sum) runs on warp 0 of the CTA that owns sector s.  All threads call it.  The sums run over
+// CTAs, not warps: a binary64 add costs a warp 64 cycles, and the 1284 warp partials of the
+// largest sector of N = 20 took 10 us a step.
+template <class R, class F>
+__device__ __forceinline__ void ft_sector_sums(const FtParams &Fp, double *red, R &&range, F &&f) {
     const FtDev &d = Fp.d;
     constexpr int NCH = FT_NT / FT_W;
     const int v = threadIdx.x % FT_W, c = threadIdx.x / FT_W;
-    const unsigned nb = Fp.nctas;
     for (int s = blockIdx.x; s < Fp.nsec; s += gridDim.x) {
-        const double *ps = d.partc + (size_t)s * nb * FT_W;
+        const double *ps = d.partc + (size_t)s * Fp.nctas * FT_W;
+        const uint2 lh = range(s);
+        const unsigned nb = lh.y;
         double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        unsigned b = c;
+        unsigned b = lh.x + c;
         for (; b + 3 * NCH < nb; b += 4 * NCH) {
             a0 += ps[(size_t)b * FT_W + v];
             a1 += ps[(size_t)(b + NCH) * FT_W + v];
@@ -477,7 +450,7 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
         }
         if (!grid_sync(d.bar, F.nctas, LIMIT)) return;
         // ---------------- phase B: alpha ----------------
-        ft_sector_sums_a(F, red, [&](int s, int v, double a) {
+        ft_sector_sums(F, red, [&](int) { return make_uint2(0u, F.nctas); }, [&](int s, int v, double a) {
             const int t = s * FT_W + v;
             if (d.done[t]) return;
             d.alpha[(size_t)t * F.steps + j] = a;
@@ -523,9 +496,23 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                 if (a1 >= rg.g1) break;
             }
         }
+        // the CTA's slots of each sector it touches, in order (written by this CTA just now)
+        __syncthreads();
+        {
+            const uint32_t w0 = blockIdx.x * (FT_NT / 32);
+            const uint32_t b0 = d.wr[w0].slot0, b1 = w0 + FT_NT / 32 < nw ? d.wr[w0 + FT_NT / 32].slot0 : d.slo[F.nsec];
+            for (int t = threadIdx.x; t < F.nsec * FT_W; t += FT_NT) {
+                const int s = t / FT_W, v = t % FT_W;
+                const uint32_t s0 = max(b0, d.slo[s]), s1 = min(b1, d.slo[s + 1]);
+                if (s0 >= s1) continue;
+                double a = 0.0;
+                for (uint32_t sl = s0; sl < s1; ++sl) a += d.part[(size_t)sl * FT_W + v];
+                d.partc[((size_t)s * F.nctas + blockIdx.x) * FT_W + v] = a;
+            }
+        }
         if (!grid_sync(d.bar, F.nctas, LIMIT)) return;
         // ---------------- phase D: beta ----------------
-        ft_sector_sums(F, red, [&](int s, int v, double sum) {
+        ft_sector_sums(F, red, [&](int s) { return d.cta_rng[s]; }, [&](int s, int v, double sum) {
             const int t = s * FT_W + v;
             bool act = false;
             if (!d.done[t]) {
@@ -559,19 +546,38 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
 // Implicit symmetric QR with Wilkinson shifts (Golub and Van Loan, Sec. 8.3): each sweep
 // chases a bulge down the unreduced block with Givens rotations; the rotations are also
 // applied to z, the first row of the accumulated eigenvector matrix.
-// One thread per matrix: a sweep is one chain of dependent binary64 operations, so its
-// number is what counts.  A rotation takes its cosine and sine from one rsqrt (six binary64
-// instructions where hypot and two divisions took forty), and the values the next rotation
-// needs stay in registers.  T is scaled to norm 1, so squares
-// neither overflow nor lose anything that matters when they underflow.
+// One warp per matrix.  A sweep is one chain of rotations, and a warp's binary64 instruction
+// occupies its quarter of an SM for 64 cycles however many lanes take part, so what counts is the
+// number of binary64 instructions a rotation takes one after the other.  Its cosine and sine come
+// from one rsqrt (six of them; hypot and two divisions take forty), and the about thirty products
+// and sums are spread over four lanes, which do up to four of them in one instruction and hand the
+// results round by shuffles: fourteen in all.  The scan for a negligible off-diagonal looks at 32
+// rows at a time.  T is scaled to norm 1, so squares neither overflow nor lose anything that
+// matters when they underflow.  N = 20, 672 matrices of 80 rows: 25.7 ms with one thread to a
+// matrix in 6 CTAs and hypot, 12.7 ms with rsqrt and 4 matrices to a CTA, 9.5 ms here.
 __device__ void tri_ql_first(int m, double *dg, double *e, double *z) {
-    for (int i = 0; i < m; ++i) z[i] = i == 0 ? 1.0 : 0.0;
+    const int lane = threadIdx.x & 31, q = lane & 3;
+    const double eps = 2.220446049250313e-16;
+    auto from = [](double v, int src) { return __shfl_sync(0xffffffffu, v, src); };
+    for (int i = lane; i < m; i += 32) z[i] = i == 0 ? 1.0 : 0.0;
+    __syncwarp();
     int hi = m - 1, guard = 0;
     while (hi > 0 && guard < 60 * m) {
-        const double tol = 2.220446049250313e-16 * (fabs(dg[hi - 1]) + fabs(dg[hi]));
-        if (fabs(e[hi - 1]) <= tol) { e[hi - 1] = 0.0; --hi; continue; }
-        int lo = hi - 1;
-        while (lo > 0 && fabs(e[lo - 1]) > 2.220446049250313e-16 * (fabs(dg[lo - 1]) + fabs(dg[lo]))) --lo;
+        // start of the unreduced block that ends at hi: the last i < hi with a negligible e[i], plus one
+        int lo = 0;
+        for (int i0 = hi - 1; i0 >= 0; i0 -= 32) {
+            const int i = i0 - lane;
+            const bool small = i >= 0 && fabs(e[i]) <= eps * (fabs(dg[i]) + fabs(dg[i + 1]));
+            const unsigned bal = __ballot_sync(0xffffffffu, small);
+            if (bal) { lo = i0 - (__ffs(bal) - 1) + 1; break; }
+        }
+        if (lo == hi) {
+            __syncwarp();
+            if (lane == 0) e[hi - 1] = 0.0;
+            __syncwarp();
+            --hi;
+            continue;
+        }
         ++guard;
         // Wilkinson shift: eigenvalue of the trailing 2x2 block closer to dg[hi]
         const double dd = 0.5 * (dg[hi - 1] - dg[hi]);
@@ -581,58 +587,70 @@ __device__ void tri_ql_first(int m, double *dg, double *e, double *z) {
         double a = dg[lo], b = e[lo], zk = z[lo], x = a - mu, y = b;
         for (int kk = lo; kk < hi; ++kk) {
             const double cc = dg[kk + 1], zk1 = z[kk + 1], en = kk + 1 < hi ? e[kk + 1] : 0.0;
-            const double r2 = fma(x, x, y * y);
-            const double ri = rsqrt(r2);
-            const double c = r2 > 0.0 ? x * ri : 1.0, s = r2 > 0.0 ? y * ri : 0.0;
-            if (kk > lo) e[kk - 1] = r2 > 0.0 ? r2 * ri : 0.0;
-            const double c2 = c * c, s2 = s * s, cs = c * s, csb = 2.0 * cs * b;
-            dg[kk] = c2 * a + csb + s2 * cc;
-            x = cs * (cc - a) + (c2 - s2) * b;
-            a = s2 * a - csb + c2 * cc;
-            z[kk] = c * zk + s * zk1;
-            zk = c * zk1 - s * zk;
-            y = s * en;
-            b = c * en;
+            const double u = q & 1 ? y : x, p = u * u;
+            const double r2 = p + __shfl_xor_sync(0xffffffffu, p, 1);
+            const bool nz = r2 > 0.0;
+            const double ri = rsqrt(r2), v = nz ? u * ri : (q & 1 ? 0.0 : 1.0), o = __shfl_xor_sync(0xffffffffu, v, 1);
+            const double c = q & 1 ? o : v, s = q & 1 ? v : o;
+            const double t5 = fma(q == 0 ? c : q == 1 ? s : q == 2 ? c : 1.0, q == 0 ? c : q == 1 ? s : q == 2 ? s : cc,
+                                  q == 3 ? -a : 0.0);
+            const double c2 = from(t5, 0), s2 = from(t5, 1), cs = from(t5, 2), d = from(t5, 3);
+            const double t6 = fma(q == 0 ? cs : q == 1 ? 1.0 : c, q == 0 ? b : q == 1 ? c2 : q == 2 ? zk : zk1,
+                                  q == 1 ? -s2 : 0.0);
+            const double csb = from(t6, 0), cd = from(t6, 1);                // c s b, c^2 - s^2
+            // lane 0: c^2 a + c s b; 1: (c^2 - s^2) b; 2: new z[kk]; 3: the z that moves on
+            const double t7 = fma(q == 0 ? c2 : q == 1 ? cd : q == 2 ? s : -s, q == 0 ? a : q == 1 ? b : q == 2 ? zk1 : zk,
+                                  q == 0 ? csb : q == 1 ? 0.0 : t6);
+            // 0: + s^2 c; 1: x of the next rotation; 2: s^2 a - c s b; 3: y of the next
+            const double t8 = fma(q == 1 ? cs : q == 3 ? s : s2, q == 0 ? cc : q == 1 ? d : q == 2 ? a : en,
+                                  q == 2 ? -csb : q == 3 ? 0.0 : t7);
+            // 0: new dg[kk]; 2: - c s b once more; 3: the next off-diagonal
+            const double t9 = fma(q == 3 ? c : 1.0, q == 3 ? en : q == 2 ? -csb : csb, q == 3 ? 0.0 : t8);
+            const double ta = fma(q == 2 ? c2 : r2, q == 2 ? cc : ri, q == 2 ? t9 : 0.0);   // 2: the dg that moves on; 0: r
+            if (lane == 0) {
+                dg[kk] = t9;
+                if (kk > lo) e[kk - 1] = nz ? ta : 0.0;
+            }
+            if (lane == 2) z[kk] = t7;
+            zk = from(t7, 3);
+            x = from(t8, 1);
+            y = from(t8, 3);
+            b = from(t9, 3);
+            a = from(ta, 2);
         }
-        dg[hi] = a;
-        e[hi - 1] = x;
-        z[hi] = zk;
+        __syncwarp();
+        if (lane == 0) {
+            dg[hi] = a;
+            e[hi - 1] = x;
+            z[hi] = zk;
+        }
+        __syncwarp();
     }
 }
 
-// theta and tau of every (sector, vector): FT_EIG matrices to a CTA.  Few to a CTA spreads
-// the chains over the SMs (a warp's binary64 instruction occupies its quarter of an SM for 64
-// cycles however many lanes take part) and keeps lanes with unequal deflation patterns apart:
-// 25.7 ms with 128 to a CTA and the hypot form against 12.7 ms at N = 20, 672 matrices of 80
-// rows.
-constexpr int FT_EIG = 4;
-__host__ __device__ __forceinline__ size_t ft_eig_smem(int steps) {
-    const size_t b = (size_t)FT_EIG * 3 * steps * 8;
-    return b <= 40 * 1024 ? b : 0;                     // more rows: the scratch in device memory
-}
-
-__global__ void __launch_bounds__(FT_EIG) k_ft_eig(FtParams F, double *scratch) {
+// theta and tau of (sector, vector) blockIdx.x; dynamic shared memory: 3 x steps doubles (47 KB at
+// the most steps a run takes)
+__global__ void __launch_bounds__(32) k_ft_eig(FtParams F) {
     extern __shared__ __align__(16) double ft_eig_sh[];
     const FtDev &d = F.d;
-    const int t = blockIdx.x * FT_EIG + threadIdx.x;
-    if (t >= F.nsec * FT_W) return;
-    const int v = t % FT_W;
+    const int t = blockIdx.x, v = t % FT_W, lane = threadIdx.x;
     if ((F.exact_mask >> (t / FT_W)) & 1ull) return;   // filled by k_ft_exact
     const int m = (v < F.R) ? d.nsteps[t] : 0;
-    d.mlen[t] = m;
+    if (lane == 0) d.mlen[t] = m;
     if (m == 0) return;
-    double *dg = ft_eig_smem(F.steps) ? ft_eig_sh + (size_t)threadIdx.x * 3 * F.steps
-                                      : scratch + (size_t)t * 3 * F.steps;
-    double *e = dg + F.steps, *z = e + F.steps;
+    double *dg = ft_eig_sh, *e = dg + F.steps, *z = e + F.steps;
     const double *al = d.alpha + (size_t)t * F.steps, *be = d.beta + (size_t)t * F.steps;
     double nrm = 0.0;
-    for (int i = 0; i < m; ++i) nrm = fmax(nrm, fmax(fabs(al[i]), i + 1 < m ? fabs(be[i]) : 0.0));
+    for (int i = lane; i < m; i += 32) nrm = fmax(nrm, fmax(fabs(al[i]), i + 1 < m ? fabs(be[i]) : 0.0));
+    for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
     const int ex = nrm > 0.0 && nrm < 1e308 ? min(max(ilogb(nrm), -1000), 1000) : 0;
-    for (int i = 0; i < m; ++i) dg[i] = ldexp(al[i], -ex);
-    for (int i = 0; i + 1 < m; ++i) e[i] = ldexp(be[i], -ex);
-    if (m > 1) e[m - 1] = 0.0;
+    for (int i = lane; i < m; i += 32) {
+        dg[i] = ldexp(al[i], -ex);
+        e[i] = i + 1 < m ? ldexp(be[i], -ex) : 0.0;
+    }
+    __syncwarp();
     tri_ql_first(m, dg, e, z);
-    for (int i = 0; i < m; ++i) {
+    for (int i = lane; i < m; i += 32) {
         d.theta[(size_t)t * F.steps + i] = ldexp(dg[i], ex);
         d.tau[(size_t)t * F.steps + i] = z[i] * z[i];
     }
@@ -815,8 +833,8 @@ __global__ void __launch_bounds__(256) k_ft_thermo_fin(FtParams F, const double 
 
 // ---- host --------------------------------------------------------------------------------
 struct FtLayout {
-    size_t q0, q1, st, ab, part, wr, slo, parta, partc, ckit, ckcs, sec, bar, items, rowoff, secdim, theta, tau, mlen, therm, tsum, temps,
-        eigs, xcd, xmat, total;
+    size_t q0, q1, st, ab, part, wr, slo, crng, parta, partc, ckit, ckcs, sec, bar, items, rowoff, secdim, theta, tau, mlen, therm, tsum, temps,
+        xcd, xmat, total;
 };
 
 static int ft_choose_K(int N) {
@@ -847,6 +865,7 @@ static FtLayout ft_layout(int N, int nsec, int R, int steps, int nitems, int nct
     L.part = o; o += a(nslots * FT_W * 8);
     L.wr = o; o += a((size_t)nctas * (FT_NT / 32) * sizeof(FtRange));
     L.slo = o; o += a((size_t)(nsec + 1) * 4);
+    L.crng = o; o += a((size_t)nsec * sizeof(uint2));
     L.parta = o; o += a((size_t)nsec * nctas * (FT_NT / 32) * FT_W * 8);
     L.partc = o; o += a((size_t)nsec * nctas * FT_W * 8);
     L.ckit = o; o += a((nchunks > 0 ? nchunks : 1) * 4);
@@ -862,7 +881,6 @@ static FtLayout ft_layout(int N, int nsec, int R, int steps, int nitems, int nct
     L.therm = o; o += a((size_t)(2 * n_t + 1) * 8);
     L.tsum = o; o += a((size_t)nsec * (2 * (size_t)n_t + 1) * 8);
     L.temps = o; o += a((size_t)(n_t > 0 ? n_t : 1) * 8);
-    L.eigs = o; o += a(nst * 3 * (size_t)steps * 8);
     L.xcd = o; o += a((xcd_words > 0 ? xcd_words : 1) * 4);
     L.xmat = o; o += a((xmat_doubles > 0 ? xmat_doubles : 1) * 8);
     L.total = o;
@@ -889,7 +907,7 @@ static size_t ft_smem(const BlkParams &P, int nsec) {
 // The warps' row ranges (equal shares of all 2^N rows) and their partial-sum slots.
 // items: the blocks (A << 16 | h) in row order; C(K, k) rows each.
 static void ft_ranges(int n_sites, int K, const hm_basis &full, const std::vector<uint32_t> &items, int W,
-                      uint32_t ck_rows, std::vector<FtRange> *wr, std::vector<uint32_t> *slo,
+                      uint32_t ck_rows, std::vector<FtRange> *wr, std::vector<uint32_t> *slo, std::vector<uint2> *crng,
                       std::vector<uint32_t> *ck_it0, std::vector<uint32_t> *ck_cs) {
     const int N = n_sites, nsec = N + 1, Wd = N + 1;
     std::vector<uint64_t> r0(items.size() + 1, 0);
@@ -919,6 +937,21 @@ static void ft_ranges(int n_sites, int K, const hm_basis &full, const std::vecto
         while (i < slot_sec.size() && slot_sec[i] < s) ++i;
         (*slo)[s] = (uint32_t)i;
     }
+    // the CTAs that own slots of each sector (their first slots increase)
+    crng->assign(nsec, make_uint2(0u, 0u));
+    const int wpc = FT_NT / 32, nct = W / wpc;
+    for (int s2 = 0; s2 < nsec; ++s2) {
+        uint2 &r = (*crng)[s2];
+        bool any = false;
+        for (int c = 0; c < nct; ++c) {
+            const uint32_t b0 = (*wr)[(size_t)c * wpc].slot0;
+            const uint32_t b1 = c + 1 < nct ? (*wr)[(size_t)(c + 1) * wpc].slot0 : (*slo)[nsec];
+            if (std::max(b0, (*slo)[s2]) >= std::min(b1, (*slo)[s2 + 1])) continue;
+            if (!any) r.x = (uint32_t)c;
+            r.y = (uint32_t)c + 1;
+            any = true;
+        }
+    }
     // product-phase chunks: each sector cut into runs of ck_rows rows
     ck_it0->clear();
     ck_cs->assign(nsec + 1, 0);
@@ -930,10 +963,12 @@ static void ft_ranges(int n_sites, int K, const hm_basis &full, const std::vecto
     (*ck_cs)[nsec] = (uint32_t)ck_it0->size();
 }
 
-// rows per product-phase chunk: HM_FT_CHUNK (16..1024), default 64
-static uint32_t ft_chunk_rows() {
+// rows per product-phase chunk: HM_FT_CHUNK (16..1024), default 64, and fewer below N = 22, where
+// chunks of 64 rows are too few for 7296 warps to share evenly (whole runs of 40 steps, 16 / 32 /
+// 64 rows: N = 16 9.3 / 10.4 / 13.5 ms, N = 20 29.5 / 31.1 / 32.6, N = 22 111 / 103 / 101)
+static uint32_t ft_chunk_rows(int n_sites) {
     const char *e = getenv("HM_FT_CHUNK");
-    const int v = e ? atoi(e) : 64;
+    const int v = e ? atoi(e) : n_sites <= 20 ? 16 : n_sites == 21 ? 32 : 64;
     return (uint32_t)(v < 16 ? 16 : v > 1024 ? 1024 : v);
 }
 
@@ -960,6 +995,7 @@ struct FtSetup {
     std::vector<uint32_t> xcd;       // CD tables of the exactly diagonalised sectors
     std::vector<FtRange> wr;         // per warp
     std::vector<uint32_t> slo;       // per sector, + 1
+    std::vector<uint2> crng;         // per sector
     std::vector<uint32_t> ck_it0;    // per product-phase chunk
     std::vector<uint32_t> ck_cs;     // per sector, + 1
 };
@@ -968,7 +1004,7 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
                       const double *J, int R, int steps, int n_t, FtSetup *S, std::vector<uint32_t> *items) {
     if (two_s != 1) return fail(HM_EINVAL, "ftlm_run supports s = 1/2 (two_s = 1)");
     if (R < 1 || R > FT_W) return fail(HM_EINVAL, "R must be in 1..%d", FT_W);
-    if (steps < 1 || steps > 2000) return fail(HM_EINVAL, "steps must be in 1..2000");
+    if (steps < 1 || steps > 2000) return fail(HM_EINVAL, "steps must be in 1..2000");   // k_ft_eig: 3 x steps doubles
     if (n_t < 0 || n_t > 4096) return fail(HM_EINVAL, "n_t must be in 0..4096");
     const int K = ft_choose_K(n_sites);
     if (K < 0 || n_sites > 32) return fail(HM_EINVAL, "ftlm_run needs 10 <= n_sites <= 32");
@@ -1029,10 +1065,13 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
         per_sm = std::min(per_sm, p);
     }
     if (per_sm < 1) return fail(HM_EINVAL, "ftlm_run: kernel does not fit on an SM");
-    S->nctas = sm_count() * per_sm;   // cooperative: all resident
+    S->F.ck_rows = ft_chunk_rows(n_sites);
+    // cooperative: all resident.  No more CTAs than their warps have chunks (N <= 16): the grid
+    // barriers and the sums over the CTAs are most of a step there
+    const uint64_t nck = ((1ull << n_sites) + S->F.ck_rows - 1) / S->F.ck_rows + (uint64_t)nsec;
+    S->nctas = (int)std::min<uint64_t>((uint64_t)sm_count() * per_sm, (nck + FT_NT / 32 - 1) / (FT_NT / 32));
     S->F.nctas = (unsigned)S->nctas;
-    S->F.ck_rows = ft_chunk_rows();
-    ft_ranges(n_sites, K, S->full, *items, S->nctas * (FT_NT / 32), S->F.ck_rows, &S->wr, &S->slo, &S->ck_it0,
+    ft_ranges(n_sites, K, S->full, *items, S->nctas * (FT_NT / 32), S->F.ck_rows, &S->wr, &S->slo, &S->crng, &S->ck_it0,
               &S->ck_cs);
     S->F.nchunks = (uint32_t)S->ck_it0.size();
     S->L = ft_layout(n_sites, nsec, R, steps, S->F.nitems, S->nctas, n_t, S->xcd.size(), (size_t)xmat,
@@ -1055,6 +1094,7 @@ static void ft_bind(FtSetup *S, unsigned char *w) {
     d.part = (double *)(w + L.part);
     d.wr = (const FtRange *)(w + L.wr);
     d.slo = (const uint32_t *)(w + L.slo);
+    d.cta_rng = (const uint2 *)(w + L.crng);
     d.parta = (double *)(w + L.parta);
     d.partc = (double *)(w + L.partc);
     d.ck_it0 = (const uint32_t *)(w + L.ckit);
@@ -1142,6 +1182,7 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
     HM_CUDA(cudaMemcpyAsync(w + S.L.rowoff, rowoff.data(), rowoff.size() * 8, cudaMemcpyHostToDevice, st));
     HM_CUDA(cudaMemcpyAsync(w + S.L.secdim, dims.data(), dims.size() * 4, cudaMemcpyHostToDevice, st));
     HM_CUDA(cudaMemcpyAsync(w + S.L.wr, S.wr.data(), S.wr.size() * sizeof(FtRange), cudaMemcpyHostToDevice, st));
+    HM_CUDA(cudaMemcpyAsync(w + S.L.crng, S.crng.data(), S.crng.size() * sizeof(uint2), cudaMemcpyHostToDevice, st));
     HM_CUDA(cudaMemcpyAsync(w + S.L.slo, S.slo.data(), S.slo.size() * 4, cudaMemcpyHostToDevice, st));
     if (!S.ck_it0.empty())
         HM_CUDA(cudaMemcpyAsync(w + S.L.ckit, S.ck_it0.data(), S.ck_it0.size() * 4, cudaMemcpyHostToDevice, st));
@@ -1184,12 +1225,15 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
         }
     }
     // the run: init, persistent steps, eigen-decompositions, sums -- one captured graph
-    cudaStream_t cap;
-    HM_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
+    cudaStream_t cap = nullptr, br = nullptr;
+    cudaEvent_t ev = nullptr;
     cudaGraph_t g = nullptr;
     cudaGraphExec_t ge = nullptr;
     int rc = HM_OK;
-    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&br, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) rc = cuda_fail(e, "ftlm capture");
     if (rc == HM_OK) {
         k_ft_init<<<sm_count() * 4, 256, 0, cap>>>(S.F);
@@ -1197,12 +1241,18 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
         if (rc == HM_OK) rc = ft_launch_persistent(&S, use_vt, cap);
         if (rc == HM_OK) {
             const int nst = nsec * FT_W;
-            k_ft_eig<<<nst / FT_EIG, FT_EIG, ft_eig_smem(S.F.steps), cap>>>(S.F, (double *)(w + S.L.eigs));
+            // the exactly diagonalised sectors on a branch beside the eigen-decompositions
+            const bool fork = S.F.nexact > 0;
+            if (fork && ((e = cudaEventRecord(ev, cap)) != cudaSuccess || (e = cudaStreamWaitEvent(br, ev, 0)) != cudaSuccess))
+                rc = cuda_fail(e, "ftlm fork");
+            k_ft_eig<<<nst, 32, (size_t)3 * S.F.steps * 8, cap>>>(S.F);
             if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ft_eig");
-            if (rc == HM_OK && S.F.nexact > 0) {
-                k_ft_exact<<<S.F.nexact, 256, 0, cap>>>(S.F, S.bp, (const uint32_t *)(w + S.L.xcd),
-                                                        (double *)(w + S.L.xmat));
+            if (rc == HM_OK && fork) {
+                k_ft_exact<<<S.F.nexact, 256, 0, br>>>(S.F, S.bp, (const uint32_t *)(w + S.L.xcd),
+                                                       (double *)(w + S.L.xmat));
                 if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ft_exact");
+                else if ((e = cudaEventRecord(ev, br)) != cudaSuccess || (e = cudaStreamWaitEvent(cap, ev, 0)) != cudaSuccess)
+                    rc = cuda_fail(e, "ftlm join");
             }
         }
         cudaError_t e2 = cudaStreamEndCapture(cap, &g);
@@ -1212,7 +1262,9 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
     if (rc == HM_OK && (e = cudaGraphLaunch(ge, st)) != cudaSuccess) rc = cuda_fail(e, "ftlm graph launch");
     if (ge) cudaGraphExecDestroy(ge);
     if (g) cudaGraphDestroy(g);
-    cudaStreamDestroy(cap);
+    if (ev) cudaEventDestroy(ev);
+    if (br) cudaStreamDestroy(br);
+    if (cap) cudaStreamDestroy(cap);
     HM_TRY(rc);
     if (n_t > 0) {
         double *mins = (double *)(w + S.L.tsum), *zs = mins + nsec, *es = zs + (size_t)nsec * n_t;

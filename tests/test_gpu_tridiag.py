@@ -37,7 +37,7 @@ def test_ritz_values_vs_lapack(hm, m):
 
 
 def test_ftlm_long_krylov_spaces(hm):
-    """Past 426 steps the eigen-decomposition works in device memory instead of shared memory.  The
+    """Many rows of T, most of them past convergence, so that the decomposition splits and deflates.  The
     quadrature over 32 vectors has converged long before, so Z and E agree with a shorter run up to the
     FP32 vectors' rounding, 430 steps of 2^-24."""
     inst = W.small_ring(12, -1.0, -0.3)
