@@ -388,8 +388,9 @@ static __device__ __forceinline__ void sums(const BlkParams &P, const BlkMeta &B
         for (int k = 0; k < 4; ++k) {
             const int i = w + k;
             if (i >= nw) break;
-            const Sv x1 = HM_XS(e4[k] & 0xFFFFu), x2 = HM_XS(e4[k] >> 16);
+            const Sv x1 = HM_XS(e4[k] & 0xFFFFu);
             if (i < ntri) {
+                const Sv x2 = HM_XS(e4[k] >> 16);
                 const int ca = P.tt_tri_ca[i], cb = P.tt_tri_cb[i];
                 if (NC == 1 || ca == cb) {
                     add(ca, x1 + x2);
@@ -401,7 +402,8 @@ static __device__ __forceinline__ void sums(const BlkParams &P, const BlkMeta &B
             } else {
                 const int s = 2 * (i - ntri);
                 add(P.tt_sgl_c[s], x1);
-                if (s + 1 < nsgl) add(P.tt_sgl_c[s + 1], x2);      // else a cross entry shares the pair
+                // else a cross entry shares the pair: a rank of another class, not a row of this block
+                if (s + 1 < nsgl) add(P.tt_sgl_c[s + 1], HM_XS(e4[k] >> 16));
             }
         }
     }
