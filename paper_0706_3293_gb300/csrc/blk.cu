@@ -505,13 +505,13 @@ int blk_target_table(hm_basis *b, BlkParams *P, int esize, bool build) {
     // per-bond plans: every slot keeps its own coefficient, so no triangles; an exchange that
     // is not allowed points at the row itself, whose difference x_i - x_t is then zero
     const bool self = P->perbond != 0;
-    struct Slot { int p, q, c; bool used; };
+    struct Slot { int p, q, c; bool used; int bond; };
     std::vector<Slot> low;
     for (int c = 0; c < P->nc; ++c)
         for (int ty = 0; ty < 3; ++ty)
             for (int k = 0; k < P->ln[c][ty]; ++k) {
                 const int p = __builtin_ctz(P->lvm[c][ty][k]);
-                low.push_back({p, p + P->ld[c][ty][k], c, false});
+                low.push_back({p, p + P->ld[c][ty][k], c, false, P->perbond ? P->pb_lb[ty][k] : 0});
             }
     auto find = [&](int x, int y) {
         for (size_t i = 0; i < low.size(); ++i)
@@ -606,7 +606,10 @@ int blk_target_table(hm_basis *b, BlkParams *P, int esize, bool build) {
         P->tt_tri_a[t] = (uint8_t)low[tris[t].e[2]].p;
         P->tt_tri_c[t] = (uint8_t)low[tris[t].e[2]].q;
     }
-    for (int i = 0; i < nsgl; ++i) P->tt_sgl_c[i] = (uint8_t)low[sgl[i]].c;
+    for (int i = 0; i < nsgl; ++i) {
+        P->tt_sgl_c[i] = (uint8_t)low[sgl[i]].c;
+        P->tt_pb[i] = (uint8_t)low[sgl[i]].bond;
+    }
     return 0;
 }
 

@@ -96,6 +96,7 @@ struct BlkParams {
     uint32_t tt_stride;
     int tt_n, tt_ncross, tt_cross_p[8];
     uint8_t tt_xe[HM_BLK_MAXC * 2 * HM_BLK_SX];   // table entry of each cross slot (index as BlkMeta::xs)
+    uint8_t tt_pb[48];                            // per-bond plan: bond of each single slot
     // the low slots as edge-disjoint triangles of bonds (a, b), (b, c), (a, c), whose spin
     // pairs hold exactly zero or two unequal pairs, so two gathers (two entries) serve three
     // slots, then single slots.  The first gathered edge of a triangle is always class

@@ -728,6 +728,48 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// v as binary64, rounded to nearest even, by integer instructions alone
+__device__ __forceinline__ double i128_round(__int128 v) {
+    const unsigned __int128 a = v < 0 ? -(unsigned __int128)v : (unsigned __int128)v;
+    const unsigned long long hi = (unsigned long long)(a >> 64), lo = (unsigned long long)a;
+    const int sh = hi ? 65 - ef::clz64(hi) : (int)(lo >> 63);    // a >> sh has at most 63 bits
+    unsigned long long m = (unsigned long long)(a >> sh);
+    if (sh) m |= (a & (((unsigned __int128)1 << sh) - 1)) != 0 ? 1ull : 0ull;
+    const unsigned long long b = ef::bits_from_int((int64_t)m, sh);
+    return ef::u2d(b | (v < 0 ? 0x8000000000000000ull : 0ull));
+}
+
+// One warp's part of a block's q.Hq from its threads' d1 (integer ratios: exact over the warp, rounded
+// once, no binary64 instruction; converting and adding in every thread took a warp twelve of them, at
+// 64 cycles each) or d1f (double-float); valid in lane 0.  blk_dot_scaled: a block's sum over its warps
+// (blk_pairwise) in true units.  They serve the whole-run kernel (lz_small.cu) too, so that it gives
+// the same bits.
+__device__ __forceinline__ double blk_dot_warp(bool exact, __int128 d1, ef::df d1f) {
+    if (exact) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long lo = __shfl_down_sync(0xffffffffu, (unsigned long long)d1, o);
+            const long long hi = __shfl_down_sync(0xffffffffu, (long long)(d1 >> 64), o);
+            d1 += ((__int128)hi << 64) | lo;         // at most 2^115 a row, 2^9 rows
+        }
+        return i128_round(d1);
+    }
+    return warp_sum((double)d1f.hi + (double)d1f.lo);
+}
+__device__ __forceinline__ double blk_dot_scaled(const BlkParams &P, bool exact, int E, double sum) {
+    return exact ? ldexp(sum * P.g0, 2 * (E - 1022 - ef::FIX_BITS)) : ldexp(sum, 2 * (E - 1023));
+}
+template <class V>
+__device__ __forceinline__ double blk_pairwise(V &&v) {  // by one thread: the order of a shuffle tree over the warps
+    double t[BLK_NT / 64];
+#pragma unroll
+    for (int w = 0; w < BLK_NT / 64; ++w) t[w] = v(w) + v(w + BLK_NT / 64);
+#pragma unroll
+    for (int o = BLK_NT / 128; o > 0; o >>= 1)
+#pragma unroll
+        for (int w = 0; w < o; ++w) t[w] += t[w + o];
+    return t[0];
+}
+
 // part[h] = (q . H q) over the rows of block h, in true units; entries of blocks that do
 // not exist stay as they are.
 // SPLIT = 1 / 2: the two passes of the split product (integer-ratio classes with a power-of-
@@ -770,15 +812,12 @@ __device__ __forceinline__ void lz64_body(const BlkParams &P, const long long *_
                     d1 += (__int128)xo * s;
                 },
                 [&](int it) {
-                    const double q_y = ldexp(i128_to_double(d1) * P.g0, 2 * u);
+                    const double a = blk_dot_warp(true, d1, ef::df{0.0f, 0.0f});
                     d1 = 0;
-                    const double a = warp_sum(q_y);
                     if ((threadIdx.x & 31) == 0) s_wpart[it & 1][threadIdx.x >> 5][0] = a;
                 },
                 [&](uint32_t h, int it) {
-                    double a = 0.0;
-                    for (int w = 0; w < BLK_NT / 32; ++w) a += s_wpart[it & 1][w][0];
-                    part[h] = a;
+                    part[h] = blk_dot_scaled(P, true, E, blk_pairwise([&](int w) { return s_wpart[it & 1][w][0]; }));
                 });
         }
         return;
@@ -825,19 +864,14 @@ __device__ __forceinline__ void lz64_body(const BlkParams &P, const long long *_
         __stcs(Y + off + r, yb);
         d1f = ef::df_add(d1f, ef::df_mul(ef::df_from_fix(xo, E, 0, E - 1023), ef::df_from_bits(yb, E - 1023)));
     };
+    constexpr bool exact = IR && !Row::kPerBond;
     auto endf = [&](int it) {
-            // true units: q.y = g0 2^(2u) sum X Tsum (integer ratios) or the double-float
-            // sum scaled back by 2^(2(E-1023))
-            const double q_y = IR && !Row::kPerBond ? ldexp(i128_to_double(d1) * P.g0, 2 * u)
-                                                    : ldexp((double)d1f.hi + (double)d1f.lo, 2 * (E - 1023));
+            const double a = blk_dot_warp(exact, d1, d1f);
             d1 = 0; d1f = ef::df{0.0f, 0.0f};
-            const double a = warp_sum(q_y);
             if ((threadIdx.x & 31) == 0) s_wpart[it & 1][threadIdx.x >> 5][0] = a;
         };
     auto flushf = [&](uint32_t h, int it) {
-            double a = 0.0;
-            for (int w = 0; w < BLK_NT / 32; ++w) a += s_wpart[it & 1][w][0];
-            part[h] = a;
+            part[h] = blk_dot_scaled(P, exact, E, blk_pairwise([&](int w) { return s_wpart[it & 1][w][0]; }));
         };
     if constexpr (Row::kPerBond)
         blk_sweep<int64_t, NC, true, Row>(P, (const unsigned char *)Xc, GFix{}, S->sched, [](uint32_t) { return 0; },

@@ -52,4 +52,12 @@ __device__ __forceinline__ double block_sum(double v, double *sh /* >= NT/32 */)
     return t;  // valid in thread 0
 }
 
+// sum of n doubles written by other CTAs, in a fixed order, by one warp; the same in every lane
+__device__ __forceinline__ double warp_sum_of(const double *part, int n) {
+    double s = 0.0;
+    for (int k = threadIdx.x & 31; k < n; k += 32) s += __ldcg(part + k);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+}
+
 }  // namespace hm

@@ -9,6 +9,7 @@
 #include "blk.cuh"
 #include "ef64.cuh"
 #include "hm_row.cuh"
+#include "lz_small.cuh"
 #include "s1blk.cuh"
 #include "tridiag.cuh"
 
@@ -49,6 +50,7 @@ struct LzLayout {
     int hpart_H;
     size_t s1part;          // s = 1 block path: one partial sum per block, s1n of them
     size_t mv;              // momentum basis: y = H q from the momentum product
+    size_t small;           // exponents and barrier of a whole run in one kernel (lz_small.cu)
     uint64_t s1n;
     bool shadow;
 };
@@ -63,7 +65,7 @@ static LzLayout lz_layout(const hm_basis *b, int dtype, int max_steps, bool grad
     size_t o = 0;
     L.buf[0] = o; o += al256(dim * es);
     L.buf[1] = o; o += al256(dim * es);
-    const size_t npart = std::max<size_t>((size_t)nblk, (size_t)sm_count() * 8);
+    const size_t npart = std::max<size_t>({(size_t)nblk, (size_t)sm_count() * 8, (size_t)1 << LZS_MAX_H});
     L.part = o; o += al256(npart * 2 * sizeof(double));
     // the block paths of FP64 runs (s = 1/2, s = 1) need y and two fixed-point copies; a
     // momentum basis takes neither block path but needs y = H q
@@ -83,6 +85,7 @@ static LzLayout lz_layout(const hm_basis *b, int dtype, int max_steps, bool grad
         const int H = b->view.N - blk_K(b, dtype == HM_F32);
         L.hpart_H = H;
         L.hpart = o; o += al256(((size_t)2 << H) * sizeof(double));
+        if (L.shadow && H <= LZS_MAX_H) { L.small = o; o += al256(lz_small_bytes(H)); }
     }
     // per-block partials of the s = 1 block path
     if ((L.s1n = s1n) > 0) { L.s1part = o; o += al256(L.s1n * sizeof(double)); }
@@ -119,6 +122,9 @@ struct hm_lanczos {
     hm::RowPlan rowp;       // its sweep form (row_blocks > 0 CTAs; 0: the table form)
     size_t row_smem;
     int row_blocks;
+    int by_blocks;          // update by blocks (lz_small_plan)
+    int use_small;          // whole runs in one kernel (lz_small.cu)
+    hm::LzSmall small;
     int use_s1;             // s = 1 block path (s1blk.cu)
     int use_mom;            // momentum basis: product k_mom_matvec, then the epilogue kernel
     hm::S1Plan s1;
@@ -345,17 +351,25 @@ k_lz_update(const T *__restrict__ qc, T *__restrict__ qp, uint64_t n, LzScalars 
 // alpha_j = sigma^2 (q.Hq) - sigma gamma (q.q_prev): q.Hq from the per-block partials of
 // the FP64 block product (exact integer dots of the fixed-point copy), q.q_prev from those
 // of the update kernel that made q (double-float), zero at the start (the Paige form
-// v.(Hv - beta v_prev))
+// v.(Hv - beta v_prev)).  few (runs by blocks): one warp adds each, in the order of the whole-run kernel
 __global__ void k_lz_alpha2(LzScalars *S, const double *__restrict__ part, int nblk, const double *__restrict__ qqp,
-                            int nq, double *alpha, int pprev) {
+                            int nq, double *alpha, int pprev, int few) {
     if (S->done) return;
     __shared__ double red[NT / 32];
     double s1 = 0.0, s2 = 0.0;
-    for (int k = threadIdx.x; k < nblk; k += NT) s1 += part[k];
-    for (int k = threadIdx.x; k < nq; k += NT) s2 += qqp[k];
-    s1 = block_sum<NT>(s1, red);
-    __syncthreads();
-    s2 = block_sum<NT>(s2, red);
+    if (few) {
+        if (threadIdx.x < 32) s1 = warp_sum_of(part, nblk);
+        else if (threadIdx.x < 64) s2 = warp_sum_of(qqp, nq);
+        if (threadIdx.x == 32) red[0] = s2;
+        __syncthreads();
+        s2 = red[0];
+    } else {
+        for (int k = threadIdx.x; k < nblk; k += NT) s1 += part[k];
+        for (int k = threadIdx.x; k < nq; k += NT) s2 += qqp[k];
+        s1 = block_sum<NT>(s1, red);
+        __syncthreads();
+        s2 = block_sum<NT>(s2, red);
+    }
     if (threadIdx.x == 0) {
         const double sg = S->sigma_cur, gm = S->beta_prev * S->sigma_prev;
         const double a = sg * sg * s1 - sg * gm * s2;
@@ -394,15 +408,7 @@ k_lz_update_y(const unsigned long long *__restrict__ Y, const float2 *__restrict
     ef::df s{0.0f, 0.0f}, dq{0.0f, 0.0f};
     uint32_t eh = 0;
     auto row = [&](unsigned long long yb, float2 q2, float2 p2) {
-        const ef::df q = ef::df{q2.x, q2.y};
-        const ef::df t1 = ef::df_mul(sg_d, ef::df_from_bits(yb, 0));
-        const ef::df t2 = ef::df_mul(as_d, q);
-        const ef::df t3 = ef::df_mul(gm_d, ef::df{p2.x, p2.y});
-        const ef::df w = ef::df_add(t1, ef::df_neg(ef::df_add(t2, t3)));
-        eh = max(eh, (ef::f2u(w.hi) >> 23) & 0xFFu);
-        s = ef::df_add(s, ef::df_mul(w, w));
-        dq = ef::df_add(dq, ef::df_mul(w, q));
-        return make_float2(w.hi, w.lo);
+        return lz_row_update(yb, q2, p2, sg_d, as_d, gm_d, s, dq, eh);
     };
     const uint64_t stride = (uint64_t)gridDim.x * NT;
     uint64_t r0 = 0;
@@ -439,12 +445,49 @@ k_lz_update_y(const unsigned long long *__restrict__ Y, const float2 *__restrict
     if ((threadIdx.x & 31) == 0 && eh) atomicMax(&S->emax[pprev], (int)eh - 127 + 1023);
 }
 
+// the same by blocks (lz_small_plan): CTA h, thread t rows t and t + BLK_NT of block h; part[h], qqp[h]
+// (those of absent blocks stay zero)
+template <bool PSI>
+__global__ void __launch_bounds__(BLK_NT)
+k_lz_update_blk(BlkParams P, const unsigned long long *__restrict__ Y, const float2 *__restrict__ qc,
+                float2 *__restrict__ qp, LzScalars *S, const double *__restrict__ alpha, double *__restrict__ part,
+                double *__restrict__ qqp, double *__restrict__ psi, const double *__restrict__ coef, int pprev) {
+    if (S->done) return;
+    const uint32_t h = blockIdx.x;
+    if (blk_h_valid(P, h)) {
+        const double sg = S->sigma_cur, gm = S->beta_prev * S->sigma_prev, as = alpha[S->j] * sg;
+        const double cj = PSI ? coef[S->j] * sg : 0.0;
+        auto todf = [](double v) { const float f = (float)v; return ef::df{f, (float)(v - (double)f)}; };
+        const ef::df sg_d = todf(sg), as_d = todf(as), gm_d = todf(gm);
+        const int k = P.A - __popc(h);
+        BlkTabs tb;
+        tb.U = nullptr; tb.R0 = nullptr;
+        tb.C = (const uint32_t *)((const unsigned char *)P.tab + P.off_C);
+        const uint32_t off = blk_off(P, tb, h, k), n = tb.C[P.K * (P.A + 1) + k];
+        ef::df nn{0.0f, 0.0f}, dq{0.0f, 0.0f};
+        uint32_t eh = 0;
+        for (uint32_t r = threadIdx.x; r < n; r += BLK_NT) {
+            const float2 q2 = qc[off + r];
+            qp[off + r] = lz_row_update(Y[off + r], q2, qp[off + r], sg_d, as_d, gm_d, nn, dq, eh);
+            if constexpr (PSI) psi[off + r] += cj * ((double)q2.x + (double)q2.y);
+        }
+        int em = 0;
+        const double t = lz_block_sums(nn, dq, eh, &em);
+        if (threadIdx.x == 0) {
+            part[h] = t;
+            if (em) atomicMax(&S->emax[pprev], em - 127 + 1023);
+        } else if (threadIdx.x == 16) {
+            qqp[h] = t;
+        }
+    }
+}
+
 // start vector of the FP64 block path, one pass: its fixed-point copy X (unit from its
 // largest exponent field, S->emax[0]) and the binary64 values turned into double-float
 // pairs in place (integer conversion, no FP64 instruction); there is no vector before it,
 // so its q.q_prev partials are zero
 __global__ void __launch_bounds__(NT) k_fix_start(unsigned long long *__restrict__ b, long long *__restrict__ X,
-                                                  uint64_t n, const LzScalars *S, double *__restrict__ qqp) {
+                                                  uint64_t n, const LzScalars *S) {
     const int E = S->emax[0];
     for (uint64_t r = blockIdx.x * (uint64_t)NT + threadIdx.x; r < n; r += (uint64_t)gridDim.x * NT) {
         const unsigned long long v = b[r];
@@ -452,7 +495,6 @@ __global__ void __launch_bounds__(NT) k_fix_start(unsigned long long *__restrict
         const ef::df d = ef::df_from_bits(v, 0);
         ((float2 *)b)[r] = make_float2(d.hi, d.lo);
     }
-    if (threadIdx.x == 0) qqp[blockIdx.x] = 0.0;
 }
 
 // fixed-point copy X of the new vector w (double-float pairs), unit from its largest
@@ -477,12 +519,17 @@ k_fixd(const float2 *__restrict__ w, long long *__restrict__ X, uint64_t n, cons
         __stcs(X + r, (long long)ef::fix_from_df(ef::df{w[r].x, w[r].y}, E, 0));
 }
 
-__global__ void k_lz_beta(LzScalars *S, const double *__restrict__ part, int nblk, double *beta, double tol) {
+// few (runs by blocks): one warp adds, in the order of the whole-run kernel
+__global__ void k_lz_beta(LzScalars *S, const double *__restrict__ part, int nblk, double *beta, double tol, int few) {
     if (S->done) return;
     __shared__ double red[NT / 32];
     double s = 0.0;
-    for (int k = threadIdx.x; k < nblk; k += NT) s += part[k];
-    s = block_sum<NT>(s, red);
+    if (few) {
+        if (threadIdx.x < 32) s = warp_sum_of(part, nblk);
+    } else {
+        for (int k = threadIdx.x; k < nblk; k += NT) s += part[k];
+        s = block_sum<NT>(s, red);
+    }
     if (threadIdx.x == 0) {
         const double b = sqrt(s);
         beta[S->j] = b;
@@ -593,12 +640,13 @@ static int enqueue_phase_t(hm_lanczos *R, int parity, int phase, cudaStream_t st
         } else if (b64 && R->use_s1) {
             double *s1part = (double *)(R->work + R->L.s1part);
             HM_TRY(s1_lz64(R->s1, xs[parity], Y, R->sc, parity, s1part, st));
-            k_lz_alpha2<<<1, NT, 0, st>>>(R->sc, s1part, R->s1.nblocks, R->qqp, nblk64, R->alpha, pprev);
+            k_lz_alpha2<<<1, NT, 0, st>>>(R->sc, s1part, R->s1.nblocks, R->qqp, nblk64, R->alpha, pprev, 0);
         } else if (b64) {
             HM_TRY(blk_lz64_launch(R->blk, xs[parity], Y, R->sc, parity, R->hpart, R->blk_blocks, st, R->jit));
             if (R->split)
                 HM_TRY(blk_lz64_launch(R->blk2, xs[parity], Y, R->sc, parity, R->hpart, R->blk_blocks2, st, R->jit2));
-            k_lz_alpha2<<<1, NT, 0, st>>>(R->sc, R->hpart, 1 << R->blk.H, R->qqp, nblk64, R->alpha, pprev);
+            k_lz_alpha2<<<1, NT, 0, st>>>(R->sc, R->hpart, 1 << R->blk.H, R->qqp, R->by_blocks ? 1 << R->blk.H : nblk64,
+                                          R->alpha, pprev, R->by_blocks);
         } else if (R->use_blk) {
             HM_TRY(blk_lz32_launch(R->blk, (const float *)qc, (float *)qp, R->sc, R->hpart, R->blk_blocks, st, R->jit));
             k_lz_alpha<<<1, NT, 0, st>>>(R->sc, R->hpart, 1 << R->blk.H, R->alpha, pprev);
@@ -618,20 +666,24 @@ static int enqueue_phase_t(hm_lanczos *R, int parity, int phase, cudaStream_t st
             k_lz_alpha<<<1, NT, 0, st>>>(R->sc, R->part, np, R->alpha, pprev);
         }
     } else if (b64) {
-        if (R->psi)
-            k_lz_update_y<true><<<nblk64, NT, 0, st>>>(Y, (const float2 *)qc, (float2 *)qp, sv.dim, R->sc, R->alpha,
-                                                       R->part, R->qqp, R->psi, R->coef, pprev);
-        else
-            k_lz_update_y<false><<<nblk64, NT, 0, st>>>(Y, (const float2 *)qc, (float2 *)qp, sv.dim, R->sc,
-                                                        R->alpha, R->part, R->qqp, nullptr, R->coef, pprev);
-        k_lz_beta<<<1, NT, 0, st>>>(R->sc, R->part, nblk64, R->beta, R->dtype == HM_F64 ? LZ_TOL : LZ_TOL32);
+        const int np = R->by_blocks ? 1 << R->blk.H : nblk64;
+        if (R->by_blocks) {
+            auto kern = R->psi ? k_lz_update_blk<true> : k_lz_update_blk<false>;
+            kern<<<np, BLK_NT, 0, st>>>(R->blk, Y, (const float2 *)qc, (float2 *)qp, R->sc, R->alpha, R->part, R->qqp,
+                                        R->psi, R->coef, pprev);
+        } else {
+            auto kern = R->psi ? k_lz_update_y<true> : k_lz_update_y<false>;
+            kern<<<np, NT, 0, st>>>(Y, (const float2 *)qc, (float2 *)qp, sv.dim, R->sc, R->alpha, R->part, R->qqp, R->psi,
+                                    R->coef, pprev);
+        }
+        k_lz_beta<<<1, NT, 0, st>>>(R->sc, R->part, np, R->beta, LZ_TOL, R->by_blocks);
         k_fixd<<<nblk, NT, 0, st>>>((const float2 *)qp, xs[pprev], sv.dim, R->sc, pprev);
     } else {
         if (R->psi)
             k_lz_update<T, true><<<nblk, NT, 0, st>>>(qc, qp, sv.dim, R->sc, R->alpha, R->part, R->psi, R->coef, pprev);
         else
             k_lz_update<T, false><<<nblk, NT, 0, st>>>(qc, qp, sv.dim, R->sc, R->alpha, R->part, nullptr, R->coef, pprev);
-        k_lz_beta<<<1, NT, 0, st>>>(R->sc, R->part, nblk, R->beta, R->dtype == HM_F64 ? LZ_TOL : LZ_TOL32);
+        k_lz_beta<<<1, NT, 0, st>>>(R->sc, R->part, nblk, R->beta, R->dtype == HM_F64 ? LZ_TOL : LZ_TOL32, 0);
     }
     HM_CUDA(cudaGetLastError());
     return HM_OK;
@@ -693,8 +745,10 @@ static int enqueue_start(hm_lanczos *R, const void *v0, uint64_t seed, cudaStrea
     else k_sumsq<float><<<nblk, NT, 0, st>>>((const float *)b0, sv.dim, R->part, nullptr);
     k_lz_start<<<1, NT, 0, st>>>(R->sc, R->part, nblk);
     if ((R->use_blk || R->use_s1) && R->dtype == HM_F64) {
-        k_fix_start<<<nblk, NT, 0, st>>>((unsigned long long *)b0, (long long *)(R->work + R->L.xs[0]), sv.dim, R->sc,
-                                         R->qqp);
+        k_fix_start<<<nblk, NT, 0, st>>>((unsigned long long *)b0, (long long *)(R->work + R->L.xs[0]), sv.dim, R->sc);
+        // no vector before the first: q.q_prev is zero (by blocks, the norms of absent blocks too)
+        HM_CUDA(cudaMemsetAsync(R->qqp, 0, (size_t)(R->by_blocks ? 1 << R->blk.H : upd64_blocks(sv.dim)) * 8, st));
+        if (R->by_blocks) HM_CUDA(cudaMemsetAsync(R->part, 0, (size_t)8 << R->blk.H, st));
     }
     HM_CUDA(cudaGetLastError());
     R->host_j = 0;
@@ -704,7 +758,7 @@ static int enqueue_start(hm_lanczos *R, const void *v0, uint64_t seed, cudaStrea
 
 static int lz_create(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v,
                      const double *J, int dtype, int max_steps, void *work, size_t work_bytes,
-                     bool grad, hm_lanczos **out) {
+                     bool grad, hm_lanczos **out, bool whole = false) {
     if (!b || !out) return fail(HM_EINVAL, "NULL argument");
     if (dtype != HM_F64 && dtype != HM_F32) return fail(HM_EINVAL, "bad dtype");
     if (max_steps < 1 || max_steps > 100000) return fail(HM_EINVAL, "steps must be in 1..100000");
@@ -732,13 +786,25 @@ static int lz_create(const hm_basis *b, int n_bonds, const int32_t *u, const int
                  R->blk.H <= 17;
     R->jit = nullptr;
     R->run = row_run_len();
+    R->use_small = 0;
+    R->by_blocks = 0;
     if (R->use_blk) {
         int jb = 0;
         const void *jk = nullptr;
         rc = blk_target_table(const_cast<hm_basis *>(b), &R->blk, dtype == HM_F64 ? 8 : 4, true);
         if (rc < 0) { delete R; return rc; }
-        if (blk_lz_jit(R->blk, dtype, &jk, &jb) == 0) { R->jit = jk; R->blk_blocks = jb; }
-        if (R->blk.perbond && !R->jit) R->use_blk = 0;   // per-bond rows run only specialised
+        // A small FP64 sector takes its update by blocks and, when the caller runs all steps at once
+        // (whole), all of it in one kernel, which needs no compilation.  HM_JIT=0 and HM_BLK_SPLIT ask
+        // for the step-wise kernels they select among
+        if (dtype == HM_F64 && R->L.small) {
+            rc = lz_small_plan(R->blk, &R->small);
+            if (rc < 0) { delete R; return rc; }
+            R->by_blocks = rc == 0;
+            const char *ej = getenv("HM_JIT"), *es = getenv("HM_BLK_SPLIT");
+            R->use_small = whole && R->by_blocks && !(ej && ej[0] == '0') && !(es && atoi(es) > 0);
+        }
+        if (!R->use_small && blk_lz_jit(R->blk, dtype, &jk, &jb) == 0) { R->jit = jk; R->blk_blocks = jb; }
+        if (R->blk.perbond && !R->jit && !R->use_small) R->use_blk = R->by_blocks = 0;  // else only specialised
     }
     R->split = 0;
     R->jit2 = nullptr;
@@ -779,9 +845,30 @@ static int lz_create(const hm_basis *b, int n_bonds, const int32_t *u, const int
     return HM_OK;
 }
 
+// all steps of a small sector in one kernel
+static int run_small(hm_lanczos *R, int steps, cudaStream_t st) {
+    LzSmallArgs a{};
+    a.X = (long long *)(R->work + R->L.xs[0]);
+    a.q0 = (const float2 *)(R->work + R->L.buf[0]);
+    a.S = R->sc;
+    a.alpha = R->alpha;
+    a.beta = R->beta;
+    a.pa = R->hpart;
+    a.pn = R->part;
+    a.pd = R->qqp;
+    a.pe = (int *)(R->work + R->L.small);
+    a.psi = R->psi;
+    a.coef = R->coef;
+    a.steps = steps;
+    a.tol = LZ_TOL;
+    a.limit_ns = 5000000000ull;
+    return lz_small_launch(R->small, a, st);
+}
+
 // steps launched as one captured graph (the recurrence state lives on the device, so
 // no host round trip is needed between steps)
 static int run_steps_graph(hm_lanczos *R, int steps, cudaStream_t st) {
+    if (R->use_small) return run_small(R, steps, st);
     cudaStream_t cap;
     HM_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
     cudaGraph_t g = nullptr;
@@ -942,6 +1029,7 @@ int lanczos_read(hm_lanczos *R, double *alpha, double *beta, int *steps_done, vo
     if (steps_done) *steps_done = S.j;
     if (alpha && S.j > 0) HM_CUDA(cudaMemcpy(alpha, R->alpha, S.j * 8, cudaMemcpyDeviceToHost));
     if (beta && S.j > 0) HM_CUDA(cudaMemcpy(beta, R->beta, S.j * 8, cudaMemcpyDeviceToHost));
+    if (S.status == HM_ETIMEOUT) return fail(S.status, "a grid barrier of the Lanczos run timed out");
     if (S.status < 0) return fail(S.status, "Lanczos start vector has zero norm");
     return S.status;
 }
@@ -970,9 +1058,10 @@ int lanczos_run(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t 
                 double *ritz, int n_ritz, void *stream) {
     if (n_ritz < 0 || n_ritz > 64 || (n_ritz > 0 && !ritz)) return fail(HM_EINVAL, "n_ritz must be in 0..64");
     hm_lanczos *R = nullptr;
-    HM_TRY(lanczos_init(b, n_bonds, u, v, J, v0, seed, dtype, steps, work, work_bytes, stream, &R));
+    HM_TRY(lz_create(b, n_bonds, u, v, J, dtype, steps, work, work_bytes, false, &R, true));
     cudaStream_t st = as_stream(stream);
-    int rc = run_steps_graph(R, steps, st);
+    int rc = enqueue_start(R, v0, seed, st);
+    if (rc == HM_OK) rc = run_steps_graph(R, steps, st);
     double *d_ritz = (double *)(R->work + R->L.ritz);
     if (rc == HM_OK && n_ritz > 0) {
         k_ritz<<<n_ritz, TRI_NT, 0, st>>>(R->sc, R->alpha, R->beta, d_ritz);
@@ -995,7 +1084,7 @@ int e0_grad(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v, 
     if (b && b->mom_k >= 0) return fail(HM_EINVAL, "e0_grad: not available on a momentum basis");
     if (!e0 || (n_bonds > 0 && !dE0_dJ)) return fail(HM_EINVAL, "NULL output");
     hm_lanczos *R = nullptr;
-    HM_TRY(lz_create(b, n_bonds, u, v, J, HM_F64, steps, work, work_bytes, true, &R));
+    HM_TRY(lz_create(b, n_bonds, u, v, J, HM_F64, steps, work, work_bytes, true, &R, true));
     cudaStream_t st = as_stream(stream);
     const SectorView &sv = b->view;
     const int nblk = grid_blocks(sv.dim, NT);
@@ -1005,7 +1094,8 @@ int e0_grad(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v, 
     int rc = HM_OK;
     // pass 1: T
     rc = enqueue_start(R, v0, seed, st);
-    for (int k = 0; k < steps && rc == HM_OK; ++k) rc = enqueue_step(R, st);
+    if (rc == HM_OK && R->use_small) rc = run_small(R, steps, st);
+    for (int k = 0; k < steps && rc == HM_OK && !R->use_small; ++k) rc = enqueue_step(R, st);
     if (rc == HM_OK) {
         // residual of the lowest Ritz pair of every leading T_k, then the shortest
         // converged length and the eigenvector of T there (no ghost copies yet)
@@ -1020,6 +1110,7 @@ int e0_grad(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v, 
         cudaError_t e = cudaMemcpyAsync(&S1, R->sc, sizeof S1, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = cuda_fail(e, "e0_grad: read pass 1");
+        if (rc == HM_OK && S1.status == HM_ETIMEOUT) rc = fail(S1.status, "a grid barrier of the Lanczos run timed out");
         if (rc == HM_OK && S1.status < 0) rc = fail(S1.status, "Lanczos start vector has zero norm");
     }
     if (rc == HM_OK) {
@@ -1027,7 +1118,8 @@ int e0_grad(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v, 
         cudaError_t e = cudaMemsetAsync(R->psi, 0, sv.dim * 8, st);
         if (e != cudaSuccess) rc = cuda_fail(e, "memset psi");
         if (rc == HM_OK) rc = enqueue_start(R, v0, seed, st);
-        for (int k = 0; k < S1.mconv && rc == HM_OK; ++k) rc = enqueue_step(R, st);
+        if (rc == HM_OK && R->use_small) rc = run_small(R, S1.mconv, st);
+        for (int k = 0; k < S1.mconv && rc == HM_OK && !R->use_small; ++k) rc = enqueue_step(R, st);
     }
     if (rc == HM_OK) {
         k_sumsq<double><<<nblk, NT, 0, st>>>(R->psi, sv.dim, R->part, nullptr);
