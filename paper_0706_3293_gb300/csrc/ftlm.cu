@@ -38,11 +38,11 @@ namespace hm {
 __host__ __device__ __forceinline__ size_t al16f(size_t x) { return (x + 15) & ~(size_t)15; }
 
 constexpr int FT_NT = 512;          // threads per CTA of the persistent kernel
-// CTAs per SM the register budget is cut for: three (40 registers; the widest tiling then
-// spills a little) ran the N = 24 run in 825 ms against 989 ms with two (64 registers): the
-// kernel waits on gather latency, and the extra resident warps hide more of it
+// CTAs per SM the register budget is cut for: with two (64 registers) the widest tiling spills little,
+// with three (40) its four gathers in flight and eight sums spill at every row: 463 against 510 us a
+// step of the N = 20 run, 151 against 178 at N = 18
 #ifndef HM_FT_CTAS
-#define HM_FT_CTAS 3
+#define HM_FT_CTAS 2
 #endif
 constexpr int FT_CTAS = HM_FT_CTAS;
 constexpr int FT_W = 32;            // row stride in floats (vectors per row, padded)
@@ -78,11 +78,12 @@ struct FtDev {
     const FtRange *wr;              // [warp]
     const uint32_t *slo;            // [nsec + 1]: sector s owns slots slo[s] .. slo[s + 1] - 1
     const uint2 *cta_rng;           // [nsec]: the CTAs [x, y) whose update rows include rows of sector s
-    int *sec_active;                // [s]
+    int *sec_active;                // [s]: four bytes, one for each eight vectors
     GridBar *bar;
     const uint32_t *items;          // (A << 16) | h, sorted by A
     const uint64_t *rowoff;         // first global row of sector A
     const uint32_t *secdim;         // D(N, A)
+    uint16_t *hops;                 // [2^K][hop_stride]: targets of each low word (k_ft_hops)
     float *q0, *q1;                 // [rows][FT_W]
     double *theta, *tau;            // [(s * FT_W + v) * steps + j]
     int *mlen;                      // Krylov length per (s, v)
@@ -109,6 +110,11 @@ struct FtParams {
     uint64_t seed;
     unsigned long long barrier_ns;  // a grid barrier gives up after this long (default 5 s)
     uint64_t exact_mask;            // bit A set: sector A is diagonalised exactly
+    // a row of d.hops (16-bit entries): the number of low targets of each class as four bytes and an entry
+    // for each of the first six low ends of cross bonds, then from hop_seg[c] on the low targets
+    // of class c, then from hop_x on the entries of the other low ends
+    int hop_stride, hop_seg[HM_BLK_MAXC], hop_x, hop_nx;
+    uint8_t hop_xp[HM_BLK_MAXB], hop_xi[HM_BLK_MAXB];   // the low ends; that of each cross bond
     int nexact;
     ExactSec ex[FT_MAXEXACT];
 };
@@ -184,7 +190,7 @@ __global__ void k_ft_init(FtParams F) {
         d.mlen[t] = 0;
     }
     if (blockIdx.x == 0 && threadIdx.x < FT_MAXS && (int)threadIdx.x < F.nsec)
-        d.sec_active[threadIdx.x] = ((F.exact_mask >> threadIdx.x) & 1ull) ? 0 : 1;
+        d.sec_active[threadIdx.x] = ((F.exact_mask >> threadIdx.x) & 1ull) ? 0 : 0x01010101;
     if (blockIdx.x == 0 && threadIdx.x == 0) { d.bar->count = 0; d.bar->gen = 0; d.bar->abort = 0; }
 }
 
@@ -207,11 +213,55 @@ __device__ __forceinline__ void ft_warp_flush(ef::df *p, double *part, uint32_t 
     }
 }
 
+constexpr int FT_XHEAD = 6;         // cross entries in the first 16 bytes of a row of the target table
+
+// Targets of the low words, once per run: thread g takes the low word at position g of the word list
+// (class k of its ones, rank r) and writes the ranks its low exchanges reach, by class and in the
+// order of the bond groups, each class's run padded to a multiple of four with r itself, and the rank of
+// l ^ 2^p for each low end p of a cross bond.  With these rows a product's target takes a
+// shift, an address and the gather; finding it took the masks, a bit scan, the xor and two
+// table lookups, which all 32 lanes did for the same few rows.  Product phase of the N = 20 run
+// 382 -> 346 us a step, where the gathers' way through L1 and L2 bounds it, not instructions.
+__global__ void k_ft_hops(FtParams F) {
+    const BlkParams &P = F.P;
+    const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= 1u << P.K) return;
+    BlkTabs tb;
+    tb.U = (const uint16_t *)((const unsigned char *)P.tab + P.off_U);
+    tb.R0 = (const uint8_t *)P.tab + P.off_R0;
+    tb.C = (const uint32_t *)((const unsigned char *)P.tab + P.off_C);
+    const uint32_t l = P.lw[g];
+    const int k = __popc(l);
+    const uint32_t r = g - (uint32_t)P.lwoff[k];
+    uint16_t *T = F.d.hops + (size_t)g * F.hop_stride;
+    for (int c = 0; c < HM_BLK_MAXC; ++c) {
+        int m = 0;
+        if (c < P.nc) {
+            uint16_t *t = T + F.hop_seg[c];
+            blk_low_hops(P, tb, c, l, r, tb.U + k * P.nb1, [&](uint32_t r2) { t[m++] = (uint16_t)r2; });
+            for (int i = m; i & 3; ++i) t[i] = (uint16_t)r;
+        }
+        ((uint8_t *)T)[c] = (uint8_t)m;
+    }
+    for (int i = 0; i < F.hop_nx; ++i) {
+        const uint32_t l2 = l ^ (1u << F.hop_xp[i]);
+        T[i < FT_XHEAD ? 2 + i : F.hop_x + i - FT_XHEAD] = (uint16_t)rank_low(P, tb, l2, __popc(l2));
+    }
+}
+
+// A warp's exchange lists of the block it works on
+struct FtHops {
+    int4 *x;              // [ncb] cross bond: {target block's rows less own, xor | test mask << 16, low end, 0}
+    int *hcd;             // [nhb] offsets (target row - own row) of the valid high exchanges
+    int *hcs;             // [HM_BLK_MAXC + 1] class c owns hcd[hcs[c] .. hcs[c+1])
+};
+
 // Hop lists of block (h, k) for one warp: the valid high exchanges as row offsets,
 // compacted by class (lane e tests bonds e and e + 32, ballots give the positions), and
 // the targets of the cross exchanges.  The caller syncs the warp before and after.
-__device__ __forceinline__ void ft_warp_setup(const BlkParams &P, const BlkTabs &tb, uint32_t h, int k, uint32_t off,
-                                              const BlkShared &sh, int lane) {
+__device__ __forceinline__ void ft_warp_setup(const FtParams &F, const BlkTabs &tb, uint32_t h, int k, uint32_t off,
+                                              const FtHops &sh, int lane) {
+    const BlkParams &P = F.P;
     int val[2] = {0, 0}, hoff[2] = {0, 0};
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
@@ -232,48 +282,64 @@ __device__ __forceinline__ void ft_warp_setup(const BlkParams &P, const BlkTabs 
                                : __popc(b0 & ((1u << e) - 1u));
     }
     for (int e = lane; e < P.ncb; e += 32) {
-        const int q = P.cb_q[e];
+        const int p = P.cb_p[e], q = P.cb_q[e];
         const uint32_t bq = (h >> q) & 1u;
         const int k2 = k + (bq ? 1 : -1);
-        const bool ok = k2 >= 0 && k2 <= P.K;
-        sh.cbq[e] = (uint8_t)bq;
-        sh.ck[e] = (int8_t)(ok ? k2 : -1);
-        sh.coff[e] = ok ? blk_off(P, tb, h ^ (1u << q), k2) : 0u;
+        const bool ok = k2 >= 0 && k2 <= P.K;     // else the test mask is empty
+        sh.x[e] = make_int4(ok ? (int)(blk_off(P, tb, h ^ (1u << q), k2) - off) : 0,
+                            (int)((bq << p) | (ok ? 1u << (p + 16) : 0u)), F.hop_xi[e], 0);
     }
 }
 
 // Per (sector, vector) sums of the CTA partials partc[s][b][v] over the CTAs b in [lo(s), hi(s))
-// in a fixed order (16 strided chunks of four running sums, then the chunks in order);
-// f(s, v, sum) runs on warp 0 of the CTA that owns sector s.  All threads call it.  The sums run over
-// CTAs, not warps: a binary64 add costs a warp 64 cycles, and the 1284 warp partials of the
-// largest sector of N = 20 took 10 us a step.
+// in a fixed order: eight vectors of a sector to a CTA, thread (chunk, vector) takes every 64th CTA, the
+// 64 chunks by shuffles over four lanes and over the warps' sums in order; f(s, v, sum) then runs
+// on 8 lanes.  All threads call it.  The sums run over CTAs, not warps, and a binary64 add costs a
+// warp 64 cycles: with one CTA and 16 chunks to a sector's 32 vectors the two grid barriers
+// around this took 20 us of a step of the N = 20 run, 7 now.
+constexpr int FT_OCT = FT_W / 8;                  // CTAs a sector
 template <class R, class F>
 __device__ __forceinline__ void ft_sector_sums(const FtParams &Fp, double *red, R &&range, F &&f) {
     const FtDev &d = Fp.d;
-    constexpr int NCH = FT_NT / FT_W;
-    const int v = threadIdx.x % FT_W, c = threadIdx.x / FT_W;
-    for (int s = blockIdx.x; s < Fp.nsec; s += gridDim.x) {
-        const double *ps = d.partc + (size_t)s * Fp.nctas * FT_W;
+    constexpr int NCH = FT_NT / 8;
+    const int v8 = threadIdx.x & 7, c = threadIdx.x >> 3, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int so = blockIdx.x; so < Fp.nsec * FT_OCT; so += gridDim.x) {
+        const int s = so / FT_OCT, v = (so % FT_OCT) * 8 + v8;
+        const double *ps = d.partc + (size_t)s * Fp.nctas * FT_W + v;
         const uint2 lh = range(s);
-        const unsigned nb = lh.y;
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        unsigned b = lh.x + c;
-        for (; b + 3 * NCH < nb; b += 4 * NCH) {
-            a0 += ps[(size_t)b * FT_W + v];
-            a1 += ps[(size_t)(b + NCH) * FT_W + v];
-            a2 += ps[(size_t)(b + 2 * NCH) * FT_W + v];
-            a3 += ps[(size_t)(b + 3 * NCH) * FT_W + v];
-        }
-        for (; b < nb; b += NCH) a0 += ps[(size_t)b * FT_W + v];
-        const double a = (a0 + a1) + (a2 + a3);
-        red[c * FT_W + v] = a;
+        double a = 0.0;
+#pragma unroll 8
+        for (unsigned b = lh.x + c; b < lh.y; b += NCH) a += __ldcg(ps + (size_t)b * FT_W);
+        a += __shfl_xor_sync(0xffffffffu, a, 8);
+        a += __shfl_xor_sync(0xffffffffu, a, 16);
+        if (lane < 8) red[warp * 8 + lane] = a;
         __syncthreads();
-        if (c == 0) {
+        if (warp == 0) {
             double t = 0.0;
-            for (int i = 0; i < NCH; ++i) t += red[i * FT_W + v];
-            f(s, v, t);
+#pragma unroll
+            for (int i = 0; i < FT_NT / 32; i += 4) t += red[(i + (lane >> 3)) * 8 + v8];
+            t += __shfl_xor_sync(0xffffffffu, t, 8);
+            t += __shfl_xor_sync(0xffffffffu, t, 16);
+            if (lane < 8) f(s, v, t);
         }
         __syncthreads();
+    }
+}
+
+// a += b where on holds, two additions to an instruction and no branch
+template <int VT>
+__device__ __forceinline__ void ft_add(float *a, const float *b, bool on = true) {
+    if constexpr (VT == 1) {
+        if (on) a[0] += b[0];
+    } else {
+#pragma unroll
+        for (int q = 0; q < VT; q += 2) {
+            unsigned long long s, t;
+            asm("mov.b64 %0, {%1, %2};" : "=l"(s) : "f"(a[q]), "f"(a[q + 1]));
+            asm("mov.b64 %0, {%1, %2};" : "=l"(t) : "f"(b[q]), "f"(b[q + 1]));
+            asm("{\n.reg .pred p;\nsetp.ne.s32 p, %2, 0;\n@p add.rn.f32x2 %0, %0, %1;\n}" : "+l"(s) : "l"(t), "r"((int)on));
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(a[q]), "=f"(a[q + 1]) : "l"(s));
+        }
     }
 }
 
@@ -291,6 +357,26 @@ __device__ __forceinline__ void ft_ld(const float *p, float *v) {
     }
 }
 
+// the same of shared memory or the buffer the kernel writes, and the store
+template <int VT>
+__device__ __forceinline__ void ft_ld_rw(const float *p, float *v) {
+    if constexpr (VT == 4) {
+        const float4 t = *(const float4 *)p;
+        v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+    } else if constexpr (VT == 2) {
+        const float2 t = *(const float2 *)p;
+        v[0] = t.x; v[1] = t.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int VT>
+__device__ __forceinline__ void ft_st(float *p, const float *v) {
+    if constexpr (VT == 4) *(float4 *)p = make_float4(v[0], v[1], v[2], v[3]);
+    else if constexpr (VT == 2) *(float2 *)p = make_float2(v[0], v[1]);
+    else *p = v[0];
+}
+
 // sector of a global row (few sectors: linear search)
 __device__ __forceinline__ int ft_sector_of(const FtDev &d, int nsec, uint64_t g) {
     int A = 0;
@@ -299,9 +385,10 @@ __device__ __forceinline__ int ft_sector_of(const FtDev &d, int nsec, uint64_t g
 }
 
 // per-warp shared slice: hop lists | sigma, gamma of the current sector | alpha sigma
-__host__ __device__ __forceinline__ size_t ft_warp_bytes(int max_block) {
-    return al16f(blk_shared_bytes(max_block)) + al16f(FT_W * 4 * 3);
+__host__ __device__ __forceinline__ size_t ft_hops_bytes(const BlkParams &P) {
+    return al16f((size_t)P.ncb * 16 + (size_t)(P.nhb + HM_BLK_MAXC + 1) * 4);
 }
+__host__ __device__ __forceinline__ size_t ft_warp_bytes(const BlkParams &P) { return ft_hops_bytes(P) + FT_W * 4 * 3; }
 
 // ---- the persistent kernel ---------------------------------------------------------------
 // Every warp owns the global rows [g0, g1) of its FtRange (rows of all sectors in order,
@@ -316,11 +403,13 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
     extern __shared__ __align__(16) unsigned char smem[];
     const BlkTabs tb = stage_blk_tables(P, smem);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const size_t wbytes = ft_warp_bytes(P.max_block);
-    unsigned char *ws = smem + al16f(P.tab_bytes) + warp * wbytes;
-    const BlkShared sh = blk_carve(ws, P.max_block);
-    float *sgw = (float *)(ws + al16f(blk_shared_bytes(P.max_block)));   // [sigma | gamma | alpha sigma][FT_W]
-    double *red = (double *)(smem + al16f(P.tab_bytes) + (FT_NT / 32) * wbytes);
+    unsigned char *ws = smem + al16f(P.tab_bytes) + warp * ft_warp_bytes(P);
+    FtHops sh;
+    sh.x = (int4 *)ws;
+    sh.hcd = (int *)(sh.x + P.ncb);
+    sh.hcs = sh.hcd + P.nhb;
+    float *sgw = (float *)(ws + ft_hops_bytes(P));  // [sigma | gamma | alpha sigma][FT_W]
+    double *red = (double *)(smem + al16f(P.tab_bytes) + (FT_NT / 32) * ft_warp_bytes(P));
     constexpr int LPR = 32 / VT;                   // lanes per row
     const int grp = lane / LPR, li = lane % LPR;   // row group in the warp, lane in row
     const int v0 = li * VT;                        // first vector of this lane
@@ -372,13 +461,13 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                     const uint32_t ra = ig0 < g0 ? (uint32_t)(g0 - ig0) : 0u;
                     const uint32_t rb = ig0 + n > g1 ? (uint32_t)(g1 - ig0) : n;
                     __syncwarp();                  // the previous block's lists are read no more
-                    ft_warp_setup(P, tb, h, k, off, sh, lane);
+                    ft_warp_setup(F, tb, h, k, off, sh, lane);
                     __syncwarp();
                     const float *Xb = qc + ig0 * FT_W + v0;   // the block's rows, this lane's vectors
-                    const uint16_t *Uk = tb.U + k * P.nb1;
-                    const uint16_t *lw = P.lw + P.lwoff[k];
                     for (uint32_t r = ra + grp; r < rb; r += VT) {
-                        const uint32_t l = __ldg(lw + r);
+                        const uint32_t g = (uint32_t)P.lwoff[k] + r, l = __ldg(P.lw + g);
+                        const uint16_t *T = d.hops + (size_t)g * F.hop_stride;
+                        const uint4 hd = __ldg((const uint4 *)T);   // counts, cross entries
                         float acc[NC][VT];
                         int cnt[NC];
 #pragma unroll
@@ -386,41 +475,60 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                             float *ac = acc[cl];
 #pragma unroll
                             for (int q = 0; q < VT; ++q) ac[q] = 0.0f;
-                            int mc = blk_low_hops(P, tb, cl, l, r, Uk, [&](uint32_t r2) {
+                            // low exchanges: four gathers in flight, added in the order of the list; the
+                            // padding reads the row itself and is not added
+                            int mc = (int)((hd.x >> (8 * cl)) & 0xFFu);
+                            const uint16_t *t = T + F.hop_seg[cl];
+                            for (int e = 0; e < mc; e += 4) {
+                                const uint2 w = __ldg((const uint2 *)(t + e));
+                                float x0[VT], x1[VT], x2[VT], x3[VT];
+                                ft_ld<VT>(Xb + (size_t)(w.x & 0xFFFFu) * FT_W, x0);
+                                ft_ld<VT>(Xb + (size_t)(w.x >> 16) * FT_W, x1);
+                                ft_ld<VT>(Xb + (size_t)(w.y & 0xFFFFu) * FT_W, x2);
+                                ft_ld<VT>(Xb + (size_t)(w.y >> 16) * FT_W, x3);
+                                ft_add<VT>(ac, x0);
+                                ft_add<VT>(ac, x1, e + 1 < mc);
+                                ft_add<VT>(ac, x2, e + 2 < mc);
+                                ft_add<VT>(ac, x3, e + 3 < mc);
+                            }
+                            for (int e = P.cb_start[cl]; e < P.cb_start[cl + 1]; ++e) {
+                                const int4 x = sh.x[e];
+                                const bool on = ((l ^ (uint32_t)x.y) & ((uint32_t)x.y >> 16)) != 0u;
+                                const uint32_t xw = x.z < 2 ? hd.y : x.z < 4 ? hd.z : hd.w;
+                                int t2 = (int)((x.z & 1) ? xw >> 16 : xw & 0xFFFFu);
+                                if (x.z >= FT_XHEAD) t2 = (int)__ldg(T + F.hop_x + x.z - FT_XHEAD);
                                 float xv[VT];
-                                ft_ld<VT>(Xb + (size_t)r2 * FT_W, xv);
-#pragma unroll
-                                for (int q = 0; q < VT; ++q) ac[q] += xv[q];
-                            });
-                            mc += blk_cross_hops(P, tb, cl, l, sh, [&](uint32_t jj) {
-                                float xv[VT];
-                                ft_ld<VT>(qc + (base + jj) * FT_W + v0, xv);
-#pragma unroll
-                                for (int q = 0; q < VT; ++q) ac[q] += xv[q];
-                            });
+                                ft_ld<VT>(Xb + (int64_t)(on ? x.x + t2 : (int)r) * FT_W, xv);
+                                ft_add<VT>(ac, xv, on);
+                                mc += (int)on;
+                            }
                             // high exchanges: four independent gathers in flight (the far ones miss L2)
                             const int e1 = sh.hcs[cl + 1];
                             int e = sh.hcs[cl];
                             for (; e + 4 <= e1; e += 4) {
                                 float x0[VT], x1[VT], x2[VT], x3[VT];
-                                ft_ld<VT>(Xb + (int64_t)((int64_t)r + sh.hcd[e]) * FT_W, x0);
-                                ft_ld<VT>(Xb + (int64_t)((int64_t)r + sh.hcd[e + 1]) * FT_W, x1);
-                                ft_ld<VT>(Xb + (int64_t)((int64_t)r + sh.hcd[e + 2]) * FT_W, x2);
-                                ft_ld<VT>(Xb + (int64_t)((int64_t)r + sh.hcd[e + 3]) * FT_W, x3);
-#pragma unroll
-                                for (int q = 0; q < VT; ++q) ac[q] += (x0[q] + x1[q]) + (x2[q] + x3[q]);
+                                ft_ld<VT>(Xb + (int64_t)((int)r + sh.hcd[e]) * FT_W, x0);
+                                ft_ld<VT>(Xb + (int64_t)((int)r + sh.hcd[e + 1]) * FT_W, x1);
+                                ft_ld<VT>(Xb + (int64_t)((int)r + sh.hcd[e + 2]) * FT_W, x2);
+                                ft_ld<VT>(Xb + (int64_t)((int)r + sh.hcd[e + 3]) * FT_W, x3);
+                                ft_add<VT>(x0, x1);
+                                ft_add<VT>(x2, x3);
+                                ft_add<VT>(x0, x2);
+                                ft_add<VT>(ac, x0);
                             }
                             for (; e < e1; ++e) {
                                 float xv[VT];
-                                ft_ld<VT>(Xb + (int64_t)((int64_t)r + sh.hcd[e]) * FT_W, xv);
-#pragma unroll
-                                for (int q = 0; q < VT; ++q) ac[q] += xv[q];
+                                ft_ld<VT>(Xb + (int64_t)((int)r + sh.hcd[e]) * FT_W, xv);
+                                    ft_add<VT>(ac, xv);
                             }
                             cnt[cl] = mc + (sh.hcs[cl + 1] - sh.hcs[cl]);
                         }
-                        const uint64_t row = ig0 + r;
-                        float xov[VT];
+                        float *up = qp + (ig0 + r) * FT_W + v0;
+                        float xov[VT], uv[VT], sg[VT], gm[VT];
                         ft_ld<VT>(Xb + (size_t)r * FT_W, xov);
+                        ft_ld_rw<VT>(up, uv);
+                        ft_ld_rw<VT>(sgw + v0, sg);
+                        ft_ld_rw<VT>(sgw + FT_W + v0, gm);
 #pragma unroll
                         for (int q = 0; q < VT; ++q) {
                             const float xo = xov[q];
@@ -428,10 +536,11 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
 #pragma unroll
                             for (int cl = 0; cl < NC; ++cl)
                                 y += P.gq[cl] * (2.0f * acc[cl][q] + (float)(P.ntot[cl] - 2 * cnt[cl]) * xo);
-                            const float u = sgw[v0 + q] * y - sgw[FT_W + v0 + q] * qp[row * FT_W + v0 + q];
-                            qp[row * FT_W + v0 + q] = u;
-                            dot[q] = ef::df_add(dot[q], ef::two_prod(sgw[v0 + q] * xo, u));
+                            const float u = sg[q] * y - gm[q] * uv[q];
+                            uv[q] = u;
+                            dot[q] = ef::df_add(dot[q], ef::two_prod(sg[q] * xo, u));
                         }
+                        ft_st<VT>(up, uv);
                     }
                 }
             }
@@ -534,9 +643,9 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                     act = true;
                 }
             }
-            // a sector stays active while any of its vectors runs (warp 0 holds one sector)
-            const unsigned any = __ballot_sync(0xffffffffu, act);
-            if (v == 0) d.sec_active[s] = any != 0u;
+            // a sector stays active while any of its vectors runs: one byte for each eight of them
+            const unsigned any = __ballot_sync(0xFFu, act);
+            if (v % 8 == 0) ((unsigned char *)(d.sec_active + s))[v / 8] = any != 0u;
         });
         if (!grid_sync(d.bar, F.nctas, LIMIT)) return;
     }
@@ -833,7 +942,7 @@ __global__ void __launch_bounds__(256) k_ft_thermo_fin(FtParams F, const double 
 
 // ---- host --------------------------------------------------------------------------------
 struct FtLayout {
-    size_t q0, q1, st, ab, part, wr, slo, crng, parta, partc, ckit, ckcs, sec, bar, items, rowoff, secdim, theta, tau, mlen, therm, tsum, temps,
+    size_t q0, q1, st, ab, part, wr, slo, crng, parta, partc, ckit, ckcs, sec, bar, items, rowoff, secdim, hops, theta, tau, mlen, therm, tsum, temps,
         xcd, xmat, total;
 };
 
@@ -850,7 +959,7 @@ static int ft_choose_K(int N) {
 }
 
 static FtLayout ft_layout(int N, int nsec, int R, int steps, int nitems, int nctas, int n_t, size_t xcd_words,
-                          size_t xmat_doubles, size_t nchunks) {
+                          size_t xmat_doubles, size_t nchunks, size_t hop_entries) {
     (void)R;
     FtLayout L{};
     auto a = [](size_t x) { return (x + 255) & ~(size_t)255; };
@@ -875,6 +984,7 @@ static FtLayout ft_layout(int N, int nsec, int R, int steps, int nitems, int nct
     L.items = o; o += a((size_t)nitems * 4);
     L.rowoff = o; o += a((size_t)(nsec + 1) * 8);
     L.secdim = o; o += a((size_t)nsec * 4);
+    L.hops = o; o += a(hop_entries * 2);
     L.theta = o; o += a(nst * (size_t)steps * 8);
     L.tau = o; o += a(nst * (size_t)steps * 8);
     L.mlen = o; o += a(nst * 4);
@@ -899,8 +1009,8 @@ static const void *pick_kernel(int nc, int vt) {
 static size_t ft_smem(const BlkParams &P, int nsec) {
     (void)nsec;
     size_t o = al16f(P.tab_bytes);
-    o += (FT_NT / 32) * ft_warp_bytes(P.max_block);
-    o += al16f((size_t)(FT_NT / FT_W) * FT_W * 8);    // sector-sum scratch
+    o += (FT_NT / 32) * ft_warp_bytes(P);
+    o += (size_t)(FT_NT / 32) * 8 * 8;    // sector-sum scratch
     return o;
 }
 
@@ -1020,6 +1130,26 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
     uint64_t mb = 1;
     for (int i = 0; i < K / 2; ++i) mb = mb * (K - i) / (i + 1);
     S->F.P.max_block = (int)mb;
+    // rows of the target table
+    {
+        FtParams &F = S->F;
+        const BlkParams &P = F.P;
+        int o = 2 + FT_XHEAD;
+        for (int c = 0; c < P.nc; ++c) {
+            int m = 0;
+            for (int g = P.lg_cs[3 * c]; g < P.lg_cs[3 * c + 3]; ++g) m += __builtin_popcount(P.lg_mask[g]);
+            F.hop_seg[c] = o;
+            o += (m + 3) & ~3;
+        }
+        F.hop_x = o;
+        for (int e = 0; e < P.ncb; ++e) {
+            int i = 0;
+            while (i < F.hop_nx && F.hop_xp[i] != P.cb_p[e]) ++i;
+            if (i == F.hop_nx) F.hop_xp[F.hop_nx++] = P.cb_p[e];
+            F.hop_xi[e] = (uint8_t)i;
+        }
+        F.hop_stride = (o + std::max(0, F.hop_nx - FT_XHEAD) + 7) & ~7;
+    }
     const int nsec = n_sites + 1;
     items->clear();
     const int H = n_sites - K;
@@ -1075,7 +1205,7 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
               &S->ck_cs);
     S->F.nchunks = (uint32_t)S->ck_it0.size();
     S->L = ft_layout(n_sites, nsec, R, steps, S->F.nitems, S->nctas, n_t, S->xcd.size(), (size_t)xmat,
-                     S->F.nchunks);
+                     S->F.nchunks, (size_t)S->F.hop_stride << K);
     return HM_OK;
 }
 
@@ -1104,6 +1234,7 @@ static void ft_bind(FtSetup *S, unsigned char *w) {
     d.items = (const uint32_t *)(w + L.items);
     d.rowoff = (const uint64_t *)(w + L.rowoff);
     d.secdim = (const uint32_t *)(w + L.secdim);
+    d.hops = (uint16_t *)(w + L.hops);
     d.theta = (double *)(w + L.theta);
     d.tau = (double *)(w + L.tau);
     d.mlen = (int *)(w + L.mlen);
@@ -1191,6 +1322,8 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
         HM_CUDA(cudaMemcpyAsync(w + S.L.xcd, S.xcd.data(), S.xcd.size() * 4, cudaMemcpyHostToDevice, st));
     double *d_temps = (double *)(w + S.L.temps);
     if (n_t > 0) HM_CUDA(cudaMemcpyAsync(d_temps, temps, n_t * 8, cudaMemcpyHostToDevice, st));
+    k_ft_hops<<<((1u << S.F.P.K) + 127) / 128, 128, 0, st>>>(S.F);
+    HM_CUDA(cudaGetLastError());
     // autotune the vectors-per-lane tiling on a short run (2 steps), once per shape
     int use_vt = vt;
     if (use_vt == 0) {

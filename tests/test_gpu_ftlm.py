@@ -170,3 +170,25 @@ def test_ftlm_barrier_gives_up_and_device_stays_usable(hm, monkeypatch):
     again = hm.ftlm_run(12, hm.bonds_of(inst), 4, 20, 3, [1.0], vt=1)
     assert again.Z[0] == ok.Z[0] and again.E[0] == ok.E[0]
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("vt", [1, 2, 4])
+@pytest.mark.parametrize("n,kind", [(10, "complete"), (11, "complete"), (13, "far")])
+def test_ftlm_target_table_rows(hm, n, kind, vt):
+    """First moments sum_j tau_j theta_j = <v|H|v> of each sector and vector, on bonds with more low ends
+    of cross bonds than the first 16 bytes of a table row hold (complete) and with classes that have no
+    low, cross or high bond (far).  An FP32 row adds at most 3 n_bonds + 4 terms, |row| <= sum |J| / 4 (3 |v|)."""
+    if kind == "complete":
+        u, v = np.triu_indices(n, 1)
+        J = np.array([-1.0, 0.6, -0.25, 0.1])[np.arange(len(u)) % 4]
+    else:
+        u, v, J = np.array([0, 0, n - 2, 3]), np.array([1, n - 1, n - 1, n - 2]), np.array([-1.0, 0.5, 0.25, -0.7])
+    R, steps, seed = 3, 12, 5
+    gpu = hm.ftlm_run(n, hm.BondList.make(u, v, J), R, steps, seed, TEMPS, vt=vt)
+    tol = (3 * len(u) + 8) * 2.0**-24 * 0.75 * np.abs(J).sum()
+    for A in range(n + 1):
+        res = oracle.ftlm_sector(oracle.Basis(n, 1, A), oracle.Bonds(u, v, J), seed, R, steps)
+        for r in range(R):
+            m = int(gpu.mlen[A, r])
+            got = float(gpu.tau[A, r, :m] @ gpu.theta[A, r, :m])
+            assert abs(got - float(np.dot(res[r][1], res[r][0]))) <= tol, (A, r)
