@@ -17,10 +17,8 @@
 //   B  alpha per (sector, vector): the sector's warp partials in order
 //   C  w = u - alpha sigma q over q_prev, |w|^2 partials
 //   D  beta, breakdown, sigma
-// Then per (sector, vector) the tridiagonal T is diagonalised on the device (implicit
-// symmetric QR with Wilkinson shifts, Golub and Van Loan, Matrix Computations, Sec. 8.3),
-// keeping the first row of the eigenvector matrix: Ritz values theta_j and weights
-// tau_j = (first component)^2.  Finally
+// Then per (sector, vector) the eigenvalues of the tridiagonal T, the Ritz values theta_j, and
+// the squares tau_j of the first components of its eigenvectors are formed on the device.  Finally
 //   Z(T) = sum_A (D_A / R) sum_r sum_j tau e^{-(theta - e_ref)/T},
 //   E(T) = [same with theta inside] / Z(T)     (Z returned relative to e^{-e_ref/T}).
 #include <algorithm>
@@ -32,6 +30,7 @@
 #include <vector>
 
 #include "blk.cuh"
+#include "tridiag.cuh"
 
 namespace hm {
 
@@ -651,117 +650,92 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
     }
 }
 
-// ---- tridiagonal eigen-decomposition with the first components -------------------------
-// Implicit symmetric QR with Wilkinson shifts (Golub and Van Loan, Sec. 8.3): each sweep
-// chases a bulge down the unreduced block with Givens rotations; the rotations are also
-// applied to z, the first row of the accumulated eigenvector matrix.
-// One warp per matrix.  A sweep is one chain of rotations, and a warp's binary64 instruction
-// occupies its quarter of an SM for 64 cycles however many lanes take part, so what counts is the
-// number of binary64 instructions a rotation takes one after the other.  Its cosine and sine come
-// from one rsqrt (six of them; hypot and two divisions take forty), and the about thirty products
-// and sums are spread over four lanes, which do up to four of them in one instruction and hand the
-// results round by shuffles: fourteen in all.  The scan for a negligible off-diagonal looks at 32
-// rows at a time.  T is scaled to norm 1, so squares neither overflow nor lose anything that
-// matters when they underflow.  N = 20, 672 matrices of 80 rows: 25.7 ms with one thread to a
-// matrix in 6 CTAs and hypot, 12.7 ms with rsqrt and 4 matrices to a CTA, 9.5 ms here.
-__device__ void tri_ql_first(int m, double *dg, double *e, double *z) {
-    const int lane = threadIdx.x & 31, q = lane & 3;
-    const double eps = 2.220446049250313e-16;
-    auto from = [](double v, int src) { return __shfl_sync(0xffffffffu, v, src); };
-    for (int i = lane; i < m; i += 32) z[i] = i == 0 ? 1.0 : 0.0;
-    __syncwarp();
-    int hi = m - 1, guard = 0;
-    while (hi > 0 && guard < 60 * m) {
-        // start of the unreduced block that ends at hi: the last i < hi with a negligible e[i], plus one
-        int lo = 0;
-        for (int i0 = hi - 1; i0 >= 0; i0 -= 32) {
-            const int i = i0 - lane;
-            const bool small = i >= 0 && fabs(e[i]) <= eps * (fabs(dg[i]) + fabs(dg[i + 1]));
-            const unsigned bal = __ballot_sync(0xffffffffu, small);
-            if (bal) { lo = i0 - (__ffs(bal) - 1) + 1; break; }
-        }
-        if (lo == hi) {
-            __syncwarp();
-            if (lane == 0) e[hi - 1] = 0.0;
-            __syncwarp();
-            --hi;
-            continue;
-        }
-        ++guard;
-        // Wilkinson shift: eigenvalue of the trailing 2x2 block closer to dg[hi]
-        const double dd = 0.5 * (dg[hi - 1] - dg[hi]);
-        const double eh = e[hi - 1];
-        const double den = dd + copysign(sqrt(dd * dd + eh * eh), dd == 0.0 ? 1.0 : dd);
-        const double mu = dg[hi] - eh * eh / den;
-        double a = dg[lo], b = e[lo], zk = z[lo], x = a - mu, y = b;
-        for (int kk = lo; kk < hi; ++kk) {
-            const double cc = dg[kk + 1], zk1 = z[kk + 1], en = kk + 1 < hi ? e[kk + 1] : 0.0;
-            const double u = q & 1 ? y : x, p = u * u;
-            const double r2 = p + __shfl_xor_sync(0xffffffffu, p, 1);
-            const bool nz = r2 > 0.0;
-            const double ri = rsqrt(r2), v = nz ? u * ri : (q & 1 ? 0.0 : 1.0), o = __shfl_xor_sync(0xffffffffu, v, 1);
-            const double c = q & 1 ? o : v, s = q & 1 ? v : o;
-            const double t5 = fma(q == 0 ? c : q == 1 ? s : q == 2 ? c : 1.0, q == 0 ? c : q == 1 ? s : q == 2 ? s : cc,
-                                  q == 3 ? -a : 0.0);
-            const double c2 = from(t5, 0), s2 = from(t5, 1), cs = from(t5, 2), d = from(t5, 3);
-            const double t6 = fma(q == 0 ? cs : q == 1 ? 1.0 : c, q == 0 ? b : q == 1 ? c2 : q == 2 ? zk : zk1,
-                                  q == 1 ? -s2 : 0.0);
-            const double csb = from(t6, 0), cd = from(t6, 1);                // c s b, c^2 - s^2
-            // lane 0: c^2 a + c s b; 1: (c^2 - s^2) b; 2: new z[kk]; 3: the z that moves on
-            const double t7 = fma(q == 0 ? c2 : q == 1 ? cd : q == 2 ? s : -s, q == 0 ? a : q == 1 ? b : q == 2 ? zk1 : zk,
-                                  q == 0 ? csb : q == 1 ? 0.0 : t6);
-            // 0: + s^2 c; 1: x of the next rotation; 2: s^2 a - c s b; 3: y of the next
-            const double t8 = fma(q == 1 ? cs : q == 3 ? s : s2, q == 0 ? cc : q == 1 ? d : q == 2 ? a : en,
-                                  q == 2 ? -csb : q == 3 ? 0.0 : t7);
-            // 0: new dg[kk]; 2: - c s b once more; 3: the next off-diagonal
-            const double t9 = fma(q == 3 ? c : 1.0, q == 3 ? en : q == 2 ? -csb : csb, q == 3 ? 0.0 : t8);
-            const double ta = fma(q == 2 ? c2 : r2, q == 2 ? cc : ri, q == 2 ? t9 : 0.0);   // 2: the dg that moves on; 0: r
-            if (lane == 0) {
-                dg[kk] = t9;
-                if (kk > lo) e[kk - 1] = nz ? ta : 0.0;
-            }
-            if (lane == 2) z[kk] = t7;
-            zk = from(t7, 3);
-            x = from(t8, 1);
-            y = from(t8, 3);
-            b = from(t9, 3);
-            a = from(ta, 2);
-        }
-        __syncwarp();
-        if (lane == 0) {
-            dg[hi] = a;
-            e[hi - 1] = x;
-            z[hi] = zk;
-        }
-        __syncwarp();
-    }
-}
-
-// theta and tau of (sector, vector) blockIdx.x; dynamic shared memory: 3 x steps doubles (47 KB at
-// the most steps a run takes)
-__global__ void __launch_bounds__(32) k_ft_eig(FtParams F) {
+// ---- tridiagonal eigenvalues and first components -----------------------------------------
+// theta and tau of (sector, vector) blockIdx.x: the eigenvalues lambda_i of T and mu_i of T without its
+// first row and column, by bisection with Sturm counts (tridiag.cuh), one eigenvalue a lane, and
+//   tau_i = prod_j (lambda_i - mu_j) / prod_{j != i} (lambda_i - lambda_j)
+// (the residues of the first diagonal entry of the resolvent; Golub and Meurant, Matrices, Moments and
+// Quadrature).  Whatever the rounding of interlacing lambda and mu, they are those of some Jacobi
+// matrix close to T, so the tau are positive and sum to one also where ghosts lie an ulp apart.  All m
+// values are found at once, where the rotations of the implicit QR algorithm form one chain of
+// m^2 times 30 dependent binary64 instructions: N = 20, 672 matrices of 80 rows 9.5 -> 2.2 ms.
+// Eigenvalues are cut to the last bit of the norm: binary32 counts to 2^-18 of it, widened by 2^-19
+// for their rounding, then binary64.  lambda and mu in dynamic shared memory (2 x steps doubles).
+constexpr int FT_EIG_NT = 192;
+__global__ void __launch_bounds__(FT_EIG_NT) k_ft_eig(FtParams F) {
     extern __shared__ __align__(16) double ft_eig_sh[];
     const FtDev &d = F.d;
-    const int t = blockIdx.x, v = t % FT_W, lane = threadIdx.x;
+    const int t = blockIdx.x, v = t % FT_W, tid = threadIdx.x, lane = tid & 31;
     if ((F.exact_mask >> (t / FT_W)) & 1ull) return;   // filled by k_ft_exact
     const int m = (v < F.R) ? d.nsteps[t] : 0;
-    if (lane == 0) d.mlen[t] = m;
+    if (tid == 0) d.mlen[t] = m;
     if (m == 0) return;
-    double *dg = ft_eig_sh, *e = dg + F.steps, *z = e + F.steps;
+    double *lam = ft_eig_sh, *mu = lam + F.steps;
     const double *al = d.alpha + (size_t)t * F.steps, *be = d.beta + (size_t)t * F.steps;
-    double nrm = 0.0;
-    for (int i = lane; i < m; i += 32) nrm = fmax(nrm, fmax(fabs(al[i]), i + 1 < m ? fabs(be[i]) : 0.0));
-    for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
-    const int ex = nrm > 0.0 && nrm < 1e308 ? min(max(ilogb(nrm), -1000), 1000) : 0;
-    for (int i = lane; i < m; i += 32) {
-        dg[i] = ldexp(al[i], -ex);
-        e[i] = i + 1 < m ? ldexp(be[i], -ex) : 0.0;
+    double *theta = d.theta + (size_t)t * F.steps, *tau = d.tau + (size_t)t * F.steps;
+    bool bad = false;
+    for (int i = tid; i < m; i += FT_EIG_NT) bad |= !isfinite(al[i]) || (i + 1 < m && !isfinite(be[i]));
+    double g0, g1;
+    tri_gershgorin(m, al, be, &g0, &g1);
+    const double bound = fmax(fabs(g0), fabs(g1));
+    if (__syncthreads_or(bad) || !(bound <= 1.7e308)) {
+        for (int i = tid; i < m; i += FT_EIG_NT) theta[i] = tau[i] = __longlong_as_double(0x7ff8000000000000ll);
+        return;
     }
-    __syncwarp();
-    tri_ql_first(m, dg, e, z);
-    for (int i = lane; i < m; i += 32) {
-        d.theta[(size_t)t * F.steps + i] = ldexp(dg[i], ex);
-        d.tau[(size_t)t * F.steps + i] = z[i] * z[i];
+    if (m == 1 || bound == 0.0) {
+        for (int i = tid; i < m; i += FT_EIG_NT) { theta[i] = al[i]; tau[i] = i == 0 ? 1.0 : 0.0; }
+        return;
+    }
+    const int ex = min(max(ilogb(bound), -1000), 1000);
+    const double s = tri_pow2(-ex);                    // s T has a norm in [1, 2)
+    const double pad = 2.0 * 2.220446049250313e-16 * bound * s;
+    const int nw = (m + 31) / 32, nw1 = (m + 30) / 32; // warps' worth of lambda, of mu
+    for (int w = tid >> 5; w < nw + nw1; w += FT_EIG_NT / 32) {
+        const bool sub = w >= nw;
+        const int mm = m - (int)sub, e = (sub ? w - nw : w) * 32 + lane + 1;
+        const double *A = al + (int)sub, *B = be + (int)sub;
+        const int ec = min(e, mm);                     // idle lanes repeat the last eigenvalue
+        float fa = __double2float_rd(g0 * s - pad), fc = __double2float_ru(g1 * s + pad);
+        for (int it = 0; it < 21; ++it) {              // 4 2^-21 < 2^-18
+            const float x = 0.5f * (fa + fc);
+            if (tri_count<float>(mm, A, B, s, x) < ec) fa = x; else fc = x;
+        }
+        double a = (double)fa - 0x1p-19, c = (double)fc + 0x1p-19;
+        for (int it = 0; it < 60; ++it) {
+            const double x = 0.5 * (a + c);
+            const bool more = c - a > 0x1p-53 && x > a && x < c;
+            if (!__any_sync(0xffffffffu, more)) break;
+            if (tri_count<double>(mm, A, B, s, x) < ec) a = more ? x : a; else c = more ? x : c;
+        }
+        if (e <= mm) (sub ? mu : lam)[e - 1] = 0.5 * (a + c);
+    }
+    __syncthreads();
+    // strictly increasing lambda (T is unreduced) at least two units of the norm's last place apart,
+    // mu between its neighbours
+    bool close = false;
+    for (int i = tid; i + 1 < m; i += FT_EIG_NT) close |= lam[i + 1] - lam[i] < 0x1p-51;
+    if (__syncthreads_or(close) && tid == 0)
+        for (int i = 1; i < m; ++i) lam[i] = fmax(lam[i], lam[i - 1] + 0x1p-51);
+    __syncthreads();
+    for (int i = tid; i + 1 < m; i += FT_EIG_NT) mu[i] = fmin(fmax(mu[i], lam[i]), lam[i + 1]);
+    __syncthreads();
+    for (int i = tid; i < m; i += FT_EIG_NT) {
+        const double x = lam[i];
+        double w = 1.0;
+        for (int j0 = 0; j0 + 1 < m; j0 += 8) {        // eight factors to a division
+            double nu = 1.0, de = 1.0;
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+                const int j = j0 + jj;
+                if (j + 1 < m) {
+                    nu *= x - mu[j];
+                    de *= x - lam[j < i ? j : j + 1];
+                }
+            }
+            w *= nu / de;
+        }
+        theta[i] = x * tri_pow2(ex);
+        tau[i] = w;
     }
 }
 
@@ -1114,7 +1088,7 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
                       const double *J, int R, int steps, int n_t, FtSetup *S, std::vector<uint32_t> *items) {
     if (two_s != 1) return fail(HM_EINVAL, "ftlm_run supports s = 1/2 (two_s = 1)");
     if (R < 1 || R > FT_W) return fail(HM_EINVAL, "R must be in 1..%d", FT_W);
-    if (steps < 1 || steps > 2000) return fail(HM_EINVAL, "steps must be in 1..2000");   // k_ft_eig: 3 x steps doubles
+    if (steps < 1 || steps > 2000) return fail(HM_EINVAL, "steps must be in 1..2000");   // k_ft_eig: 2 x steps doubles
     if (n_t < 0 || n_t > 4096) return fail(HM_EINVAL, "n_t must be in 0..4096");
     const int K = ft_choose_K(n_sites);
     if (K < 0 || n_sites > 32) return fail(HM_EINVAL, "ftlm_run needs 10 <= n_sites <= 32");
@@ -1378,7 +1352,7 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
             const bool fork = S.F.nexact > 0;
             if (fork && ((e = cudaEventRecord(ev, cap)) != cudaSuccess || (e = cudaStreamWaitEvent(br, ev, 0)) != cudaSuccess))
                 rc = cuda_fail(e, "ftlm fork");
-            k_ft_eig<<<nst, 32, (size_t)3 * S.F.steps * 8, cap>>>(S.F);
+            k_ft_eig<<<nst, FT_EIG_NT, (size_t)2 * S.F.steps * 8, cap>>>(S.F);
             if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ft_eig");
             if (rc == HM_OK && fork) {
                 k_ft_exact<<<S.F.nexact, 256, 0, br>>>(S.F, S.bp, (const uint32_t *)(w + S.L.xcd),

@@ -1,5 +1,7 @@
 """GPU tests of the tridiagonal eigensolvers (csrc/tridiag.cuh, the Ritz values of lanczos_run, and
 the finite-temperature eigen-decomposition) at the edges of their 32-row chunks."""
+import math
+
 import numpy as np
 import pytest
 
@@ -71,3 +73,25 @@ def test_arnoldi_gram_schmidt_tiles(hm, n, two_m, steps):
         dense = torch.stack([hm.matvec(b, hm.bonds_of(inst), eye[k].contiguous()) for k in range(b.dim)])
         e0 = np.linalg.eigvalsh(dense.cpu().numpy())[0]
         assert abs(r.ritz[0] - e0) <= 1e-11 * abs(e0)
+
+
+@pytest.mark.parametrize("m", [3, 31, 32, 33, 64, 65, 96, 97, 130])
+def test_ftlm_quadrature_moments(hm, m):
+    """An m-step run and a 2-step run of the same vectors share alpha_0, beta_0 and alpha_1, so their moments
+    sum_j tau_j theta_j^k, k <= 3, agree: the weights of interlacing values add up to one but for 16 roundings
+    a factor, and the values lie within 10 eps of the norm of T's (bound: sum |J| 3/4).  Sectors of at most m
+    states are diagonalised instead, without FP32 vectors."""
+    inst = W.small_ring(12, -1.0, -0.3)
+    bonds = hm.bonds_of(inst)
+    two, run = (hm.ftlm_run(12, bonds, 2, k, 9, [1.0]) for k in (2, m))
+    nrm = 0.75 * np.abs(inst.J).sum()
+    for A in range(13):
+        for r in range(2):
+            n2, n = int(two.mlen[A, r]), int(run.mlen[A, r])
+            if n2 < 2 or n < 3 or math.comb(12, A) <= m:
+                continue
+            t2, t = two.theta[A, r, :n2], run.theta[A, r, :n]
+            assert (run.tau[A, r, :n] >= 0).all()
+            for k in range(4):
+                a, b = two.tau[A, r, :n2] @ t2**k, run.tau[A, r, :n] @ t**k
+                assert abs(a - b) <= (16 * n + 10 * k + 64) * np.finfo(float).eps * nrm**k, (A, r, k)
