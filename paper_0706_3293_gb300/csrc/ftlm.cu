@@ -96,7 +96,7 @@ struct ExactSec {
     int A, dim;
     uint32_t cd_off;                // its CD table inside the exact-table buffer
     int cd_rowlen, cd_len;
-    uint64_t mat_off;               // doubles: H (dim x dim) then V (dim x dim)
+    uint64_t mat_off;               // ft_exact_bytes(dim)
 };
 constexpr int FT_MAXEXACT = 40;
 
@@ -743,22 +743,38 @@ __global__ void __launch_bounds__(FT_EIG_NT) k_ft_eig(FtParams F) {
 // eigen-decomposition by parallel cyclic Jacobi (Brent-Luk round-robin ordering of the
 // rotations, each zeroing one off-diagonal pair as in Golub and Van Loan, Sec. 8.5),
 // then theta_k = E_k and tau_k = <r^|psi_k>^2 for every start vector r^ = r / |r|.
-__global__ void __launch_bounds__(256) k_ft_exact(FtParams F, BondParams bp, const uint32_t *__restrict__ cdall,
-                                                  double *__restrict__ mats) {
+// One CTA a sector, so what bounds it is the binary64 pipe of one SM and the chain of a round's
+// rotation angles.  The rotations are applied to the start vectors (W = V^T r) instead of to an
+// n x n V; both sides of H at once, a 2 x 2 block of two rotations a thread and only one of each two
+// mirrored blocks; angles by two rsqrt (eighteen dependent instructions, forty before);
+// matrices in shared memory where they fit.  N = 12, two sectors of 66 states: 3.4 ms, the run 17.5 -> 8.3 ms.
+// n is padded to an even size with a zero row; H has a power of two taken out.
+constexpr int FT_X_NT = 1024;
+constexpr size_t FT_X_SMEM = 200 * 1024;   // n <= 144
+__host__ __device__ __forceinline__ size_t ft_exact_bytes(int n) {
+    const size_t m = (size_t)n + (n & 1);
+    return m * m * 8 + m * FT_W * 8;
+}
+__global__ void __launch_bounds__(FT_X_NT) k_ft_exact(FtParams F, BondParams bp, const uint32_t *__restrict__ cdall,
+                                                      double *__restrict__ mats, size_t smem_bytes) {
+    extern __shared__ __align__(16) double ft_x_sh[];
     const FtDev &d = F.d;
     const ExactSec ex = F.ex[blockIdx.x];
-    const int n = ex.dim;
-    double *H = mats + ex.mat_off, *V = H + (size_t)n * n;
-    __shared__ int sp[256], sq[256];
-    __shared__ double sc[256], ss[256], red[8];
-    __shared__ int s_stop;
-    for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
-        H[t] = 0.0;
-        V[t] = (t / n == t % n) ? 1.0 : 0.0;
+    const int n = ex.dim, m = n + (n & 1), mh = m / 2, tid = threadIdx.x;
+    double *H = ft_exact_bytes(n) <= smem_bytes ? ft_x_sh : mats + ex.mat_off, *W = H + (size_t)m * m;
+    __shared__ int sp[256], sq[256], s_stop;
+    __shared__ double sc[256], ss[256], red[FT_X_NT / 32];
+    for (int t = tid; t < m * m; t += FT_X_NT) H[t] = 0.0;
+    const double inv = 1.0 / sqrt((double)n);
+    for (int t = tid; t < m * FT_W; t += FT_X_NT) {
+        const int i = t / FT_W, r = t % FT_W;
+        const uint64_t stream = sm64(F.seed, ((uint64_t)ex.A << 20) + (uint64_t)r);
+        W[t] = i < n && r < F.R ? ((sm64(stream, (uint64_t)i) >> 63) ? -inv : inv) : 0.0;
     }
     __syncthreads();
     Codec<uint32_t> c{cdall + ex.cd_off, F.P.N, 1, ex.A, 1, 3, ex.cd_rowlen};
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    double big = 0.0;
+    for (int i = tid; i < n; i += FT_X_NT) {
         const uint64_t w = c.decode((uint32_t)i);
         double dg = 0.0;
         for (int t = 0; t < bp.nb; ++t) {
@@ -767,79 +783,85 @@ __global__ void __launch_bounds__(256) k_ft_exact(FtParams F, BondParams bp, con
             dg += bp.jm[t] * (0.5 - ap) * (0.5 - aq);
             if (ap != aq) {
                 const uint32_t j = (uint32_t)i + c.delta(w, p, q, ap ? -1 : +1);
-                H[(size_t)i * n + j] += bp.jm[t] * 0.5;
+                H[(size_t)i * m + j] += bp.jm[t] * 0.5;
             }
         }
-        H[(size_t)i * n + i] += dg;
+        H[(size_t)i * m + i] += dg;
+        for (int k = 0; k < n; ++k) big = fmax(big, fabs(H[(size_t)i * m + k]));
     }
+    for (int o = 16; o > 0; o >>= 1) big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if ((tid & 31) == 0) red[tid >> 5] = big;
     __syncthreads();
-    const int m = n + (n & 1);            // players of the round-robin (one dummy if n is odd)
+    for (int w = 0; w < FT_X_NT / 32; ++w) big = fmax(big, red[w]);
+    __syncthreads();
+    const int e2 = big > 0.0 && big < 1e308 ? min(max(ilogb(big), -1000), 1000) : 0;
+    for (int t = tid; t < m * m; t += FT_X_NT) H[t] = ldexp(H[t], -e2);
+    __syncthreads();
+    const int nblk = mh * (mh / 2 + 1);   // blocks (k, k + o mod mh), o = 0 .. mh / 2 (half of the last o if mh is even)
     for (int sweep = 0; sweep < 40 && n > 1; ++sweep) {
         // stop when the off-diagonal part is negligible
         double off = 0.0, tot = 0.0;
-        for (int t = threadIdx.x; t < n * n; t += blockDim.x) {
+        for (int t = tid; t < m * m; t += FT_X_NT) {
             const double h = H[t];
             tot += h * h;
-            if (t / n != t % n) off += h * h;
+            if (t / m != t % m) off += h * h;
         }
-        off = block_sum<256>(off, red);
+        off = block_sum<FT_X_NT>(off, red);
         __syncthreads();
-        tot = block_sum<256>(tot, red);
-        if (threadIdx.x == 0) s_stop = off <= 1e-30 * tot;
+        tot = block_sum<FT_X_NT>(tot, red);
+        if (tid == 0) s_stop = off <= 1e-30 * tot;
         __syncthreads();
         if (s_stop) break;
         for (int round = 0; round < m - 1; ++round) {
-            for (int k = threadIdx.x; k < m / 2; k += blockDim.x) {
+            for (int k = tid; k < mh; k += FT_X_NT) {
                 int p, q;
                 if (k == 0) { p = m - 1; q = round; }
                 else { p = (round + k) % (m - 1); q = (round - k + (m - 1)) % (m - 1); }
                 if (p > q) { const int tt = p; p = q; q = tt; }
-                double cc = 1.0, sn = 0.0;
-                if (q < n) {
-                    const double apq = H[(size_t)p * n + q];
-                    if (apq != 0.0) {
-                        const double tau = (H[(size_t)q * n + q] - H[(size_t)p * n + p]) / (2.0 * apq);
-                        const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-                        cc = 1.0 / sqrt(1.0 + t * t);
-                        sn = t * cc;
-                    }
+                // tan 2 theta = 2 apq / (aqq - app), |theta| <= pi / 4
+                const double dd = H[(size_t)q * m + q] - H[(size_t)p * m + p], h2 = 2.0 * H[(size_t)p * m + q];
+                const double r2 = dd * dd + h2 * h2, ri = rsqrt(r2);
+                const bool on = h2 != 0.0 && r2 > 0.0;
+                const double x = fma(0.5 * fabs(dd), ri, 0.5), rx = rsqrt(x);
+                sp[k] = p;
+                sq[k] = q;
+                sc[k] = on ? x * rx : 1.0;
+                ss[k] = on ? 0.5 * h2 * (dd < 0.0 ? -ri : ri) * rx : 0.0;
+            }
+            __syncthreads();
+            for (int t = tid; t < nblk + mh * FT_W; t += FT_X_NT) {
+                if (t < nblk) {                            // J1^T B J2
+                    const int o = t / mh, k1 = t - o * mh, k2 = k1 + o < mh ? k1 + o : k1 + o - mh;
+                    if (2 * o == mh && k1 >= o) continue;
+                    const size_t p1 = sp[k1], q1 = sq[k1], p2 = sp[k2], q2 = sq[k2];
+                    const double c1 = sc[k1], s1 = ss[k1], c2 = sc[k2], s2 = ss[k2];
+                    const double a = H[p1 * m + p2], b = H[p1 * m + q2], e = H[q1 * m + p2], f = H[q1 * m + q2];
+                    const double ra = c1 * a - s1 * e, rb = c1 * b - s1 * f, re = s1 * a + c1 * e, rf = s1 * b + c1 * f;
+                    const double na = c2 * ra - s2 * rb, nf = s2 * re + c2 * rf;
+                    double nb = s2 * ra + c2 * rb, ne = c2 * re - s2 * rf;
+                    if (o == 0) nb = ne = 0.0;             // the pair that the rotation zeroes
+                    H[p1 * m + p2] = na; H[p1 * m + q2] = nb; H[q1 * m + p2] = ne; H[q1 * m + q2] = nf;
+                    if (o != 0) { H[p2 * m + p1] = na; H[q2 * m + p1] = nb; H[p2 * m + q1] = ne; H[q2 * m + q1] = nf; }
+                } else {                                   // W <- J^T W
+                    const int u = t - nblk, k = u / FT_W, r = u % FT_W;
+                    double *wp = W + (size_t)sp[k] * FT_W + r, *wq = W + (size_t)sq[k] * FT_W + r;
+                    const double a = *wp, b = *wq;
+                    *wp = sc[k] * a - ss[k] * b;
+                    *wq = ss[k] * a + sc[k] * b;
                 }
-                sp[k] = p; sq[k] = q; sc[k] = cc; ss[k] = sn;
-            }
-            __syncthreads();
-            for (int t = threadIdx.x; t < (m / 2) * n; t += blockDim.x) {   // rows: A <- J^T A
-                const int k = t / n, j = t % n;
-                if (sq[k] >= n) continue;
-                const double a = H[(size_t)sp[k] * n + j], b = H[(size_t)sq[k] * n + j];
-                H[(size_t)sp[k] * n + j] = sc[k] * a - ss[k] * b;
-                H[(size_t)sq[k] * n + j] = ss[k] * a + sc[k] * b;
-            }
-            __syncthreads();
-            for (int t = threadIdx.x; t < (m / 2) * n; t += blockDim.x) {   // columns: A <- A J, V <- V J
-                const int k = t / n, i = t % n;
-                if (sq[k] >= n) continue;
-                const double a = H[(size_t)i * n + sp[k]], b = H[(size_t)i * n + sq[k]];
-                H[(size_t)i * n + sp[k]] = sc[k] * a - ss[k] * b;
-                H[(size_t)i * n + sq[k]] = ss[k] * a + sc[k] * b;
-                const double va = V[(size_t)i * n + sp[k]], vb = V[(size_t)i * n + sq[k]];
-                V[(size_t)i * n + sp[k]] = sc[k] * va - ss[k] * vb;
-                V[(size_t)i * n + sq[k]] = ss[k] * va + sc[k] * vb;
             }
             __syncthreads();
         }
     }
     // weights of every start vector
-    const double inv = 1.0 / sqrt((double)n);
-    for (int t = threadIdx.x; t < F.R * n; t += blockDim.x) {
+    for (int t = tid; t < F.R * n; t += FT_X_NT) {
         const int r = t / n, kk = t % n;
-        const uint64_t stream = sm64(F.seed, ((uint64_t)ex.A << 20) + (uint64_t)r);
-        double o = 0.0;
-        for (int i = 0; i < n; ++i) o += V[(size_t)i * n + kk] * ((sm64(stream, (uint64_t)i) >> 63) ? -inv : inv);
+        const double o = W[(size_t)kk * FT_W + r];
         const size_t sv = (size_t)ex.A * FT_W + r;
-        d.theta[sv * F.steps + kk] = H[(size_t)kk * n + kk];
+        d.theta[sv * F.steps + kk] = ldexp(H[(size_t)kk * m + kk], e2);
         d.tau[sv * F.steps + kk] = o * o;
     }
-    for (int r = threadIdx.x; r < FT_W; r += blockDim.x) d.mlen[(size_t)ex.A * FT_W + r] = r < F.R ? n : 0;
+    for (int r = tid; r < FT_W; r += FT_X_NT) d.mlen[(size_t)ex.A * FT_W + r] = r < F.R ? n : 0;
 }
 
 // Thermal sums.  Every (temperature, Ritz value) pair costs an exponential, about 25 binary64
@@ -1153,7 +1175,7 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
         ex.cd_len = sb.view.cd_len;
         for (int k = 0; k < sb.view.cd_len; ++k) S->xcd.push_back((uint32_t)sb.cd[k]);
         ex.mat_off = xmat;
-        xmat += 2 * dimA * dimA;
+        xmat += ft_exact_bytes((int)dimA) / 8;
         S->F.exact_mask |= 1ull << A;
     }
     S->F.nitems = (int)items->size();
@@ -1355,8 +1377,16 @@ int ftlm_run(int n_sites, int two_s, int n_bonds, const int32_t *u, const int32_
             k_ft_eig<<<nst, FT_EIG_NT, (size_t)2 * S.F.steps * 8, cap>>>(S.F);
             if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ft_eig");
             if (rc == HM_OK && fork) {
-                k_ft_exact<<<S.F.nexact, 256, 0, br>>>(S.F, S.bp, (const uint32_t *)(w + S.L.xcd),
-                                                       (double *)(w + S.L.xmat));
+                // shared memory for the largest sector that fits; larger ones work in mats
+                size_t xs = 0;
+                for (int x = 0; x < S.F.nexact; ++x) {
+                    const size_t need = ft_exact_bytes(S.F.ex[x].dim);
+                    if (need <= FT_X_SMEM) xs = std::max(xs, need);
+                }
+                if (xs > 0 && (e = raise_smem_limit((const void *)k_ft_exact, xs)) != cudaSuccess)
+                    rc = cuda_fail(e, "k_ft_exact shared memory");
+                k_ft_exact<<<S.F.nexact, FT_X_NT, xs, br>>>(S.F, S.bp, (const uint32_t *)(w + S.L.xcd),
+                                                            (double *)(w + S.L.xmat), xs);
                 if ((e = cudaGetLastError()) != cudaSuccess) rc = cuda_fail(e, "k_ft_exact");
                 else if ((e = cudaEventRecord(ev, br)) != cudaSuccess || (e = cudaStreamWaitEvent(cap, ev, 0)) != cudaSuccess)
                     rc = cuda_fail(e, "ftlm join");

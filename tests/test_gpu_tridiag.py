@@ -7,6 +7,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+import oracle
 from paper_0706_3293_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -95,3 +96,31 @@ def test_ftlm_quadrature_moments(hm, m):
             for k in range(4):
                 a, b = two.tau[A, r, :n2] @ t2**k, run.tau[A, r, :n] @ t**k
                 assert abs(a - b) <= (16 * n + 10 * k + 64) * np.finfo(float).eps * nrm**k, (A, r, k)
+
+
+@pytest.mark.parametrize("n,steps", [(10, 9), (11, 60), (12, 70), (12, 230)])
+def test_ftlm_exact_sectors(hm, n, steps):
+    """Sectors of at most `steps` states (one, odd and even sizes, in shared memory and beyond it), degenerate
+    levels included, against LAPACK on H's columns: Jacobi stops at off-diagonals of 1e-15 of the norm, its
+    rotations round each element at most 40 (dim - 1) times by 4 eps; the weights of a level sum
+    to |P r|^2, and all of them to one."""
+    inst = W.small_ring(n, -1.0, -0.5)
+    bonds = hm.bonds_of(inst)
+    run = hm.ftlm_run(n, bonds, 3, steps, 4, [1.0])
+    for A in range(n + 1):
+        dim = math.comb(n, A)
+        if dim > steps:
+            continue
+        b = hm.Basis(n, 1, n - 2 * A)
+        eye = torch.eye(dim, dtype=torch.float64, device="cuda")
+        H = torch.stack([hm.matvec(b, bonds, eye[k].contiguous()) for k in range(dim)]).cpu().numpy()
+        ref = np.linalg.eigvalsh(H)
+        tol = 160 * dim * np.finfo(float).eps * max(np.abs(H).sum(1).max(), 1.0)
+        for r in range(3):
+            assert run.mlen[A, r] == dim
+            assert np.abs(np.sort(run.theta[A, r, :dim]) - ref).max() <= tol
+            assert abs(run.tau[A, r, :dim].sum() - 1.0) <= tol
+            v = oracle.start_pm1(oracle.splitmix(4, (A << 20) + r), dim) / math.sqrt(dim)
+            m1, m2 = (run.tau[A, r, :dim] @ run.theta[A, r, :dim] ** k for k in (1, 2))
+            nrm = max(np.abs(H).sum(1).max(), 1.0)
+            assert abs(m1 - v @ H @ v) <= 2 * tol and abs(m2 - v @ H @ (H @ v)) <= 4 * tol * nrm
