@@ -9,7 +9,7 @@
 #include <tuple>
 #include <type_traits>
 
-#include "blk.cuh"
+#include "blk_hops.cuh"
 #include "blk_sweep.cuh"
 
 namespace hm {
@@ -772,18 +772,27 @@ const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int 
     return jit_mv_kernel(P, dtype, &k) == 0 ? "k_blk_matvec_jit" : nullptr;
 }
 
+// several vectors at once (blk_multi.cu)
+int blk_hop_table(hm_basis *b, const BlkParams &P, const HopTab &H, bool build, const uint16_t **table);
+int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table, const double *gd, const void *x, void *y,
+                     int dtype, int nvec, cudaStream_t st);
+
 // The plan of y = H x for one bond list.  Planning takes 20 to 60 us of host time (groups, table
 // layout, the source text that names a run-time compiled kernel), more than the product itself
 // below N = 22, so a basis keeps its last BLK_MV_PLANS of them, found by the values of the bonds
 // (never by an address), the type and the environment knobs that enter.
 struct BlkMvPlan {
-    int nb, dtype, K, env;
+    int nb, dtype, K, env, multi;
     unsigned char p[HM_BLK_MAXB], q[HM_BLK_MAXB];
     double jm[HM_BLK_MAXB];
     BlkParams P;
     const void *kern;
     size_t smem;
     int blocks;
+    // multi: several vectors (blk_multi.cu)
+    HopTab hop;
+    const uint16_t *hops;
+    double gd[HM_BLK_MAXC];          // -J_c / 4
 };
 constexpr unsigned BLK_MV_PLANS = 8;
 
@@ -794,14 +803,14 @@ static int blk_env() {
 }
 
 // 0 and the plan, or 1 when the block path does not apply
-static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, cudaStream_t st,
+static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi, cudaStream_t st,
                        std::shared_ptr<const BlkMvPlan> *out) {
     if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB) return 1;
     const int K = blk_K(b, false), env = blk_env(), nb = bp.nb;
     {
         std::lock_guard<std::mutex> lk(b->tab_mu);
         for (const auto &m : b->mv_plans)
-            if (m->nb == nb && m->dtype == dtype && m->K == K && m->env == env && !memcmp(m->p, bp.p, nb) &&
+            if (m->nb == nb && m->dtype == dtype && m->K == K && m->env == env && m->multi == (int)multi && !memcmp(m->p, bp.p, nb) &&
                 !memcmp(m->q, bp.q, nb) && !memcmp(m->jm, bp.jm, nb * sizeof(double))) {
                 *out = m;
                 return 0;
@@ -812,8 +821,10 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, cudaStream_
     const int rc = blk_plan(b, bp, K, &P);
     if (rc != 0) return rc;
     const int es = dtype == HM_F64 ? 8 : 4;
+    m->multi = multi;
     m->smem = blk_row_smem_bytes(P, es, BLK_XPAD);
-    if (!P.rows_ok || m->smem > 200 * 1024) return 1;
+    // several vectors: class plans; a plain basis only, as the general rows
+    if (multi ? P.perbond || P.par : !P.rows_ok || m->smem > 200 * 1024) return 1;
     // target tables: built on the first product of a layout, but for class plans neither inside a
     // stream capture (no allocation there) nor without end on a basis that sees many bond lists; the
     // generic rows then serve, with the same result (FP64: the same exact sums)
@@ -824,24 +835,37 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, cudaStream_
         std::lock_guard<std::mutex> lk(b->tab_mu);
         build = cs == cudaStreamCaptureStatusNone && b->blk_ttabs.size() < 32;
     }
-    const int trc = blk_target_table(b, &P, es, build);
+    if (multi) {
+        m->hop = hop_layout(P);
+        HM_TRY(blk_hop_table(b, P, m->hop, build, &m->hops));
+        if (!m->hops) return 1;
+        for (int t = 0, c = 0; t < nb; ++t) {                // class c: the c-th distinct coupling
+            bool seen = false;
+            for (int i = 0; i < t && !seen; ++i) seen = bp.jm[i] == bp.jm[t];
+            if (!seen) m->gd[c++] = bp.jm[t] / 4.0;
+        }
+    }
+    const int trc = multi ? 1 : blk_target_table(b, &P, es, build);
     if (trc < 0) return trc;
-    if (P.perbond) {
+    if (multi) {
+    } else if (P.perbond) {
         if (jit_mv_kernel(P, dtype, &m->kern) != 0) return 1;
     } else if (dtype == HM_F64) {
         m->kern = P.tt ? blk_mv_kernel<double, true>(P.nc) : blk_mv_kernel<double, false>(P.nc);
     } else {
         m->kern = P.tt ? blk_mv_kernel<float, true>(P.nc) : blk_mv_kernel<float, false>(P.nc);
     }
-    HM_CUDA(raise_smem_limit(m->kern, m->smem));
-    int per = 0;
-    HM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, m->kern, BLK_NT, m->smem));
-    m->blocks = std::min<int>(sm_count() * std::max(per, 1), 1 << P.H);
+    if (!multi) {
+        HM_CUDA(raise_smem_limit(m->kern, m->smem));
+        int per = 0;
+        HM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, m->kern, BLK_NT, m->smem));
+        m->blocks = std::min<int>(sm_count() * std::max(per, 1), 1 << P.H);
+    }
     m->nb = nb; m->dtype = dtype; m->K = K; m->env = env;
     memcpy(m->p, bp.p, nb);
     memcpy(m->q, bp.q, nb);
     memcpy(m->jm, bp.jm, nb * sizeof(double));
-    if (P.perbond || P.tt || cs == cudaStreamCaptureStatusNone) {   // a capture's plan without its table is not kept
+    if (P.perbond || P.tt || multi || cs == cudaStreamCaptureStatusNone) {   // a capture's plan without its table is not kept
         std::lock_guard<std::mutex> lk(b->tab_mu);
         if (b->mv_plans.size() < BLK_MV_PLANS) b->mv_plans.push_back(m);
         else b->mv_plans[b->mv_next++ % BLK_MV_PLANS] = m;
@@ -853,10 +877,10 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, cudaStream_
 // returns 1 when the block path does not apply (caller falls back to the row kernel)
 int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dtype, int nvec,
                cudaStream_t st) {
-    if (nvec != 1) return 1;
     std::shared_ptr<const BlkMvPlan> m;
-    const int rc = blk_mv_plan(b, bp, dtype, st, &m);
+    const int rc = blk_mv_plan(b, bp, dtype, nvec > 1, st, &m);
     if (rc != 0) return rc;
+    if (nvec > 1) return blk_multi_launch(m->P, m->hop, m->hops, m->gd, x, y, dtype, nvec, st);
     int *Ed = nullptr, nE = 0;
     if (dtype == HM_F64) HM_TRY(launch_max_exp(b, x, m->P.dim, &Ed, &nE, st));
     void *args[] = {(void *)&m->P, (void *)&x, (void *)&y, (void *)&Ed, (void *)&nE};

@@ -29,7 +29,7 @@
 #include <map>
 #include <vector>
 
-#include "blk.cuh"
+#include "blk_hops.cuh"
 #include "tridiag.cuh"
 
 namespace hm {
@@ -82,7 +82,7 @@ struct FtDev {
     const uint32_t *items;          // (A << 16) | h, sorted by A
     const uint64_t *rowoff;         // first global row of sector A
     const uint32_t *secdim;         // D(N, A)
-    uint16_t *hops;                 // [2^K][hop_stride]: targets of each low word (k_ft_hops)
+    uint16_t *hops;                 // [2^K][hop.stride]: targets of each low word (k_ft_hops)
     float *q0, *q1;                 // [rows][FT_W]
     double *theta, *tau;            // [(s * FT_W + v) * steps + j]
     int *mlen;                      // Krylov length per (s, v)
@@ -109,11 +109,7 @@ struct FtParams {
     uint64_t seed;
     unsigned long long barrier_ns;  // a grid barrier gives up after this long (default 5 s)
     uint64_t exact_mask;            // bit A set: sector A is diagonalised exactly
-    // a row of d.hops (16-bit entries): the number of low targets of each class as four bytes and an entry
-    // for each of the first six low ends of cross bonds, then from hop_seg[c] on the low targets
-    // of class c, then from hop_x on the entries of the other low ends
-    int hop_stride, hop_seg[HM_BLK_MAXC], hop_x, hop_nx;
-    uint8_t hop_xp[HM_BLK_MAXB], hop_xi[HM_BLK_MAXB];   // the low ends; that of each cross bond
+    HopTab hop;
     int nexact;
     ExactSec ex[FT_MAXEXACT];
 };
@@ -212,82 +208,12 @@ __device__ __forceinline__ void ft_warp_flush(ef::df *p, double *part, uint32_t 
     }
 }
 
-constexpr int FT_XHEAD = 6;         // cross entries in the first 16 bytes of a row of the target table
-
-// Targets of the low words, once per run: thread g takes the low word at position g of the word list
-// (class k of its ones, rank r) and writes the ranks its low exchanges reach, by class and in the
-// order of the bond groups, each class's run padded to a multiple of four with r itself, and the rank of
-// l ^ 2^p for each low end p of a cross bond.  With these rows a product's target takes a
-// shift, an address and the gather; finding it took the masks, a bit scan, the xor and two
-// table lookups, which all 32 lanes did for the same few rows.  Product phase of the N = 20 run
-// 382 -> 346 us a step, where the gathers' way through L1 and L2 bounds it, not instructions.
+// The target table (blk_hops.cuh), once per run.  With the targets found by all 32 lanes for the same few
+// rows, a row took 429 warp instructions and the product was issue-bound.  Product phase of the
+// N = 20 run 382 -> 346 us a step, where the gathers' way through L1 and L2 bounds it, not instructions.
 __global__ void k_ft_hops(FtParams F) {
-    const BlkParams &P = F.P;
     const uint32_t g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= 1u << P.K) return;
-    BlkTabs tb;
-    tb.U = (const uint16_t *)((const unsigned char *)P.tab + P.off_U);
-    tb.R0 = (const uint8_t *)P.tab + P.off_R0;
-    tb.C = (const uint32_t *)((const unsigned char *)P.tab + P.off_C);
-    const uint32_t l = P.lw[g];
-    const int k = __popc(l);
-    const uint32_t r = g - (uint32_t)P.lwoff[k];
-    uint16_t *T = F.d.hops + (size_t)g * F.hop_stride;
-    for (int c = 0; c < HM_BLK_MAXC; ++c) {
-        int m = 0;
-        if (c < P.nc) {
-            uint16_t *t = T + F.hop_seg[c];
-            blk_low_hops(P, tb, c, l, r, tb.U + k * P.nb1, [&](uint32_t r2) { t[m++] = (uint16_t)r2; });
-            for (int i = m; i & 3; ++i) t[i] = (uint16_t)r;
-        }
-        ((uint8_t *)T)[c] = (uint8_t)m;
-    }
-    for (int i = 0; i < F.hop_nx; ++i) {
-        const uint32_t l2 = l ^ (1u << F.hop_xp[i]);
-        T[i < FT_XHEAD ? 2 + i : F.hop_x + i - FT_XHEAD] = (uint16_t)rank_low(P, tb, l2, __popc(l2));
-    }
-}
-
-// A warp's exchange lists of the block it works on
-struct FtHops {
-    int4 *x;              // [ncb] cross bond: {target block's rows less own, xor | test mask << 16, low end, 0}
-    int *hcd;             // [nhb] offsets (target row - own row) of the valid high exchanges
-    int *hcs;             // [HM_BLK_MAXC + 1] class c owns hcd[hcs[c] .. hcs[c+1])
-};
-
-// Hop lists of block (h, k) for one warp: the valid high exchanges as row offsets,
-// compacted by class (lane e tests bonds e and e + 32, ballots give the positions), and
-// the targets of the cross exchanges.  The caller syncs the warp before and after.
-__device__ __forceinline__ void ft_warp_setup(const FtParams &F, const BlkTabs &tb, uint32_t h, int k, uint32_t off,
-                                              const FtHops &sh, int lane) {
-    const BlkParams &P = F.P;
-    int val[2] = {0, 0}, hoff[2] = {0, 0};
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int e = lane + 32 * half;
-        if (e < P.nhb) {
-            const int p = P.hb_p[e], q = P.hb_q[e];
-            val[half] = (((h >> p) ^ (h >> q)) & 1u) ? 1 : 0;
-            if (val[half]) hoff[half] = (int)(blk_off(P, tb, h ^ ((1u << p) | (1u << q)), k) - off);
-        }
-    }
-    const uint32_t b0 = __ballot_sync(0xffffffffu, val[0]), b1 = __ballot_sync(0xffffffffu, val[1]);
-    const uint32_t below = (1u << lane) - 1u;
-    if (val[0]) sh.hcd[__popc(b0 & below)] = hoff[0];
-    if (val[1]) sh.hcd[__popc(b0) + __popc(b1 & below)] = hoff[1];
-    if (lane <= HM_BLK_MAXC) {                    // class c starts at the valid ones before hb_start[c]
-        const int e = P.hb_start[lane];
-        sh.hcs[lane] = e >= 32 ? __popc(b0) + __popc(e >= 64 ? b1 : b1 & ((1u << (e - 32)) - 1u))
-                               : __popc(b0 & ((1u << e) - 1u));
-    }
-    for (int e = lane; e < P.ncb; e += 32) {
-        const int p = P.cb_p[e], q = P.cb_q[e];
-        const uint32_t bq = (h >> q) & 1u;
-        const int k2 = k + (bq ? 1 : -1);
-        const bool ok = k2 >= 0 && k2 <= P.K;     // else the test mask is empty
-        sh.x[e] = make_int4(ok ? (int)(blk_off(P, tb, h ^ (1u << q), k2) - off) : 0,
-                            (int)((bq << p) | (ok ? 1u << (p + 16) : 0u)), F.hop_xi[e], 0);
-    }
+    if (g < 1u << F.P.K) hop_fill(F.P, F.hop, g, F.d.hops);
 }
 
 // Per (sector, vector) sums of the CTA partials partc[s][b][v] over the CTAs b in [lo(s), hi(s))
@@ -384,10 +310,7 @@ __device__ __forceinline__ int ft_sector_of(const FtDev &d, int nsec, uint64_t g
 }
 
 // per-warp shared slice: hop lists | sigma, gamma of the current sector | alpha sigma
-__host__ __device__ __forceinline__ size_t ft_hops_bytes(const BlkParams &P) {
-    return al16f((size_t)P.ncb * 16 + (size_t)(P.nhb + HM_BLK_MAXC + 1) * 4);
-}
-__host__ __device__ __forceinline__ size_t ft_warp_bytes(const BlkParams &P) { return ft_hops_bytes(P) + FT_W * 4 * 3; }
+__host__ __device__ __forceinline__ size_t ft_warp_bytes(const BlkParams &P) { return hops_bytes(P) + FT_W * 4 * 3; }
 
 // ---- the persistent kernel ---------------------------------------------------------------
 // Every warp owns the global rows [g0, g1) of its FtRange (rows of all sectors in order,
@@ -403,11 +326,8 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
     const BlkTabs tb = stage_blk_tables(P, smem);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char *ws = smem + al16f(P.tab_bytes) + warp * ft_warp_bytes(P);
-    FtHops sh;
-    sh.x = (int4 *)ws;
-    sh.hcd = (int *)(sh.x + P.ncb);
-    sh.hcs = sh.hcd + P.nhb;
-    float *sgw = (float *)(ws + ft_hops_bytes(P));  // [sigma | gamma | alpha sigma][FT_W]
+    const Hops sh = hops_carve(P, ws);
+    float *sgw = (float *)(ws + hops_bytes(P));     // [sigma | gamma | alpha sigma][FT_W]
     double *red = (double *)(smem + al16f(P.tab_bytes) + (FT_NT / 32) * ft_warp_bytes(P));
     constexpr int LPR = 32 / VT;                   // lanes per row
     const int grp = lane / LPR, li = lane % LPR;   // row group in the warp, lane in row
@@ -460,12 +380,12 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                     const uint32_t ra = ig0 < g0 ? (uint32_t)(g0 - ig0) : 0u;
                     const uint32_t rb = ig0 + n > g1 ? (uint32_t)(g1 - ig0) : n;
                     __syncwarp();                  // the previous block's lists are read no more
-                    ft_warp_setup(F, tb, h, k, off, sh, lane);
+                    hops_setup(P, F.hop, tb, h, k, off, sh, lane);
                     __syncwarp();
                     const float *Xb = qc + ig0 * FT_W + v0;   // the block's rows, this lane's vectors
                     for (uint32_t r = ra + grp; r < rb; r += VT) {
                         const uint32_t g = (uint32_t)P.lwoff[k] + r, l = __ldg(P.lw + g);
-                        const uint16_t *T = d.hops + (size_t)g * F.hop_stride;
+                        const uint16_t *T = d.hops + (size_t)g * F.hop.stride;
                         const uint4 hd = __ldg((const uint4 *)T);   // counts, cross entries
                         float acc[NC][VT];
                         int cnt[NC];
@@ -477,7 +397,7 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                             // low exchanges: four gathers in flight, added in the order of the list; the
                             // padding reads the row itself and is not added
                             int mc = (int)((hd.x >> (8 * cl)) & 0xFFu);
-                            const uint16_t *t = T + F.hop_seg[cl];
+                            const uint16_t *t = T + F.hop.seg[cl];
                             for (int e = 0; e < mc; e += 4) {
                                 const uint2 w = __ldg((const uint2 *)(t + e));
                                 float x0[VT], x1[VT], x2[VT], x3[VT];
@@ -492,12 +412,10 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                             }
                             for (int e = P.cb_start[cl]; e < P.cb_start[cl + 1]; ++e) {
                                 const int4 x = sh.x[e];
-                                const bool on = ((l ^ (uint32_t)x.y) & ((uint32_t)x.y >> 16)) != 0u;
-                                const uint32_t xw = x.z < 2 ? hd.y : x.z < 4 ? hd.z : hd.w;
-                                int t2 = (int)((x.z & 1) ? xw >> 16 : xw & 0xFFFFu);
-                                if (x.z >= FT_XHEAD) t2 = (int)__ldg(T + F.hop_x + x.z - FT_XHEAD);
+                                int t2;
+                                const bool on = hop_cross(F.hop, x, hd, T, l, &t2);
                                 float xv[VT];
-                                ft_ld<VT>(Xb + (int64_t)(on ? x.x + t2 : (int)r) * FT_W, xv);
+                                ft_ld<VT>(Xb + (int64_t)(on ? t2 : (int)r) * FT_W, xv);
                                 ft_add<VT>(ac, xv, on);
                                 mc += (int)on;
                             }
@@ -1126,26 +1044,7 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
     uint64_t mb = 1;
     for (int i = 0; i < K / 2; ++i) mb = mb * (K - i) / (i + 1);
     S->F.P.max_block = (int)mb;
-    // rows of the target table
-    {
-        FtParams &F = S->F;
-        const BlkParams &P = F.P;
-        int o = 2 + FT_XHEAD;
-        for (int c = 0; c < P.nc; ++c) {
-            int m = 0;
-            for (int g = P.lg_cs[3 * c]; g < P.lg_cs[3 * c + 3]; ++g) m += __builtin_popcount(P.lg_mask[g]);
-            F.hop_seg[c] = o;
-            o += (m + 3) & ~3;
-        }
-        F.hop_x = o;
-        for (int e = 0; e < P.ncb; ++e) {
-            int i = 0;
-            while (i < F.hop_nx && F.hop_xp[i] != P.cb_p[e]) ++i;
-            if (i == F.hop_nx) F.hop_xp[F.hop_nx++] = P.cb_p[e];
-            F.hop_xi[e] = (uint8_t)i;
-        }
-        F.hop_stride = (o + std::max(0, F.hop_nx - FT_XHEAD) + 7) & ~7;
-    }
+    S->F.hop = hop_layout(S->F.P);
     const int nsec = n_sites + 1;
     items->clear();
     const int H = n_sites - K;
@@ -1201,7 +1100,7 @@ static int ft_prepare(int n_sites, int two_s, int n_bonds, const int32_t *u, con
               &S->ck_cs);
     S->F.nchunks = (uint32_t)S->ck_it0.size();
     S->L = ft_layout(n_sites, nsec, R, steps, S->F.nitems, S->nctas, n_t, S->xcd.size(), (size_t)xmat,
-                     S->F.nchunks, (size_t)S->F.hop_stride << K);
+                     S->F.nchunks, (size_t)S->F.hop.stride << K);
     return HM_OK;
 }
 
