@@ -225,14 +225,15 @@ int lanczos_kernel_name(const hm_lanczos *run, char *name, int cap);
  * (s = 1/2 block kernel, up to 4 distinct couplings), "k_blk_matvec_jit" (block kernel
  * compiled at run time for a bond list with more distinct couplings), "k_s1_mv_jit" /
  * "k_s1_mv" (s = 1 block kernel compiled for the bond list / generic; FP32, one vector) or
- * "k_matvec" (general row kernel).  name: host buffer of cap bytes. */
+ * "k_matvec" (every other form: general rows, several vectors).  name: host buffer of cap bytes. */
 int matvec_kernel_name(const hm_basis *basis, int n_bonds, const int32_t *u, const int32_t *v,
                        const double *J, int dtype, int nvec, char *name, int cap);
 
-/* A whole run: steps steps captured in one CUDA graph and launched once, then the
- * n_ritz lowest eigenvalues of T (Sturm bisection on the device).  Host outputs:
- * alpha[steps], beta[steps], *steps_done, ritz[n_ritz].  Returns HM_OK or
- * HM_BREAKDOWN. */
+/* A whole run: steps steps captured in one CUDA graph and launched once (FP64 runs of s = 1/2
+ * sectors small enough to stay on the chip: one cooperative kernel for all steps, whose grid
+ * barriers wait at most 5 s, then the call returns HM_ETIMEOUT), then the n_ritz lowest
+ * eigenvalues of T (Sturm counts on the device).  Host outputs: alpha[steps], beta[steps],
+ * *steps_done, ritz[n_ritz].  Returns HM_OK or HM_BREAKDOWN. */
 int lanczos_run(const hm_basis *basis, int n_bonds, const int32_t *u, const int32_t *v,
                 const double *J, const void *v0, uint64_t seed, int steps, int dtype,
                 void *work, size_t work_bytes, double *alpha, double *beta,
@@ -328,7 +329,8 @@ int sym_eigenvalues(int n, const double *a, double *ev);
  * eigenvectors, the limit the Lanczos quadrature reaches; its mlen = D_A).  Everything
  * runs in one CUDA graph: start vectors, one
  * cooperative persistent kernel for all steps (grid barriers wait at most 5 s, then the
- * call returns HM_ETIMEOUT), and the tridiagonal eigensolves on the device.  Outputs (host):
+ * call returns HM_ETIMEOUT), and the eigenvalues and weights of each T on the device
+ * (theta ascending).  Outputs (host):
  * e_ref = lowest Ritz value; for each temperature T = temps[i]:
  *   Z[i] = sum_A (D_A/R) sum_r sum_j tau_j e^{-(theta_j - e_ref)/T}  (partition function
  *          divided by e^{-e_ref/T}),  E[i] = energy expectation;
