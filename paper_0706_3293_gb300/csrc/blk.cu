@@ -806,7 +806,11 @@ static int blk_env() {
 static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi, cudaStream_t st,
                        std::shared_ptr<const BlkMvPlan> *out) {
     if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB) return 1;
-    const int K = blk_K(b, false), env = blk_env(), nb = bp.nb;
+    // Blocks of several vectors are cut into parts, so their split has no reason to keep them small: 13 low
+    // sites, fewer blocks to set up and fewer scattered cross exchanges (N = 20, eight vectors, FP64:
+    // K = 11 / 12 / 13 / 14 90 / 86 / 80 / 80 us; N = 23 531 / 527 / 523 / 520)
+    const int K = multi && !getenv("HM_BLK_K") ? std::min(13, b->view.N - 2) : blk_K(b, false);
+    const int env = blk_env(), nb = bp.nb;
     {
         std::lock_guard<std::mutex> lk(b->tab_mu);
         for (const auto &m : b->mv_plans)

@@ -9,7 +9,7 @@
 // order of the bond groups, padded to a multiple of four with the row's own rank, then from
 // xs on the entries of the other low ends.  A target then takes a shift, an address and the gather;
 // finding it takes masks, a bit scan, an xor and two table lookups, by all lanes of the row.
-// High and cross exchanges are listed once per block (hops_setup).
+// High and cross exchanges are listed once per block (hops_setup_high, hops_setup_cross).
 #pragma once
 
 #include "blk.cuh"
@@ -87,9 +87,9 @@ __device__ __forceinline__ Hops hops_carve(const BlkParams &P, void *p) {
 
 // Hop lists of block (h, k), by one warp: the valid high exchanges as row offsets,
 // compacted by class (lane e tests bonds e and e + 32, ballots give the positions), and
-// the targets of the cross exchanges.  The caller syncs before and after.
-__device__ __forceinline__ void hops_setup(const BlkParams &P, const HopTab &H, const BlkTabs &tb, uint32_t h, int k,
-                                           uint32_t off, const Hops &sh, int lane) {
+// the targets of the cross exchanges (hops_setup_cross).  The caller syncs before and after.
+__device__ __forceinline__ void hops_setup_high(const BlkParams &P, const BlkTabs &tb, uint32_t h, int k, uint32_t off,
+                                                const Hops &sh, int lane) {
     int val[2] = {0, 0}, hoff[2] = {0, 0};
 #pragma unroll
     for (int half = 0; half < 2; ++half) {
@@ -109,6 +109,9 @@ __device__ __forceinline__ void hops_setup(const BlkParams &P, const HopTab &H, 
         sh.hcs[lane] = e >= 32 ? __popc(b0) + __popc(e >= 64 ? b1 : b1 & ((1u << (e - 32)) - 1u))
                                : __popc(b0 & ((1u << e) - 1u));
     }
+}
+__device__ __forceinline__ void hops_setup_cross(const BlkParams &P, const HopTab &H, const BlkTabs &tb, uint32_t h, int k,
+                                                 uint32_t off, const Hops &sh, int lane) {
     for (int e = lane; e < P.ncb; e += 32) {
         const int p = P.cb_p[e], q = P.cb_q[e];
         const uint32_t bq = (h >> q) & 1u;

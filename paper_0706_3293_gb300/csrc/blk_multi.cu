@@ -13,8 +13,8 @@
 // of its row where a binary64 sum rounds at every addition.  Both sums of a class and the diagonal
 // meet in one integer, and a class takes a conversion, a scaling and a multiply-add.  Rows with
 // infinities or NaN, and those whose largest value is below 2^-959 or above 2^1007, are added in
-// binary64.  Adding the high exchanges in binary64 beside the integers was slower (100 against 95 us below).
-// Measured on GB300, J1-J2 ring, whole calls: N = 20, eight vectors FP64 135 -> 93 us, FP32 71 -> 41;
+// binary64.  Adding the high exchanges in binary64 beside the integers was slower (100 against 95 us, before the last tuning).
+// Measured on GB300, J1-J2 ring, whole calls: N = 20, eight vectors FP64 135 -> 80 us, FP32 71 -> 41;
 // 16 vectors 315 -> 175 and 178 -> 56; 33 vectors (rows of no 16 bytes' alignment) 492 -> 344 and 243 -> 193.
 #include <algorithm>
 #include <cstdlib>
@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(MV_NT, 4) k_blk_multi(BlkParams P, HopTab Hp, 
     tb.C = (const uint32_t *)((const unsigned char *)P.tab + P.off_C);
     const uint32_t off = blk_off(P, tb, h, k), n = tb.C[P.K * (P.A + 1) + k];
     const Hops sh = hops_carve(P, smem);
-    if (warp == 0) hops_setup(P, Hp, tb, h, k, off, sh, lane);
+    if (warp == 0) hops_setup_high(P, tb, h, k, off, sh, lane);
+    else if (warp == 1) hops_setup_cross(P, Hp, tb, h, k, off, sh, lane);
     __syncthreads();
     // row of the warp's and the lane's columns; idle lanes repeat the last column group
     const int rpw = 32 >> a.lsh, grp = lane >> a.lsh, li = (lane & ((1 << a.lsh) - 1)) * V;

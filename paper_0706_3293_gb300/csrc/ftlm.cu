@@ -380,7 +380,8 @@ __global__ void __launch_bounds__(FT_NT, FT_CTAS) k_ftlm(FtParams F) {
                     const uint32_t ra = ig0 < g0 ? (uint32_t)(g0 - ig0) : 0u;
                     const uint32_t rb = ig0 + n > g1 ? (uint32_t)(g1 - ig0) : n;
                     __syncwarp();                  // the previous block's lists are read no more
-                    hops_setup(P, F.hop, tb, h, k, off, sh, lane);
+                    hops_setup_high(P, tb, h, k, off, sh, lane);
+                    hops_setup_cross(P, F.hop, tb, h, k, off, sh, lane);
                     __syncwarp();
                     const float *Xb = qc + ig0 * FT_W + v0;   // the block's rows, this lane's vectors
                     for (uint32_t r = ra + grp; r < rb; r += VT) {
