@@ -58,12 +58,14 @@ int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, siz
 // than grid_blocks, for which the workspaces' partial sums are sized
 template <class F>
 inline int row_grid(uint64_t rows, F kern, size_t smem) {
+    const int need = grid_blocks(rows, ROW_NT);
+    if (need <= sm_count()) return need;             // one CTA an SM always fits: no query (about 1 us of a call's 27)
     int per = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, ROW_NT, smem) != cudaSuccess) {
         cudaGetLastError();
         per = 1;
     }
-    const int wave = sm_count() * (per < 1 ? 1 : per), need = grid_blocks(rows, ROW_NT);
+    const int wave = sm_count() * (per < 1 ? 1 : per);
     return need < wave ? need : wave;
 }
 

@@ -375,7 +375,7 @@ int mom_matvec(const hm_basis *b, const BondParams &bp, const void *x, void *y, 
     size_t sm = 0;
     if (row_plan(sv, bp, 8, &P, &sm) == 0) {
         auto run = [&](auto kern, auto *xv, auto *yv) -> int {
-            HM_CUDA(raise_smem_limit(kern, sm));
+            if (sm > 16 * 1024) HM_CUDA(raise_smem_limit(kern, sm));   // below, 48 KB hold it and the static part
             kern<<<row_grid(b->view.dim, kern, sm), ROW_NT, sm, st>>>(sv, P, kpi, b->view.dim, reps, map, xv, yv);
             HM_CUDA(cudaGetLastError());
             return HM_OK;
