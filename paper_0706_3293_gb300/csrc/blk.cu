@@ -9,6 +9,7 @@
 #include <tuple>
 #include <type_traits>
 
+#include "blk_fit.h"
 #include "blk_hops.cuh"
 #include "blk_sweep.cuh"
 
@@ -112,18 +113,17 @@ static int blk_tables(hm_basis *b, int K, const void **dev, int *bytes, int *oU,
 // integer coefficient of a per-bond plan: round(h 2^pb_s)
 static long long pb_coef(const BlkParams &P, double h) { return std::llround(std::ldexp(h, P.pb_s)); }
 
-// Compile-time slots of the thread-per-row kernels (BlkParams::ln ..).  Sets rows_ok = 0
-// when a class has more bonds of one kind than the slots hold.
+// Compile-time slots of the thread-per-row kernels (BlkParams::ln ..), when they hold the list (rows_ok).
 static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int K, BlkParams *P) {
-    P->rows_ok = K <= 15 ? 1 : 0;
+    P->rows_ok = blk_slots_fit(bp.nb, bp.p, bp.q, bc.data(), K, HM_BLK_SL, HM_BLK_SX, HM_BLK_SG) ? 1 : 0;
     P->kshift = K - 6;
+    if (!P->rows_ok) return;
     std::map<std::pair<int, int>, uint32_t> cgroups;      // (class, d) -> mask of p
     for (int t = 0; t < bp.nb; ++t) {
         const int c = bc[t], p = bp.p[t], q = bp.q[t];    // p < q
         if (q < K) {
             const int ty = q < 8 ? 0 : (p >= 8 ? 1 : 2);
             int &n = P->ln[c][ty];
-            if (n == HM_BLK_SL) { P->rows_ok = 0; continue; }
             const uint32_t pat = (1u << p) | (1u << q);
             P->ld[c][ty][n] = (uint8_t)(q - p);
             if (P->perbond) P->pb_lb[ty][n] = (uint8_t)t;
@@ -135,7 +135,6 @@ static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int
         } else if (p < K) {
             const int ty = p < 8 ? 0 : 1;
             int &n = P->xn[c][ty];
-            if (n == HM_BLK_SX) { P->rows_ok = 0; continue; }
             P->xxa[c][ty][n] = (uint16_t)(ty == 0 ? (1u << p) << 2 : (1u << (p - 8)) << 2);
             if (P->perbond) P->pb_xb[ty][n] = (uint8_t)t;
             P->xf_p[P->nxf] = (uint8_t)p;
@@ -147,7 +146,6 @@ static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int
     }
     for (auto &kv : cgroups) {
         const int c = kv.first.first;
-        if (P->lgn[c] == HM_BLK_SG) { P->rows_ok = 0; continue; }
         P->lgd[c][P->lgn[c]] = (uint8_t)kv.first.second;
         P->lgm[c][P->lgn[c]] = kv.second;
         ++P->lgn[c];
@@ -155,6 +153,22 @@ static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int
 }
 
 static int blk_plan_bonds(hm_basis *b, const BondParams &bp, const std::vector<int> &bc, int K, BlkParams *P);
+
+// coupling classes: the distinct J and the class of each bond.  With more than HM_BLK_MAXC of them every
+// bond keeps its own coefficient (per-bond rows, class 0 slots): true, no classes
+static bool blk_classes_of(const BondParams &bp, bool bond_corr, std::vector<double> *cls, std::vector<int> *bc) {
+    bc->assign(bp.nb, 0);
+    for (int t = 0; t < bp.nb; ++t) {
+        const double J = -bp.jm[t];
+        const int c = (int)(std::find(cls->begin(), cls->end(), J) - cls->begin());
+        if (c == (int)cls->size()) cls->push_back(J);
+        (*bc)[t] = c;
+    }
+    if ((int)cls->size() <= HM_BLK_MAXC && !bond_corr) return false;
+    cls->clear();
+    bc->assign(bp.nb, 0);
+    return true;
+}
 
 int blk_plan(hm_basis *b, const BondParams &bp_all, int K, BlkParams *P, bool bond_corr, uint64_t use) {
     const SectorView &sv = b->view;
@@ -166,21 +180,11 @@ int blk_plan(hm_basis *b, const BondParams &bp_all, int K, BlkParams *P, bool bo
     P->N = sv.N; P->K = K; P->H = sv.N - K; P->A = sv.A; P->nb1 = 1 << (K - 8);
     P->dim = (uint32_t)sv.dim;
     P->par = b->parity;
-    // coupling classes: distinct J values; with more than HM_BLK_MAXC of them every bond
-    // keeps its own coefficient (per-bond rows, class 0 slots)
     std::vector<double> cls;
-    std::vector<int> bc(bp.nb);
-    for (int t = 0; t < bp.nb; ++t) {
-        const double J = -bp.jm[t];
-        int c = (int)(std::find(cls.begin(), cls.end(), J) - cls.begin());
-        if (c == (int)cls.size()) cls.push_back(J);
-        bc[t] = c;
-    }
-    if ((int)cls.size() > HM_BLK_MAXC || bond_corr) {
+    std::vector<int> bc;
+    if (blk_classes_of(bp, bond_corr, &cls, &bc)) {
         P->perbond = 1;
         P->bcmode = bond_corr ? 1 : 0;
-        cls.clear();
-        std::fill(bc.begin(), bc.end(), 0);
         double g0 = 0.0, mx = 0.0;
         for (int t = 0; t < bp.nb; ++t) {
             g0 += bp.jm[t] / 4.0;                                 // -J_b / 4
@@ -401,11 +405,24 @@ static const void *blk_mv_kernel(int nc) {
 // fp32_run: FP32 Lanczos runs keep K = 15.  The split decides the order in which a float row adds
 // its exchanges, and a run carries a changed rounding into every alpha and beta (FP64 rows are
 // exact integer sums, whatever the order).
-// The Lanczos workspace sizes its per-block partials (2^(N-K) blocks) with the same function.
+// The Lanczos workspace sizes its per-block partials (2^(N-K) blocks) with this K.
 int blk_K(const hm_basis *b, bool fp32_run) {
     int K = fp32_run ? 15 : std::max(8, std::min(15, b->view.N / 2 + 2));
     if (const char *e = getenv("HM_BLK_K")) K = std::max(8, std::min(15, atoi(e)));
     return std::min(K, b->view.N - 2);
+}
+
+// The split of a bond list: blk_K, or the next larger K whose slots hold the list (fewer blocks, so the
+// workspaces sized by blk_K hold them; HM_BLK_K is taken as it is).  The smallest is the fastest also where
+// it has no target table and a larger one does (FP64 Lanczos product and alpha, us: square 6 x 3 at
+// K = 12 / 15 38 / 51, honeycomb of 20 sites at K = 12 / 14 49 / 54).
+static int blk_K_of(const hm_basis *b, const BondParams &bp, bool fp32_run, bool bond_corr) {
+    const int k0 = blk_K(b, fp32_run);
+    if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB || getenv("HM_BLK_K")) return k0;
+    std::vector<double> cls;
+    std::vector<int> bc;
+    blk_classes_of(bp, bond_corr, &cls, &bc);
+    return blk_fitting_K(bp.nb, bp.p, bp.q, bc.data(), k0, std::min(15, b->view.N - 2), HM_BLK_SL, HM_BLK_SX, HM_BLK_SG);
 }
 
 // f(kernel) for the FP64 block-product instance of the plan (class count, integer ratios)
@@ -429,7 +446,7 @@ static int set_smem(K_t kern, size_t sm) {
 
 // Lanczos hooks: plan (0 = block path usable), attribute setup, launch
 int blk_lz_plan(hm_basis *b, const BondParams &bp, int dtype, BlkParams *P, int *blocks) {
-    int rc = blk_plan(b, bp, blk_K(b, dtype == HM_F32), P);
+    int rc = blk_plan(b, bp, blk_K_of(b, bp, dtype == HM_F32, false), P);
     if (rc != 0) return rc;
     const size_t sm = blk_row_smem_bytes(*P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
     if (!P->rows_ok || sm > 200 * 1024) return 1;
@@ -731,7 +748,7 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
             bc.jm[i] = bp.jm[c0 + i]; bc.jmf[i] = bp.jmf[c0 + i];
         }
         BlkParams &P = plans[c];
-        if (blk_plan(b, bc, blk_K(b, false), &P, true) != 0 || !P.rows_ok) return 1;
+        if (blk_plan(b, bc, blk_K_of(b, bc, false, true), &P, true) != 0 || !P.rows_ok) return 1;
         const size_t sm = blk_row_smem_bytes(P, es, BLK_XPAD);
         if (sm > 200 * 1024 || jit_bc_kernel(P, dtype, nbk, &kerns[c]) != 0) return 1;
         if (raise_smem_limit(kerns[c], (int)sm) != cudaSuccess) {
@@ -765,7 +782,7 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
 const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int nvec) {
     if (nvec != 1) return nullptr;
     BlkParams P;
-    if (blk_plan(b, bp, blk_K(b, false), &P) != 0) return nullptr;
+    if (blk_plan(b, bp, blk_K_of(b, bp, false, false), &P) != 0) return nullptr;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return nullptr;
     if (!P.perbond) return "k_blk_matvec";
     const void *k = nullptr;
@@ -796,10 +813,10 @@ struct BlkMvPlan {
 };
 constexpr unsigned BLK_MV_PLANS = 8;
 
-// what of the environment enters a plan besides the split
+// what of the environment enters a plan besides the value of blk_K, by which it is found
 static int blk_env() {
     const char *row = getenv("HM_JIT_ROW"), *jit = getenv("HM_JIT");
-    return (row && *row && strcmp(row, "table") != 0 ? 1 : 0) | (jit && jit[0] == '0' ? 2 : 0);
+    return (row && *row && strcmp(row, "table") != 0 ? 1 : 0) | (jit && jit[0] == '0' ? 2 : 0) | (getenv("HM_BLK_K") ? 4 : 0);
 }
 
 // 0 and the plan, or 1 when the block path does not apply
@@ -822,7 +839,7 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
     }
     auto m = std::make_shared<BlkMvPlan>();
     BlkParams &P = m->P;
-    const int rc = blk_plan(b, bp, K, &P);
+    const int rc = blk_plan(b, bp, multi ? K : blk_K_of(b, bp, false, false), &P);
     if (rc != 0) return rc;
     const int es = dtype == HM_F64 ? 8 : 4;
     m->multi = multi;
