@@ -845,6 +845,18 @@ static int lz_create(const hm_basis *b, int n_bonds, const int32_t *u, const int
     return HM_OK;
 }
 
+// time limit of a grid-barrier wait of the whole-run kernel: 5 s, or less by HM_LZ_BARRIER_NS ("ns" or
+// "ns,ns": the second pass of e0_grad has the second limit; a test sets 0 so that the first wait gives up)
+static unsigned long long lz_barrier_ns(bool pass2) {
+    const unsigned long long most = 5000000000ull;
+    const char *e = getenv("HM_LZ_BARRIER_NS");
+    if (!e || !*e) return most;
+    char *end = nullptr;
+    unsigned long long v = strtoull(e, &end, 10);
+    if (pass2 && *end == ',') v = strtoull(end + 1, nullptr, 10);
+    return std::min(v, most);
+}
+
 // all steps of a small sector in one kernel
 static int run_small(hm_lanczos *R, int steps, cudaStream_t st) {
     LzSmallArgs a{};
@@ -861,7 +873,7 @@ static int run_small(hm_lanczos *R, int steps, cudaStream_t st) {
     a.coef = R->coef;
     a.steps = steps;
     a.tol = LZ_TOL;
-    a.limit_ns = 5000000000ull;
+    a.limit_ns = lz_barrier_ns(R->psi != nullptr);
     return lz_small_launch(R->small, a, st);
 }
 
@@ -1146,8 +1158,11 @@ int e0_grad(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *v, 
     if (rc == HM_OK) {
         cudaError_t e = cudaMemcpyAsync(rz, d_ritz, 16, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess && n_bonds > 0) e = cudaMemcpyAsync(dE0_dJ, d_out, n_bonds * 8, cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&S1, R->sc, sizeof S1, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) rc = cuda_fail(e, "e0_grad: results");
+        // a second pass that gave up leaves a psi of some of its steps only
+        if (rc == HM_OK && S1.status == HM_ETIMEOUT) rc = fail(S1.status, "a grid barrier of the Lanczos run timed out");
     }
     delete R;
     if (rc < 0) return rc;

@@ -59,16 +59,20 @@ __device__ __forceinline__ PbSum lzs_row_pb(const BlkParams &P, const BlkMeta &B
 }
 
 // all CTAs past their writes; false when a barrier gave up.  bar[0] counts arrivals (never reset:
-// barrier k ends at k ctas), bar[1] is the abort flag
+// barrier k ends at k ctas), bar[1] is the abort flag.  A limit of 0 waits for nobody: the CTA that
+// arrives first gives up
 __device__ __forceinline__ bool lzs_barrier(unsigned *bar, unsigned target, unsigned long long limit_ns) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(bar, 1u);
+        const unsigned here = atomicAdd(bar, 1u) + 1u;
         volatile unsigned *v = bar;
         int ok = 1;
-        if (*v < target) {
+        if (here < target && limit_ns == 0) {
+            atomicExch(bar + 1, 1u);
+            ok = 0;
+        } else if (here < target) {
             unsigned long long t0, t;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
             for (unsigned spin = 1; *v < target; ++spin) {
