@@ -319,11 +319,12 @@ int basis_build(int n_sites, int two_s, int two_m, hm_basis **out) {
     }
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_cd, bytes > 0 ? bytes : 8);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_scratch, (size_t)HM_ESLOTS * HM_EPART * sizeof(int));
+    b->eslots = std::make_shared<ExpSlots>();
+    if (e == cudaSuccess) e = cudaMalloc(&b->eslots->dev, (size_t)HM_ESLOTS * HM_EPART * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(b->d_cd, src, bytes, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         if (b->d_cd) cudaFree(b->d_cd);
-        if (b->d_scratch) cudaFree(b->d_scratch);
+        if (b->eslots->dev) cudaFree(b->eslots->dev);
         delete b;
         return cuda_fail(e, "basis_build: device tables");
     }
@@ -348,7 +349,12 @@ int basis_free(hm_basis *b) {
     if (!b) return HM_OK;
     cudaError_t e = cudaSuccess, e2;
     if (b->d_cd && (e2 = cudaFree(b->d_cd)) != cudaSuccess) e = e2;
-    if (b->d_scratch && (e2 = cudaFree(b->d_scratch)) != cudaSuccess) e = e2;
+    if (b->eslots) {
+        std::lock_guard<std::mutex> lk(b->eslots->mu);
+        if (b->eslots->dev && (e2 = cudaFree(b->eslots->dev)) != cudaSuccess) e = e2;
+        for (int *p : b->eslots->captured)
+            if ((e2 = cudaFree(p)) != cudaSuccess) e = e2;
+    }
     for (auto &kv : b->blk_tabs)
         if (kv.second.dev && (e2 = cudaFree(kv.second.dev)) != cudaSuccess) e = e2;
     for (auto &kv : b->s1_tabs)

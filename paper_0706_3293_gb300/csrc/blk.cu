@@ -375,13 +375,92 @@ __global__ void __launch_bounds__(256) k_max_exp(const unsigned long long *__res
     }
 }
 
-// enqueues k_max_exp of x into the next exponent slot of the basis; its partial maxima are at *part,
-// *n of them
-static int launch_max_exp(hm_basis *b, const void *x, uint64_t n, int **part, int *np, cudaStream_t st) {
-    *part = (int *)b->d_scratch + (size_t)(b->eslot.fetch_add(1) % HM_ESLOTS) * HM_EPART;
-    const uint64_t want = (n + 2047) / 2048;                  // four loads a thread
-    *np = (int)std::min<uint64_t>(std::min(HM_EPART, sm_count() * 3), want ? want : 1);
-    k_max_exp<<<*np, 256, 0, st>>>((const unsigned long long *)x, n, *part);
+// The partial exponent maxima of one call's vector (ExpSlots): enqueue() runs k_max_exp of x, whose n
+// partials at part are the kernel's until the object goes
+struct ExpPart {
+    int *part = nullptr, n = 0;
+    int enqueue(hm_basis *b, const void *x, uint64_t rows, cudaStream_t stream);
+    ~ExpPart() { if (pooled) cudaFreeAsync(part, st); }
+
+  private:
+    int take(hm_basis *b);
+    cudaStream_t st = nullptr;
+    bool pooled = false;
+};
+
+// a slot for a captured call, given back with the graph
+static int exp_slot_of_graph(const std::shared_ptr<ExpSlots> &s, cudaGraph_t graph, int **part) {
+    struct Held {
+        std::shared_ptr<ExpSlots> s;
+        int *part;
+    };
+    int *p = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(s->mu);
+        if (s->free.empty()) {
+            const CaptureRelaxed relaxed;
+            int *chunk = nullptr;
+            HM_CUDA(cudaMalloc(&chunk, (size_t)HM_ESLOTS * HM_EPART * sizeof(int)));
+            s->captured.push_back(chunk);
+            for (int k = 0; k < HM_ESLOTS; ++k) s->free.push_back(chunk + (size_t)k * HM_EPART);
+        }
+        p = s->free.back();
+        s->free.pop_back();
+    }
+    auto give_back = [](void *v) {                            // host only: no CUDA call is allowed here
+        std::unique_ptr<Held> h((Held *)v);
+        std::lock_guard<std::mutex> lk(h->s->mu);
+        h->s->free.push_back(h->part);
+    };
+    Held *h = new Held{s, p};
+    cudaUserObject_t obj = nullptr;
+    cudaError_t e = cudaUserObjectCreate(&obj, h, give_back, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) {
+        give_back(h);
+        return cuda_fail(e, "exponent slot");
+    }
+    e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+    if (e != cudaSuccess) {
+        cudaUserObjectRelease(obj, 1);
+        return cuda_fail(e, "exponent slot");
+    }
+    *part = p;
+    return HM_OK;
+}
+
+int ExpPart::take(hm_basis *b) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    HM_CUDA(cudaStreamIsCapturing(st, &cs));
+    if (cs == cudaStreamCaptureStatusActive) {
+        cudaGraph_t graph = nullptr;
+        HM_CUDA(cudaStreamGetCaptureInfo(st, &cs, nullptr, &graph));
+        return exp_slot_of_graph(b->eslots, graph, &part);
+    }
+    // the per-thread handle names another stream in each thread
+    if (st != cudaStreamPerThread) {
+        unsigned long long id = 0;
+        HM_CUDA(cudaStreamGetId(st, &id));
+        ExpSlots &s = *b->eslots;
+        std::lock_guard<std::mutex> lk(s.mu);
+        int k = 0;
+        while (k < s.streams && s.owner[k] != id) ++k;
+        if (k == s.streams && k < HM_ESLOTS) s.owner[s.streams++] = id;
+        if (k < HM_ESLOTS) {
+            part = s.dev + (size_t)k * HM_EPART;
+            return HM_OK;
+        }
+    }
+    HM_CUDA(cudaMallocAsync((void **)&part, (size_t)HM_EPART * sizeof(int), st));
+    pooled = true;
+    return HM_OK;
+}
+
+int ExpPart::enqueue(hm_basis *b, const void *x, uint64_t rows, cudaStream_t stream) {
+    st = stream;
+    HM_TRY(take(b));
+    const uint64_t want = (rows + 2047) / 2048;               // four loads a thread
+    n = (int)std::min<uint64_t>(std::min(HM_EPART, sm_count() * 3), want ? want : 1);
+    k_max_exp<<<n, 256, 0, st>>>((const unsigned long long *)x, rows, part);
     HM_CUDA(cudaGetLastError());
     return HM_OK;
 }
@@ -763,15 +842,15 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
         blocks[c] = std::min<int>(sm_count() * std::min(per, 4), 1 << P.H);
         if (!work || work_bytes < (size_t)blocks[c] * (nbk + 1) * sizeof(double)) return 1;
     }
-    int *Ed = nullptr, nE = 0;
-    if (dtype == HM_F64) HM_TRY(launch_max_exp(b, x, sv.dim, &Ed, &nE, st));
+    ExpPart E;
+    if (dtype == HM_F64) HM_TRY(E.enqueue(b, x, sv.dim, st));
     double *part = (double *)work;
     for (int c = 0; c < nch; ++c) {
         const int nbk = std::min(BC_CHUNK, bp.nb - c * BC_CHUNK);
         const size_t sm = blk_row_smem_bytes(plans[c], es, BLK_XPAD);
-        void *args[] = {(void *)&plans[c], (void *)&x, (void *)&g, (void *)&Ed, (void *)&nE, (void *)&part};
+        void *args[] = {(void *)&plans[c], (void *)&x, (void *)&g, (void *)&E.part, (void *)&E.n, (void *)&part};
         HM_CUDA(cudaLaunchKernel(kerns[c], dim3(blocks[c]), dim3(BLK_NT), args, sm, st));
-        k_bc_final<<<1, 32 * (BC_CHUNK + 1), 0, st>>>(part, blocks[c], nbk, Ed, nE, sign, div, out + c * BC_CHUNK);
+        k_bc_final<<<1, 32 * (BC_CHUNK + 1), 0, st>>>(part, blocks[c], nbk, E.part, E.n, sign, div, out + c * BC_CHUNK);
         HM_CUDA(cudaGetLastError());
     }
     return HM_OK;
@@ -902,9 +981,9 @@ int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dt
     const int rc = blk_mv_plan(b, bp, dtype, nvec > 1, st, &m);
     if (rc != 0) return rc;
     if (nvec > 1) return blk_multi_launch(m->P, m->hop, m->hops, m->gd, x, y, dtype, nvec, st);
-    int *Ed = nullptr, nE = 0;
-    if (dtype == HM_F64) HM_TRY(launch_max_exp(b, x, m->P.dim, &Ed, &nE, st));
-    void *args[] = {(void *)&m->P, (void *)&x, (void *)&y, (void *)&Ed, (void *)&nE};
+    ExpPart E;
+    if (dtype == HM_F64) HM_TRY(E.enqueue(b, x, m->P.dim, st));
+    void *args[] = {(void *)&m->P, (void *)&x, (void *)&y, (void *)&E.part, (void *)&E.n};
     HM_CUDA(cudaLaunchKernel(m->kern, dim3(m->blocks), dim3(BLK_NT), args, m->smem, st));
     return HM_OK;
 }

@@ -7,7 +7,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <map>
 #include <memory>
 #include <mutex>
@@ -84,18 +83,38 @@ struct S1Tab {                      // tables of the s = 1 block path (s1blk.cu)
 
 namespace hm {
 struct BlkMvPlan;
-}
+
+// allocations and copies of tables while a stream of this or another thread is being captured: none of
+// them touches the captured streams
+struct CaptureRelaxed {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    CaptureRelaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~CaptureRelaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    CaptureRelaxed(const CaptureRelaxed &) = delete;
+};
+
+// Slots of HM_EPART ints for the exponent maxima of a product's vector, from the kernel that forms them to
+// the product that reads them (blk.cu, ExpPart).  No two calls that may run at the same time share one:
+//   * the first HM_ESLOTS streams that a basis sees have one each (calls of one stream are in order);
+//     calls of any other stream take theirs from the stream's memory pool;
+//   * a captured call has one of its own, given back when the last graph that holds the call is gone.
 constexpr int HM_ESLOTS = 16, HM_EPART = 512;
+struct ExpSlots {
+    std::mutex mu;
+    int *dev = nullptr;                     // HM_ESLOTS slots (owned)
+    unsigned long long owner[HM_ESLOTS];    // stream ids, which are never used again
+    int streams = 0;
+    std::vector<int *> captured;            // chunks of HM_ESLOTS slots for captured calls (owned)
+    std::vector<int *> free;                // those of them that no graph holds
+};
+}  // namespace hm
 
 struct hm_basis {
     hm::SectorView view;
     std::vector<uint64_t> D;        // host D(k, a), (N+1) x (S2*N+1)
     std::vector<uint64_t> cd;       // host CD, cd_len entries
     void *d_cd = nullptr;           // device copy (owned)
-    // device scratch (owned): HM_ESLOTS slots of HM_EPART ints for the exponent maxima of a product's
-    // vector; a call takes the next slot, so calls in flight on several streams do not share one
-    void *d_scratch = nullptr;
-    std::atomic<unsigned> eslot{0};
+    std::shared_ptr<hm::ExpSlots> eslots;   // graphs that hold a slot keep the host part alive
     std::mutex tab_mu;              // guards blk_tabs, blk_ttabs and mv_plans (built on first use)
     std::vector<std::shared_ptr<const hm::BlkMvPlan>> mv_plans;   // the last plans of y = H x (blk.cu)
     unsigned mv_next = 0;
