@@ -870,8 +870,9 @@ const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int 
 
 // several vectors at once (blk_multi.cu)
 int blk_hop_table(hm_basis *b, const BlkParams &P, const HopTab &H, bool build, const uint16_t **table);
-int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table, const double *gd, const void *x, void *y,
-                     int dtype, int nvec, cudaStream_t st);
+bool blk_multi_orders(const double *gd, int nc, int *oc);
+int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table, const double *gd, const int *oc,
+                     const void *x, void *y, int dtype, int nvec, cudaStream_t st);
 
 // The plan of y = H x for one bond list.  Planning takes 20 to 60 us of host time (groups, table
 // layout, the source text that names a run-time compiled kernel), more than the product itself
@@ -888,7 +889,8 @@ struct BlkMvPlan {
     // multi: several vectors (blk_multi.cu)
     HopTab hop;
     const uint16_t *hops;
-    double gd[HM_BLK_MAXC];          // -J_c / 4
+    double gd[HM_BLK_MAXC] = {};     // -J_c / 4
+    int oc[HM_BLK_MAXC] = {};        // binary orders of |J_c| below the largest
 };
 constexpr unsigned BLK_MV_PLANS = 8;
 
@@ -917,14 +919,20 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
             }
     }
     auto m = std::make_shared<BlkMvPlan>();
+    if (multi) {             // class plans of a plain basis only, as the general rows; decided before any planning
+        std::vector<double> cls;
+        std::vector<int> bc;
+        if (b->parity || blk_classes_of(bp, false, &cls, &bc)) return 1;
+        for (size_t c = 0; c < cls.size(); ++c) m->gd[c] = -cls[c] / 4.0;
+        if (dtype == HM_F64 && !blk_multi_orders(m->gd, (int)cls.size(), m->oc)) return 1;
+    }
     BlkParams &P = m->P;
     const int rc = blk_plan(b, bp, multi ? K : blk_K_of(b, bp, false, false), &P);
     if (rc != 0) return rc;
     const int es = dtype == HM_F64 ? 8 : 4;
     m->multi = multi;
     m->smem = blk_row_smem_bytes(P, es, BLK_XPAD);
-    // several vectors: class plans; a plain basis only, as the general rows
-    if (multi ? P.perbond || P.par : !P.rows_ok || m->smem > 200 * 1024) return 1;
+    if (!multi && (!P.rows_ok || m->smem > 200 * 1024)) return 1;
     // target tables: built on the first product of a layout, but for class plans neither inside a
     // stream capture (no allocation there) nor without end on a basis that sees many bond lists; the
     // generic rows then serve, with the same result (FP64: the same exact sums)
@@ -939,11 +947,6 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
         m->hop = hop_layout(P);
         HM_TRY(blk_hop_table(b, P, m->hop, build, &m->hops));
         if (!m->hops) return 1;
-        for (int t = 0, c = 0; t < nb; ++t) {                // class c: the c-th distinct coupling
-            bool seen = false;
-            for (int i = 0; i < t && !seen; ++i) seen = bp.jm[i] == bp.jm[t];
-            if (!seen) m->gd[c++] = bp.jm[t] / 4.0;
-        }
     }
     const int trc = multi ? 1 : blk_target_table(b, &P, es, build);
     if (trc < 0) return trc;
@@ -980,7 +983,7 @@ int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dt
     std::shared_ptr<const BlkMvPlan> m;
     const int rc = blk_mv_plan(b, bp, dtype, nvec > 1, st, &m);
     if (rc != 0) return rc;
-    if (nvec > 1) return blk_multi_launch(m->P, m->hop, m->hops, m->gd, x, y, dtype, nvec, st);
+    if (nvec > 1) return blk_multi_launch(m->P, m->hop, m->hops, m->gd, m->oc, x, y, dtype, nvec, st);
     ExpPart E;
     if (dtype == HM_F64) HM_TRY(E.enqueue(b, x, m->P.dim, st));
     void *args[] = {(void *)&m->P, (void *)&x, (void *)&y, (void *)&E.part, (void *)&E.n};

@@ -8,15 +8,20 @@
 // What bounds the FP64 product is arithmetic: a warp's binary64 instruction occupies its quarter of
 // an SM for 64 cycles, and a multiply-add for each of the 40 bonds of a J1-J2 ring kept that pipe 72%
 // busy (k_row_matvec).  Here the exchange sums are integers: every gathered value is aligned to the
-// largest exponent among those seen so far in its row and column (the sums move along when a larger
-// one comes), with two bits below the last place, so a value is cut at 2^-54 of the largest one
-// of its row where a binary64 sum rounds at every addition.  Both sums of a class and the diagonal
-// meet in one integer, and a class takes a conversion, a scaling and a multiply-add.  Rows with
-// infinities or NaN, and those whose largest value is below 2^-959 or above 2^1007, are added in
-// binary64.  Adding the high exchanges in binary64 beside the integers was slower (100 against 95 us, before the last tuning).
-// Measured on GB300, J1-J2 ring, whole calls: N = 20, eight vectors FP64 135 -> 80 us, FP32 71 -> 41;
-// 16 vectors 315 -> 175 and 178 -> 56; 33 vectors (rows of no 16 bytes' alignment) 492 -> 344 and 243 -> 193.
+// largest term of its row and column so far, in powers of two of |J_c| |x_j| (the sums move along when a
+// larger one comes), with four bits below the last place.  So a value is cut at 2^-55 of the row's largest
+// term -J_c/2 x_j, however far apart the couplings lie, where a binary64 sum rounds at every addition.
+// A class's low, cross and high sums meet in one integer, and a class takes a conversion, a scaling
+// and a multiply-add; the diagonal term is a binary64 product.  Rows with infinities or NaN, and those whose
+// largest term is near the ends of binary64's range, are added in binary64; couplings more than 2^MULTI_SPREAD
+// apart, or zero, take the general rows.  Adding the high exchanges in binary64 beside the integers was
+// slower (100 against 95 us, before the last tuning).
+// Measured on GB300, J1-J2 ring, N = 20, against k_matvec (general rows): eight vectors FP64 255 -> 81 us (unit
+// vectors, whose rows are nearly all zeros, 255 -> 112), FP32 78 -> 25; 16 vectors FP64 361 -> 142; 33
+// vectors (rows of no 16 bytes' alignment) 723 -> 330.
 #include <algorithm>
+#include <climits>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <string>
@@ -29,6 +34,7 @@ namespace hm {
 namespace {
 
 constexpr int MV_NT = 256;
+constexpr int MULTI_SPREAD = 60;   // FP64: binary orders between the largest and the smallest |J_c|
 
 __device__ __forceinline__ int hi32(double v) { return __double2hiint(v); }
 __device__ __forceinline__ int lo32(double v) { return __double2loint(v); }
@@ -36,6 +42,7 @@ __device__ __forceinline__ int lo32(double v) { return __double2loint(v); }
 struct MultiArgs {
     const uint16_t *hops;
     double gd[HM_BLK_MAXC];        // -J_c / 4
+    int oc[HM_BLK_MAXC];           // binary orders of |J_c| below the largest
     int ld, c0, w, parts;          // columns c0 .. c0 + w - 1 of ld; CTAs a block
     int lsh;                       // 2^lsh lanes a row
 };
@@ -64,70 +71,97 @@ __device__ __forceinline__ void multi_st(T *p, const T *v) {
     else *(float4 *)p = make_float4(v[0], v[1], v[2], v[3]);
 }
 
-// one row and column in binary64, for the rows the integers do not serve
+// f(row offset) for every target of class cl of row r; returns their number
+template <class F>
+__device__ __forceinline__ int multi_targets(const BlkParams &P, const HopTab &Hp, const Hops &sh, const uint16_t *T,
+                                             uint4 hd, uint32_t l, uint32_t r, int cl, F &&f) {
+    int cnt = (int)((hd.x >> (8 * cl)) & 0xFFu);
+    for (int e = 0; e < cnt; ++e) f((int)__ldg(T + Hp.seg[cl] + e));
+    for (int e = P.cb_start[cl]; e < P.cb_start[cl + 1]; ++e) {
+        int t2;
+        if (!hop_cross(Hp, sh.x[e], hd, T, l, &t2)) continue;
+        f(t2);
+        ++cnt;
+    }
+    for (int e = sh.hcs[cl]; e < sh.hcs[cl + 1]; ++e) f((int)r + sh.hcd[e]);
+    return cnt + sh.hcs[cl + 1] - sh.hcs[cl];
+}
+
+// whether all targets of a row hold zeros in the lane's columns (blocks of unit vectors are made of such rows)
+template <int NC, int V>
+__device__ __noinline__ bool multi_row_zeros(const BlkParams &P, const HopTab &Hp, const MultiArgs &a, const Hops &sh,
+                                             const double *Xb, const uint16_t *T, uint4 hd, uint32_t l, uint32_t r) {
+    unsigned bits = 0u;
+    for (int cl = 0; cl < NC; ++cl)
+        multi_targets(P, Hp, sh, T, hd, l, r, cl, [&](int t) {
+            double v[V];
+            multi_ld<double, V>(Xb + (ptrdiff_t)t * a.ld, v);
+#pragma unroll
+            for (int q = 0; q < V; ++q) bits |= (unsigned)hi32(v[q]) << 1 | (unsigned)lo32(v[q]);
+        });
+    return bits == 0u;
+}
+
+// one row and column in binary64, for the rows the integers do not serve; a term at a time, so that large values
+// under small couplings do not overflow
 template <int NC>
 __device__ __noinline__ double multi_row_f64(const BlkParams &P, const HopTab &Hp, const MultiArgs &a, const Hops &sh,
                                              const double *Xb, const uint16_t *T, uint4 hd, uint32_t l, uint32_t r) {
-    const double xo = __ldg(Xb + (ptrdiff_t)r * a.ld);
     double y = 0.0, dg = 0.0;
     for (int cl = 0; cl < NC; ++cl) {
-        double s = 0.0;
-        int cnt = (int)((hd.x >> (8 * cl)) & 0xFFu);
-        for (int e = 0; e < cnt; ++e) s += __ldg(Xb + (ptrdiff_t)__ldg(T + Hp.seg[cl] + e) * a.ld);
-        for (int e = P.cb_start[cl]; e < P.cb_start[cl + 1]; ++e) {
-            int t2;
-            if (!hop_cross(Hp, sh.x[e], hd, T, l, &t2)) continue;
-            s += __ldg(Xb + (ptrdiff_t)t2 * a.ld);
-            ++cnt;
-        }
-        for (int e = sh.hcs[cl]; e < sh.hcs[cl + 1]; ++e) s += __ldg(Xb + (ptrdiff_t)((int)r + sh.hcd[e]) * a.ld);
-        cnt += sh.hcs[cl + 1] - sh.hcs[cl];
+        const double g2 = 2.0 * a.gd[cl];
+        const int cnt = multi_targets(P, Hp, sh, T, hd, l, r, cl,
+                                      [&](int t) { y = fma(g2, __ldg(Xb + (ptrdiff_t)t * a.ld), y); });
         dg += a.gd[cl] * (double)(P.ntot[cl] - 2 * cnt);
-        y += 2.0 * a.gd[cl] * s;
     }
-    return dg * xo + y;
+    return fma(dg, __ldg(Xb + (ptrdiff_t)r * a.ld), y);
 }
 
-// running sums of one row and column: FP32 plainly, FP64 as integers in units of 2^(E - 1077)
+// running sums of one row and column: FP32 plainly, FP64 as integers, class c in units of 2^(E + oc - 1079)
 template <class T, int NC> struct MultiAcc;
 template <int NC> struct MultiAcc<float, NC> {
-    float s[NC], own;
-    __device__ __forceinline__ void start(float xo) {
-        own = xo;
+    float s[NC];
+    __device__ __forceinline__ void start() {
 #pragma unroll
         for (int c = 0; c < NC; ++c) s[c] = 0.0f;
     }
+    __device__ __forceinline__ void to_class(int) {}
     __device__ __forceinline__ void add(int c, float v, bool on) { s[c] += on ? v : 0.0f; }
 };
 template <int NC> struct MultiAcc<double, NC> {
+    // E serves from E_LO + 1 to E_HI: above, all shifts and scales are those of normal numbers, and a value
+    // that is not finite has an exponent field above E_HI + oc
+    static constexpr int E_LO = 64, E_HI = 2030 - MULTI_SPREAD;
     long long s[NC];
-    int E;
-    double own;
-    __device__ __forceinline__ void start(double xo) {
-        own = xo;
-        E = (hi32(xo) >> 20) & 0x7FF;
+    int E;                         // of the largest term so far; plus oc while a class is added
+    __device__ __forceinline__ void start() {
+        E = E_LO;
 #pragma unroll
         for (int c = 0; c < NC; ++c) s[c] = 0;
     }
+    __device__ __forceinline__ void to_class(int d) { E += d; }
     __device__ __forceinline__ static long long fixed(int hi, int lo, int E) {
         const int e = (hi >> 20) & 0x7FF;
-        const unsigned long long M = ((unsigned long long)(unsigned)((hi & 0xFFFFF) | 0x100000) << 32 | (unsigned)lo) << 2;
+        const unsigned long long M = ((unsigned long long)(unsigned)((hi & 0xFFFFF) | 0x100000) << 32 | (unsigned)lo) << 4;
         unsigned long long q;
         asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(M), "r"(E - e));       // zero from 64 on
         const long long m = (long long)q, sg = hi >> 31;
         return (m ^ sg) - sg;
     }
-    // a value that is not on counts as zero (exponent 0: shifted out whenever E serves)
+    // a value that is not on counts as zero (exponent field 0: shifted out, as E is at least E_LO)
     __device__ __forceinline__ void add(int c, double v, bool on) {
-        const int hi = on ? hi32(v) : 0, e = (hi >> 20) & 0x7FF;
+        const int hi = on ? hi32(v) : 0, lo = lo32(v), e = (hi >> 20) & 0x7FF;
         if (e > E) {
             const int d = min(e - E, 63);
 #pragma unroll
             for (int k = 0; k < NC; ++k) s[k] >>= d;
             E = e;
         }
-        s[c] += fixed(hi, lo32(v), E);
+        s[c] += fixed(hi, lo, E);
     }
+    __device__ __forceinline__ bool low() const { return E == E_LO; }
+    // the integers hold the sums: a largest term in range, or only zeros
+    __device__ __forceinline__ bool serves(bool zeros) const { return low() ? zeros : E <= E_HI; }
 };
 
 template <class T, int NC, int V>
@@ -159,15 +193,14 @@ __global__ void __launch_bounds__(MV_NT, 4) k_blk_multi(BlkParams P, HopTab Hp, 
         const uint16_t *Tr = a.hops + (size_t)g * Hp.stride;
         const uint4 hd = __ldg((const uint4 *)Tr);
         MultiAcc<T, NC> acc[V];
-        {
-            T v[V];
-            row((int)r, v);
 #pragma unroll
-            for (int q = 0; q < V; ++q) acc[q].start(v[q]);
-        }
+        for (int q = 0; q < V; ++q) acc[q].start();
         int nd[NC];
 #pragma unroll
         for (int cl = 0; cl < NC; ++cl) {
+            const int oc = a.oc[cl];
+#pragma unroll
+            for (int q = 0; q < V; ++q) acc[q].to_class(oc);
             auto add = [&](const T *v, bool on) {
 #pragma unroll
                 for (int q = 0; q < V; ++q) acc[q].add(cl, v[q], on);
@@ -213,23 +246,37 @@ __global__ void __launch_bounds__(MV_NT, 4) k_blk_multi(BlkParams P, HopTab Hp, 
                 add(v, true);
             }
             nd[cl] = P.ntot[cl] - 2 * (mc + e1 - e0);
+#pragma unroll
+            for (int q = 0; q < V; ++q) acc[q].to_class(-oc);
         }
-        T yv[V];
+        T yv[V], own[V], dg = T(0);
+        bool zeros = false;
+        row((int)r, own);
+        if constexpr (sizeof(T) == 8) {
+#pragma unroll
+            for (int cl = 0; cl < NC; ++cl) dg = fma(a.gd[cl], (double)nd[cl], dg);
+            bool low = false;
+#pragma unroll
+            for (int q = 0; q < V; ++q) low |= acc[q].low();
+            if (low) zeros = multi_row_zeros<NC, V>(P, Hp, a, sh, Xb, Tr, hd, l, r);
+        }
 #pragma unroll
         for (int q = 0; q < V; ++q) {
             if constexpr (sizeof(T) == 4) {
                 yv[q] = 0.0f;
 #pragma unroll
-                for (int cl = 0; cl < NC; ++cl) yv[q] += P.gq[cl] * (2.0f * acc[q].s[cl] + (float)nd[cl] * acc[q].own);
-            } else if (acc[q].E < 64 || acc[q].E > 2030) {
+                for (int cl = 0; cl < NC; ++cl) yv[q] += P.gq[cl] * (2.0f * acc[q].s[cl] + (float)nd[cl] * own[q]);
+            } else if (!acc[q].serves(zeros)) {
                 yv[q] = multi_row_f64<NC>(P, Hp, a, sh, Xb + q, Tr, hd, l, r);
             } else {
-                // |2 s + nd xo| < 3 64 2^55
-                const long long xo = MultiAcc<T, NC>::fixed(hi32(acc[q].own), lo32(acc[q].own), acc[q].E);
-                const double sc = ef::u2d((uint64_t)(acc[q].E - 1077 + 1023) << 52);
                 yv[q] = 0.0;
 #pragma unroll
-                for (int cl = 0; cl < NC; ++cl) yv[q] = fma(a.gd[cl], (double)(2 * acc[q].s[cl] + nd[cl] * xo) * sc, yv[q]);
+                for (int cl = 0; cl < NC; ++cl) {                // at most 64 values below 2^57; 2 s in the scale
+                    const double t = (double)acc[q].s[cl];
+                    const int th = hi32(t);
+                    yv[q] = fma(a.gd[cl], __hiloint2double(th ? th + ((acc[q].E + a.oc[cl] - 1078) << 20) : 0, lo32(t)), yv[q]);
+                }
+                yv[q] = fma(dg, own[q], yv[q]);
             }
         }
         if (on_col) multi_st<T, V>(y + ((size_t)off + r) * a.ld + a.c0 + li, yv);
@@ -273,12 +320,29 @@ int blk_hop_table(hm_basis *b, const BlkParams &P, const HopTab &H, bool build, 
     return HM_OK;
 }
 
+// binary orders of each |J_c| below the largest (gd: the -J_c / 4 of nc classes); false when the integer sums
+// do not serve them
+bool blk_multi_orders(const double *gd, int nc, int *oc) {
+    int most = INT_MIN;
+    for (int c = 0; c < nc; ++c) {
+        if (gd[c] == 0.0) return false;
+        oc[c] = std::ilogb(gd[c]);
+        most = std::max(most, oc[c]);
+    }
+    for (int c = 0; c < HM_BLK_MAXC; ++c) {
+        oc[c] = c < nc ? most - oc[c] : 0;
+        if (oc[c] > MULTI_SPREAD) return false;
+    }
+    return true;
+}
+
 // y = H x, columns 0 .. nvec - 1 of rows of nvec elements, 32 at a time
-int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table, const double *gd, const void *x, void *y,
-                     int dtype, int nvec, cudaStream_t st) {
+int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table, const double *gd, const int *oc,
+                     const void *x, void *y, int dtype, int nvec, cudaStream_t st) {
     MultiArgs a{};
     a.hops = table;
     memcpy(a.gd, gd, sizeof a.gd);
+    memcpy(a.oc, oc, sizeof a.oc);
     a.ld = nvec;
     int valid = 0;
     for (uint32_t h = 0; h < (1u << P.H); ++h) {
