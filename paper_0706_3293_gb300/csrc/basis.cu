@@ -179,14 +179,14 @@ int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, siz
     uint16_t bc[ROW_MB];
     int last[HM_MAX_SITES], slot_of[HM_MAX_SITES], freed[HM_MAX_SITES], nf = 0;    // last[q]: lowest partner below q
     for (int r = 0; r < N; ++r) last[r] = N;
-    double mx = 0.0;
+    double most = 0.0;
     int count[HM_MAX_SITES] = {};
     for (int t = 0; t < bp.nb; ++t) {
         int c = t > 0 && bp.jm[t] == bp.jm[t - 1] ? bc[t - 1] : 0;
         while (c < P->nc && P->jm[c] != bp.jm[t]) ++c;
         if (c == P->nc) P->jm[P->nc++] = bp.jm[t];
         bc[t] = (uint16_t)c;
-        mx = std::max(mx, std::fabs(bp.jm[t] / 4.0));
+        most += std::fabs(bp.jm[t] / 4.0);
         last[bp.q[t]] = std::min(last[bp.q[t]], (int)bp.p[t]);
         ++count[bp.p[t]];
     }
@@ -208,17 +208,29 @@ int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, siz
     }
     for (int t = 0; t < bp.nb; ++t)
         P->bond[at[bp.p[t]]++] = (uint32_t)(bp.q[t] * sv.bits) | ((uint32_t)slot_of[bp.q[t]] << 8) | ((uint32_t)bc[t] << 16);
-    // diagonal sum_b dC_b k_b with |k_b| <= S2^2, below 2^62; taken when that leaves the largest
-    // coupling 52 bits or more (a binary64 sum of the terms rounds no finer)
+    // diagonal sum_b dC_b k_b with |k_b| <= S2^2 in two parts, dC 2^-s below 2^62 and the remainder dL 2^-(s+t)
+    // below 2^30; taken when they hold every coupling as exactly as a binary64 (binary32) term does: a digit can
+    // make the term of a large coupling zero (integer spins), and terms of large couplings can cancel
     int ex = 0, kb = 0;
-    std::frexp(mx, &ex);                             // mx < 2^ex
-    while ((1 << kb) < S2 * S2 * std::max(1, bp.nb)) ++kb;
-    const int s = 62 - kb - ex;
-    if (62 - kb < 52 || s <= -1000 || s >= 1000) return 1;
+    std::frexp(most * S2 * S2, &ex);                 // sum of |J_b| / 4 S2^2 < 2^ex
+    while ((1 << kb) < S2 * S2 * bp.nb) ++kb;
+    const int s = 62 - ex, t = 30 - kb;
+    if (kb > 10 || s <= -900 || s >= 900) return 1;
     P->dscale = std::ldexp(1.0, -s);
-    for (int c = 0; c < P->nc; ++c) P->dC[c] = std::llround(std::ldexp(P->jm[c] / 4.0, s));
+    P->dscale_low = std::ldexp(1.0, -s - t);
+    P->dlow = 0;
+    for (int c = 0; c < P->nc; ++c) {
+        const double v = std::ldexp(P->jm[c] / 4.0, s);
+        P->dC[c] = std::llround(v);
+        const double rem = std::ldexp(v - (double)P->dC[c], t);
+        P->dL[c] = (int)std::lround(rem);
+        // one class at s > 1/2: ROW_ONE, without dC
+        if (std::fabs(rem - (double)P->dL[c]) > std::ldexp(std::fabs(v), t - (es == 8 ? 53 : 29)) && !(P->nc == 1 && S2 > 1))
+            return 1;
+        P->dlow |= P->dL[c] != 0;
+    }
     P->dsum = 0;
-    for (int t = 0; t < bp.nb; ++t) P->dsum += P->dC[bc[t]];
+    for (int b = 0; b < bp.nb; ++b) P->dsum += P->dC[bc[b]];
     const size_t tabs = sv.idx64 ? row_tab_bytes<uint64_t>(sv) : row_tab_bytes<uint32_t>(sv);
     *smem = row_coef_bytes(*P, S2, es) + tabs + (size_t)P->nslots * ROW_NT * (sv.idx64 ? 16 : 8);
     // at least two CTAs on an SM; more shared memory than that leaves the table form ahead

@@ -7,6 +7,8 @@
 // larger tables and the successor-rule row runs (HM_ROW_RUN).
 #pragma once
 
+#include <type_traits>
+
 #include "hm_internal.cuh"
 
 namespace hm {
@@ -34,24 +36,26 @@ constexpr int ROW_NT = 256;          // threads per CTA of the row kernels
 constexpr int ROW_SLOT_NONE = 255;
 
 // Lists of more than ROW_MB bonds take the table form: a kernel's parameters are copied at every
-// launch (3.9 KB here)
+// launch (4.4 KB here)
 constexpr int ROW_MB = 128;
 struct RowPlan {
     int nslots, nc;
-    double dscale;                   // 2^-s of dC
+    double dscale, dscale_low;       // 2^-s of dC, 2^-(s+t) of dL
     // per position: first bond whose lower end it is | their number << 10 | slot of its R << 20
     // (ROW_SLOT_NONE: not the upper end of a bond)
     uint32_t pos[HM_MAX_SITES];
     uint32_t bond[ROW_MB];           // bit offset of the upper end's digit | its slot << 8 | class << 16
     double jm[ROW_MB];               // by class (distinct coupling): -J
-    long long dC[ROW_MB];            // by class: round(-J / 4 2^s)
+    long long dC[ROW_MB];            // by class: round(-J / 4 2^s), and the remainder 2^-t dL; dlow: some dL is not zero
+    int dL[ROW_MB];
+    int dlow;
     long long dsum;                  // sum of dC over the bonds (s = 1/2: the diagonal is dsum - 2 sum over unequal spins)
     double hs_pdn[64], hs_pup[64];   // as in BondParams
 };
 
 // the plan of a bond list; 0, or 1 when the table form has to serve: more than ROW_MB bonds, tables
-// above the shared memory, couplings the integer diagonal does not hold to 52 bits, or row
-// runs (HM_ROW_RUN).  *smem: dynamic shared memory of a CTA for accumulation type size es
+// above the shared memory, couplings so far apart that the integer diagonal does not hold
+// them exactly, or row runs (HM_ROW_RUN).  *smem: dynamic shared memory of a CTA for accumulation type size es
 int row_plan(const SectorView &sv, const BondParams &bp, int es, RowPlan *P, size_t *smem);
 
 // CTAs of a row kernel: one resident wave at most (every CTA stages the tables), and no more
@@ -153,8 +157,25 @@ __device__ __forceinline__ void row_sweep(const SectorView &sv, const RowPlan &P
 
 // (H x)_i for NV columns: *dg the diagonal element, acc the exchange sums.  MODE: ROW_ONE one class
 // of couplings (a ring, a uniform lattice); ROW_HALF s = 1/2, where a bond allows one direction at
-// most, so one gather and one multiply-add serve it; ROW_ANY the rest
-enum { ROW_ANY = 0, ROW_ONE = 1, ROW_HALF = 2 };
+// most, so one gather and one multiply-add serve it; ROW_ANY the rest; ROW_LOW any list whose diagonal has a
+// low part (of its own, since a test for it costs the others 5%)
+enum { ROW_ANY = 0, ROW_ONE = 1, ROW_HALF = 2, ROW_LOW = 3 };
+// f(std::integral_constant<int, MODE>) for the plan's mode
+template <class F>
+inline auto row_dispatch(const SectorView &sv, const RowPlan &P, F &&f) {
+    if (P.nc == 1 && sv.S2 > 1) return f(std::integral_constant<int, ROW_ONE>());
+    if (P.dlow) return f(std::integral_constant<int, ROW_LOW>());
+    if (sv.S2 == 1) return f(std::integral_constant<int, ROW_HALF>());
+    return f(std::integral_constant<int, ROW_ANY>());
+}
+template <int MODE>
+__device__ __forceinline__ double row_diag(const RowPlan &P, long long di, int dl, int k1) {
+    if constexpr (MODE == ROW_ONE) return 0.25 * P.jm[0] * (double)k1;
+    if constexpr (MODE == ROW_HALF)
+        return (double)(long long)((unsigned long long)P.dsum - 2ull * (unsigned long long)di) * P.dscale;
+    const double d = (double)di * P.dscale;
+    return MODE == ROW_LOW ? fma((double)dl, P.dscale_low, d) : d;
+}
 template <class I, class T, class Acc, int NV, int MODE>
 __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P, const RowTabs<I, Acc> &Tb, I i,
                                          const T *__restrict__ x, int ld, int c0, Acc *acc, Acc *dg) {
@@ -162,7 +183,7 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
     Acc cp[2] = {Acc(0), Acc(0)};                  // the bond before: coefficients and gathered values
     T vp[2][NV];
     long long di = 0;
-    int k1 = 0;
+    int k1 = 0, dl = 0;
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
         acc[k] = Acc(0);
@@ -187,7 +208,10 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
         } else {
             const int kk = (S2 - 2 * ap) * (S2 - 2 * aq);
             if constexpr (MODE == ROW_ONE) k1 += kk;
-            else di += P.dC[c] * kk;
+            else {
+                di += P.dC[c] * kk;
+                if constexpr (MODE == ROW_LOW) dl += P.dL[c] * kk;
+            }
             const Acc *co = Tb.coef + ap * n1 + aq;
             if constexpr (MODE != ROW_ONE) co += c * 2 * n2;
             const bool dn = ap >= 1 && aq < S2, up = ap < S2 && aq >= 1;
@@ -216,8 +240,7 @@ __device__ __forceinline__ void row_hops(const SectorView &sv, const RowPlan &P,
         acc[k] = fma(cp[0], (Acc)vp[0][k], acc[k]);
         if constexpr (MODE != ROW_HALF) acc[k] = fma(cp[1], (Acc)vp[1][k], acc[k]);
     }
-    if constexpr (MODE == ROW_HALF) di = P.dsum - 2 * di;
-    *dg = MODE == ROW_ONE ? (Acc)(0.25 * P.jm[0] * (double)k1) : (Acc)((double)di * P.dscale);
+    *dg = (Acc)row_diag<MODE>(P, di, dl, k1);
 }
 
 // ---- the table form ------------------------------------------------------------------------

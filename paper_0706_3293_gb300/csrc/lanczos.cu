@@ -614,7 +614,7 @@ __global__ void k_store_nrm2(LzScalars *S, const double *__restrict__ part, int 
 // ---------------------------------------------------------------------------------------
 template <class I>
 static auto lz_row_kernel(const hm_lanczos *R) {
-    return R->basis->view.S2 == 1 ? k_lz_row<I, ROW_HALF> : R->rowp.nc == 1 ? k_lz_row<I, ROW_ONE> : k_lz_row<I, ROW_ANY>;
+    return row_dispatch(R->basis->view, R->rowp, [](auto mode) { return k_lz_row<I, mode()>; });
 }
 
 template <class I, class T, class Acc>

@@ -57,9 +57,7 @@ static int launch_matvec(const SectorView &sv, const BondParams &bp, const T *x,
             HM_CUDA(cudaGetLastError());
             return HM_OK;
         };
-        if (sv.S2 == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_HALF>);
-        if (P.nc == 1) return run(k_row_matvec<I, T, Acc, NV, ROW_ONE>);
-        return run(k_row_matvec<I, T, Acc, NV, ROW_ANY>);
+        return row_dispatch(sv, P, [&](auto mode) -> int { return run(k_row_matvec<I, T, Acc, NV, mode()>); });
     }
     sm = row_smem_bytes<I>(sv);
     HM_CUDA(raise_smem_limit(k_matvec<I, T, Acc, NV>, (int)sm));

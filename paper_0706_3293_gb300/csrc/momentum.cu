@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(ROW_NT) k_mom_row(SectorView sv, RowPlan P, in
         uint2 e0 = make_uint2(0u, none);
         T x1 = T(0);
         long long di = 0;
-        int k1 = 0;
+        int k1 = 0, dl = 0;
         bool other = false;                        // a target of shorter period was met
         auto step = [&](double cn, uint2 en) {
             acc = fma(c1, (double)x1, acc);
@@ -273,7 +273,10 @@ __global__ void __launch_bounds__(ROW_NT) k_mom_row(SectorView sv, RowPlan P, in
             } else {
                 const int kk = (S2 - 2 * ap) * (S2 - 2 * aq);
                 if constexpr (MODE == ROW_ONE) k1 += kk;
-                else di += P.dC[c] * kk;
+                else {
+                    di += P.dC[c] * kk;
+                    if constexpr (MODE == ROW_LOW) dl += P.dL[c] * kk;
+                }
                 const double *co = Tb.coef + (MODE == ROW_ONE ? 0 : c * 2 * n2) + ap * n1 + aq;
                 const bool dn = ap >= 1 && aq < S2, up = ap < S2 && aq >= 1;
                 step(co[0], entry(dn, jm));
@@ -294,8 +297,7 @@ __global__ void __launch_bounds__(ROW_NT) k_mom_row(SectorView sv, RowPlan P, in
                     acc = fma(kpi && (e.y & 1u) ? -f : f, (double)__ldg(x + e.x), acc);
                 }
             });
-        if constexpr (MODE == ROW_HALF) di = P.dsum - 2 * di;
-        const double dg = MODE == ROW_ONE ? 0.25 * P.jm[0] * (double)k1 : (double)di * P.dscale;
+        const double dg = row_diag<MODE>(P, di, dl, k1);
         y[r] = (T)(dg * (double)x[r] + sq[own >> 8] * acc);
     }
 }
@@ -380,19 +382,10 @@ int mom_matvec(const hm_basis *b, const BondParams &bp, const void *x, void *y, 
             HM_CUDA(cudaGetLastError());
             return HM_OK;
         };
-        const int mode = sv.S2 == 1 ? ROW_HALF : P.nc == 1 ? ROW_ONE : ROW_ANY;
-        if (dtype == HM_F64) {
-            const double *xv = (const double *)x;
-            double *yv = (double *)y;
-            if (mode == ROW_HALF) return run(k_mom_row<double, ROW_HALF>, xv, yv);
-            if (mode == ROW_ONE) return run(k_mom_row<double, ROW_ONE>, xv, yv);
-            return run(k_mom_row<double, ROW_ANY>, xv, yv);
-        }
-        const float *xv = (const float *)x;
-        float *yv = (float *)y;
-        if (mode == ROW_HALF) return run(k_mom_row<float, ROW_HALF>, xv, yv);
-        if (mode == ROW_ONE) return run(k_mom_row<float, ROW_ONE>, xv, yv);
-        return run(k_mom_row<float, ROW_ANY>, xv, yv);
+        return row_dispatch(sv, P, [&](auto mode) -> int {
+            if (dtype == HM_F64) return run(k_mom_row<double, mode()>, (const double *)x, (double *)y);
+            return run(k_mom_row<float, mode()>, (const float *)x, (float *)y);
+        });
     }
     if (dtype == HM_F64)
         k_mom_matvec<double><<<nblk, MOM_NT, 0, st>>>(sv, bp, kpi, b->view.dim, reps, map, (const double *)x,
