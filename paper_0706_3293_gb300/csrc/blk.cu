@@ -263,8 +263,21 @@ static int blk_plan_bonds(hm_basis *b, const BondParams &bp, const std::vector<i
             const long long C = pb_coef(*P, -bp.jm[t] / 2.0);
             P->pb_cl[t] = (int)(C & ((1ll << 27) - 1));
             P->pb_ch[t] = (int)(C >> 27);
+            P->pb_cw[t] = (float)(std::ldexp(-bp.jm[t] / 2.0, P->pb_s) - (double)C);
+            P->pb_wide |= P->pb_cw[t] != 0.0f;
             P->pb_cf[t] = (float)(-bp.jm[t] / 2.0);
         }
+    // g0 of the coefficients themselves, -sum_b (C_b + pb_cw) / 2, when their low parts count
+    if (P->pb_wide) {
+        long long c = 0;
+        double low = 0.0;
+        for (int t = 0; t < bp.nb; ++t) {
+            c += ((long long)P->pb_ch[t] << 27) + P->pb_cl[t];
+            low += (double)P->pb_cw[t];
+        }
+        P->pb_c0 = -(c >> 1);
+        P->pb_c0w = (float)(-0.5 * (low + (double)(c & 1)));
+    }
     // low groups keyed by (class, type, d); high and cross bonds by class
     std::map<std::tuple<int, int, int>, uint32_t> groups;
     std::vector<std::tuple<int, int, int>> hi[HM_BLK_MAXC], cr[HM_BLK_MAXC];   // (p, q, bond)
@@ -527,6 +540,7 @@ static int set_smem(K_t kern, size_t sm) {
 int blk_lz_plan(hm_basis *b, const BondParams &bp, int dtype, BlkParams *P, int *blocks) {
     int rc = blk_plan(b, bp, blk_K_of(b, bp, dtype == HM_F32, false), P);
     if (rc != 0) return rc;
+    if (dtype == HM_F32) P->pb_wide = 0;          // float rows read the float coefficients alone
     const size_t sm = blk_row_smem_bytes(*P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
     if (!P->rows_ok || sm > 200 * 1024) return 1;
     int per = 1;
@@ -862,6 +876,7 @@ const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int 
     if (nvec != 1) return nullptr;
     BlkParams P;
     if (blk_plan(b, bp, blk_K_of(b, bp, false, false), &P) != 0) return nullptr;
+    if (dtype == HM_F32) P.pb_wide = 0;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return nullptr;
     if (!P.perbond) return "k_blk_matvec";
     const void *k = nullptr;
@@ -929,6 +944,7 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
     BlkParams &P = m->P;
     const int rc = blk_plan(b, bp, multi ? K : blk_K_of(b, bp, false, false), &P);
     if (rc != 0) return rc;
+    if (dtype == HM_F32) P.pb_wide = 0;           // float rows read the float coefficients alone
     const int es = dtype == HM_F64 ? 8 : 4;
     m->multi = multi;
     m->smem = blk_row_smem_bytes(P, es, BLK_XPAD);

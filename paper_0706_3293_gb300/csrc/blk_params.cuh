@@ -74,14 +74,17 @@ struct BlkParams {
     // coefficients are integers scaled by 2^pb_s: C_b = round(h_b 2^pb_s), |C_b| < 2^56, so that
     // couplings down to 1/16 of the largest keep all 53 bits, pb_c0 = round(g0 2^pb_s), and a
     // row is one exact 128-bit sum, rounded once (PbSum, blk_sweep.cuh).  C_b is kept as the pair
-    // {C & (2^27 - 1), C >> 27}
+    // {C & (2^27 - 1), C >> 27}.  pb_wide: some coupling needs more, and pb_cw (pb_c0w for g0) is
+    // what C_b leaves of h_b 2^pb_s, |pb_cw| <= 1/2
     int perbond;
-    int pb_s;
+    int pb_s, pb_wide;
+    float pb_c0w;
     long long pb_c0;
     double pb_g0;
     uint8_t pb_lb[3][HM_BLK_SL], pb_xb[2][HM_BLK_SX];   // bond index of each low / cross slot
     uint8_t pb_hbb[HM_BLK_MAXB];                      // bond index of each high bond
     int pb_cl[HM_BLK_MAXB], pb_ch[HM_BLK_MAXB];       // C_b of each bond (bond order)
+    float pb_cw[HM_BLK_MAXB];
     float pb_cf[HM_BLK_MAXB];                         // h_b of each bond
     // bond-correlation plan (one chunk of bonds, per-bond slots): the block setup keeps the
     // high targets uncompacted, hbi[j] for high bond j or ~0 when its spins are parallel

@@ -62,8 +62,8 @@ struct BlkMetaXF {
 };
 struct BlkMetaX : BlkMetaXF {
     // per-bond plan (a spin-flip plan with classes allocates only the BlkMetaXF part):
-    // coefficient of each entry of hbi and of hbf, integer pair (C_b, FP64 rows) and float (FP32
-    // rows)
+    // coefficient of each entry of hbi and of hbf: FP64 rows C_b as a pair and pb_cw in hbcf / hbfcf,
+    // FP32 rows the float there
     int2 hbc[BLK_HBI], hbfc[HM_BLK_MAXB];
     float hbcf[BLK_HBI], hbfcf[HM_BLK_MAXB];
 };
@@ -146,9 +146,27 @@ struct PbSum {
     __device__ __forceinline__ __int128 value() const {
         return (__int128)s0 + ((__int128)(long long)(s1 - (unsigned long long)s0 - (unsigned long long)s2) << 27) + ((__int128)s2 << 54);
     }
+    // the whole row, with g0 x_i
+    __device__ __forceinline__ __int128 row(const BlkParams &P, int64_t xo) const { return (__int128)P.pb_c0 * xo + value(); }
 };
-template <class Sv> struct PbAcc { using T = PbSum; };
-template <> struct PbAcc<float> { using T = float; };
+// The same with the low parts of the coefficients (BlkParams::pb_wide: couplings less than 1/16 of the largest
+// whose bits reach below the unit).  Their sum is at most 2^-57 of the largest coupling times x, so a float of 24 bits and
+// the upper 22 bits of d do: no 64-bit product, one register.  Products N = 24 181 -> 198 us, N = 26 684 -> 735; with
+// the low parts as two more 64-bit sums 247 and 934.
+struct PbSumW : PbSum {
+    float w;                                          // in units of 2^32
+    __device__ __forceinline__ PbSumW(int) : PbSum(0), w(0.0f) {}
+    // d >> 32 as a float, |d| <= 2^54 (1.5 2^23 holds it in its low bits)
+    static __device__ __forceinline__ float upper(int64_t d) { return __int_as_float(0x4B400000 + (int)(d >> 32)) - 12582912.0f; }
+    __device__ __forceinline__ __int128 row(const BlkParams &P, int64_t xo) const {
+        return PbSum::row(P, xo) + (long long)(fmaf(P.pb_c0w, upper(xo), w) * 4294967296.0f);
+    }
+};
+template <class Sv, bool W> struct PbAcc { using T = PbSum; };
+template <class Sv> struct PbAcc<Sv, true> { using T = PbSumW; };
+template <> struct PbAcc<float, false> { using T = float; };
+template <> struct PbAcc<float, true> { using T = float; };
+// a += the coefficient times d: C_b = {c0, c1} and cf = pb_cw for integers, cf = h_b for floats
 __device__ __forceinline__ PbSum pb_mac(int c0, int c1, float, int64_t d, PbSum a) {
     const int d0 = (int)d & 0x7FFFFFF, d1 = (int)(d >> 27);
     a.s0 += (long long)c0 * d0;
@@ -156,7 +174,12 @@ __device__ __forceinline__ PbSum pb_mac(int c0, int c1, float, int64_t d, PbSum 
     a.s2 += (long long)c1 * d1;
     return a;
 }
-__device__ __forceinline__ float pb_mac(int, int, float Cf, float d, float a) { return fmaf(Cf, d, a); }
+__device__ __forceinline__ PbSumW pb_mac(int c0, int c1, float cf, int64_t d, PbSumW a) {
+    (PbSum &)a = pb_mac(c0, c1, 0.0f, d, (const PbSum &)a);
+    a.w = fmaf(cf, PbSumW::upper(d), a.w);
+    return a;
+}
+__device__ __forceinline__ float pb_mac(int, int, float cf, float d, float a) { return fmaf(cf, d, a); }
 
 __device__ __forceinline__ double i128_to_double(__int128 v) {
     const long long hi = (long long)(v >> 64);
@@ -166,15 +189,14 @@ __device__ __forceinline__ double i128_to_double(__int128 v) {
 
 // high exchanges of a per-bond plan (class 0 lists), four gathers at a time; flipped
 // targets carry the parity
-template <class Sv, class G>
-__device__ __forceinline__ typename PbAcc<Sv>::T blk_high_pb(const BlkParams &P, const BlkMeta &B,
-                                                             const unsigned char *Xg, uint32_t r, const G &gx,
-                                                             Sv xo, typename PbAcc<Sv>::T a) {
+template <class Sv, class G, class A>
+__device__ __forceinline__ A blk_high_pb(const BlkParams &P, const BlkMeta &B, const unsigned char *Xg, uint32_t r,
+                                         const G &gx, Sv xo, A a) {
     const BlkMetaX &X = *B.x;
     const int e1 = B.he[0];
     const uint4 *h4 = reinterpret_cast<const uint4 *>(B.hbi);
     auto mac = [&](int e, Sv v) {
-        if constexpr (sizeof(Sv) == 8) a = pb_mac(X.hbc[e].x, X.hbc[e].y, 0.0f, xo - v, a);
+        if constexpr (sizeof(Sv) == 8) a = pb_mac(X.hbc[e].x, X.hbc[e].y, X.hbcf[e], xo - v, a);
         else a = pb_mac(0, 0, X.hbcf[e], xo - v, a);
     };
     int e = B.hs[0];
@@ -552,7 +574,7 @@ __device__ __forceinline__ void blk_sweep(const BlkParams &P, const unsigned cha
                 const int f0 = popc_below(fm, P.hb_start[c]), f1 = popc_below(fm, P.hb_start[c + 1]);
                 if (tid >= P.hb_start[c] && tid < P.hb_start[c + 1]) {
                     const int pb = P.pb_hbb[tid];
-                    const float cf = P.pb_cf[pb];
+                    const float cf = sizeof(Sv) == 8 ? P.pb_cw[pb] : P.pb_cf[pb];
                     if (hval) {
                         B.hbi[start + popc_below(hm, tid) - b0] = hidx;
                         if (P.perbond) {
@@ -683,9 +705,8 @@ __device__ __forceinline__ void matvec_body(const BlkParams &P, const T *__restr
         if constexpr (Row::kPerBond) {
             const double sy = ef::pow2d(u - P.pb_s);
             blk_sweep<int64_t, NC, false, Row>(P, (const unsigned char *)x, GF64{E}, nullptr, [](uint32_t) { return 0; },
-                                          [&](uint32_t off, uint32_t r, int64_t xo, const PbSum &sv, int) {
-                                              const __int128 t = (__int128)P.pb_c0 * xo + sv.value();
-                                              yb[off + r] = ef::d2u(i128_to_double(t) * sy);
+                                          [&](uint32_t off, uint32_t r, int64_t xo, const typename Row::template PbT<int64_t> &sv, int) {
+                                              yb[off + r] = ef::d2u(i128_to_double(sv.row(P, xo)) * sy);
                                           },
                                           [](int) {}, [](uint32_t, int) {});
         } else {
@@ -858,12 +879,6 @@ __device__ __forceinline__ void lz64_body(const BlkParams &P, const long long *_
         }
     };
     const double sy = ef::pow2d(u - P.pb_s);
-    auto rowb = [&](uint32_t off, uint32_t r, int64_t xo, const PbSum &sv, int) {
-        const __int128 t = (__int128)P.pb_c0 * xo + sv.value();
-        const unsigned long long yb = ef::d2u(i128_to_double(t) * sy);
-        __stcs(Y + off + r, yb);
-        d1f = ef::df_add(d1f, ef::df_mul(ef::df_from_fix(xo, E, 0, E - 1023), ef::df_from_bits(yb, E - 1023)));
-    };
     constexpr bool exact = IR && !Row::kPerBond;
     auto endf = [&](int it) {
             const double a = blk_dot_warp(exact, d1, d1f);
@@ -873,10 +888,15 @@ __device__ __forceinline__ void lz64_body(const BlkParams &P, const long long *_
     auto flushf = [&](uint32_t h, int it) {
             part[h] = blk_dot_scaled(P, exact, E, blk_pairwise([&](int w) { return s_wpart[it & 1][w][0]; }));
         };
-    if constexpr (Row::kPerBond)
+    if constexpr (Row::kPerBond) {
+        auto rowb = [&](uint32_t off, uint32_t r, int64_t xo, const typename Row::template PbT<int64_t> &sv, int) {
+            const unsigned long long yb = ef::d2u(i128_to_double(sv.row(P, xo)) * sy);
+            __stcs(Y + off + r, yb);
+            d1f = ef::df_add(d1f, ef::df_mul(ef::df_from_fix(xo, E, 0, E - 1023), ef::df_from_bits(yb, E - 1023)));
+        };
         blk_sweep<int64_t, NC, true, Row>(P, (const unsigned char *)Xc, GFix{}, S->sched, [](uint32_t) { return 0; },
                                           rowb, endf, flushf);
-    else
+    } else
         blk_sweep<int64_t, NC, true, Row>(P, (const unsigned char *)Xc, GFix{}, S->sched, [](uint32_t) { return 0; },
                                           rowc, endf, flushf);
 }

@@ -290,20 +290,24 @@ std::string gen_row_table(const BlkParams &P) {
 // a fixed address (a broadcast) and adds a zero difference.
 std::string gen_row_pb_table(const BlkParams &P);
 
+// coefficient arguments of hm::pb_mac: C_b (integer, FP64 rows) and pb_cw (wide FP64 rows) or h_b (FP32 rows), read
+// from the kernel parameters; the accumulator of the rows
+std::string pb_args(const BlkParams &P, int t) {
+    const std::string i = std::to_string(t);
+    return "P.pb_cl[" + i + "], P.pb_ch[" + i + "], " + (P.pb_wide ? "P.pb_cw[" : "P.pb_cf[") + i + "]";
+}
+std::string pb_acc(const BlkParams &P) { return P.pb_wide ? "typename hm::PbAcc<Sv, true>::T" : "typename hm::PbAcc<Sv, false>::T"; }
+
 std::string gen_row_pb(const BlkParams &P) {
     if (P.tt) return gen_row_pb_table(P);
-    // coefficient arguments of hm::pb_mac: C_b (integer, FP64 rows) and h_b (float, FP32 rows),
-    // read from the kernel parameters
-    auto cf = [&](int t) {
-        const std::string i = std::to_string(t);
-        return "P.pb_cl[" + i + "], P.pb_ch[" + i + "], P.pb_cf[" + i + "]";
-    };
+    auto cf = [&](int t) { return pb_args(P, t); };
     std::string s;
     s += "struct RowJit {\n"
          "static constexpr int kPad = hm::BLK_XPAD;\n"
          "static constexpr bool kRelUS = false;\n"
          "static constexpr bool kPerBond = true;\n"
          "static constexpr bool kBC = false;\n"
+         "template <class Sv> using PbT = " + pb_acc(P) + ";\n"
          "template <class Sv>\n"
          "static __device__ __forceinline__ void stage(const hm::BlkParams &P, unsigned char *dyn) {\n"
          "    hm::RowGeneric<1>::stage<Sv>(P, dyn);\n"
@@ -311,14 +315,14 @@ std::string gen_row_pb(const BlkParams &P) {
          "template <class Sv>\n"
          "static __device__ __forceinline__ void block(const hm::BlkParams &, uint32_t) {}\n"
          "template <class Sv, class G>\n"
-         "static __device__ __forceinline__ typename hm::PbAcc<Sv>::T sums_pb(const hm::BlkParams &P,\n"
+         "static __device__ __forceinline__ PbT<Sv> sums_pb(const hm::BlkParams &P,\n"
          "        const hm::BlkMeta &B, const unsigned char *Xsb, const unsigned char *Xg, uint32_t l, uint32_t r,\n"
          "        const G &gx, Sv xo) {\n"
          "    const uint32_t l4 = l << 2, lh4 = (l >> 8) << 2, lh4k = lh4 | B.kofs;\n"
          "    const uint32_t R0own = hm::r0s_at(l4 & 0x3FCu), R1own = hm::us_at(lh4k);\n"
          "    const uint32_t zo = (uint32_t)((P.max_block + hm::BLK_XPAD - 1) * sizeof(Sv));   // fixed address\n"
          "    (void)R0own; (void)R1own; (void)lh4; (void)gx; (void)zo;\n"
-         "    typename hm::PbAcc<Sv>::T a(0);\n";
+         "    PbT<Sv> a(0);\n";
     std::set<int> ds;
     for (int t = 0; t < 3; ++t)
         for (int k = 0; k < P.ln[0][t]; ++k) ds.insert(P.ld[0][t][k]);
@@ -359,27 +363,25 @@ std::string gen_row_pb(const BlkParams &P) {
 // exchange is not allowed, so that h_b (x_i - x_t) is zero without a test -- and cross slots
 // take the rank of l ^ 2^p from the table.
 std::string gen_row_pb_table(const BlkParams &P) {
-    auto cf = [&](int t) {
-        const std::string i = std::to_string(t);
-        return "P.pb_cl[" + i + "], P.pb_ch[" + i + "], P.pb_cf[" + i + "]";
-    };
+    auto cf = [&](int t) { return pb_args(P, t); };
     std::string s;
     s += "struct RowJit {\n"
          "static constexpr int kPad = hm::BLK_XPAD;\n"
          "static constexpr bool kRelUS = false;\n"
          "static constexpr bool kPerBond = true;\n"
          "static constexpr bool kBC = false;\n"
+         "template <class Sv> using PbT = " + pb_acc(P) + ";\n"
          "template <class Sv>\n"
          "static __device__ __forceinline__ void stage(const hm::BlkParams &, unsigned char *) {}\n"
          "template <class Sv>\n"
          "static __device__ __forceinline__ void block(const hm::BlkParams &, uint32_t) {}\n"
          "template <class Sv, class G>\n"
-         "static __device__ __forceinline__ typename hm::PbAcc<Sv>::T sums_pb(const hm::BlkParams &P,\n"
+         "static __device__ __forceinline__ PbT<Sv> sums_pb(const hm::BlkParams &P,\n"
          "        const hm::BlkMeta &B, const unsigned char *Xsb, const unsigned char *Xg, uint32_t l, uint32_t r,\n"
          "        const G &gx, Sv xo) {\n"
          "    (void)l; (void)Xg;\n"
          "    const uint4 *tt = P.tt + (B.lwo + r);\n"
-         "    typename hm::PbAcc<Sv>::T a(0);\n";
+         "    PbT<Sv> a(0);\n";
     const int nch = (P.tt_n + 7) / 8;
     for (int j = 0; j < nch; ++j) put(s, "    const uint4 q%d = hm::ldg_v4(tt + %uu);\n", j, (unsigned)j * P.tt_stride);
     static const char *comp[4] = {"x", "y", "z", "w"};

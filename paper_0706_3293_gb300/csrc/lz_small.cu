@@ -27,11 +27,12 @@ struct GFixCg {                      // fixed-point copy, written during the ker
     }
 };
 
-// row sum of a per-bond plan with its target table: low slots, cross slots, high list
-__device__ __forceinline__ PbSum lzs_row_pb(const BlkParams &P, const BlkMeta &B, const unsigned char *Xsb,
-                                            const unsigned char *Xg, uint32_t l, uint32_t r, int64_t xo) {
+// row sum of a per-bond plan with its target table: low slots, cross slots, high list (A: PbSum or PbSumW)
+template <class A>
+__device__ __forceinline__ A lzs_row_pb(const BlkParams &P, const BlkMeta &B, const unsigned char *Xsb,
+                                        const unsigned char *Xg, uint32_t l, uint32_t r, int64_t xo) {
     const GFixCg gx;
-    PbSum a(0);
+    A a(0);
     const uint32_t g = B.lwo + r;
     const uint4 *tt = P.tt + g;
     for (int e0 = 0; e0 < P.tt_nsgl; e0 += 8, tt += P.tt_stride) {
@@ -42,7 +43,7 @@ __device__ __forceinline__ PbSum lzs_row_pb(const BlkParams &P, const BlkMeta &B
             if (e0 + k >= P.tt_nsgl) break;
             const uint32_t o = k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xFFFFu;
             const int b = P.tt_pb[e0 + k];
-            a = pb_mac(P.pb_cl[b], P.pb_ch[b], 0.0f, xo - *(const int64_t *)(Xsb + o), a);
+            a = pb_mac(P.pb_cl[b], P.pb_ch[b], P.pb_cw[b], xo - *(const int64_t *)(Xsb + o), a);
         }
     }
     for (int t = 0; t < 2; ++t)
@@ -52,7 +53,7 @@ __device__ __forceinline__ PbSum lzs_row_pb(const BlkParams &P, const BlkMeta &B
             if ((l ^ x_.wm) & x_.vm) {
                 const int e = P.tt_xe[d], b = P.pb_xb[t][s];
                 const uint32_t v_ = __ldg((const uint16_t *)P.tt + ((size_t)(e >> 3) * P.tt_stride + g) * 8 + (e & 7));
-                a = pb_mac(P.pb_cl[b], P.pb_ch[b], 0.0f, xo - gx(x_.base + v_), a);
+                a = pb_mac(P.pb_cl[b], P.pb_ch[b], P.pb_cw[b], xo - gx(x_.base + v_), a);
             }
         }
     return blk_high_pb<int64_t>(P, B, Xg, r, gx, xo, a);
@@ -88,13 +89,13 @@ __device__ __forceinline__ bool lzs_barrier(unsigned *bar, unsigned target, unsi
     return s_ok != 0;
 }
 
-// NC: coupling classes (1, 2, 4), or 0 for a per-bond plan
+// NC: coupling classes (1, 2, 4), or 0 for a per-bond plan, -1 for one with low parts (pb_wide)
 template <int NC, bool PSI>
 __global__ void __launch_bounds__(BLK_NT, 2) k_lz_small(BlkParams P, LzSmallArgs a) {
     if (a.S->done) return;
     extern __shared__ __align__(16) unsigned char smem[];
-    constexpr bool PB = NC == 0;
-    constexpr int NCA = NC == 0 ? 1 : NC;
+    constexpr bool PB = NC <= 0;
+    constexpr int NCA = PB ? 1 : NC;
     const int tid = threadIdx.x, nt = blockDim.x, ctas = gridDim.x, nh = 1 << P.H;
     int64_t *Xs = (int64_t *)smem;
     BlkMeta &B = *(BlkMeta *)(smem + blk_row_xs_bytes(P, 8, BLK_XPAD));
@@ -151,7 +152,10 @@ __global__ void __launch_bounds__(BLK_NT, 2) k_lz_small(BlkParams P, LzSmallArgs
             if (e < P.nhb && e >= P.hb_start[c] && e < P.hb_start[c + 1] && ((hm >> e) & 1ull)) {
                 const int i = start + popc_below(hm, e) - b0;
                 B.hbi[i] = blk_off(P, tb, h ^ ((1u << P.hb_p[e]) | (1u << P.hb_q[e])), k);
-                if (PB) BX->hbc[i] = make_int2(P.pb_cl[P.pb_hbb[e]], P.pb_ch[P.pb_hbb[e]]);
+                if (PB) {
+                    BX->hbc[i] = make_int2(P.pb_cl[P.pb_hbb[e]], P.pb_ch[P.pb_hbb[e]]);
+                    BX->hbcf[i] = P.pb_cw[P.pb_hbb[e]];
+                }
             }
             if (e == c) {
                 B.hs[c] = start;
@@ -204,8 +208,8 @@ __global__ void __launch_bounds__(BLK_NT, 2) k_lz_small(BlkParams P, LzSmallArgs
             if (r >= n) continue;
             const int64_t xo = Xs[r];
             if constexpr (PB) {
-                const __int128 t = (__int128)P.pb_c0 * xo + lzs_row_pb(P, B, smem, Xg, low[j], r, xo).value();
-                yb[j] = ef::d2u(i128_to_double(t) * sy);
+                const auto sv = lzs_row_pb<typename PbAcc<int64_t, NC == -1>::T>(P, B, smem, Xg, low[j], r, xo);
+                yb[j] = ef::d2u(i128_to_double(sv.row(P, xo)) * sy);
             } else {
                 int64_t acc[NCA], Tc[NCA], ts = 0;
                 int cnt[NCA];
@@ -311,6 +315,7 @@ __global__ void __launch_bounds__(BLK_NT, 2) k_lz_small(BlkParams P, LzSmallArgs
 }
 
 const void *lzs_kernel(const BlkParams &P, bool psi) {
+    if (P.perbond && P.pb_wide) return psi ? (const void *)k_lz_small<-1, true> : (const void *)k_lz_small<-1, false>;
     if (P.perbond) return psi ? (const void *)k_lz_small<0, true> : (const void *)k_lz_small<0, false>;
     if (P.nc == 1) return psi ? (const void *)k_lz_small<1, true> : (const void *)k_lz_small<1, false>;
     if (P.nc == 2) return psi ? (const void *)k_lz_small<2, true> : (const void *)k_lz_small<2, false>;
