@@ -29,7 +29,8 @@ namespace hm {
 // diagonal is an exact integer sum, converted once a row.  The gathers of one bond are in flight
 // while those of the bond before are added.  Measured (s = 3/2 ring, N = 12, 1.7 M rows, FP64):
 // k_matvec, the table form, 362 us; this form 110 us.
-template <class I> struct alignas(4 * sizeof(I)) RowEF { I ep, fp, em, fm; };
+// Aligned to a 16-byte shared load at most: the tables start on 16 bytes, behind the coefficients.
+template <class I> struct alignas(16) RowEF { I ep, fp, em, fm; };
 template <class I> struct alignas(2 * sizeof(I)) RowG { I gp, gm; };
 
 constexpr int ROW_NT = 256;          // threads per CTA of the row kernels
