@@ -92,6 +92,30 @@ int build_tables(int n_sites, int two_s, int two_m, hm_basis *b) {
     return HM_OK;
 }
 
+int upload_table(const void *host, size_t bytes, void **dev, const char *what) {
+    const CaptureRelaxed relaxed;
+    HM_CUDA(cudaMalloc(dev, bytes));
+    // a copy on the null stream would join the capture of a blocking stream
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(cudaStreamLegacy, &cs);
+    if (e == cudaErrorStreamCaptureImplicit) {
+        cudaGetLastError();
+        cudaStream_t st = nullptr;
+        e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(*dev, host, bytes, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+        if (st) cudaStreamDestroy(st);
+    } else if (e == cudaSuccess) {
+        e = cudaMemcpy(*dev, host, bytes, cudaMemcpyHostToDevice);
+    }
+    if (e != cudaSuccess) {
+        cudaFree(*dev);
+        *dev = nullptr;
+        return cuda_fail(e, what);
+    }
+    return HM_OK;
+}
+
 int sm_count() {
     static int n = 0;
     if (n == 0) {

@@ -94,9 +94,7 @@ static int blk_tables(hm_basis *b, int K, const void **dev, int *bytes, int *oU,
         memcpy(host.data() + t.oR0, R0.data(), 256);
         memcpy(host.data() + t.oC, C.data(), C.size() * 4);
         memcpy(host.data() + olw, lw.data(), lw.size() * 2);
-        HM_CUDA(cudaMalloc(&t.dev, total));
-        cudaError_t e = cudaMemcpy(t.dev, host.data(), total, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) { cudaFree(t.dev); return cuda_fail(e, "block tables"); }
+        HM_TRY(upload_table(host.data(), total, &t.dev, "block tables"));
         t.lw = (uint16_t *)((unsigned char *)t.dev + olw);
         it = b->blk_tabs.emplace(K, t).first;
     }
@@ -696,9 +694,7 @@ int blk_target_table(hm_basis *b, BlkParams *P, int esize, bool build) {
                 put(2 * ntri + nsgl + (int)i, rank[l ^ (1u << cps[i])] * (uint32_t)esize);
         }
         void *dev = nullptr;
-        HM_CUDA(cudaMalloc(&dev, host.size() * 2));
-        cudaError_t e = cudaMemcpy(dev, host.data(), host.size() * 2, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) { cudaFree(dev); return cuda_fail(e, "target table"); }
+        HM_TRY(upload_table(host.data(), host.size() * 2, &dev, "target table"));
         it = b->blk_ttabs.emplace(key, dev).first;
     }
     P->tt = (const uint4 *)it->second;
@@ -933,6 +929,12 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
                 return 0;
             }
     }
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    HM_CUDA(cudaStreamIsCapturing(st, &cs));
+    if (multi && cs != cudaStreamCaptureStatusNone) {         // no table of this split: none for the list either
+        std::lock_guard<std::mutex> lk(b->tab_mu);
+        if (!b->blk_tabs.count(K)) return 1;
+    }
     auto m = std::make_shared<BlkMvPlan>();
     if (multi) {             // class plans of a plain basis only, as the general rows; decided before any planning
         std::vector<double> cls;
@@ -950,11 +952,9 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
     m->smem = blk_row_smem_bytes(P, es, BLK_XPAD);
     if (!multi && (!P.rows_ok || m->smem > 200 * 1024)) return 1;
     // target tables: built on the first product of a layout, but for class plans neither inside a
-    // stream capture (no allocation there) nor without end on a basis that sees many bond lists; the
+    // stream capture (work there is the caller's) nor without end on a basis that sees many bond lists; the
     // generic rows then serve, with the same result (FP64: the same exact sums)
     bool build = true;
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    HM_CUDA(cudaStreamIsCapturing(st, &cs));
     if (!P.perbond) {
         std::lock_guard<std::mutex> lk(b->tab_mu);
         build = cs == cudaStreamCaptureStatusNone && b->blk_ttabs.size() < 32;

@@ -93,6 +93,9 @@ struct CaptureRelaxed {
     CaptureRelaxed(const CaptureRelaxed &) = delete;
 };
 
+// device copy of a host table (the caller's to free), also while streams are being captured
+int upload_table(const void *host, size_t bytes, void **dev, const char *what);
+
 // Slots of HM_EPART ints for the exponent maxima of a product's vector, from the kernel that forms them to
 // the product that reads them (blk.cu, ExpPart).  No two calls that may run at the same time share one:
 //   * the first HM_ESLOTS streams that a basis sees have one each (calls of one stream are in order);
