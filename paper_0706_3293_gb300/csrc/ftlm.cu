@@ -737,10 +737,11 @@ __global__ void __launch_bounds__(FT_X_NT) k_ft_exact(FtParams F, BondParams bp,
                 if (k == 0) { p = m - 1; q = round; }
                 else { p = (round + k) % (m - 1); q = (round - k + (m - 1)) % (m - 1); }
                 if (p > q) { const int tt = p; p = q; q = tt; }
-                // tan 2 theta = 2 apq / (aqq - app), |theta| <= pi / 4
+                // tan 2 theta = 2 apq / (aqq - app), |theta| <= pi / 4.  The largest element is in [1, 2): an apq
+                // below 2^-500 counts as zero, as r2 would otherwise leave the normal numbers and c^2 + s^2 one
                 const double dd = H[(size_t)q * m + q] - H[(size_t)p * m + p], h2 = 2.0 * H[(size_t)p * m + q];
                 const double r2 = dd * dd + h2 * h2, ri = rsqrt(r2);
-                const bool on = h2 != 0.0 && r2 > 0.0;
+                const bool on = fabs(h2) > 0x1p-500;
                 const double x = fma(0.5 * fabs(dd), ri, 0.5), rx = rsqrt(x);
                 sp[k] = p;
                 sq[k] = q;
