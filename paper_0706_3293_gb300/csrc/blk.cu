@@ -79,13 +79,15 @@ static int blk_tables(hm_basis *b, int K, const void **dev, int *bytes, int *oU,
         // popcount numerically)
         std::vector<uint16_t> lw((size_t)1 << K);
         {
-            size_t w = 0;
+            int at[17];                               // next place of each popcount (K <= 16)
+            uint64_t c = 1;
+            t.lwoff[0] = 0;
             for (int k = 0; k <= K; ++k) {
-                t.lwoff[k] = (int)w;
-                for (uint32_t l = 0; l < (1u << K); ++l)
-                    if (__builtin_popcount(l) == k) lw[w++] = (uint16_t)l;
+                at[k] = t.lwoff[k];
+                t.lwoff[k + 1] = t.lwoff[k] + (int)c;
+                c = c * (K - k) / (k + 1);
             }
-            t.lwoff[K + 1] = (int)w;
+            for (uint32_t l = 0; l < (1u << K); ++l) lw[at[__builtin_popcount(l)]++] = (uint16_t)l;
         }
         const size_t olw = al16(t.bytes);
         const size_t total = olw + lw.size() * 2;
