@@ -883,6 +883,7 @@ const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int 
 
 // several vectors at once (blk_multi.cu)
 int blk_hop_table(hm_basis *b, const BlkParams &P, const HopTab &H, bool build, const uint16_t **table);
+bool blk_multi_serves(uint64_t dim, int H, int K, int A, int nvec);
 bool blk_multi_orders(const double *gd, int nc, int *oc);
 int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table, const double *gd, const int *oc,
                      const void *x, void *y, int dtype, int nvec, cudaStream_t st);
@@ -914,14 +915,16 @@ static int blk_env() {
 }
 
 // 0 and the plan, or 1 when the block path does not apply
-static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi, cudaStream_t st,
+static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, int nvec, cudaStream_t st,
                        std::shared_ptr<const BlkMvPlan> *out) {
-    if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB) return 1;
+    const bool multi = nvec > 1;
+    if (b->view.S2 != 1 || b->view.N < 10 || b->view.N > 32 || bp.nb > HM_BLK_MAXB) return 1;
     // Blocks of several vectors are cut into parts, so their split has no reason to keep them small: 13 low
     // sites, fewer blocks to set up and fewer scattered cross exchanges (N = 20, eight vectors, FP64:
     // K = 11 / 12 / 13 / 14 90 / 86 / 80 / 80 us; N = 23 531 / 527 / 523 / 520)
     const int K = multi && !getenv("HM_BLK_K") ? std::min(13, b->view.N - 2) : blk_K(b, false);
     const int env = blk_env(), nb = bp.nb;
+    if (multi && !blk_multi_serves(b->view.dim, b->view.N - K, K, b->view.A, nvec)) return 1;
     {
         std::lock_guard<std::mutex> lk(b->tab_mu);
         for (const auto &m : b->mv_plans)
@@ -999,7 +1002,7 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, bool multi,
 int blk_matvec(hm_basis *b, const BondParams &bp, const void *x, void *y, int dtype, int nvec,
                cudaStream_t st) {
     std::shared_ptr<const BlkMvPlan> m;
-    const int rc = blk_mv_plan(b, bp, dtype, nvec > 1, st, &m);
+    const int rc = blk_mv_plan(b, bp, dtype, nvec, st, &m);
     if (rc != 0) return rc;
     if (nvec > 1) return blk_multi_launch(m->P, m->hop, m->hops, m->gd, m->oc, x, y, dtype, nvec, st);
     ExpPart E;

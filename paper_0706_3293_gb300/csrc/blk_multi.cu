@@ -320,6 +320,27 @@ int blk_hop_table(hm_basis *b, const BlkParams &P, const HopTab &H, bool build, 
     return HM_OK;
 }
 
+// blocks of the sector: high words that leave 0 .. K ones to the low part
+static int blk_multi_blocks(int H, int K, int A) {
+    int valid = 0;
+    for (int c = std::max(0, A - K); c <= std::min(H, A); ++c) {
+        uint64_t b = 1;
+        for (int i = 0; i < c; ++i) b = b * (H - i) / (i + 1);
+        valid += (int)b;
+    }
+    return valid;
+}
+
+// Whether blocks are the faster form for nvec vectors: a CTA sets a block up and takes 256 / (lanes a row) rows
+// at a time, so sectors far from M = 0, whose blocks have few rows, leave it idle.  The line is at
+// rows a block times (vectors + 4) = 480.  Measured (J1-J2 ring, FP64, us, blocks / general rows):
+//   N = 32, 5 ones (12 rows a block): 2 vectors 1228 / 65, 8 vectors 1253 / 211, 32 vectors 1367 / 903
+//   N = 30, 7 ones (49): 610 / 492, 1146 / 1698, 3275 / 7673    N = 28, 7 ones (72): 243 / 269, 592 / 934, 1922 / 4268
+//   N = 24, 5 ones (42): 42 / 23, 51 / 59, 117 / 247            N = 26, 8 ones (220): 209 / 324, 683 / 1147, 2490 / 5429
+bool blk_multi_serves(uint64_t dim, int H, int K, int A, int nvec) {
+    return dim * (uint64_t)(std::min(nvec, 32) + 4) >= 480ull * (uint64_t)blk_multi_blocks(H, K, A);
+}
+
 // binary orders of each |J_c| below the largest (gd: the -J_c / 4 of nc classes); false when the integer sums
 // do not serve them
 bool blk_multi_orders(const double *gd, int nc, int *oc) {
@@ -344,11 +365,7 @@ int blk_multi_launch(const BlkParams &P, const HopTab &H, const uint16_t *table,
     memcpy(a.gd, gd, sizeof a.gd);
     memcpy(a.oc, oc, sizeof a.oc);
     a.ld = nvec;
-    int valid = 0;
-    for (uint32_t h = 0; h < (1u << P.H); ++h) {
-        const int k = P.A - __builtin_popcount(h);
-        valid += k >= 0 && k <= P.K;
-    }
+    const int valid = blk_multi_blocks(P.H, P.K, P.A);
     const size_t sm = hops_bytes(P);
     for (a.c0 = 0; a.c0 < nvec; a.c0 += a.w) {
         a.w = std::min(32, nvec - a.c0);

@@ -135,14 +135,15 @@ def test_many_high_sites(hm, n, two_m, nvec):
     assert (np.abs(got - y) <= (len(u) + 16) * 3 * 2.0**-24 * (bound + np.abs(J).sum() / 4 * np.abs(x32))).all()
 
 
-@pytest.mark.parametrize("n,two_m", [(24, 0), (30, 16), (32, 20)])
-def test_up_to_nineteen_high_sites(hm, n, two_m):
-    """Against the products of single vectors, exact sums rounded once: row sums of |H| are at most 3/4 sum |J|."""
+@pytest.mark.parametrize("n,two_m,nvec", [(24, 0, 2), (30, 16, 32), (32, 20, 32), (32, 20, 2), (32, -22, 33)])
+def test_up_to_nineteen_high_sites(hm, n, two_m, nvec):
+    """Against the products of single vectors, exact sums rounded once: row sums of |H| are at most 3/4 sum |J|.
+    The last two sectors have too few rows a block and take the general rows."""
     b = hm.Basis(n, 1, two_m)
     u, v, J = W.ring_bonds(n, -1.0, -0.3)
     bl = hm.BondList.make(u, v, J)
-    x = torch.rand((b.dim, 2), dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n)) - 0.5
+    x = torch.rand((b.dim, nvec), dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(n)) - 0.5
     got = hm.matvec(b, bl, x)
-    for k in range(2):
+    for k in {0, 1, nvec - 1}:
         ref = hm.matvec(b, bl, x[:, k].contiguous())
         assert (got[:, k] - ref).abs().max().item() <= rounding(u, J) * 0.75 * np.abs(J).sum() * 0.5
