@@ -507,7 +507,8 @@ int blk_K(const hm_basis *b, bool fp32_run) {
 // The split of a bond list: blk_K, or the next larger K whose slots hold the list (fewer blocks, so the
 // workspaces sized by blk_K hold them; HM_BLK_K is taken as it is).  The smallest is the fastest also where
 // it has no target table and a larger one does (FP64 Lanczos product and alpha, us: square 6 x 3 at
-// K = 12 / 15 38 / 51, honeycomb of 20 sites at K = 12 / 14 49 / 54).
+// K = 12 / 15 38 / 51, honeycomb of 20 sites at K = 12 / 14 49 / 54).  -1: no split holds the list, so that it
+// leaves for the general rows before any planning.
 static int blk_K_of(const hm_basis *b, const BondParams &bp, bool fp32_run, bool bond_corr) {
     const int k0 = blk_K(b, fp32_run);
     if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB || getenv("HM_BLK_K")) return k0;
@@ -538,7 +539,9 @@ static int set_smem(K_t kern, size_t sm) {
 
 // Lanczos hooks: plan (0 = block path usable), attribute setup, launch
 int blk_lz_plan(hm_basis *b, const BondParams &bp, int dtype, BlkParams *P, int *blocks) {
-    int rc = blk_plan(b, bp, blk_K_of(b, bp, dtype == HM_F32, false), P);
+    const int K = blk_K_of(b, bp, dtype == HM_F32, false);
+    if (K < 0) return 1;
+    int rc = blk_plan(b, bp, K, P);
     if (rc != 0) return rc;
     if (dtype == HM_F32) P->pb_wide = 0;          // float rows read the float coefficients alone
     const size_t sm = blk_row_smem_bytes(*P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
@@ -839,7 +842,8 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
             bc.jm[i] = bp.jm[c0 + i]; bc.jmf[i] = bp.jmf[c0 + i];
         }
         BlkParams &P = plans[c];
-        if (blk_plan(b, bc, blk_K_of(b, bc, false, true), &P, true) != 0 || !P.rows_ok) return 1;
+        const int K = blk_K_of(b, bc, false, true);
+        if (K < 0 || blk_plan(b, bc, K, &P, true) != 0 || !P.rows_ok) return 1;
         const size_t sm = blk_row_smem_bytes(P, es, BLK_XPAD);
         if (sm > 200 * 1024 || jit_bc_kernel(P, dtype, nbk, &kerns[c]) != 0) return 1;
         if (raise_smem_limit(kerns[c], (int)sm) != cudaSuccess) {
@@ -873,7 +877,8 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
 const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int nvec) {
     if (nvec != 1) return nullptr;
     BlkParams P;
-    if (blk_plan(b, bp, blk_K_of(b, bp, false, false), &P) != 0) return nullptr;
+    const int K = blk_K_of(b, bp, false, false);
+    if (K < 0 || blk_plan(b, bp, K, &P) != 0) return nullptr;
     if (dtype == HM_F32) P.pb_wide = 0;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return nullptr;
     if (!P.perbond) return "k_blk_matvec";
@@ -934,6 +939,8 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, int nvec, c
                 return 0;
             }
     }
+    const int Kp = multi ? K : blk_K_of(b, bp, false, false);
+    if (Kp < 0) return 1;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     HM_CUDA(cudaStreamIsCapturing(st, &cs));
     if (multi && cs != cudaStreamCaptureStatusNone) {         // no table of this split: none for the list either
@@ -949,7 +956,7 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, int nvec, c
         if (dtype == HM_F64 && !blk_multi_orders(m->gd, (int)cls.size(), m->oc)) return 1;
     }
     BlkParams &P = m->P;
-    const int rc = blk_plan(b, bp, multi ? K : blk_K_of(b, bp, false, false), &P);
+    const int rc = blk_plan(b, bp, Kp, &P);
     if (rc != 0) return rc;
     if (dtype == HM_F32) P.pb_wide = 0;           // float rows read the float coefficients alone
     const int es = dtype == HM_F64 ? 8 : 4;

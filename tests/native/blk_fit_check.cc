@@ -13,7 +13,7 @@ int main() {
         for (int t = 0; t < nb; ++t)
             if (scanf("%hhu %hhu %d", &p[t], &q[t], &c[t]) != 3) return 1;
         const int K = hm::blk_fitting_K(nb, p.data(), q.data(), c.data(), k0, kmax, sl, sx, sg);
-        printf("%d %d\n", K, (int)hm::blk_slots_fit(nb, p.data(), q.data(), c.data(), K, sl, sx, sg));
+        printf("%d %d\n", K, (int)(K >= 0 && hm::blk_slots_fit(nb, p.data(), q.data(), c.data(), K, sl, sx, sg)));
     }
     return 0;
 }

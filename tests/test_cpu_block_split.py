@@ -52,5 +52,5 @@ def test_split_of_lattices(chosen, name, every_own):
     cls = [0] * len(bonds) if every_own else cls
     k0, kmax = min(max(8, min(15, n // 2 + 2)), n - 2), min(15, n - 2)
     want = [K for K in range(k0, kmax + 1) if fits(bonds, cls, K)]
-    assert chosen(bonds, cls, k0, kmax) == ((want[0], 1) if want else (k0, 0))
+    assert chosen(bonds, cls, k0, kmax) == ((want[0], 1) if want else (-1, 0))
     assert every_own or want[0] == K_classes
