@@ -167,29 +167,31 @@ int make_bonds(const hm_basis *b, int n_bonds, const int32_t *u, const int32_t *
 
 // the device tables of a basis: CD, then per entry (p, S, a) the rank changes {E+, F+, E-, F-}
 // and {G+, G-} of the exchanges that the row sweep reads (hm_row.cuh), zero where there is none
-static std::vector<uint64_t> row_tables(const hm_basis *b) {
+template <class I>
+static std::vector<I> row_tables(const hm_basis *b) {
     const SectorView &v = b->view;
-    const size_t n = (size_t)v.cd_len;
-    std::vector<uint64_t> t(7 * n, 0);
-    std::copy(b->cd.begin(), b->cd.end(), t.begin());
-    auto at = [&](int p, int S, int a) { return b->cd[(size_t)p * v.cd_rowlen + (size_t)S * v.cd_w + a]; };
+    const size_t n = (size_t)v.cd_len, w = (size_t)v.cd_w;
+    std::vector<I> t(7 * n, 0);
+    for (size_t k = 0; k < n; ++k) t[k] = (I)b->cd[k];
     for (int p = 1; p < v.N; ++p)                    // position 0 has no rank term
-        for (int S = 0; S <= v.A; ++S)
-            for (int a = 0; a <= std::min(S, v.S2); ++a) {
-                const uint64_t c = at(p, S, a);
-                uint64_t *e = t.data() + n + 4 * ((size_t)p * v.cd_rowlen + (size_t)S * v.cd_w + a);
-                uint64_t *g = t.data() + 5 * n + 2 * ((size_t)p * v.cd_rowlen + (size_t)S * v.cd_w + a);
-                if (S < v.A) {
-                    if (a < v.S2) e[0] = at(p, S + 1, a + 1) - c;
-                    g[0] = at(p, S + 1, a) - c;
+        for (int S = std::max(0, v.A - v.S2 * (v.N - 1 - p)); S <= std::min(v.A, v.S2 * (p + 1)); ++S) {
+            const size_t k0 = (size_t)p * v.cd_rowlen + (size_t)S * w;
+            const I *c = t.data() + k0, *up = S < v.A ? c + w : nullptr, *dn = S >= 1 ? c - w : nullptr;
+            I *e = t.data() + n + 4 * k0, *g = t.data() + 5 * n + 2 * k0;
+            const int most = std::min(S, v.S2);
+            for (int a = 0; a <= most; ++a) {
+                if (up) {
+                    if (a < v.S2) e[4 * a] = up[a + 1] - c[a];
+                    g[2 * a] = up[a] - c[a];
                 }
-                if (a >= 1) e[1] = at(p, S, a - 1) - c;
-                if (S >= 1) {
-                    if (a >= 1) e[2] = at(p, S - 1, a - 1) - c;
-                    g[1] = at(p, S - 1, a) - c;
+                if (a >= 1) e[4 * a + 1] = c[a - 1] - c[a];
+                if (dn) {
+                    if (a >= 1) e[4 * a + 2] = dn[a - 1] - c[a];
+                    g[2 * a + 1] = dn[a] - c[a];
                 }
-                if (a < v.S2) e[3] = at(p, S, a + 1) - c;
+                if (a < v.S2) e[4 * a + 3] = c[a + 1] - c[a];
             }
+        }
     return t;
 }
 
@@ -362,15 +364,10 @@ int basis_build(int n_sites, int two_s, int two_m, hm_basis **out) {
     int rc = build_tables(n_sites, two_s, two_m, b);
     if (rc < 0) { delete b; return rc; }
     SectorView &v = b->view;
-    const std::vector<uint64_t> tab = row_tables(b);
-    size_t bytes = v.idx64 ? tab.size() * 8 : tab.size() * 4;
-    std::vector<uint32_t> c32;
-    const void *src = tab.data();
-    if (!v.idx64) {
-        c32.resize(tab.size());
-        for (size_t k = 0; k < tab.size(); ++k) c32[k] = (uint32_t)tab[k];
-        src = c32.data();
-    }
+    const std::vector<uint64_t> t64 = v.idx64 ? row_tables<uint64_t>(b) : std::vector<uint64_t>();
+    const std::vector<uint32_t> t32 = v.idx64 ? std::vector<uint32_t>() : row_tables<uint32_t>(b);
+    const size_t bytes = t64.size() * 8 + t32.size() * 4;
+    const void *src = v.idx64 ? (const void *)t64.data() : (const void *)t32.data();
     cudaError_t e = cudaGetDevice(&b->device);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_cd, bytes > 0 ? bytes : 8);
     b->eslots = std::make_shared<ExpSlots>();
