@@ -115,10 +115,10 @@ static long long pb_coef(const BlkParams &P, double h) { return std::llround(std
 
 // Compile-time slots of the thread-per-row kernels (BlkParams::ln ..), when they hold the list (rows_ok).
 static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int K, BlkParams *P) {
-    P->rows_ok = blk_slots_fit(bp.nb, bp.p, bp.q, bc.data(), K, HM_BLK_SL, HM_BLK_SX, HM_BLK_SG) ? 1 : 0;
+    P->rows_ok = blk_slots_fit(bp.nb, bp.p, bp.q, bc.data(), P->perbond, K, HM_BLK_SL, HM_BLK_SX, HM_BLK_SG) ? 1 : 0;
     P->kshift = K - 6;
     if (!P->rows_ok) return;
-    std::map<std::pair<int, int>, uint32_t> cgroups;      // (class, d) -> mask of p
+    std::map<std::tuple<int, int, int>, uint32_t> cgroups;      // (class, d, repetition) -> mask of p
     for (int t = 0; t < bp.nb; ++t) {
         const int c = bc[t], p = bp.p[t], q = bp.q[t];    // p < q
         if (q < K) {
@@ -131,7 +131,7 @@ static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int
             P->lxa[c][ty][n] = (uint16_t)(ty == 0 ? (pat & 255u) << 2 : ty == 2 ? (1u << p) << 2 : 0u);
             P->lxb[c][ty][n] = (uint16_t)(ty == 1 ? (pat >> 8) << 2 : ty == 2 ? (1u << (q - 8)) << 2 : 0u);
             ++n;
-            cgroups[{c, q - p}] |= 1u << p;
+            cgroups[{c, q - p, P->perbond ? 0 : blk_repetition(bp.p, bp.q, bc.data(), t)}] |= 1u << p;
         } else if (p < K) {
             const int ty = p < 8 ? 0 : 1;
             int &n = P->xn[c][ty];
@@ -145,8 +145,8 @@ static void blk_plan_slots(const BondParams &bp, const std::vector<int> &bc, int
         }
     }
     for (auto &kv : cgroups) {
-        const int c = kv.first.first;
-        P->lgd[c][P->lgn[c]] = (uint8_t)kv.first.second;
+        const int c = std::get<0>(kv.first);
+        P->lgd[c][P->lgn[c]] = (uint8_t)std::get<1>(kv.first);
         P->lgm[c][P->lgn[c]] = kv.second;
         ++P->lgn[c];
     }
@@ -278,14 +278,14 @@ static int blk_plan_bonds(hm_basis *b, const BondParams &bp, const std::vector<i
         P->pb_c0 = -(c >> 1);
         P->pb_c0w = (float)(-0.5 * (low + (double)(c & 1)));
     }
-    // low groups keyed by (class, type, d); high and cross bonds by class
-    std::map<std::tuple<int, int, int>, uint32_t> groups;
+    // low groups keyed by (class, type, d, repetition); high and cross bonds by class
+    std::map<std::tuple<int, int, int, int>, uint32_t> groups;
     std::vector<std::tuple<int, int, int>> hi[HM_BLK_MAXC], cr[HM_BLK_MAXC];   // (p, q, bond)
     for (int t = 0; t < bp.nb; ++t) {
         const int p = bp.p[t], q = bp.q[t];  // p < q
         if (q < K) {
             const int type = q < 8 ? 0 : (p >= 8 ? 1 : 2);
-            groups[std::make_tuple(bc[t], type, q - p)] |= 1u << p;
+            groups[std::make_tuple(bc[t], type, q - p, P->perbond ? 0 : blk_repetition(bp.p, bp.q, bc.data(), t))] |= 1u << p;
         } else if (p >= K) {
             hi[bc[t]].push_back({p - K, q - K, t});
         } else {
@@ -514,8 +514,8 @@ static int blk_K_of(const hm_basis *b, const BondParams &bp, bool fp32_run, bool
     if (b->view.S2 != 1 || bp.nb > HM_BLK_MAXB || getenv("HM_BLK_K")) return k0;
     std::vector<double> cls;
     std::vector<int> bc;
-    blk_classes_of(bp, bond_corr, &cls, &bc);
-    return blk_fitting_K(bp.nb, bp.p, bp.q, bc.data(), k0, std::min(15, b->view.N - 2), HM_BLK_SL, HM_BLK_SX, HM_BLK_SG);
+    const bool own = blk_classes_of(bp, bond_corr, &cls, &bc);
+    return blk_fitting_K(bp.nb, bp.p, bp.q, bc.data(), own, k0, std::min(15, b->view.N - 2), HM_BLK_SL, HM_BLK_SX, HM_BLK_SG);
 }
 
 // f(kernel) for the FP64 block-product instance of the plan (class count, integer ratios)

@@ -20,7 +20,7 @@ def ring(n, *distances):
             [k for k in range(len(distances)) for _ in range(n)])
 
 
-# name: (lattice, the split K that holds it with one class for each kind of bond)
+# name: (lattice, the split K that holds it with one class for each kind of bond, if any does)
 LATTICES = {
     "triangular 4x4": (cluster(4, 4, triangular=True), 12),
     "square 6x3": (cluster(6, 3), 12),
@@ -35,4 +35,8 @@ LATTICES = {
     "ring 18, J1 J2": (ring(18, 1, 2), 11),
     "square 4x4": (cluster(4, 4), 10),
     "square 6x4": (cluster(6, 4), 14),
+    # two sites wide: the bonds along y come twice
+    "square 6x2 torus": (cluster(6, 2), 9),
+    "square 8x2 torus": (cluster(8, 2), 12),
+    "triangular 6x2 torus": (cluster(6, 2, triangular=True), None),
 }

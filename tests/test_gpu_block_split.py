@@ -20,7 +20,7 @@ def hm():
     return api
 
 
-SMALL = [k for k in LATTICES if LATTICES[k][0][0] <= 21]
+SMALL = [k for k in LATTICES if LATTICES[k][0][0] <= 21 and LATTICES[k][1]]
 J = [-1.0, -0.625]
 
 
