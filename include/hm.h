@@ -215,17 +215,22 @@ int lanczos_free(hm_lanczos *run);
  * blocks with the top sites varying fastest; bit for bit the one-pass result), "k_blk_lz64" / "k_blk_lz32" (the same block
  * product reading its bonds from the parameters; used when NVRTC is unavailable or the
  * environment sets HM_JIT=0), "k_s1_lz64_jit" / "k_s1_lz32_jit" (s = 1 block product
- * compiled for the bond list), "k_s1_lz32" (its generic FP32 form) or "k_lz_matvec" (row
- * kernel of Eq. E-4-b for any s).  No counterpart in the paper: it reports an
+ * compiled for the bond list), "k_s1_lz32" (its generic FP32 form), "k_lz_matvec" (the
+ * general rows of Eq. E-4-b for any s, by whichever of their two kernels serves: the row sweep
+ * k_lz_row in FP64, else the table form) or "k_mom_matvec" (a momentum basis, likewise
+ * k_mom_row or the table form).  A whole FP64 run of a small sector (lanczos_run) forms the same
+ * rows in one kernel of its own.  No counterpart in the paper: it reports an
  * implementation choice.  HM_EINVAL on NULL. */
 int lanczos_kernel_name(const hm_lanczos *run, char *name, int cap);
 
-/* Name of the kernel `matvec` launches for these arguments (the same dispatch; nothing
+/* Name of the path `matvec` takes for these arguments (the same dispatch; nothing
  * is launched, though a kernel specialised to the bonds may be compiled): "k_blk_matvec"
  * (s = 1/2 block kernel, up to 4 distinct couplings), "k_blk_matvec_jit" (block kernel
  * compiled at run time for a bond list with more distinct couplings), "k_s1_mv_jit" /
  * "k_s1_mv" (s = 1 block kernel compiled for the bond list / generic; FP32, one vector) or
- * "k_matvec" (every other form: general rows, several vectors).  name: host buffer of cap bytes. */
+ * "k_matvec" (every other form: the general rows, by the sweep k_row_matvec or the table form, and
+ * several vectors, whose blocks k_blk_multi takes) or "k_mom_matvec" (a momentum basis: k_mom_row or its
+ * table form).  name: host buffer of cap bytes. */
 int matvec_kernel_name(const hm_basis *basis, int n_bonds, const int32_t *u, const int32_t *v,
                        const double *J, int dtype, int nvec, char *name, int cap);
 
