@@ -60,20 +60,20 @@ __device__ __forceinline__ A lzs_row_pb(const BlkParams &P, const BlkMeta &B, co
 }
 
 // all CTAs past their writes; false when a barrier gave up.  bar[0] counts arrivals (never reset:
-// barrier k ends at k ctas), bar[1] is the abort flag.  A limit of 0 waits for nobody: the CTA that
-// arrives first gives up
+// barrier k ends at k ctas), bar[1] is the abort flag.  A limit of 0 waits for nobody: CTAs that
+// are not alone give up
 __device__ __forceinline__ bool lzs_barrier(unsigned *bar, unsigned target, unsigned long long limit_ns) {
     __shared__ int s_ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        const unsigned here = atomicAdd(bar, 1u) + 1u;
+        atomicAdd(bar, 1u);
         volatile unsigned *v = bar;
         int ok = 1;
-        if (here < target && limit_ns == 0) {
+        if (limit_ns == 0 && gridDim.x > 1) {
             atomicExch(bar + 1, 1u);
             ok = 0;
-        } else if (here < target) {
+        } else if (*v < target) {
             unsigned long long t0, t;
             asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
             for (unsigned spin = 1; *v < target; ++spin) {
