@@ -28,8 +28,8 @@ struct BlkParams {
     double g0;
     float g0_hi, g0_lo;
     // low bonds grouped by (class, byte type, distance d): mask of start positions p;
-    // type 0: both ends in byte 0, 1: both in byte 1, 2: across the bytes.  Groups of
-    // class c and type t are [lg_cs[3c+t], lg_cs[3c+t+1]).
+    // type 0: both ends in byte 0, 1: both in byte 1, 2: across the bytes; the second copy of a
+    // repeated bond is in a group of its own.  Groups of class c and type t are [lg_cs[3c+t], lg_cs[3c+t+1]).
     int nlg, lg_cs[3 * HM_BLK_MAXC + 1];
     uint32_t lg_mask[HM_BLK_MAXG];
     uint8_t lg_d[HM_BLK_MAXG];

@@ -1,5 +1,5 @@
-"""GPU test of the bounded grid barriers of the whole-run kernel (csrc/lz_small.cu): with a limit of 0 ns the
-CTA that arrives first gives up, every CTA returns, and the call reports HM_ETIMEOUT (no fault, no hang);
+"""GPU test of the bounded grid barriers of the whole-run kernel (csrc/lz_small.cu): with a limit of 0 ns no
+CTA waits for another, every CTA returns, and the call reports HM_ETIMEOUT (no fault, no hang);
 the next call on the same device is correct."""
 import numpy as np
 import pytest
