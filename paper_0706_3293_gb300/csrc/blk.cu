@@ -518,6 +518,33 @@ static int blk_K_of(const hm_basis *b, const BondParams &bp, bool fp32_run, bool
     return blk_fitting_K(bp.nb, bp.p, bp.q, bc.data(), own, k0, std::min(15, b->view.N - 2), HM_BLK_SL, HM_BLK_SX, HM_BLK_SG);
 }
 
+// The same, and the list to plan: where no split holds the bonds as they come, those of a repeated pair as one with the
+// sum of their couplings (fewer slots), in merged.
+static int blk_K_and_list(const hm_basis *b, const BondParams &bp, bool fp32_run, BondParams *merged, const BondParams **list) {
+    *list = &bp;
+    const int K = blk_K_of(b, bp, fp32_run, false);
+    if (K >= 0) return K;
+    merged->nb = 0;
+    for (int t = 0; t < bp.nb; ++t) {
+        int i = 0;
+        while (i < merged->nb && (merged->p[i] != bp.p[t] || merged->q[i] != bp.q[t])) ++i;
+        if (i == merged->nb) {
+            merged->p[i] = bp.p[t];
+            merged->q[i] = bp.q[t];
+            merged->jm[i] = 0.0;
+            ++merged->nb;
+        }
+        merged->jm[i] += bp.jm[t];
+    }
+    if (merged->nb == bp.nb) return -1;
+    merged->S2 = bp.S2;
+    memcpy(merged->hs_pdn, bp.hs_pdn, sizeof merged->hs_pdn);
+    memcpy(merged->hs_pup, bp.hs_pup, sizeof merged->hs_pup);
+    for (int t = 0; t < merged->nb; ++t) merged->jmf[t] = (float)merged->jm[t];
+    *list = merged;
+    return blk_K_of(b, *merged, fp32_run, false);
+}
+
 // f(kernel) for the FP64 block-product instance of the plan (class count, integer ratios)
 template <class F>
 static int lz64_dispatch(const BlkParams &P, F &&f) {
@@ -539,9 +566,11 @@ static int set_smem(K_t kern, size_t sm) {
 
 // Lanczos hooks: plan (0 = block path usable), attribute setup, launch
 int blk_lz_plan(hm_basis *b, const BondParams &bp, int dtype, BlkParams *P, int *blocks) {
-    const int K = blk_K_of(b, bp, dtype == HM_F32, false);
+    BondParams merged;
+    const BondParams *list;
+    const int K = blk_K_and_list(b, bp, dtype == HM_F32, &merged, &list);
     if (K < 0) return 1;
-    int rc = blk_plan(b, bp, K, P);
+    int rc = blk_plan(b, *list, K, P);
     if (rc != 0) return rc;
     if (dtype == HM_F32) P->pb_wide = 0;          // float rows read the float coefficients alone
     const size_t sm = blk_row_smem_bytes(*P, dtype == HM_F64 ? 8 : 4, BLK_XPAD);
@@ -877,8 +906,10 @@ int blk_bond_corr(hm_basis *b, const BondParams &bp, const void *g, const void *
 const char *blk_matvec_kernel(hm_basis *b, const BondParams &bp, int dtype, int nvec) {
     if (nvec != 1) return nullptr;
     BlkParams P;
-    const int K = blk_K_of(b, bp, false, false);
-    if (K < 0 || blk_plan(b, bp, K, &P) != 0) return nullptr;
+    BondParams merged;
+    const BondParams *list;
+    const int K = blk_K_and_list(b, bp, false, &merged, &list);
+    if (K < 0 || blk_plan(b, *list, K, &P) != 0) return nullptr;
     if (dtype == HM_F32) P.pb_wide = 0;
     if (!P.rows_ok || blk_row_smem_bytes(P, dtype == HM_F64 ? 8 : 4, BLK_XPAD) > 200 * 1024) return nullptr;
     if (!P.perbond) return "k_blk_matvec";
@@ -939,7 +970,9 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, int nvec, c
                 return 0;
             }
     }
-    const int Kp = multi ? K : blk_K_of(b, bp, false, false);
+    BondParams merged;
+    const BondParams *list = &bp;
+    const int Kp = multi ? K : blk_K_and_list(b, bp, false, &merged, &list);
     if (Kp < 0) return 1;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     HM_CUDA(cudaStreamIsCapturing(st, &cs));
@@ -956,7 +989,7 @@ static int blk_mv_plan(hm_basis *b, const BondParams &bp, int dtype, int nvec, c
         if (dtype == HM_F64 && !blk_multi_orders(m->gd, (int)cls.size(), m->oc)) return 1;
     }
     BlkParams &P = m->P;
-    const int rc = blk_plan(b, bp, Kp, &P);
+    const int rc = blk_plan(b, *list, Kp, &P);
     if (rc != 0) return rc;
     if (dtype == HM_F32) P.pb_wide = 0;           // float rows read the float coefficients alone
     const int es = dtype == HM_F64 ? 8 : 4;

@@ -81,12 +81,19 @@ def test_products_and_runs(hm, name, row, monkeypatch):
 
 
 @pytest.mark.parametrize("parity", [1, -1])
-@pytest.mark.parametrize("name", [k for k in NAMES if "triangular" not in k])
+@pytest.mark.parametrize("name", NAMES)                  # the triangular torus fits with its repeated bonds as one
 def test_spin_flip_blocks(hm, name, parity):
     n, bl, obl = case(hm, name)
     b, ob = hm.Basis(n, 1, 0, parity=parity), oracle.Basis(n, 1, n // 2)
     x = oracle.start_uniform(3, b.dim)
-    assert rel(hm.matvec(b, bl, torch.from_numpy(x).cuda()).cpu().numpy(), oracle.flip_matvec(ob, obl, x, parity)) <= 1e-12
+    xd = torch.from_numpy(x).cuda()
+    ref = oracle.flip_matvec(ob, obl, x, parity)
+    assert rel(hm.matvec(b, bl, xd).cpu().numpy(), ref) <= 1e-12
+    assert rel(hm.matvec(b, bl, xd.float()).double().cpu().numpy(), ref) <= 1e-5
+    q = x / np.linalg.norm(x)
+    first = q @ oracle.flip_matvec(ob, obl, q, parity)
+    for dt, tol in ((torch.float64, 1e-11), (torch.float32, 2e-5)):
+        assert abs(hm.lanczos_run(b, bl, 4, v0=xd.to(dt), dtype=dt).alpha[0] - first) <= tol * np.abs(bl.J).sum()
 
 
 @pytest.mark.parametrize("name", [k for k in NAMES if k.split()[0] == "12" and "bonds" not in k] + ["square 6x2 torus"])
